@@ -256,8 +256,8 @@ d2o_status d2o_full_decode_step(int32_t dtype, int32_t d_head, int32_t n_slices,
  * process whose memory pool has already claimed the whole device, in a plugin that is handed
  * tensors but no allocator, or between the steps of a latency-critical loop where an allocation
  * would synchronise the device.  d2o_layer_stats needs a scratch buffer for the softmax row
- * normalisers of the prompt attention; here that buffer is a fixed array of
- * D2O_STATIC_LSE_FLOATS floats (4 MiB) that is part of the library image, so every GPU that
+ * normalisers of the prompt attention; here that buffer is a fixed array of about
+ * D2O_STATIC_LSE_FLOATS floats (4.75 MiB with the padding of its rows) that is part of the library image, so every GPU that
  * loads the library carries it until the process exits.  No context, no workspace: the caller
  * passes the inputs and the outputs only.
  *
@@ -265,11 +265,10 @@ d2o_status d2o_full_decode_step(int32_t dtype, int32_t d_head, int32_t n_slices,
  *   colsum DEVICE float [B, Hq, P] (out: column sums of the causal prompt attention, Eq. 4);
  *   density DEVICE double [B, Hq] (out: F_v = Var(colsum) per query head).
  *
- * It always runs the generic kernels (fp32 arithmetic on CUDA cores, any dtype, any prompt
- * length).  d2o_layer_stats runs the same kernels, and then returns bit-identical results, for
- * fp32 inputs, for a prompt length that is not a multiple of 4, or with stats_path = 1; for
- * 16-bit inputs it otherwise takes its tensor-core kernels, which are several times faster and
- * agree with this entry point to rounding (column sums within 2e-4 relative).
+ * It runs the kernels that d2o_layer_stats runs with its default tuning (tensor cores for 16-bit
+ * inputs, fp32 arithmetic on CUDA cores for fp32 inputs; any prompt length) and returns
+ * bit-identical results.  It has no error word: should a device-side wait run out, the column sums
+ * concerned are NaN.
  *
  * Limit: batch * n_q_heads * prompt_len <= D2O_STATIC_LSE_FLOATS and batch * n_q_heads <= 65535,
  * else D2O_ERR_TOO_LARGE and nothing is launched.  The call neither allocates nor frees device

@@ -358,7 +358,7 @@ def d2o_layer_stats_static(Q: torch.Tensor, K: torch.Tensor, colsum: torch.Tenso
 
     For callers that must not allocate device memory while the library works (a serving process
     whose pool owns the whole GPU, a plugin without an allocator): the library's only scratch is
-    a fixed 4 MiB array inside its own image.  The caller provides every tensor, outputs included:
+    a fixed array of about 4.75 MiB inside its own image.  The caller provides every tensor, outputs included:
     Q [B, Hq, P, d], K [B, Hkv, P, d], colsum float32 [B, Hq, P], density float64 [B, Hq].
     Raises D2OError (status 7) if B * Hq * P exceeds STATIC_LSE_FLOATS.  Calls that overlap on the
     GPU share the scratch array and race; make the first call on a device outside stream capture."""

@@ -31,12 +31,15 @@ constexpr int kCsStages = 4;                 // B ring
 enum { kSweepRows = 0, kSweepCols = 1 };
 
 struct ColsumTcArgs {
-  float* lse2;                               // [B, Hq, P] log2-domain row normalisers (written by sweep 1, read by sweep 2)
+  float* lse2;                               // [B * Hq][lse_row(P)] log2-domain row normalisers (sweep 1 -> sweep 2)
   float* colsum;                             // [B, Hq, P] (sweep 2)
-  uint32_t* status;
-  const int32_t* plen;                       // [B] prompt length of every sequence (<= P)
+  uint32_t* status;                          // NULL: no error word (the allocation-free entry point)
+  const int32_t* plen;                       // [B] prompt length of every sequence (<= P); NULL: all P
   int P, Hq, group;                          // P: the length the tensors are laid out for
 };
+
+// Row stride of the normalisers: the bulk copies of sweep 2 start on 16-byte boundaries whatever the prompt length.
+__host__ __device__ __forceinline__ size_t lse_row(int P) { return (size_t)((P + 3) & ~3); }
 
 namespace tc {
 // global -> this CTA's shared memory, 16-byte aligned on both sides, size a multiple of 16
@@ -79,7 +82,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int bh = blockIdx.x;                                 // b * Hq + hq (fastest index: all heads of the heaviest pair first)
   const int b = bh / a.Hq, hq = bh % a.Hq;
-  const int P = a.plen[b];                                   // this sequence's prompt; rows beyond it are padding
+  const int P = a.plen ? a.plen[b] : a.P;                                   // this sequence's prompt; rows beyond it are padding
   const int n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile);
   const int n_tiles = (P + kCsTile - 1) / kCsTile;
   if ((int)blockIdx.y >= n_pairs) return;                    // the grid is sized for the longest prompt
@@ -94,7 +97,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   const int bt1 = SWEEP == kSweepRows ? min(n_tiles, (a0 + 2 * kCsTile) / kCsTile) : n_tiles;
   const int n_jobs = bt1 - bt0;
   if ((tc::smem_u32(cs_smem) & 1023u) != 0u) {               // swizzled tiles need 1024-byte aligned shared memory
-    if (tid == 0) report_error(a.status, D2O_ERR_STATE, 0xC5C10000u);
+    if (tid == 0 && a.status) report_error(a.status, D2O_ERR_STATE, 0xC5C10000u);
     return;
   }
 
@@ -137,7 +140,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         tc::mbar_expect_tx(&b_full[s], bytes);
         for (int kb = 0; kb < KB; ++kb)
           tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
-        if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, a.lse2 + (size_t)bh * a.P + r0, (uint32_t)(n_lse * 4), &b_full[s]);
+        if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, a.lse2 + bh * lse_row(a.P) + r0, (uint32_t)(n_lse * 4), &b_full[s]);
       }
     }
   } else if (warp == 1) {
@@ -251,7 +254,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         if (lane == 0) tc::mbar_arrive(&b_empty[s]);
       }
     }
-    // combine the two warps that share an A row (B-row halves), fixed order
+    // combine the two warps that share an A row (B-row halves), fixed order; after a wait that ran out: NaN
     const int r = quarter * 32 + lane;
     if (SWEEP == kSweepRows) {
       if (bhalf == 1) { s_comb[(at * 2 + 0) * kCsTile + r] = m_run; s_comb[(at * 2 + 1) * kCsTile + r] = l_run; }
@@ -261,13 +264,14 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         const float mm = fmaxf(m_run, m2);
         const float ll = (m_run > -INFINITY ? l_run * exp2f((m_run - mm) * c) : 0.f) +
                          (m2 > -INFINITY ? l2 * exp2f((m2 - mm) * c) : 0.f);
-        a.lse2[(size_t)bh * a.P + arow] = fmaf(mm, c, log2f(ll));
+        a.lse2[bh * lse_row(a.P) + arow] = s_fail ? NAN : fmaf(mm, c, log2f(ll));
       }
     } else {
       double* dcomb = reinterpret_cast<double*>(s_comb);
       if (bhalf == 1) dcomb[at * kCsTile + r] = col_acc;
       asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
-      if (bhalf == 0 && arow < P) a.colsum[(size_t)bh * a.P + arow] = (float)(col_acc + dcomb[at * kCsTile + r]);
+      if (bhalf == 0 && arow < P) 
+        a.colsum[(size_t)bh * a.P + arow] = s_fail ? NAN : (float)(col_acc + dcomb[at * kCsTile + r]);
     }
   }
   tc::fence_before_sync();
@@ -276,39 +280,39 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem_base, 512);
   }
-  if (tid == 0 && s_fail) report_error(a.status, D2O_ERR_TIMEOUT, 0xC5C00000u | (uint32_t)(bh & 0xfffff));
+  if (tid == 0 && s_fail && a.status) report_error(a.status, D2O_ERR_TIMEOUT, 0xC5C00000u | (uint32_t)(bh & 0xfffff));
 }
 
-// natural-log row normalisers supplied by the caller -> log2 domain
-__global__ void lse_to_log2_kernel(const float* __restrict__ lse, float* __restrict__ lse2, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) lse2[i] = lse[i] * kLog2e;
+// natural-log row normalisers supplied by the caller -> log2 domain, padded rows; one (sequence, head) per blockIdx.x
+__global__ void lse_to_log2_kernel(const float* __restrict__ lse, float* __restrict__ lse2, int P) {
+  const int i = blockIdx.y * blockDim.x + threadIdx.x;
+  if (i < P) lse2[blockIdx.x * lse_row(P) + i] = lse[(size_t)blockIdx.x * P + i] * kLog2e;
 }
 
-bool colsum_tc_supported(const d2o_config* cfg) {
-  return cfg->dtype != D2O_F32 && cfg->prompt_len % 4 == 0;
-}
+size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P) { return (size_t)batch * n_q_heads * lse_row(P) * 4; }
 
-// Column sums of one layer on the tensor cores.  `lse_in` (natural log, may be NULL) replaces sweep 1.
-cudaError_t launch_colsum_tc(const d2o_ctx* c, const void* Q, const void* K, const float* lse_in, float* colsum,
-                             cudaStream_t st, int lane) {
-  const d2o_config& g = c->cfg;
-  const int B = g.batch, Hq = g.n_q_heads, Hkv = g.n_kv_heads, P = g.prompt_len, D = g.d_head;
+// Column sums of one layer of 16-bit Q, K on the tensor cores.  `lse_in` (natural log, may be NULL) replaces sweep 1;
+// `lse2` is scratch of colsum_tc_lse_bytes(); `plen` (DEVICE, may be NULL) holds every sequence's prompt length,
+// `status` (may be NULL) the error word.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that
+// are not a multiple of four used to take the FFMA kernels: 17.5 ms instead of 1.1 for two layers of 6001 tokens.)
+cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
+                             const float* lse_in, float* lse2, float* colsum, const int32_t* plen, uint32_t* status,
+                             cudaStream_t st) {
   CUtensorMap map_q, map_k;
-  if (!encode_rows_2d(&map_q, g.dtype, Q, (uint64_t)B * Hq * P, D, kCsTile)) return cudaErrorNotSupported;
-  if (!encode_rows_2d(&map_k, g.dtype, K, (uint64_t)B * Hkv * P, D, kCsTile)) return cudaErrorNotSupported;
+  if (!encode_rows_2d(&map_q, dtype, Q, (uint64_t)B * Hq * P, D, kCsTile)) return cudaErrorNotSupported;
+  if (!encode_rows_2d(&map_k, dtype, K, (uint64_t)B * Hkv * P, D, kCsTile)) return cudaErrorNotSupported;
   ColsumTcArgs a;
-  a.lse2 = (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride);
+  a.lse2 = lse2;
   a.colsum = colsum;
-  a.status = (uint32_t*)(c->state + c->lay.status);
-  a.P = P; a.Hq = Hq; a.group = c->group;
-  a.plen = (const int32_t*)(c->state + c->lay.plen);
+  a.status = status;
+  a.P = P; a.Hq = Hq; a.group = Hq / Hkv;
+  a.plen = plen;
   const int KB = D / 64;
   const size_t smem = (size_t)(2 + kCsStages) * KB * kCsTile * 128 + (size_t)kCsStages * kCsTile * 4 + 4 * kCsTile * 4;
   const int n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile);
   // heaviest CTAs first over the whole launch: the pair index is the slow grid dimension
   dim3 grid(B * Hq, n_pairs);
-  const int fmt = g.dtype == D2O_F16 ? 0 : 1;
+  const int fmt = dtype == D2O_F16 ? 0 : 1;
   cudaError_t e;
 #define D2O_LAUNCH_CS(DD, FF, SW)                                                                                  \
   do {                                                                                                             \
@@ -322,8 +326,7 @@ cudaError_t launch_colsum_tc(const d2o_ctx* c, const void* Q, const void* K, con
     else          { if (fmt == 0) D2O_LAUNCH_CS(64, 0, SW); else D2O_LAUNCH_CS(64, 1, SW); }     \
   } while (0)
   if (lse_in) {
-    const size_t n = (size_t)B * Hq * P;
-    lse_to_log2_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(lse_in, a.lse2, n);
+    lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256)), 256, 0, st>>>(lse_in, lse2, P);
   } else {
     D2O_LAUNCH_CS_ALL(kSweepRows);
   }

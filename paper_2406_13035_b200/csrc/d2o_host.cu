@@ -118,7 +118,7 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   l->vpool = take(rows * d * e);
   l->end = o;
   o = 0;
-  s->lse = take(B * Hq * P * 4);
+  s->lse = take(colsum_tc_lse_bytes(c->batch, c->n_q_heads, c->prompt_len));
   s->lse_stride = o - s->lse;
   o += (size_t)(kStatsLanes - 1) * s->lse_stride;
   s->evict_idx = take(B * Hkv * P * 4);

@@ -390,8 +390,10 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
   float* colsum = (float*)(c->state + c->lay.colsum) + (size_t)layer * B * Hq * P;
   double* density = (double*)(c->state + c->lay.density);
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
-  if (c->stats_path == 0 && colsum_tc_supported(&g)) {
-    cudaError_t e = launch_colsum_tc(c, Q, K, lse_in, colsum, st, lane);
+  if (c->stats_path == 0 && g.dtype != D2O_F32) {
+    cudaError_t e = launch_colsum_tc(g.dtype, D, B, Hq, g.n_kv_heads, P, Q, K, lse_in,
+                                     (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride), colsum, plen,
+                                     (uint32_t*)(c->state + c->lay.status), st);
     if (e != cudaSuccess) return e;
     density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, g.n_layers, layer, plen);
     return cudaGetLastError();
@@ -444,14 +446,22 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
 }
 
 // ------------------------------------------------------------------------------------ allocation-free variant
-// Scratch for the row normalisers of d2o_layer_stats_static: part of the library image, one copy per GPU.
-static __device__ __align__(256) float g_static_lse[D2O_STATIC_LSE_FLOATS];
+// Scratch for the row normalisers of d2o_layer_stats_static: part of the library image, one copy per GPU.  The
+// tensor-core kernels pad every (sequence, head) row to a multiple of four floats.
+constexpr int kStaticMaxRows = 65535;                // (sequence, head) pairs: one grid row of the generic kernels each
+static __device__ __align__(256) float g_static_lse[D2O_STATIC_LSE_FLOATS + 3 * kStaticMaxRows];
 constexpr int kMaxDevices = 64;
 static float* g_static_lse_addr[kMaxDevices];        // device address of g_static_lse, per device (host-side cache)
 
 template <typename T, int D>
-static cudaError_t run_stats_static(const void* Q, const void* K, float* lse_buf, float* colsum, double* density, int B,
-                                    int Hq, int group, int P, cudaStream_t st) {
+static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, float* lse_buf, float* colsum, double* density,
+                                    int B, int Hq, int group, int P, cudaStream_t st) {
+  if (sizeof(T) == 2) {
+    cudaError_t e = launch_colsum_tc(dtype, D, B, Hq, Hq / group, P, Q, K, nullptr, lse_buf, colsum, nullptr, nullptr, st);
+    if (e != cudaSuccess) return e;
+    density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
+    return cudaGetLastError();
+  }
   const int nT = (P + kTile - 1) / kTile;
   dim3 grid(nT, B * Hq);
   const size_t sm = (size_t)2 * D * kTile * sizeof(float);
@@ -480,7 +490,7 @@ extern "C" d2o_status d2o_layer_stats_static(int32_t dtype, int32_t d_head, int3
   if (!aligned16(Q) || !aligned16(K) || !aligned16(colsum) || !density || ((uintptr_t)density & 7)) return D2O_ERR_INVALID_ARG;
   if ((unsigned long long)batch * n_q_heads * prompt_len > (unsigned long long)D2O_STATIC_LSE_FLOATS)
     return D2O_ERR_TOO_LARGE;
-  if ((long long)batch * n_q_heads > 65535) return D2O_ERR_TOO_LARGE;      // one grid row per (sequence, head)
+  if ((long long)batch * n_q_heads > kStaticMaxRows) return D2O_ERR_TOO_LARGE;      // one grid row per (sequence, head)
   // set-up, once per device: in host code `g_static_lse` is only a handle, the kernels need its device address
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
@@ -496,16 +506,16 @@ extern "C" d2o_status d2o_layer_stats_static(int32_t dtype, int32_t d_head, int3
   cudaStream_t st = (cudaStream_t)stream;
   switch (dtype) {
     case D2O_F32:
-      e = d_head == 64 ? run_stats_static<float, 64>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
-                       : run_stats_static<float, 128>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
+      e = d_head == 64 ? run_stats_static<float, 64>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
+                       : run_stats_static<float, 128>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
       break;
     case D2O_F16:
-      e = d_head == 64 ? run_stats_static<__half, 64>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
-                       : run_stats_static<__half, 128>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
+      e = d_head == 64 ? run_stats_static<__half, 64>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
+                       : run_stats_static<__half, 128>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
       break;
     default:
-      e = d_head == 64 ? run_stats_static<__nv_bfloat16, 64>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
-                       : run_stats_static<__nv_bfloat16, 128>(Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
+      e = d_head == 64 ? run_stats_static<__nv_bfloat16, 64>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st)
+                       : run_stats_static<__nv_bfloat16, 128>(dtype, Q, K, lse_buf, colsum, density, batch, n_q_heads, group, prompt_len, st);
   }
   if (e != cudaSuccess) return record_cuda_error(e, "d2o_layer_stats_static launch");
   return D2O_OK;

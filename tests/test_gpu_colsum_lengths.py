@@ -1,0 +1,51 @@
+"""Column sums of the prompt attention (Eq. 4) at prompt lengths around the tile edges of the tensor-core kernels and at
+lengths that are no multiple of anything, against the attention in float64.
+
+Tolerance: the logits are exact products of 16-bit values summed in fp32 (relative error about d * 2^-24 of the sum of
+their magnitudes, here below 4e-6 of a logit of magnitude ~10), one exponential (2^-22) and fp32 / fp64 sums: 2e-5 of a
+column sum covers it four times."""
+import math
+
+import pytest
+import torch
+
+from paper_2406_13035_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+def _reference(Q, K):
+    q, k = Q.double(), K.double().repeat_interleave(Q.shape[1] // K.shape[1], 1)
+    x = q @ k.transpose(-1, -2) / math.sqrt(Q.shape[-1])
+    P = Q.shape[2]
+    x = x.masked_fill(torch.ones(P, P, dtype=torch.bool, device=x.device).triu(1), float("-inf"))
+    return x, torch.softmax(x, -1).sum(-2)
+
+
+def _context(dtype, b, hq, hkv, d, P):
+    return B.D2OContext(B.make_config(n_layers=1, batch=b, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=P,
+                                      max_new_tokens=8, rho=1.0, n_sink=0, min_budget=1))
+
+
+@pytest.mark.parametrize("P", [1, 2, 31, 63, 64, 65, 127, 129, 191, 255, 257, 321, 383, 514, 769, 1023, 1281])
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f16", 64)])
+def test_colsum_at_any_prompt_length(cuda_device, dtype, d, P):
+    b, hq, hkv = 2, 4, 2
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    Q = (1.5 * torch.randn(b, hq, P, d, generator=g, device=cuda_device)).to(td)
+    K = torch.randn(b, hkv, P, d, generator=g, device=cuda_device).to(td)
+    logits, ref = _reference(Q, K)
+    ctx = _context(dtype, b, hq, hkv, d, P)
+    ctx.d2o_layer_stats(0, Q, K)
+    own = ctx.colsum(0).clone()
+    assert float(((own.double() - ref).abs() / ref).max()) < 2e-5
+    # the normalisers of the caller's own attention kernel; rounded to fp32 (2^-24 of about 10) by the caller
+    ctx.d2o_layer_stats(0, Q, K, torch.logsumexp(logits, -1).float().contiguous())
+    assert float(((ctx.colsum(0).double() - ref).abs() / ref).max()) < 2e-5
+    assert ctx.d2o_get_stats().error_word == 0
+    # the allocation-free entry point runs the same kernels
+    cs = torch.empty(b, hq, P, device=cuda_device)
+    F = torch.empty(b, hq, dtype=torch.float64, device=cuda_device)
+    B.d2o_layer_stats_static(Q, K, cs, F)
+    assert torch.equal(cs, own)
