@@ -166,6 +166,7 @@ struct d2o_ctx {
   int elem_size;
   int max_budget;
   int n_sms;                   // multiprocessors of the device the context was created on
+  int max_cluster;             // largest thread-block cluster of decode_split_kernel there
   int64_t total_budget;        // S_tot per sequence = round(rho * L * P)
   int64_t pool_rows;           // B * Hkv * S_tot
   d2o::Layout lay;
@@ -183,6 +184,7 @@ struct d2o_ctx {
   uint8_t* layer_fed;          // [L] stats seen
   uint8_t* layer_compressed;   // [L]
   int32_t* layer_steps;        // [L] decode steps taken
+  uint8_t* layer_published;    // [L] the slices' step counters of the last decode step were (or will be) written
   int32_t* h_plen;             // [B] prompt length of every sequence (prompt_len unless d2o_set_prompt_lens was called)
   int32_t* h_sim_count;        // [L] work items of the tensor-core similarity kernel per layer
   int4* h_sim_items;           // host copy of the work lists (device copy in `state`)

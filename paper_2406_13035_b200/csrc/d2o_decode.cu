@@ -32,6 +32,7 @@
 #include <cuda/std/type_traits>
 
 #include "d2o_common.cuh"
+#include "d2o_decode.cuh"
 #include "d2o_tc.cuh"
 
 namespace d2o {
@@ -42,125 +43,10 @@ namespace d2o {
 // vectors per stage.
 __host__ __device__ constexpr int stage_bytes_of(int cw) { return 4 * cw * 32 * 16; }
 constexpr int kMaxStages = 12;
-constexpr unsigned long long kWaitNs = 1000000000ull;   // an mbarrier wait gives up after 1 s
 constexpr int kTensorMinG = 2;                          // query heads per KV head from which the tensor-core path is used
-constexpr uint32_t kSuspendNs = 4000u;                  // a waiting thread may stay suspended this long before it looks again
 
-struct DecodeArgs {
-  const int32_t* budgets; const int32_t* windows; const int64_t* row_off;   // [B, L, Hkv]
-  int32_t* pos; float* score; float* rnorm;                                  // pool-wide
-  int32_t* len; float* tau;                                                  // [L, B, Hkv]
-  unsigned long long* counters; uint32_t* status;
-  const int32_t* plen;              // [B] prompt length of every sequence
-  int L, l0, B, Hkv, T, step;       // step = number of tokens generated before this one: its position is plen[b] + step
-  float beta, tau_override;
-  int row_cap;                      // rows of a slice whose logits / probabilities live in shared memory (multiple of 8)
-  float* spill;                     // the same for rows >= row_cap: [(row0 + 8 slice) G + g (stride(S) + 8) + row], stays in L2
-  int stages;                       // stages of the ring
-  int l2_hints;                     // 1: the streamed rows are marked evict-first in L2 (each is read once per step)
-  const int32_t* order;             // NULL: CTAs take (layer, b, h) in index order; else (layer * B + b) per group of Hkv CTAs
-  int pair_base;                    // first entry of `order` this launch works on
-  int average;                      // 1: average merge (both rows weigh 1/2) instead of the weights of Eq. 12
-  unsigned long long wait_ns;       // a wait for a stage gives up after this long
-  int stop_stage;                   // failure-detection tests: the producer issues no copy from this stage on (-1: never)
-  long long pool_rows;              // rows of the cache pool (bounds of the checked build)
-  int32_t* steps_done;              // [L, B, Hkv] decode steps completed on the slice: written as a CTA's last act
-  int chained;                      // 1: the previous step's grids may still be running (see slice_ready)
-  int publish;                      // 1: a chained step follows: the CTA publishes the slice's step counter at its end
-};
-
-// ----------------------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long global_ns() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
 template <int CW>
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(CW * 32) : "memory"); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs) : "memory");
-  return ok != 0;
-}
-// Wait for a stage in the kernel's loops: one probe when the phase is already complete (the common case); otherwise
-// poll until it completes, another thread has recorded a timeout, or this one does.
-__device__ __forceinline__ void stage_wait(unsigned long long* bar, uint32_t parity, volatile int* timeout,
-                                           unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return;
-  const unsigned long long t0 = global_ns();
-  while (*timeout == 0) {
-    if (mbar_try_wait(bar, parity)) return;
-    if (global_ns() - t0 > limit_ns) { *timeout = 2; return; }
-  }
-}
-// The same without giving up early when another thread has recorded a timeout: used by the producer to see its own
-// copies land before it leaves.  false = the limit ran out.
-__device__ __forceinline__ bool landed_wait(unsigned long long* bar, uint32_t parity, unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (global_ns() - t0 > limit_ns) return false;
-  return true;
-}
-// Waits, with a limit, until the slice's step counter has reached `want`: the CTA that ran the slice's previous
-// decode step has finished and its stores are visible.  0: ready; 1: an anomaly was recorded meanwhile (the state is
-// no longer trusted); 2: the wait ran out.
-__device__ __forceinline__ int slice_ready(const int32_t* flag, int want, const uint32_t* status, unsigned long long limit_ns) {
-  const unsigned long long t0 = global_ns();
-  for (;;) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-    if (v >= want) return 0;
-    if (*reinterpret_cast<const volatile uint32_t*>(status) != 0u) return 1;
-    if (global_ns() - t0 > limit_ns) return 2;
-    __nanosleep(200);
-  }
-}
-// Similarity as an ordered key: -0 (a zero-norm row times a negative dot product) must count as +0, or equal
-// similarities would not tie.
-__device__ __forceinline__ uint32_t sim_ord(float u) { return float_ord(__fadd_rn(u, 0.f)); }
-// d = a * b + c on two fp32 lanes at once (one issue slot instead of two)
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<const unsigned long long*>(&a)), "l"(*reinterpret_cast<const unsigned long long*>(&b)),
-        "l"(*reinterpret_cast<const unsigned long long*>(&c)));
-  return *reinterpret_cast<float2*>(&d);
-}
-// dot product of two pieces of N floats each, accumulated in two interleaved fp32 chains
-template <int N>
-__device__ __forceinline__ float dot_pairs(const float (&a)[N], const float (&b)[N]) {
-  float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int i = 0; i < N; i += 2) acc = ffma2(make_float2(a[i], a[i + 1]), make_float2(b[i], b[i + 1]), acc);
-  return acc.x + acc.y;
-}
-// next slot of the ring; the parity flips on wrap-around
-__device__ __forceinline__ void ring_next(int& slot, uint32_t& ph, int stages) {
-  if (++slot == stages) { slot = 0; ph ^= 1u; }
-}
-// global -> this CTA's shared memory, 16-byte aligned on both sides, size a multiple of 16
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32_t bytes, unsigned long long* bar,
-                                              unsigned long long policy) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy) : "memory");
-}
 
 // 2-D tiled load with an L2 eviction-priority hint; x = innermost coordinate (elements), y = row
 __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y, unsigned long long* bar,
@@ -189,25 +75,6 @@ __device__ __forceinline__ void block_arg_extreme(unsigned long long key, int li
     }
     *s_out_key = b; *s_out_li = bl;
   }
-}
-
-// Sums four values, each spread over the LPR lanes of a row group, with 3 + log2(LPR/4) shuffles instead of
-// 4*log2(LPR): lanes trade halves of the batch first.  Lane `lig` returns the total of value lig / (LPR/4).
-// All 32 lanes of the warp must call it.
-template <int LPR>
-__device__ __forceinline__ float reduce4(float s0, float s1, float s2, float s3, int lig) {
-  const bool hi = (lig & (LPR / 2)) != 0;
-  float k0 = hi ? s2 : s0, k1 = hi ? s3 : s1;
-  const float t0 = hi ? s0 : s2, t1 = hi ? s1 : s3;
-  k0 += __shfl_xor_sync(0xffffffffu, t0, LPR / 2);
-  k1 += __shfl_xor_sync(0xffffffffu, t1, LPR / 2);
-  const bool hi2 = (lig & (LPR / 4)) != 0;
-  float k = hi2 ? k1 : k0;
-  const float t = hi2 ? k0 : k1;
-  k += __shfl_xor_sync(0xffffffffu, t, LPR / 4);
-#pragma unroll
-  for (int o = LPR / 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  return k;
 }
 
 // One warp-level tensor-core step for the logits of 16 rows against up to 8 heads: acc (16 x 8, fp32) += A (16 rows x
@@ -1375,6 +1242,26 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     return min(c->h_pair_max[(pr % B) * L + pr / B], t_now) + 1;
   };
 
+  // Few slices: a cluster of CTAs for each (the knobs of d2o_set_tuning belong to the kernel below)
+  if (c->decode_warps == 0 && c->decode_stages == 0 && c->decode_smem_rows == 0 && c->decode_long_pairs == 0) {
+    const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows);
+    if (C > 0) {
+      bool published = true;                                          // the last step of every layer of the call
+      for (int l = l0; l < l1; ++l) published = published && c->layer_published[l];
+      a.early = published ? 1 : 0;
+      a.publish = 1;
+      c->decode_launches += 1;
+      const cudaError_t e = launch_decode_split(c, a, C, n_pairs * Hkv, max_rows, q, k, v, out, kpool, vpool, st);
+      if (e == cudaSuccess) memset(c->layer_published + l0, 1, l1 - l0);
+      return e;
+    }
+  }
+  memset(c->layer_published + l0, 0, l1 - l0);                          // set again below once the launch has succeeded
+  auto launched = [&](cudaError_t e) {
+    if (publish && e == cudaSuccess && *why == D2O_OK) memset(c->layer_published + l0, 1, l1 - l0);
+    return e;
+  };
+
   // A step takes at least as long as its longest slice takes in one CTA, and in a chain of steps a slice's CTAs
   // follow one another.  On the tensor path, where a few layers hold several times the mean budget and an
   // eight-warp CTA streams about 15 GB/s, the longest slices go into a launch of their own with sixteen consumer
@@ -1455,7 +1342,7 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     int rest_max = rows_of_pair(n_long);
     const int cw = (c->decode_warps == 4 || c->decode_warps == 8) ? c->decode_warps
                    : ((G <= 2 && rest >= 8 * c->n_sms * 4 && rest_max <= 2304) ? 4 : 8);
-    return launch_class(n_long, n_pairs, cw, true);
+    return launched(launch_class(n_long, n_pairs, cw, true));
   }
   // Consumer warps per CTA.  One head per KV head and enough small slices for seven and more CTAs on every SM:
   // four warps (measured on the serving-shaped config, 8192 slices of ~410 rows: 350 vs 370 us per step; with the
@@ -1470,7 +1357,7 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     if (G <= 2 && n_slices >= 8 * c->n_sms * 4 && max_rows <= 2304) cw = 4;
     if (G >= 4 && n_slices <= c->n_sms * 8 && max_rows > 2.0 * mean_rows) cw = 16;
   }
-  return launch_class(0, n_pairs, cw, chained);
+  return launched(launch_class(0, n_pairs, cw, chained));
 }
 
 }  // namespace d2o

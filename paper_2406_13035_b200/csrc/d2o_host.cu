@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "d2o_common.cuh"
+#include "d2o_decode.cuh"
 
 using namespace d2o;
 
@@ -184,6 +185,7 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
       return D2O_ERR_CUDA;
     }
     c->n_sms = sms;
+    c->max_cluster = decode_split_max_cluster();
   }
   c->state = (char*)state; c->scratch = (char*)scratch;
   c->state_bytes = state_bytes; c->scratch_bytes = scratch_bytes;
@@ -197,6 +199,7 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
   c->layer_fed = (uint8_t*)calloc(cfg->n_layers, 1);
   c->layer_compressed = (uint8_t*)calloc(cfg->n_layers, 1);
   c->layer_steps = (int32_t*)calloc(cfg->n_layers, 4);
+  c->layer_published = (uint8_t*)calloc(cfg->n_layers, 1);
   c->h_order = (int32_t*)calloc(BL, 4);
   c->h_plen = (int32_t*)calloc(cfg->batch, 4);
   c->h_sim_count = (int32_t*)calloc(cfg->n_layers, 4);
@@ -225,7 +228,7 @@ extern "C" void d2o_destroy(d2o_ctx* c) {
     cudaEventDestroy(c->lane_fork);
   }
   free(c->h_budgets); free(c->h_windows); free(c->h_row_off); free(c->h_pair_max); free(c->h_pair_sum);
-  free(c->layer_fed); free(c->layer_compressed); free(c->layer_steps); free(c->h_order); free(c->h_plen); free(c->h_sim_count); free(c->h_sim_items);
+  free(c->layer_fed); free(c->layer_compressed); free(c->layer_steps); free(c->layer_published); free(c->h_order); free(c->h_plen); free(c->h_sim_count); free(c->h_sim_items);
   free(c);
 }
 
@@ -364,6 +367,7 @@ extern "C" d2o_status d2o_prefill_compress(d2o_ctx* c, int32_t layer, const void
   CUDA_TRY(launch_prefill_compress(c, layer, K, V, (cudaStream_t)stream));
   c->layer_compressed[layer] = 1;
   c->layer_steps[layer] = 0;
+  c->layer_published[layer] = 1;                              // the compression sets the step counters to zero
   return D2O_OK;
 }
 
@@ -392,7 +396,7 @@ extern "C" d2o_status d2o_prefill_compress_layers(d2o_ctx* c, int32_t l0, int32_
       CUDA_TRY(cudaStreamWaitEvent(st, c->lane_done[i], 0));
     }
   }
-  for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; }
+  for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; c->layer_published[l] = 1; }
   return D2O_OK;
 }
 
