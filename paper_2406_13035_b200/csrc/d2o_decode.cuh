@@ -1,8 +1,11 @@
 // Pieces shared by the two decode kernels (d2o_decode.cu: one CTA per slice; d2o_decode_split.cu: one cluster per
-// slice): launch arguments, mbarrier and bulk-copy wrappers with bounded waits, packed fp32 arithmetic.
+// slice): launch arguments, mbarrier and bulk-copy wrappers with bounded waits, packed fp32 arithmetic, the mma.sync steps.
 #pragma once
 
+#include <cuda/std/type_traits>
+
 #include "d2o_common.cuh"
+#include "d2o_tc.cuh"
 
 namespace d2o {
 
@@ -35,7 +38,7 @@ struct DecodeArgs {
 
 // d2o_decode_split.cu
 int decode_split_max_cluster();
-int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows);
+int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows);
 cudaError_t launch_decode_split(const d2o_ctx* c, DecodeArgs a, int C, int n_slices, int max_rows, const void* q,
                                 const void* k, const void* v, void* out, void* kpool, void* vpool, cudaStream_t st);
 
@@ -146,6 +149,97 @@ __device__ __forceinline__ float reduce4(float s0, float s1, float s2, float s3,
 #pragma unroll
   for (int o = LPR / 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
   return k;
+}
+
+// 2-D tiled load with an L2 eviction-priority hint; x = innermost coordinate (elements), y = row
+__device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* map, int x, int y, unsigned long long* bar,
+                                                 unsigned long long policy) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
+               ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy) : "memory");
+}
+
+// One warp-level tensor-core step for the logits of 16 rows against up to 8 heads: acc (16 x 8, fp32) += A (16 rows x
+// 16 elements of d, from the row-major stage) * B (16 elements x 8 heads, the queries).  Both operands take their
+// 16-byte pieces from the same offsets of their rows, so the order of the elements inside a step is free and a
+// thread's piece is one contiguous vector load.
+// the same step with a zero accumulator on input: d = a * b
+template <typename T>
+__device__ __forceinline__ void mma_16x8x16_zero(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                 uint32_t b0, uint32_t b1) {
+  if constexpr (sizeof(T) == 2 && !cuda::std::is_same<T, __nv_bfloat16>::value) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+  } else {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+  }
+}
+template <typename T>
+__device__ __forceinline__ void mma_16x8x16(float (&acc)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                            uint32_t b0, uint32_t b1) {
+  if constexpr (sizeof(T) == 2 && !cuda::std::is_same<T, __nv_bfloat16>::value) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  } else {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+}
+
+// (hi, lo) 16-bit pairs of two fp32 weights, hi + lo carrying 16 (bf16) or 22 (fp16) significant bits: x -> low half
+template <typename T>
+__device__ __forceinline__ void split_pair(float x, float y, uint32_t& hi, uint32_t& lo) {
+  if constexpr (cuda::std::is_same<T, __nv_bfloat16>::value) {
+    // hi = the upper 16 bits (the subtraction is then exact), lo = the remainder rounded
+    const uint32_t xb = __float_as_uint(x) & 0xffff0000u, yb = __float_as_uint(y) & 0xffff0000u;
+    hi = (xb >> 16) | yb;
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(xb), y - __uint_as_float(yb));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+  } else {
+    const __half xh = __float2half_rn(x), yh = __float2half_rn(y);
+    const __half2 h = __halves2half2(xh, yh);
+    const __half2 l = __halves2half2(__float2half_rn(x - __half2float(xh)), __float2half_rn(y - __half2float(yh)));
+    hi = *reinterpret_cast<const uint32_t*>(&h); lo = *reinterpret_cast<const uint32_t*>(&l);
+  }
+}
+// four 8x8 16-bit matrices, transposed on the way into registers (value rows become the A operand's columns)
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(saddr) : "memory");
+}
+
+// Dot products of the 16 rows of tile `tile` of a swizzled stage ([d half][SR rows][128 bytes], 16-byte chunk c of
+// row r at chunk c ^ (r & 7)) with the (up to 8) vectors whose fragments are in `qb`.  Thread (gid, tig) reads chunk
+// 2 tig + (j & 1) of half j / 2 of rows gid and gid + 8 in step j: with the swizzle the eight lanes of a quarter-warp
+// hit eight different bank groups.  The order of the elements inside a step is free as long as both operands agree,
+// so a thread's piece is one vector load; `qb[j]` holds the same chunk of vector gid.
+// acc[0], acc[1] = row gid of the tile against vectors 2 tig, 2 tig + 1; acc[2], acc[3] = row gid + 8.
+template <typename T, int D, int SR>
+__device__ __forceinline__ void tile_dots(const unsigned char* stage, int tile, const uint4 (&qb)[D / 32], float (&acc)[4]) {
+  const int gid = (threadIdx.x & 31) >> 2, tig = threadIdx.x & 3;
+  // all fragments first, then one tensor-core step per 16 elements of d, each into its own accumulator: neither
+  // the loads nor the steps wait for one another
+  uint4 A0[D / 32], A1[D / 32];
+#pragma unroll
+  for (int j = 0; j < D / 32; ++j) {
+    const unsigned char* row = stage + (size_t)(j >> 1) * SR * 128 + (size_t)(tile * 16 + gid) * 128 +
+                               (((2 * tig + (j & 1)) ^ gid) << 4);
+    A0[j] = *reinterpret_cast<const uint4*>(row);
+    A1[j] = *reinterpret_cast<const uint4*>(row + 8 * 128);
+  }
+  float part[D / 16][4];
+#pragma unroll
+  for (int j = 0; j < D / 32; ++j) {
+    mma_16x8x16_zero<T>(part[2 * j], A0[j].x, A1[j].x, A0[j].y, A1[j].y, qb[j].x, qb[j].y);
+    mma_16x8x16_zero<T>(part[2 * j + 1], A0[j].z, A1[j].z, A0[j].w, A1[j].w, qb[j].z, qb[j].w);
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < D / 16; ++i) t += part[i][e];
+    acc[e] = t;
+  }
 }
 
 }  // namespace d2o
