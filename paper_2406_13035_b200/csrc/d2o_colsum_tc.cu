@@ -2,7 +2,7 @@
 // 5th-generation tensor cores.  The P x P probability matrix is never stored: two sweeps recompute the
 // logits tile by tile with tcgen05.mma (fp32 accumulators in tensor memory) and reduce them on the fly.
 //
-//   sweep 1 (rows)     lse2_i = log2 sum_{j<=i} 2^{c q_i.k_j},  c = log2(e)/sqrt(d)
+//   sweep 1 (rows)     lse2_i = log2 sum_{j<=i} 2^{c q_i.k_j},  c = log2(e)/sqrt(d); stored negated
 //                      A = 256 query rows of one head (resident), B = key tiles 0 .. diagonal (streamed)
 //   sweep 2 (columns)  s_j = sum_{i>=j} 2^{c q_i.k_j - lse2_i}
 //                      A = 256 keys (resident), B = query tiles diagonal .. end (streamed, with their lse2)
@@ -16,7 +16,15 @@
 //   warp 0      TMA producer (A once; B tiles and, in sweep 2, their lse2 through a 4-stage ring)
 //   warp 1      tensor-memory allocation, MMA issue
 //   warps 2-17  epilogue: four warps per quarter of the lanes; warp parts 0,1 take the first A tile
-//               (B rows 0-63 / 64-127), parts 2,3 the second; exp2 on the MUFU pipe is what bounds a job
+//               (B rows 0-63 / 64-127), parts 2,3 the second
+//
+// What bounds a job: one exponential per logit.  The special-function unit takes 8 cycles for a warp's 32 of them, 2048
+// cycles per job and SM quarter, twice the job's tensor-pipe time; and the instructions around them, so scale, sum and
+// the normaliser's addition are packed (two logits per issue slot) and masked tiles (the diagonal, the end of the prompt)
+// have a path of their own.  One pair of logits in four takes a polynomial on the FMA pipe instead (exp2_poly_pair): more
+// and the issue slots become the limit.  P = 8192, 32 fp16 heads, us per sweep (ncu): 482 / 417 with scalar arithmetic
+// and the mask inside the loop, 369 / 370 with every exponential on the special-function unit, 337 / 348 with every fourth
+// pair as a polynomial (xu 67 %, issue 61 %, tensor 44 %).  Two layers of 32768 tokens: 24.0, 20.7 and 20.2 ms (power cap).
 #include <math.h>
 
 #include "d2o_common.cuh"
@@ -31,7 +39,7 @@ constexpr int kCsStages = 4;                 // B ring
 enum { kSweepRows = 0, kSweepCols = 1 };
 
 struct ColsumTcArgs {
-  float* lse2;                               // [B * Hq][lse_row(P)] log2-domain row normalisers (sweep 1 -> sweep 2)
+  float* neg_lse2;                           // [B * Hq][lse_row(P)] negated log2-domain row normalisers (sweep 1 -> sweep 2)
   float* colsum;                             // [B, Hq, P] (sweep 2)
   uint32_t* status;                          // NULL: no error word (the allocation-free entry point)
   const int32_t* plen;                       // [B] prompt length of every sequence (<= P); NULL: all P
@@ -41,7 +49,33 @@ struct ColsumTcArgs {
 // Row stride of the normalisers: the bulk copies of sweep 2 start on 16-byte boundaries whatever the prompt length.
 __host__ __device__ __forceinline__ size_t lse_row(int P) { return (size_t)((P + 3) & ~3); }
 
+constexpr int kPolyPairs = 0x11;             // of eight pairs of logits, those whose exponentials go to the FMA pipe
+
 namespace tc {
+// two fp32 lanes in one 64-bit register, and the packed operations on them (one issue slot each)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// maximum that keeps a NaN
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
 // global -> this CTA's shared memory, 16-byte aligned on both sides, size a multiple of 16
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -61,6 +95,73 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 }
 }  // namespace tc
 
+// acc += (2^x, 2^y) on the FMA pipe.  x = n + f with n the nearest integer and |f| <= 1/2 (adding 1.5 * 2^23 rounds to
+// the nearest integer and leaves n in the low mantissa bits), 2^f by the polynomial of degree 5 with constant term 1
+// whose largest relative error on [-1/2, 1/2] is smallest (9.1e-8; found as a linear program over 4001 Chebyshev points;
+// 1.7e-7 with the fp32 roundings of Horner's rule, the same size as the special-function unit's), 2^n as exponent bits.
+// Exponents below -127 count as -127, whose exponent bits are those of zero: such a term is 0.  A NaN stays one.
+__device__ __forceinline__ tc::f32x2 exp2_poly_pair(tc::f32x2 xy, tc::f32x2 acc) {
+  const float kRound = 12582912.0f;
+  float x, y;
+  tc::unpack2(xy, x, y);
+  xy = tc::pack2(tc::max_nan(x, -127.f), tc::max_nan(y, -127.f));
+  const tc::f32x2 t = tc::add2(xy, tc::pack2(kRound, kRound));
+  const tc::f32x2 n = tc::add2(t, tc::pack2(-kRound, -kRound));
+  const tc::f32x2 f = tc::fma2(n, tc::pack2(-1.f, -1.f), xy);                 // exact
+  tc::f32x2 p = tc::pack2(0.001326472731307149f, 0.001326472731307149f);
+  p = tc::fma2(p, f, tc::pack2(0.009671512991189957f, 0.009671512991189957f));
+  p = tc::fma2(p, f, tc::pack2(0.05550733581185341f, 0.05550733581185341f));
+  p = tc::fma2(p, f, tc::pack2(0.24022242426872253f, 0.24022242426872253f));
+  p = tc::fma2(p, f, tc::pack2(0.6931470036506653f, 0.6931470036506653f));
+  p = tc::fma2(p, f, tc::pack2(1.f, 1.f));
+  float t0, t1;
+  tc::unpack2(t, t0, t1);
+  const tc::f32x2 s = tc::pack2(__uint_as_float((__float_as_uint(t0) << 23) + 0x3f800000u),
+                                __uint_as_float((__float_as_uint(t1) << 23) + 0x3f800000u));
+  return tc::fma2(p, s, acc);
+}
+
+// Which pairs of 64 logits take the polynomial.
+__host__ __device__ constexpr bool poly_pair(int k) { return (kPolyPairs >> (k & 7)) & 1; }
+
+// Sum of 2^{c s_i + b_i} over the 64 logits s_i of one accumulator row (in two register blocks).  Rows: every b_i is
+// `b`; columns: b_i comes from shared memory (the negated normalisers of the 64 streamed rows).
+template <bool PER_ROW>
+__device__ __forceinline__ float exp_sum_64(const uint32_t (&ra)[32], const uint32_t (&rb)[32], float c, float b,
+                                            const float* s_b) {
+  const tc::f32x2 c2 = tc::pack2(c, c), b2 = tc::pack2(b, b);
+  tc::f32x2 acc[2] = {0ull, 0ull}, pac[2] = {0ull, 0ull};
+#pragma unroll
+  for (int i4 = 0; i4 < 8; ++i4) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      tc::f32x2 bb[2] = {b2, b2};
+      if (PER_ROW) {
+        const float4 v = *reinterpret_cast<const float4*>(s_b + half * 32 + i4 * 4);
+        bb[0] = tc::pack2(v.x, v.y); bb[1] = tc::pack2(v.z, v.w);
+      }
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const int i = i4 * 4 + w * 2;
+        const tc::f32x2 s = half == 0 ? tc::pack2(__uint_as_float(ra[i]), __uint_as_float(ra[i + 1]))
+                                      : tc::pack2(__uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
+        const tc::f32x2 x = tc::fma2(s, c2, bb[w]);
+        if (poly_pair(i4 * 4 + half * 2 + w)) {
+          pac[w] = exp2_poly_pair(x, pac[w]);
+        } else {
+          float x0, x1;
+          tc::unpack2(x, x0, x1);
+          acc[w] = tc::add2(acc[w], tc::pack2(tc::ex2(x0), tc::ex2(x1)));
+        }
+      }
+    }
+  }
+  const tc::f32x2 t = tc::add2(tc::add2(acc[0], acc[1]), tc::add2(pac[0], pac[1]));
+  float lo, hi;
+  tc::unpack2(t, lo, hi);
+  return lo + hi;
+}
+
 template <int D, int FMT, int SWEEP>
 __global__ void __launch_bounds__(kCsThreads, 1)
 attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k) {
@@ -73,7 +174,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   extern __shared__ __align__(1024) unsigned char cs_smem[];
   unsigned char* sA = cs_smem;                               // [2 tiles][KB][128 rows][128 B]
   unsigned char* sB = cs_smem + 2 * TILE;                    // [stages][KB][128 rows][128 B]
-  float* s_lse = reinterpret_cast<float*>(sB + kCsStages * TILE);   // [stages][128] lse2 of the B rows (sweep 2)
+  float* s_lse = reinterpret_cast<float*>(sB + kCsStages * TILE);   // [stages][128] negated lse2 of the B rows (sweep 2)
   float* s_comb = s_lse + kCsStages * kCsTile;               // [2][2][128] partner values for the final combination
   __shared__ unsigned long long a_full, b_full[kCsStages], b_empty[kCsStages], tm_full[2], tm_empty[2];
   __shared__ uint32_t s_tmem;
@@ -140,7 +241,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         tc::mbar_expect_tx(&b_full[s], bytes);
         for (int kb = 0; kb < KB; ++kb)
           tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
-        if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, a.lse2 + bh * lse_row(a.P) + r0, (uint32_t)(n_lse * 4), &b_full[s]);
+        if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, a.neg_lse2 + bh * lse_row(a.P) + r0, (uint32_t)(n_lse * 4), &b_full[s]);
       }
     }
   } else if (warp == 1) {
@@ -176,7 +277,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
     const int part = e >> 2;                                 // 0,1: first A tile, B rows 0-63 / 64-127; 2,3: second A tile
     const int at = part >> 1, bhalf = part & 1;
     const int arow = a0 + at * kCsTile + quarter * 32 + lane;    // position of this thread's A row (query or key)
-    // sweep 1: running maximum of the raw logits and sum of 2^{c (s - m)}; sweep 2: column sum
+    // sweep 1: running maximum m of the log2-domain logits and sum of 2^{c s - m}; sweep 2: column sum
     float m_run = -INFINITY, l_run = 0.f;
     double col_acc = 0.0;
     uint32_t ra[32], rb[32];
@@ -197,62 +298,43 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
       if (lane == 0) tc::mbar_arrive(&tm_empty[buf]);
       if (SWEEP == kSweepRows) {
         // B rows are keys: valid iff key <= query (keys >= P are > every stored query)
-        const bool need_mask = brow0 + 63 > a0 + at * kCsTile + quarter * 32;     // warp-uniform
+        if (brow0 + 63 > a0 + at * kCsTile + quarter * 32) {   // warp-uniform: the diagonal
+          const int last = arow - brow0;                       // the row's last valid column of the 64
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            if (i > last) ra[i] = 0xff800000u;
+            if (i + 32 > last) rb[i] = 0xff800000u;
+          }
+        }
         // four independent chains of three-input maxima: the block maximum is on every thread's critical path
         float bmx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          float x = __uint_as_float(ra[i]), y = __uint_as_float(rb[i]);
-          if (need_mask) {
-            if (brow0 + i > arow) x = -INFINITY;
-            if (brow0 + 32 + i > arow) y = -INFINITY;
-            ra[i] = __float_as_uint(x); rb[i] = __float_as_uint(y);
-          }
-          bmx[i & 3] = tc::max3(bmx[i & 3], x, y);
-        }
-        const float bm = fmaxf(fmaxf(bmx[0], bmx[1]), fmaxf(bmx[2], bmx[3]));
-        if (bm > m_run) { l_run *= exp2f((m_run - bm) * c); m_run = bm; }      // exp2f(-inf) = 0 on the first block
-        if (m_run > -INFINITY) {
-          const float mc = m_run * c;
-          float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            l0 += tc::ex2(fmaf(__uint_as_float(ra[i]), c, -mc));
-            l1 += tc::ex2(fmaf(__uint_as_float(rb[i]), c, -mc));
-          }
-          l_run += l0 + l1;
-        }
+        for (int i = 0; i < 32; ++i) bmx[i & 3] = tc::max3(bmx[i & 3], __uint_as_float(ra[i]), __uint_as_float(rb[i]));
+        const float bm = fmaxf(fmaxf(bmx[0], bmx[1]), fmaxf(bmx[2], bmx[3])) * c;     // in the log2 domain, rounded once
+        if (bm > m_run) { l_run *= exp2f(m_run - bm); m_run = bm; }            // exp2f(-inf) = 0 on the first block
+        if (m_run > -INFINITY) l_run += exp_sum_64<false>(ra, rb, c, -m_run, nullptr);
       } else {
         // B rows are queries: valid iff query >= key and query < P
         const float* ls = s_lse + s * kCsTile + bhalf * 64;
-        const bool need_mask = (brow0 < a0 + at * kCsTile + quarter * 32 + 32) || (brow0 + 64 > P);   // warp-uniform
-        float p0 = 0.f, p1 = 0.f;
-        const float4* l4 = reinterpret_cast<const float4*>(ls);
+        float part;
+        if (brow0 >= a0 + at * kCsTile + quarter * 32 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
+          part = exp_sum_64<true>(ra, rb, c, 0.f, ls);
+        } else {
+          const int first = arow - brow0, end = P - brow0;     // the row's valid columns of the 64
+          float p0 = 0.f, p1 = 0.f;
 #pragma unroll
-        for (int i4 = 0; i4 < 8; ++i4) {
-          const float4 la = l4[i4], lb = l4[8 + i4];
-          const float lav[4] = {la.x, la.y, la.z, la.w}, lbv[4] = {lb.x, lb.y, lb.z, lb.w};
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const int i = i4 * 4 + w;
-            float x = tc::ex2(fmaf(__uint_as_float(ra[i]), c, -lav[w]));
-            float y = tc::ex2(fmaf(__uint_as_float(rb[i]), c, -lbv[w]));
-            if (need_mask) {
-              const int qa = brow0 + i, qb = brow0 + 32 + i;
-              if (qa < arow || qa >= P) x = 0.f;
-              if (qb < arow || qb >= P) y = 0.f;
-            }
-            p0 += x; p1 += y;
+          for (int i = 0; i < 32; ++i) {
+            const float x = tc::ex2(fmaf(__uint_as_float(ra[i]), c, ls[i]));
+            const float y = tc::ex2(fmaf(__uint_as_float(rb[i]), c, ls[32 + i]));
+            p0 += i >= first && i < end ? x : 0.f;
+            p1 += i + 32 >= first && i + 32 < end ? y : 0.f;
           }
+          part = p0 + p1;
         }
-        col_acc += (double)(p0 + p1);
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&b_empty[s]);         // this warp is done with the stage's lse2
+        col_acc += (double)part;
       }
-      if (SWEEP == kSweepRows) {
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&b_empty[s]);
-      }
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&b_empty[s]);           // this warp is done with the stage (sweep 2: its normalisers)
     }
     // combine the two warps that share an A row (B-row halves), fixed order; after a wait that ran out: NaN
     const int r = quarter * 32 + lane;
@@ -262,9 +344,9 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
       if (bhalf == 0 && arow < P) {
         const float m2 = s_comb[(at * 2 + 0) * kCsTile + r], l2 = s_comb[(at * 2 + 1) * kCsTile + r];
         const float mm = fmaxf(m_run, m2);
-        const float ll = (m_run > -INFINITY ? l_run * exp2f((m_run - mm) * c) : 0.f) +
-                         (m2 > -INFINITY ? l2 * exp2f((m2 - mm) * c) : 0.f);
-        a.lse2[bh * lse_row(a.P) + arow] = s_fail ? NAN : fmaf(mm, c, log2f(ll));
+        const float ll = (m_run > -INFINITY ? l_run * exp2f(m_run - mm) : 0.f) +
+                         (m2 > -INFINITY ? l2 * exp2f(m2 - mm) : 0.f);
+        a.neg_lse2[bh * lse_row(a.P) + arow] = s_fail ? NAN : -(mm + log2f(ll));
       }
     } else {
       double* dcomb = reinterpret_cast<double*>(s_comb);
@@ -283,26 +365,26 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   if (tid == 0 && s_fail && a.status) report_error(a.status, D2O_ERR_TIMEOUT, 0xC5C00000u | (uint32_t)(bh & 0xfffff));
 }
 
-// natural-log row normalisers supplied by the caller -> log2 domain, padded rows; one (sequence, head) per blockIdx.x
-__global__ void lse_to_log2_kernel(const float* __restrict__ lse, float* __restrict__ lse2, int P) {
+// natural-log row normalisers supplied by the caller -> negated log2 domain, padded rows; one (sequence, head) per blockIdx.x
+__global__ void lse_to_log2_kernel(const float* __restrict__ lse, float* __restrict__ neg_lse2, int P) {
   const int i = blockIdx.y * blockDim.x + threadIdx.x;
-  if (i < P) lse2[blockIdx.x * lse_row(P) + i] = lse[(size_t)blockIdx.x * P + i] * kLog2e;
+  if (i < P) neg_lse2[blockIdx.x * lse_row(P) + i] = -(lse[(size_t)blockIdx.x * P + i] * kLog2e);
 }
 
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P) { return (size_t)batch * n_q_heads * lse_row(P) * 4; }
 
 // Column sums of one layer of 16-bit Q, K on the tensor cores.  `lse_in` (natural log, may be NULL) replaces sweep 1;
-// `lse2` is scratch of colsum_tc_lse_bytes(); `plen` (DEVICE, may be NULL) holds every sequence's prompt length,
+// `neg_lse2` is scratch of colsum_tc_lse_bytes(); `plen` (DEVICE, may be NULL) holds every sequence's prompt length,
 // `status` (may be NULL) the error word.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that
 // are not a multiple of four used to take the FFMA kernels: 17.5 ms instead of 1.1 for two layers of 6001 tokens.)
 cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
-                             const float* lse_in, float* lse2, float* colsum, const int32_t* plen, uint32_t* status,
+                             const float* lse_in, float* neg_lse2, float* colsum, const int32_t* plen, uint32_t* status,
                              cudaStream_t st) {
   CUtensorMap map_q, map_k;
   if (!encode_rows_2d(&map_q, dtype, Q, (uint64_t)B * Hq * P, D, kCsTile)) return cudaErrorNotSupported;
   if (!encode_rows_2d(&map_k, dtype, K, (uint64_t)B * Hkv * P, D, kCsTile)) return cudaErrorNotSupported;
   ColsumTcArgs a;
-  a.lse2 = lse2;
+  a.neg_lse2 = neg_lse2;
   a.colsum = colsum;
   a.status = status;
   a.P = P; a.Hq = Hq; a.group = Hq / Hkv;
@@ -326,7 +408,7 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, co
     else          { if (fmt == 0) D2O_LAUNCH_CS(64, 0, SW); else D2O_LAUNCH_CS(64, 1, SW); }     \
   } while (0)
   if (lse_in) {
-    lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256)), 256, 0, st>>>(lse_in, lse2, P);
+    lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256)), 256, 0, st>>>(lse_in, neg_lse2, P);
   } else {
     D2O_LAUNCH_CS_ALL(kSweepRows);
   }

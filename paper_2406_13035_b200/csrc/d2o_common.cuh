@@ -233,7 +233,7 @@ size_t sim_tc_max_items(const d2o_config* cfg, int max_budget);
 void sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count);
 // tensor-core column sums of the prompt attention for 16-bit Q/K (d2o_colsum_tc.cu)
 cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
-                             const float* lse_in, float* lse2, float* colsum, const int32_t* plen, uint32_t* status,
+                             const float* lse_in, float* neg_lse2, float* colsum, const int32_t* plen, uint32_t* status,
                              cudaStream_t st);
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P);      // its row normalisers
 
