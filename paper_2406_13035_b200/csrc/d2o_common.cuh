@@ -176,6 +176,7 @@ struct d2o_ctx {
   size_t state_bytes, scratch_bytes;
   // host mirrors, valid after d2o_layer_budgets
   bool have_budgets;
+  char* h_tables;              // the three tables below, laid out as in `state`
   int32_t* h_budgets;          // [B, L, Hkv]
   int32_t* h_windows;          // [B, L, Hkv]
   int64_t* h_row_off;          // [B, L, Hkv]
@@ -187,6 +188,7 @@ struct d2o_ctx {
   uint8_t* layer_published;    // [L] the slices' step counters of the last decode step were (or will be) written
   int32_t* h_plen;             // [B] prompt length of every sequence (prompt_len unless d2o_set_prompt_lens was called)
   int32_t* h_sim_count;        // [L] work items of the tensor-core similarity kernel per layer
+  int32_t* h_sim_off;          // [L] first item of the layer in the work list
   int4* h_sim_items;           // host copy of the work lists (device copy in `state`)
   int32_t* h_order;            // [L * B] (layer * B + b) sorted by cache size, largest first (device copy in `state`)
   int decode_stages;           // tuning: stages of the decode kernel's ring, 0 = auto
@@ -230,7 +232,7 @@ cudaError_t launch_full_decode(int dtype, int d, int n_slices, int group, int ca
 cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, const void* K, int max_S, cudaStream_t st, int lane = 0);
 size_t sim_tc_part_key_bytes(const d2o_config* cfg, int max_budget);
 size_t sim_tc_max_items(const d2o_config* cfg, int max_budget);
-void sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count);
+size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count, int32_t* first);
 // tensor-core column sums of the prompt attention for 16-bit Q/K (d2o_colsum_tc.cu)
 cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
                              const float* lse_in, float* neg_lse2, float* colsum, const int32_t* plen, uint32_t* status,

@@ -191,9 +191,12 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
   c->state_bytes = state_bytes; c->scratch_bytes = scratch_bytes;
   const size_t BL = (size_t)cfg->batch * cfg->n_layers;
   const size_t BLH = BL * cfg->n_kv_heads;
-  c->h_budgets = (int32_t*)calloc(BLH, 4);
-  c->h_windows = (int32_t*)calloc(BLH, 4);
-  c->h_row_off = (int64_t*)calloc(BLH, 8);
+  // budgets, windows and row offsets lie one after another in `state`; the host mirror has the same layout, so that
+  // they travel in one copy
+  c->h_tables = (char*)calloc(l.order - l.budgets, 1);
+  c->h_budgets = (int32_t*)c->h_tables;
+  c->h_windows = (int32_t*)(c->h_tables + (l.windows - l.budgets));
+  c->h_row_off = (int64_t*)(c->h_tables + (l.row_off - l.budgets));
   c->h_pair_max = (int32_t*)calloc(BL, 4);
   c->h_pair_sum = (int64_t*)calloc(BL, 8);
   c->layer_fed = (uint8_t*)calloc(cfg->n_layers, 1);
@@ -203,6 +206,7 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
   c->h_order = (int32_t*)calloc(BL, 4);
   c->h_plen = (int32_t*)calloc(cfg->batch, 4);
   c->h_sim_count = (int32_t*)calloc(cfg->n_layers, 4);
+  c->h_sim_off = (int32_t*)calloc(cfg->n_layers, 4);
   c->h_sim_items = cfg->dtype == D2O_F32 ? nullptr
       : (int4*)malloc((size_t)cfg->n_layers * sim_tc_max_items(cfg, maxb) * sizeof(int4));
   for (int b = 0; b < cfg->batch; ++b) c->h_plen[b] = cfg->prompt_len;
@@ -227,7 +231,7 @@ extern "C" void d2o_destroy(d2o_ctx* c) {
     for (int i = 0; i < kCompressLanes; ++i) { cudaStreamDestroy(c->lane_stream[i]); cudaEventDestroy(c->lane_done[i]); }
     cudaEventDestroy(c->lane_fork);
   }
-  free(c->h_budgets); free(c->h_windows); free(c->h_row_off); free(c->h_pair_max); free(c->h_pair_sum);
+  free(c->h_tables); free(c->h_sim_off); free(c->h_pair_max); free(c->h_pair_sum);
   free(c->layer_fed); free(c->layer_compressed); free(c->layer_steps); free(c->layer_published); free(c->h_order); free(c->h_plen); free(c->h_sim_count); free(c->h_sim_items);
   free(c);
 }
@@ -321,9 +325,8 @@ extern "C" d2o_status d2o_layer_budgets(d2o_ctx* c, int32_t* budgets_host, void*
                           (uint32_t*)(c->state + c->lay.status), (const int32_t*)(c->state + c->lay.plen), st));
   const size_t BL = (size_t)g.batch * g.n_layers;
   const size_t Hkv = g.n_kv_heads, BLH = BL * Hkv;
-  CUDA_TRY(cudaMemcpyAsync(c->h_budgets, d_b, BLH * 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(c->h_windows, d_w, BLH * 4, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(c->h_row_off, d_o, BLH * 8, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(c->h_tables, c->state + c->lay.budgets, c->lay.row_off + BLH * 8 - c->lay.budgets,
+                           cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   // the device computed offsets for the pool; make sure they fit what the caller gave us
   for (size_t i = 0; i < BLH; ++i) {
@@ -349,12 +352,11 @@ extern "C" d2o_status d2o_layer_budgets(d2o_ctx* c, int32_t* budgets_host, void*
   CUDA_TRY(cudaMemcpyAsync(c->state + c->lay.order, c->h_order, BL * 4, cudaMemcpyHostToDevice, st));
   if (c->h_sim_items) {
     // work lists of the tensor-core similarity kernel for every layer (the budgets are all it needs)
-    sim_tc_build_items(c, c->n_sms, c->h_sim_items, c->h_sim_count);
-    CUDA_TRY(cudaMemcpyAsync(c->state + c->lay.sim_items, c->h_sim_items,
-                             (size_t)g.n_layers * sim_tc_max_items(&g, c->max_budget) * sizeof(int4),
-                             cudaMemcpyHostToDevice, st));
+    const size_t n_items = sim_tc_build_items(c, c->n_sms, c->h_sim_items, c->h_sim_count, c->h_sim_off);
+    if (n_items > 0)
+      CUDA_TRY(cudaMemcpyAsync(c->state + c->lay.sim_items, c->h_sim_items, n_items * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
-  CUDA_TRY(cudaStreamSynchronize(st));
+  // (the two host arrays change again only in a later call, behind its own synchronisation above)
   c->have_budgets = true;
   if (budgets_host) memcpy(budgets_host, c->h_budgets, BLH * 4);
   return D2O_OK;

@@ -445,17 +445,20 @@ size_t sim_tc_max_items(const d2o_config* cfg, int max_budget) {
 
 // The work lists of all layers, built on the host once the budgets are known: every (slice, chunk of retained rows)
 // is cut into ranges of prompt tiles of about equal work (tiles x columns), so that one launch is several full waves
-// of CTAs of the same length whatever the spread of the budgets; longest first.  `items` has room for
-// n_layers * sim_tc_max_items() entries, `count[layer]` receives the entries of each layer.
-void sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count) {
+// of CTAs of the same length whatever the spread of the budgets; longest first.  The lists lie one after another in
+// `items` (room for n_layers * sim_tc_max_items() entries); `count[layer]` and `first[layer]` describe each.  Returns the
+// entries of all layers.
+size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count, int32_t* first) {
   const d2o_config& g = c->cfg;
   const int B = g.batch, Hkv = g.n_kv_heads, L = g.n_layers;
   const size_t cap = sim_tc_max_items(&g, c->max_budget);
   struct Piece { int slice, chunk, tiles, cols; };
-  Piece* pieces = (Piece*)malloc(sizeof(Piece) * (size_t)B * Hkv * ((c->max_budget + kChunkN - 1) / kChunkN + 1));
+  std::vector<Piece> pieces;
+  std::vector<std::pair<double, int4>> list;
+  size_t n = 0;
   for (int layer = 0; layer < L; ++layer) {
-    int4* out = items + (size_t)layer * cap;
-    size_t n_pieces = 0;
+    pieces.clear();
+    list.clear();
     double total = 0.0;
     for (int b = 0; b < B; ++b)
       for (int h = 0; h < Hkv; ++h) {
@@ -467,34 +470,31 @@ void sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count
         for (int nc = 0; nc < n_chunks; ++nc) {
           const int cols = min(cc, S - nc * cc);
           if (cols <= 0) continue;
-          pieces[n_pieces++] = {b * Hkv + h, nc, tiles, cols};
+          pieces.push_back({b * Hkv + h, nc, tiles, cols});
           total += (double)tiles * (cols + 64);                // + a per-tile cost that does not depend on the columns
         }
       }
-    size_t n = 0;
-    if (n_pieces > 0) {
-      // aim at five waves of equal items, at least eight tiles each (a CTA first loads its chunk of retained rows and keeps four tiles in flight)
-      const double target = total / ((double)n_sms * 5.0);
-      std::vector<std::pair<double, int4>> list;
-      for (size_t i = 0; i < n_pieces; ++i) {
-        const Piece& p = pieces[i];
-        const double work = (double)p.tiles * (p.cols + 64);
-        int k = (int)(work / target + 0.5);
-        k = max(1, min(k, max(1, p.tiles / 8)));
-        if (list.size() + k + (n_pieces - i) > cap) k = 1;     // never more entries than the list holds
-        for (int j = 0; j < k; ++j) {
-          const int t0 = (int)((long long)p.tiles * j / k), t1 = (int)((long long)p.tiles * (j + 1) / k);
-          if (t1 > t0) list.push_back({(double)(t1 - t0) * (p.cols + 64), make_int4(p.slice, p.chunk, t0, t1)});
-        }
+    // aim at five waves of equal items, at least eight tiles each (a CTA first loads its chunk of retained rows and keeps four tiles in flight)
+    const double target = total / ((double)n_sms * 5.0);
+    for (size_t i = 0; i < pieces.size(); ++i) {
+      const Piece& p = pieces[i];
+      const double work = (double)p.tiles * (p.cols + 64);
+      int k = (int)(work / target + 0.5);
+      k = max(1, min(k, max(1, p.tiles / 8)));
+      if (list.size() + k + (pieces.size() - i) > cap) k = 1;  // never more entries than the list holds
+      for (int j = 0; j < k; ++j) {
+        const int t0 = (int)((long long)p.tiles * j / k), t1 = (int)((long long)p.tiles * (j + 1) / k);
+        if (t1 > t0) list.push_back({(double)(t1 - t0) * (p.cols + 64), make_int4(p.slice, p.chunk, t0, t1)});
       }
-      // longest first; ties keep the slice order
-      std::stable_sort(list.begin(), list.end(),
-                       [](const std::pair<double, int4>& x, const std::pair<double, int4>& y) { return x.first > y.first; });
-      for (const auto& e : list) out[n++] = e.second;
     }
-    count[layer] = (int32_t)n;
+    // longest first; ties keep the slice order
+    std::stable_sort(list.begin(), list.end(),
+                     [](const std::pair<double, int4>& x, const std::pair<double, int4>& y) { return x.first > y.first; });
+    first[layer] = (int32_t)n;
+    count[layer] = (int32_t)list.size();
+    for (const auto& e : list) items[n++] = e.second;
   }
-  free(pieces);
+  return n;
 }
 
 size_t sim_tc_part_key_bytes(const d2o_config* cfg, int max_budget) {
@@ -525,7 +525,7 @@ cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, const void* K, int
   a.status = (uint32_t*)(S + c->lay.status);
   a.plen = (const int32_t*)(S + c->lay.plen);
   a.L = g.n_layers; a.layer = layer; a.Hkv = Hkv; a.P = P; a.n_chunks_max = n_chunks_max;
-  a.items = (const int4*)(S + c->lay.sim_items) + (size_t)layer * sim_tc_max_items(&g, c->max_budget);
+  a.items = (const int4*)(S + c->lay.sim_items) + c->h_sim_off[layer];
   const int KB = D / 64;
   const size_t smem = (size_t)KB * kChunkN * 128 + (size_t)kParts * KB * kTileM * 128 + kChunkN * 4;
   dim3 grid((unsigned)n_items);

@@ -8,7 +8,7 @@
 //                   columns and walks down the rows, so the column reduction needs neither
 //                   atomics nor scratch and is bit-reproducible
 //   density_kernel  warp-shuffle mean / variance of s per query head (double accumulation)
-//   budget_kernel   Eq. 5 with clamping and exact-sum integerisation, one thread per sequence
+//   budget_kernel   Eq. 5 with clamping and exact-sum integerisation, one CTA per sequence
 // The two attention sweeps here are the generic FFMA implementation (any dtype, fp32 math);
 // 16-bit inputs take the tensor-core path of d2o_colsum_tc.cu.
 #include <math.h>
@@ -224,101 +224,136 @@ density_kernel(const float* __restrict__ colsum, double* __restrict__ density, i
 // Cache sizes from the densities.  budget_rule 0 (Eq. 5): S_l = clip(lambda * w_l, S_min, S_max) with
 // sum_l S_l = S_tot, then floor + largest remainder; rule 1 (per-head sizes of Appendix A.5): the same over the
 // (layer, KV head) units; rule 2 (exponential-decay allocation of the ablation): S_l = round(mean_h exp(-F/gamma) P),
-// clamped, no fixed total.  One thread per sequence; its work arrays (w, kinks, x) live in dynamic shared memory.
-// Output tables are [B, L, Hkv]; the per-layer rules give every KV head of a layer the same size.
+// clamped, no fixed total.  Output tables are [B, L, Hkv]; the per-layer rules give every KV head of a layer the same size.
+//
+// One CTA per sequence.  The integers must not depend on how the work is divided, so every sum runs in one thread in the
+// order of the units; what runs side by side are different sums: the weights of different units, the totals at different
+// values of lambda (all kinks at once, or a many-way search where there are more of them than threads), the rank of every
+// remainder.
+constexpr int kBudgetThreads = 256;
 __device__ inline double clipd(double v, double lo, double hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-__global__ void budget_kernel(const double* __restrict__ density, int B, int L, int H, int Hkv, int Pmax, double rho,
-                              int min_budget, int max_budget_cfg, double gamma, int head_reduce, int budget_rule,
-                              int n_sink, int window, double nm_ratio, int32_t* __restrict__ budgets,
-                              int32_t* __restrict__ windows, int64_t* __restrict__ row_off, uint32_t* status_word,
-                              const int32_t* __restrict__ plen) {
+// minimum over the CTA; every thread gets it
+__device__ inline double block_min(double v, double* part) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { const double t = __shfl_xor_sync(0xffffffffu, v, o); v = t < v ? t : v; }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = part[0];
+  for (int w = 1; w < kBudgetThreads / 32; ++w) v = part[w] < v ? part[w] : v;
+  return v;
+}
+
+__global__ void __launch_bounds__(kBudgetThreads)
+budget_kernel(const double* __restrict__ density, int L, int H, int Hkv, int Pmax, double rho, int min_budget,
+              int max_budget_cfg, double gamma, int head_reduce, int budget_rule, int n_sink, int window, double nm_ratio,
+              int32_t* __restrict__ budgets, int32_t* __restrict__ windows, uint32_t* status_word,
+              const int32_t* __restrict__ plen) {
   extern __shared__ __align__(16) double dsm[];
   const int n = budget_rule == 1 ? L * Hkv : L;                       // allocation units
   const int G = H / Hkv;
-  double* w = dsm + (size_t)threadIdx.x * 4 * n;
-  double* kinks = w + n;        // [2n]
-  double* x = kinks + 2 * n;    // [n]
+  int n_pad = 2;                                                      // kinks, padded for the sort
+  while (n_pad < 2 * n) n_pad *= 2;
+  double* w = dsm;              // [n] weights
+  double* x = w + n;            // [n] scaled sizes, then remainders
+  double* kinks = x + n;        // [n_pad]
+  __shared__ double part[kBudgetThreads / 32], s_lam;
+  __shared__ int s_lo, s_hi, s_open;
+  __shared__ long long s_left;
+  const int tid = threadIdx.x, b = blockIdx.x;
   const double lo = (double)min_budget;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const int P = plen ? plen[b] : Pmax;                              // this sequence's prompt length
-    const int max_budget = max_budget_cfg > 0 ? max_budget_cfg : P;   // no clamp given: a layer cannot hold more than the prompt
-    const double hi = (double)max_budget;
-    const long long S_tot = (long long)floor(rho * (double)n * (double)P + 0.5);
-    const double* F = density + (size_t)b * L * H;
-    int32_t* bud = budgets + (size_t)b * L * Hkv;
-    // unit u -> its (first) entry of the [L, Hkv] table
-    auto slot_of = [&](int u) { return budget_rule == 1 ? u : u * Hkv; };
-    if (budget_rule == 2) {
-      for (int l = 0; l < L; ++l) {
+  const int P = plen ? plen[b] : Pmax;                                // this sequence's prompt length
+  const int max_budget = max_budget_cfg > 0 ? max_budget_cfg : P;     // no clamp given: a layer cannot hold more than the prompt
+  const double hi = (double)max_budget;
+  const long long S_tot = (long long)floor(rho * (double)n * (double)P + 0.5);
+  const double* F = density + (size_t)b * L * H;
+  int32_t* bud = budgets + (size_t)b * L * Hkv;
+  // unit u -> its (first) entry of the [L, Hkv] table
+  auto slot_of = [&](int u) { return budget_rule == 1 ? u : u * Hkv; };
+  if (budget_rule == 2) {
+    for (int l = tid; l < L; l += kBudgetThreads) {
+      double a = 0.0;
+      for (int h = 0; h < H; ++h) a = __dadd_rn(a, exp(-__ddiv_rn(F[l * H + h], gamma)));
+      const double s = floor(__dadd_rn(__dmul_rn(__ddiv_rn(a, (double)H), (double)P), 0.5));
+      bud[l * Hkv] = (int32_t)clipd(s, lo, hi);
+    }
+  } else {
+    if (budget_rule == 1 || head_reduce == 0) {
+      double fmin = INFINITY;
+      for (int i = tid; i < L * H; i += kBudgetThreads) fmin = F[i] < fmin ? F[i] : fmin;
+      fmin = block_min(fmin, part);
+      const int heads = budget_rule == 1 ? G : H;                     // query heads of a unit
+      for (int u = tid; u < n; u += kBudgetThreads) {
         double a = 0.0;
-        for (int h = 0; h < H; ++h) a = __dadd_rn(a, exp(-__ddiv_rn(F[l * H + h], gamma)));
-        const double s = floor(__dadd_rn(__dmul_rn(__ddiv_rn(a, (double)H), (double)P), 0.5));
-        bud[l * Hkv] = (int32_t)clipd(s, lo, hi);
+        for (int g = 0; g < heads; ++g) a = __dadd_rn(a, exp(-__ddiv_rn(__dadd_rn(F[u * heads + g], -fmin), gamma)));
+        w[u] = a;
+      }
+    } else if (head_reduce == 2) {
+      // reciprocal of the variance, per head (a zero variance counts as the smallest positive one)
+      for (int l = tid; l < L; l += kBudgetThreads) {
+        double a = 0.0;
+        for (int h = 0; h < H; ++h) {
+          const double f = F[l * H + h];
+          a = __dadd_rn(a, __ddiv_rn(1.0, f > 1e-300 ? f : 1e-300));
+        }
+        w[l] = a;
       }
     } else {
-      if (budget_rule == 1) {
-        double fmin = F[0];
-        for (int i = 1; i < L * H; ++i) fmin = fmin < F[i] ? fmin : F[i];
-        for (int u = 0; u < n; ++u) {
-          double a = 0.0;
-          for (int g = 0; g < G; ++g) a = __dadd_rn(a, exp(-__ddiv_rn(__dadd_rn(F[u * G + g], -fmin), gamma)));
-          w[u] = a;
-        }
-      } else if (head_reduce == 0) {
-        double fmin = F[0];
-        for (int i = 1; i < L * H; ++i) fmin = fmin < F[i] ? fmin : F[i];
-        for (int l = 0; l < L; ++l) {
-          double a = 0.0;
-          for (int h = 0; h < H; ++h) a = __dadd_rn(a, exp(-__ddiv_rn(__dadd_rn(F[l * H + h], -fmin), gamma)));
-          w[l] = a;
-        }
-      } else if (head_reduce == 2) {
-        // reciprocal of the variance, per head (a zero variance counts as the smallest positive one)
-        for (int l = 0; l < L; ++l) {
-          double a = 0.0;
-          for (int h = 0; h < H; ++h) {
-            const double f = F[l * H + h];
-            a = __dadd_rn(a, __ddiv_rn(1.0, f > 1e-300 ? f : 1e-300));
+      double fmin = INFINITY;
+      for (int l = tid; l < L; l += kBudgetThreads) {
+        double a = 0.0;
+        for (int h = 0; h < H; ++h) a = __dadd_rn(a, F[l * H + h]);
+        x[l] = __ddiv_rn(a, (double)H);
+        fmin = fmin < x[l] ? fmin : x[l];
+      }
+      fmin = block_min(fmin, part);
+      for (int l = tid; l < L; l += kBudgetThreads) {                 // x[l] was written by this thread
+        if (head_reduce == 1) w[l] = exp(-__ddiv_rn(__dadd_rn(x[l], -fmin), gamma));
+        else w[l] = __ddiv_rn(1.0, x[l] > 1e-300 ? x[l] : 1e-300);
+      }
+    }
+    // kinks of the piecewise-linear total(lambda), ascending
+    for (int u = tid; u < n; u += kBudgetThreads) {
+      w[u] = w[u] > 1e-300 ? (w[u] < 1e300 ? w[u] : 1e300) : 1e-300;
+      kinks[2 * u] = __ddiv_rn(lo, w[u]);
+      kinks[2 * u + 1] = __ddiv_rn(hi, w[u]);
+    }
+    for (int i = 2 * n + tid; i < n_pad; i += kBudgetThreads) kinks[i] = INFINITY;
+    for (int k = 2; k <= n_pad; k *= 2)                               // bitonic sort
+      for (int j = k / 2; j > 0; j /= 2) {
+        __syncthreads();
+        for (int i = tid; i < n_pad; i += kBudgetThreads) {
+          const int o = i ^ j;
+          if (o > i) {
+            const double p = kinks[i], q = kinks[o];
+            if ((p > q) == ((i & k) == 0)) { kinks[i] = q; kinks[o] = p; }
           }
-          w[l] = a;
-        }
-      } else {
-        double fmin = INFINITY;
-        for (int l = 0; l < L; ++l) {
-          double a = 0.0;
-          for (int h = 0; h < H; ++h) a = __dadd_rn(a, F[l * H + h]);
-          x[l] = __ddiv_rn(a, (double)H);
-          fmin = fmin < x[l] ? fmin : x[l];
-        }
-        if (head_reduce == 1) {
-          for (int l = 0; l < L; ++l) w[l] = exp(-__ddiv_rn(__dadd_rn(x[l], -fmin), gamma));
-        } else {
-          for (int l = 0; l < L; ++l) w[l] = __ddiv_rn(1.0, x[l] > 1e-300 ? x[l] : 1e-300);
         }
       }
-      for (int u = 0; u < n; ++u) w[u] = w[u] > 1e-300 ? (w[u] < 1e300 ? w[u] : 1e300) : 1e-300;
-      // kinks of the piecewise-linear total(lambda), ascending (insertion sort)
-      int nk = 0;
-      for (int u = 0; u < n; ++u) {
-        const double cand[2] = {__ddiv_rn(lo, w[u]), __ddiv_rn(hi, w[u])};
-        for (int c = 0; c < 2; ++c) {
-          int i = nk++;
-          while (i > 0 && kinks[i - 1] > cand[c]) { kinks[i] = kinks[i - 1]; --i; }
-          kinks[i] = cand[c];
-        }
+    const int nk = 2 * n;
+    auto total = [&](double lam) {
+      double t = 0.0;
+      for (int u = 0; u < n; ++u) t = __dadd_rn(t, clipd(__dmul_rn(lam, w[u]), lo, hi));
+      return t;
+    };
+    // total() is non-decreasing: the first kink that reaches S_tot, in [s_lo, s_hi]
+    if (tid == 0) { s_lo = 0; s_hi = nk; }
+    __syncthreads();
+    while (s_lo < s_hi) {                                             // uniform: written before a barrier
+      const int from = s_lo, to = s_hi, step = (to - from + kBudgetThreads - 1) / kBudgetThreads;
+      const int at = min(from + (tid + 1) * step - 1, to - 1);        // last kink of this thread's stretch
+      const bool below = from + tid * step < to && total(kinks[at]) < (double)S_tot;
+      // stretches whose last kink stays below the total are passed over; the next one holds the answer
+      const int passed = __syncthreads_count(below);
+      if (tid == 0) {
+        s_lo = min(from + passed * step, to);
+        s_hi = step == 1 ? s_lo : min(s_lo + step - 1, to);
       }
-      auto total = [&](double lam) {
-        double t = 0.0;
-        for (int u = 0; u < n; ++u) t = __dadd_rn(t, clipd(__dmul_rn(lam, w[u]), lo, hi));
-        return t;
-      };
-      // total() is non-decreasing: the first kink that reaches S_tot, by bisection
-      int k = 0, k_hi = nk;
-      while (k < k_hi) {
-        const int mid = (k + k_hi) >> 1;
-        if (total(kinks[mid]) < (double)S_tot) k = mid + 1; else k_hi = mid;
-      }
+      __syncthreads();
+    }
+    if (tid == 0) {
+      const int k = s_lo;
       double lam;
       if (k == 0) lam = kinks[0];
       else if (k == nk) lam = kinks[nk - 1];
@@ -334,50 +369,72 @@ __global__ void budget_kernel(const double* __restrict__ density, int B, int L, 
         lam = wf > 0.0 ? __ddiv_rn(__dadd_rn((double)S_tot, -fixed), wf) : bb;
         lam = lam < a ? a : (lam > bb ? bb : lam);
       }
-      long long sum = 0;
-      for (int u = 0; u < n; ++u) {
-        x[u] = clipd(__dmul_rn(lam, w[u]), lo, hi);
-        const double fl = floor(x[u]);
-        bud[slot_of(u)] = (int32_t)fl;
-        x[u] = x[u] - fl;                                   // remainder
-        sum += (long long)fl;
-      }
-      long long left = S_tot - sum;
-      if (left < 0 || left > n) { report_error(status_word, D2O_ERR_STATE, 0xB0000000u | (uint32_t)b); left = 0; }
-      while (left > 0) {                                     // largest remainder first, ties -> lower unit
-        int best = -1;
-        for (int u = 0; u < n; ++u)
-          if (x[u] >= 0.0 && bud[slot_of(u)] < max_budget && (best < 0 || x[u] > x[best])) best = u;
-        if (best < 0) { report_error(status_word, D2O_ERR_STATE, 0xB1000000u | (uint32_t)b); break; }
-        bud[slot_of(best)] += 1;
-        x[best] = -1.0;                                      // taken
-        --left;
-      }
+      s_lam = lam;
+      s_left = S_tot;
+      s_open = 0;
     }
-    if (budget_rule != 1) {                                  // one size per layer: every KV head gets it
-      for (int l = 0; l < L; ++l)
-        for (int h = 1; h < Hkv; ++h) bud[l * Hkv + h] = bud[l * Hkv];
+    __syncthreads();
+    const double lam = s_lam;
+    for (int u = tid; u < n; u += kBudgetThreads) {
+      const double v = clipd(__dmul_rn(lam, w[u]), lo, hi), fl = floor(v);
+      bud[slot_of(u)] = (int32_t)fl;
+      x[u] = (int32_t)fl < max_budget ? v - fl : -1.0;                // remainder; a unit at the upper clamp takes no further row
+      if (x[u] >= 0.0) atomicAdd(&s_open, 1);
+      atomicAdd((unsigned long long*)&s_left, (unsigned long long)(-(long long)fl));
     }
+    __syncthreads();
+    long long left = s_left;
+    if (left < 0 || left > n) {
+      if (tid == 0) report_error(status_word, D2O_ERR_STATE, 0xB0000000u | (uint32_t)b);
+      left = 0;
+    }
+    if (left > s_open && tid == 0) report_error(status_word, D2O_ERR_STATE, 0xB1000000u | (uint32_t)b);
+    // largest remainder first, ties -> lower unit: the first `left` in that order get one more row
+    if (left > 0)
+      for (int u = tid; u < n; u += kBudgetThreads) {
+        const double xu = x[u];
+        if (xu < 0.0) continue;
+        int rank = 0;
+        for (int v = 0; v < n; ++v) rank += x[v] > xu || (x[v] == xu && v < u) ? 1 : 0;
+        if (rank < left) bud[slot_of(u)] += 1;
+      }
+  }
+  __syncthreads();                                                    // the CTA's own writes to `bud` are read below
+  for (int i = tid; i < L * Hkv; i += kBudgetThreads) {
+    const int S = budget_rule == 1 ? bud[i] : bud[i / Hkv * Hkv];     // one size per layer: every KV head gets it
+    if (budget_rule != 1 && i % Hkv != 0) bud[i] = S;
     if (windows) {
-      for (int i = 0; i < L * Hkv; ++i) {
-        const int S = bud[i];
-        const int T = n_sink < S ? n_sink : S;
-        int M = window > 0 ? window : (int)floor((double)(S - T) / (1.0 + nm_ratio) + 0.5);
-        M = M < 0 ? 0 : (M > S - T ? S - T : M);
-        windows[(size_t)b * L * Hkv + i] = M;
-      }
+      const int T = n_sink < S ? n_sink : S;
+      int M = window > 0 ? window : (int)floor((double)(S - T) / (1.0 + nm_ratio) + 0.5);
+      M = M < 0 ? 0 : (M > S - T ? S - T : M);
+      windows[(size_t)b * L * Hkv + i] = M;
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0 && row_off) {                       // cache rows laid out layer-major, then sequence, then head
-    long long o = 0;
-    for (int l = 0; l < L; ++l)
-      for (int b = 0; b < B; ++b)
-        for (int h = 0; h < Hkv; ++h) {
-          const size_t i = ((size_t)b * L + l) * Hkv + h;
-          row_off[i] = o;
-          o += (long long)slice_stride(budgets[i]);
-        }
+}
+
+// First cache row of every slice: rows are laid out layer-major, then sequence, then head.
+__global__ void __launch_bounds__(1024)
+row_offset_kernel(const int32_t* __restrict__ budgets, int B, int L, int Hkv, int64_t* __restrict__ row_off) {
+  __shared__ long long s_warp[32], s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_base = 0;
+  const int n = L * B * Hkv;
+  for (int i0 = 0; i0 < n; i0 += 1024) {
+    const int i = i0 + threadIdx.x;
+    const int l = i / (B * Hkv), b = i / Hkv % B, h = i % Hkv;
+    const size_t e = ((size_t)b * L + l) * Hkv + h;
+    const long long v = i < n ? (long long)slice_stride(budgets[e]) : 0;
+    long long inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const long long t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    long long before = s_base;
+    for (int k = 0; k < warp; ++k) before += s_warp[k];
+    if (i < n) row_off[e] = before + inc - v;
+    __syncthreads();
+    if (threadIdx.x == 1023) s_base = before + inc;
+    __syncthreads();
   }
 }
 
@@ -431,17 +488,17 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
                            int max_budget, float gamma, int head_reduce, int budget_rule, int n_sink, int window,
                            float nm_ratio, int32_t* budgets, int32_t* windows, int64_t* row_off, uint32_t* status_word,
                            const int32_t* plen, cudaStream_t st) {
-  const size_t n_units = budget_rule == 1 ? (size_t)L * Hkv : (size_t)L;
-  const size_t per_thread = 4 * n_units * sizeof(double);
-  int threads = B < 32 ? B : 32;
-  while (threads > 1 && per_thread * threads > 160 * 1024) threads /= 2;
-  const size_t sm = per_thread * threads;
+  const size_t n = budget_rule == 1 ? (size_t)L * Hkv : (size_t)L;
+  size_t n_pad = 2;
+  while (n_pad < 2 * n) n_pad *= 2;
+  const size_t sm = (2 * n + n_pad) * sizeof(double);
   if (sm > 200 * 1024) return cudaErrorInvalidValue;          // more allocation units than the work arrays hold
   cudaError_t e = cudaFuncSetAttribute(budget_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  budget_kernel<<<1, threads, sm, st>>>(density, B, L, H, Hkv, P, (double)rho, min_budget, max_budget, (double)gamma,
-                                        head_reduce, budget_rule, n_sink, window, (double)nm_ratio, budgets, windows,
-                                        row_off, status_word, plen);
+  budget_kernel<<<B, kBudgetThreads, sm, st>>>(density, L, H, Hkv, P, (double)rho, min_budget, max_budget, (double)gamma,
+                                               head_reduce, budget_rule, n_sink, window, (double)nm_ratio, budgets, windows,
+                                               status_word, plen);
+  if (row_off) row_offset_kernel<<<1, 1024, 0, st>>>(budgets, B, L, Hkv, row_off);
   return cudaGetLastError();
 }
 
