@@ -153,7 +153,8 @@ d2o_status d2o_layer_stats(d2o_ctx* ctx, int32_t layer, const void* Q, const voi
 
 /* The same for layers [l0, l1) in one call (Eq. 4 acts per layer; a caller that holds several
  * layers' Q and K can hand them over together).  Q, K: HOST arrays of l1-l0 DEVICE pointers;
- * lse: NULL, or a HOST array of l1-l0 DEVICE pointers (entries may be NULL).  Two layers are
+ * lse: NULL, or a HOST array of l1-l0 DEVICE pointers (entries may be NULL).  16-bit inputs: up to
+ * eight layers share a launch, so that short prompts fill the GPU.  fp32 inputs: two layers are
  * worked on side by side on streams of the library's own (as d2o_prefill_compress_layers does,
  * same fork / join on `stream`, same first-call creation of streams and events), each with its
  * own row-normaliser scratch, so that one layer's last CTAs share the GPU with the next layer's

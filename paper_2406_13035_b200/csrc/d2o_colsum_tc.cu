@@ -11,7 +11,10 @@
 // atomics, a fixed order, bit-reproducible.  Across jobs the per-thread partials are added in fp64
 // (sweep 2) so that a column which receives up to P probabilities keeps full fp32 accuracy.
 //
-// One CTA = (head, 256 A rows).  One job = one streamed tile of 128 B rows against both 128-row A
+// One item = (head, 256 A rows); a CTA per SM works through its items (see CsItem), so that one item's first loads and
+// products run beside the epilogue of the one before it (one CTA per item: the prologue and the last combination, about
+// 4 us of every CTA, were most of a short prompt's time: 32 layers of 1200 tokens 976 -> 724 us for both sweeps, eight
+// layers of 4096 tokens with the caller's normalisers 811 -> 730).  One job = one streamed tile of 128 B rows against both 128-row A
 // tiles: two 128 x 128 x d MMAs whose accumulators fill one of two 256-column tensor-memory buffers.
 //   warp 0      TMA producer (A once; B tiles and, in sweep 2, their lse2 through a 4-stage ring)
 //   warp 1      tensor-memory allocation, MMA issue
@@ -27,6 +30,8 @@
 // pair as a polynomial (xu 67 %, issue 61 %, tensor 44 %).  Two layers of 32768 tokens: 24.0, 20.7 and 20.2 ms (power cap).
 #include <math.h>
 
+#include <algorithm>
+
 #include "d2o_common.cuh"
 #include "d2o_tc.cuh"
 
@@ -39,11 +44,20 @@ constexpr int kCsStages = 4;                 // B ring
 enum { kSweepRows = 0, kSweepCols = 1 };
 
 struct ColsumTcArgs {
-  float* neg_lse2;                           // [B * Hq][lse_row(P)] negated log2-domain row normalisers (sweep 1 -> sweep 2)
-  float* colsum;                             // [B, Hq, P] (sweep 2)
+  float* neg_lse2;                           // [layers][B * Hq][lse_row(P)] negated log2-domain row normalisers (sweep 1 -> sweep 2)
+  float* colsum;                             // [layers][B, Hq, P] (sweep 2)
+  size_t lse_stride;                         // floats between the normalisers of two layers
+  int n_items, n_pairs;                      // items of the launch; pairs of tiles of the longest prompt
+  uint32_t* sched;                           // [2] items handed out beyond the first of every CTA; CTAs done (both 0 between launches)
   uint32_t* status;                          // NULL: no error word (the allocation-free entry point)
   const int32_t* plen;                       // [B] prompt length of every sequence (<= P); NULL: all P
-  int P, Hq, group;                          // P: the length the tensors are laid out for
+  int P, Hq, group, BHq;                     // P: the length the tensors are laid out for; BHq: (sequence, head) pairs of a layer
+};
+
+// Layers of one launch: a short prompt's layer alone (32 heads, 1200 tokens: 160 items) is little more than one item per
+// SM.
+struct ColsumTcMaps {
+  CUtensorMap q[kColsumLayers], k[kColsumLayers];
 };
 
 // Row stride of the normalisers: the bulk copies of sweep 2 start on 16-byte boundaries whatever the prompt length.
@@ -162,9 +176,35 @@ __device__ __forceinline__ float exp_sum_64(const uint32_t (&ra)[32], const uint
   return lo + hi;
 }
 
+// One item: 256 A rows of one (layer, sequence, head).  Items of a layer are numbered heaviest first (sweep 1: the last
+// rows see the most keys; sweep 2: the first keys see the most rows), all heads of a pair of tiles next to one another so
+// that the CTAs at work share the streamed tiles in L2, the layers one after another.  CTA i begins with item i and takes
+// the next free one from a counter from then on.
+template <int SWEEP>
+struct CsItem {
+  int layer, bh, P, a0, bt0, n_jobs;                         // n_jobs = 0: the sequence has no such rows
+  __device__ __forceinline__ void decode(const ColsumTcArgs& a, int i) {
+    n_jobs = 0;
+    bh = i % a.BHq;
+    const int y = i / a.BHq % a.n_pairs;
+    layer = i / a.BHq / a.n_pairs;
+    P = a.plen ? a.plen[bh / a.Hq] : a.P;                    // this sequence's prompt; rows beyond it are padding
+    const int n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile), n_tiles = (P + kCsTile - 1) / kCsTile;
+    if (y >= n_pairs) return;                                // the numbering is for the longest prompt
+    a0 = (SWEEP == kSweepRows ? n_pairs - 1 - y : y) * 2 * kCsTile;          // first A row (query or key position)
+    // streamed tiles: sweep 1 keys [0, a0 + 256), sweep 2 queries [a0, P)
+    bt0 = SWEEP == kSweepRows ? 0 : a0 / kCsTile;
+    n_jobs = (SWEEP == kSweepRows ? min(n_tiles, (a0 + 2 * kCsTile) / kCsTile) : n_tiles) - bt0;
+  }
+  __device__ __forceinline__ int q_base(const ColsumTcArgs& a) const { return bh * a.P; }     // first row of the head in the views
+  __device__ __forceinline__ int k_base(const ColsumTcArgs& a) const {
+    return (bh / a.Hq * (a.Hq / a.group) + bh % a.Hq / a.group) * a.P;
+  }
+};
+
 template <int D, int FMT, int SWEEP>
 __global__ void __launch_bounds__(kCsThreads, 1)
-attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k) {
+attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   constexpr int KB = D / 64;                                 // 64-element (128-byte) blocks along d
   constexpr int BLOCK = kCsTile * 128;                       // bytes of one k-block of one 128-row tile
   constexpr int TILE = KB * BLOCK;                           // bytes of one 128-row tile
@@ -175,28 +215,13 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   unsigned char* sA = cs_smem;                               // [2 tiles][KB][128 rows][128 B]
   unsigned char* sB = cs_smem + 2 * TILE;                    // [stages][KB][128 rows][128 B]
   float* s_lse = reinterpret_cast<float*>(sB + kCsStages * TILE);   // [stages][128] negated lse2 of the B rows (sweep 2)
-  float* s_comb = s_lse + kCsStages * kCsTile;               // [2][2][128] partner values for the final combination
-  __shared__ unsigned long long a_full, b_full[kCsStages], b_empty[kCsStages], tm_full[2], tm_empty[2];
+  float* s_comb = s_lse + kCsStages * kCsTile;               // [2][2][2][128] partner values for the final combination
+  __shared__ unsigned long long a_full, a_empty, b_full[kCsStages], b_empty[kCsStages], tm_full[2], tm_empty[2], it_full[2], it_empty[2];
+  __shared__ int s_item[2];                                  // the CTA's current and next item, -1: no more
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int bh = blockIdx.x;                                 // b * Hq + hq (fastest index: all heads of the heaviest pair first)
-  const int b = bh / a.Hq, hq = bh % a.Hq;
-  const int P = a.plen ? a.plen[b] : a.P;                                   // this sequence's prompt; rows beyond it are padding
-  const int n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile);
-  const int n_tiles = (P + kCsTile - 1) / kCsTile;
-  if ((int)blockIdx.y >= n_pairs) return;                    // the grid is sized for the longest prompt
-  const int Hkv = a.Hq / a.group;
-  const int q_base = bh * a.P;                               // first row of this head in the [B*Hq*P, d] view of Q
-  const int k_base = (b * Hkv + hq / a.group) * a.P;
-  // heaviest CTAs first: sweep 1 -> the last rows see the most keys; sweep 2 -> the first keys see the most rows
-  const int pair = SWEEP == kSweepRows ? n_pairs - 1 - (int)blockIdx.y : (int)blockIdx.y;
-  const int a0 = pair * 2 * kCsTile;                         // first A row (query position or key position)
-  // streamed tiles: sweep 1 keys [0, a0 + 256), sweep 2 queries [a0, P)
-  const int bt0 = SWEEP == kSweepRows ? 0 : a0 / kCsTile;
-  const int bt1 = SWEEP == kSweepRows ? min(n_tiles, (a0 + 2 * kCsTile) / kCsTile) : n_tiles;
-  const int n_jobs = bt1 - bt0;
   if ((tc::smem_u32(cs_smem) & 1023u) != 0u) {               // swizzled tiles need 1024-byte aligned shared memory
     if (tid == 0 && a.status) report_error(a.status, D2O_ERR_STATE, 0xC5C10000u);
     return;
@@ -204,9 +229,10 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
 
   if (tid == 0) {
     s_fail = 0;
-    tc::mbar_init(&a_full, 1);
+    tc::mbar_init(&a_full, 1); tc::mbar_init(&a_empty, 1);
     for (int s = 0; s < kCsStages; ++s) { tc::mbar_init(&b_full[s], 1); tc::mbar_init(&b_empty[s], 1 + kCsEpiWarps); }
-    for (int i = 0; i < 2; ++i) { tc::mbar_init(&tm_full[i], 1); tc::mbar_init(&tm_empty[i], kCsEpiWarps); }
+    for (int i = 0; i < 2; ++i) { tc::mbar_init(&tm_full[i], 1); tc::mbar_init(&tm_empty[i], kCsEpiWarps);
+                                  tc::mbar_init(&it_full[i], 1); tc::mbar_init(&it_empty[i], 1 + kCsEpiWarps); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -219,40 +245,81 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
   tc::fence_after_sync();
   const uint32_t tmem_base = s_tmem;
 
+  // The k-th item of this CTA as the consumers see it; false: no more.  All lanes of an epilogue warp, or the MMA thread.
+  auto next_item = [&](int k, CsItem<SWEEP>& it) {
+    if (!tc::mbar_wait(&it_full[k & 1], (uint32_t)((k >> 1) & 1))) { s_fail = 1; return false; }
+    const int i = s_item[k & 1];
+    if (i < 0) return false;
+    it.decode(a, i);
+    return true;
+  };
+
   if (warp == 0) {
     // ======================================================================= TMA producer
     if (lane == 0) {
-      const CUtensorMap* map_a = SWEEP == kSweepRows ? &map_q : &map_k;
-      const CUtensorMap* map_b = SWEEP == kSweepRows ? &map_k : &map_q;
-      const int a_base = SWEEP == kSweepRows ? q_base : k_base;
-      const int b_base = SWEEP == kSweepRows ? k_base : q_base;
-      tc::mbar_expect_tx(&a_full, (uint32_t)(2 * TILE));
-      for (int t = 0; t < 2; ++t)
-        for (int kb = 0; kb < KB; ++kb)
-          tc::tma_load_2d(sA + t * TILE + kb * BLOCK, map_a, kb * 64, a_base + a0 + t * kCsTile, &a_full);
-      for (int job = 0; job < n_jobs; ++job) {
-        const int s = job % kCsStages;
-        if (job >= kCsStages && !s_fail && !tc::mbar_wait(&b_empty[s], (uint32_t)(((job / kCsStages) - 1) & 1))) s_fail = 1;
-        const int r0 = (bt0 + job) * kCsTile;                // first B row of the tile
-        uint32_t bytes = (uint32_t)TILE;
-        // 16-byte granules: up to three entries past the prompt come from the row's padding and are masked
-        const int n_lse = SWEEP == kSweepCols ? min(kCsTile, ((P + 3) & ~3) - r0) : 0;
-        bytes += (uint32_t)(n_lse * 4);
-        tc::mbar_expect_tx(&b_full[s], bytes);
-        for (int kb = 0; kb < KB; ++kb)
-          tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
-        if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, a.neg_lse2 + bh * lse_row(a.P) + r0, (uint32_t)(n_lse * 4), &b_full[s]);
+      CsItem<SWEEP> it{};
+      int jb = 0, ia = 0;                                    // jobs and items so far
+      int item = (int)blockIdx.x;
+      for (int k = 0;; ++k) {
+        if (k >= 2 && !tc::mbar_wait(&it_empty[k & 1], (uint32_t)(((k >> 1) - 1) & 1))) s_fail = 1;
+        s_item[k & 1] = item < a.n_items ? item : -1;
+        tc::mbar_arrive(&it_full[k & 1]);
+        if (item >= a.n_items) break;
+        it.decode(a, item);
+        if (s_fail) it.n_jobs = 0;                           // after a wait that ran out: the epilogue writes NaN
+        const CUtensorMap* map_a = SWEEP == kSweepRows ? &maps.q[it.layer] : &maps.k[it.layer];
+        const CUtensorMap* map_b = SWEEP == kSweepRows ? &maps.k[it.layer] : &maps.q[it.layer];
+        const int a_row = (SWEEP == kSweepRows ? it.q_base(a) : it.k_base(a)) + it.a0;
+        const int b_base = SWEEP == kSweepRows ? it.k_base(a) : it.q_base(a);
+        const float* neg_lse2 = a.neg_lse2 + it.layer * a.lse_stride + it.bh * lse_row(a.P);
+        for (int job = 0; job < it.n_jobs; ++job, ++jb) {
+          // the first streamed tile goes ahead of the resident ones: its stage is free earlier than they are
+          const int s = jb % kCsStages;
+          if (jb >= kCsStages && !s_fail && !tc::mbar_wait(&b_empty[s], (uint32_t)(((jb / kCsStages) - 1) & 1))) s_fail = 1;
+          if (s_fail) break;
+          const int r0 = (it.bt0 + job) * kCsTile;           // first B row of the tile
+          // 16-byte granules: up to three entries past the prompt come from the row's padding and are masked
+          const int n_lse = SWEEP == kSweepCols ? min(kCsTile, ((it.P + 3) & ~3) - r0) : 0;
+          tc::mbar_expect_tx(&b_full[s], (uint32_t)(TILE + n_lse * 4));
+          for (int kb = 0; kb < KB; ++kb)
+            tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
+          if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, neg_lse2 + r0, (uint32_t)(n_lse * 4), &b_full[s]);
+          if (job == 0) {
+            if (ia >= 1 && !tc::mbar_wait(&a_empty, (uint32_t)((ia - 1) & 1))) { s_fail = 1; ++jb; break; }
+            tc::mbar_expect_tx(&a_full, (uint32_t)(2 * TILE));
+            for (int t = 0; t < 2; ++t)
+              for (int kb = 0; kb < KB; ++kb)
+                tc::tma_load_2d(sA + t * TILE + kb * BLOCK, map_a, kb * 64, a_row + t * kCsTile, &a_full);
+            ++ia;
+          }
+        }
+        // Not earlier: this thread is up to four tiles ahead of the epilogue, which covers the counter's latency, and an
+        // item taken at the beginning of a long one would wait while other CTAs run out of work (2048 tokens, 32 heads:
+        // 80 us instead of 62).
+        item = (int)(gridDim.x + atomicAdd(&a.sched[0], 1u));
+      }
+      if (s_fail) {                                          // see the copies on their way land before the CTA may end
+        for (int i = max(0, jb - kCsStages); i < jb; ++i)
+          if (!tc::mbar_wait(&b_full[i % kCsStages], (uint32_t)((i / kCsStages) & 1))) break;
+        if (ia > 0) (void)tc::mbar_wait(&a_full, (uint32_t)((ia - 1) & 1));
       }
     }
   } else if (warp == 1) {
     // ======================================================================= MMA issuer
     if (lane == 0) {
-      if (!tc::mbar_wait(&a_full, 0)) s_fail = 1;
-      for (int job = 0; job < n_jobs; ++job) {
-        const int s = job % kCsStages, buf = job & 1;
-        if (!s_fail && !tc::mbar_wait(&b_full[s], (uint32_t)((job / kCsStages) & 1))) s_fail = 1;
+      CsItem<SWEEP> it;
+      int jb = 0, ia = 0;
+      for (int k = 0; next_item(k, it); ++k) {
+      tc::mbar_arrive(&it_empty[k & 1]);
+      if (it.n_jobs == 0) continue;
+      if (!s_fail && !tc::mbar_wait(&a_full, (uint32_t)(ia & 1))) s_fail = 1;
+      ++ia;
+      for (int job = 0; job < it.n_jobs && !s_fail; ++job, ++jb) {
+        const int s = jb % kCsStages, buf = jb & 1;
+        if (!s_fail && !tc::mbar_wait(&b_full[s], (uint32_t)((jb / kCsStages) & 1))) s_fail = 1;
         // the epilogue must have drained this buffer (the first use of each buffer passes at once)
-        if (!s_fail && !tc::mbar_wait(&tm_empty[buf], (uint32_t)(((job >> 1) & 1) ^ 1))) s_fail = 1;
+        if (!s_fail && !tc::mbar_wait(&tm_empty[buf], (uint32_t)(((jb >> 1) & 1) ^ 1))) s_fail = 1;
+        if (s_fail) break;
         tc::fence_after_sync();
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
@@ -268,6 +335,8 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         }
         tc::mma_commit(&tm_full[buf]);
         tc::mma_commit(&b_empty[s]);                         // one of the 17 arrivals that free the stage
+        if (job == it.n_jobs - 1) tc::mma_commit(&a_empty);  // the resident tiles have been read
+      }
       }
     }
   } else {
@@ -276,16 +345,25 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
     const int quarter = warp & 3;                            // tensor-memory lanes this warp may read: 32*quarter ..
     const int part = e >> 2;                                 // 0,1: first A tile, B rows 0-63 / 64-127; 2,3: second A tile
     const int at = part >> 1, bhalf = part & 1;
-    const int arow = a0 + at * kCsTile + quarter * 32 + lane;    // position of this thread's A row (query or key)
+    CsItem<SWEEP> it;
+    int jb = 0, ia = 0;
+    uint32_t ra[32], rb[32];
+#pragma unroll 1
+    for (int k = 0; next_item(k, it); ++k) {
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&it_empty[k & 1]);
+    if (it.n_jobs == 0) continue;
+    const int P = it.P, w0 = it.a0 + at * kCsTile + quarter * 32;        // first A row of this warp
+    const int arow = w0 + lane;                              // position of this thread's A row (query or key)
     // sweep 1: running maximum m of the log2-domain logits and sum of 2^{c s - m}; sweep 2: column sum
     float m_run = -INFINITY, l_run = 0.f;
     double col_acc = 0.0;
-    uint32_t ra[32], rb[32];
 #pragma unroll 1
-    for (int job = 0; job < n_jobs; ++job) {
-      const int s = job % kCsStages, buf = job & 1;
-      const int brow0 = (bt0 + job) * kCsTile + bhalf * 64;   // position of the first B row this warp looks at
-      if (!s_fail && !tc::mbar_wait(&tm_full[buf], (uint32_t)((job >> 1) & 1))) s_fail = 1;
+    for (int job = 0; job < it.n_jobs && !s_fail; ++job, ++jb) {
+      const int s = jb % kCsStages, buf = jb & 1;
+      const int brow0 = (it.bt0 + job) * kCsTile + bhalf * 64;   // position of the first B row this warp looks at
+      if (!tc::mbar_wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1))) s_fail = 1;
+      __syncwarp();
       tc::fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + at * kCsTile + bhalf * 64);
       tc::tmem_ld32_issue(taddr, ra);
@@ -296,9 +374,11 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&tm_empty[buf]);
-      if (SWEEP == kSweepRows) {
+      if (SWEEP == kSweepRows ? brow0 > w0 + 31 : brow0 + 63 < w0 || brow0 >= P) {
+        // nothing of this warp's block is valid (warp-uniform)
+      } else if (SWEEP == kSweepRows) {
         // B rows are keys: valid iff key <= query (keys >= P are > every stored query)
-        if (brow0 + 63 > a0 + at * kCsTile + quarter * 32) {   // warp-uniform: the diagonal
+        if (brow0 + 63 > w0) {                                 // warp-uniform: the diagonal
           const int last = arow - brow0;                       // the row's last valid column of the 64
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -317,7 +397,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
         // B rows are queries: valid iff query >= key and query < P
         const float* ls = s_lse + s * kCsTile + bhalf * 64;
         float part;
-        if (brow0 >= a0 + at * kCsTile + quarter * 32 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
+        if (brow0 >= w0 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
           part = exp_sum_64<true>(ra, rb, c, 0.f, ls);
         } else {
           const int first = arow - brow0, end = P - brow0;     // the row's valid columns of the 64
@@ -336,24 +416,28 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&b_empty[s]);           // this warp is done with the stage (sweep 2: its normalisers)
     }
-    // combine the two warps that share an A row (B-row halves), fixed order; after a wait that ran out: NaN
+    // combine the two warps that share an A row (B-row halves), fixed order; after a wait that ran out: NaN.  The exchange
+    // area alternates between items: whoever writes it again has passed the barrier of the item in between.
     const int r = quarter * 32 + lane;
+    float* comb = s_comb + (ia & 1) * 4 * kCsTile;
+    ++ia;
     if (SWEEP == kSweepRows) {
-      if (bhalf == 1) { s_comb[(at * 2 + 0) * kCsTile + r] = m_run; s_comb[(at * 2 + 1) * kCsTile + r] = l_run; }
+      if (bhalf == 1) { comb[(at * 2 + 0) * kCsTile + r] = m_run; comb[(at * 2 + 1) * kCsTile + r] = l_run; }
       asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
       if (bhalf == 0 && arow < P) {
-        const float m2 = s_comb[(at * 2 + 0) * kCsTile + r], l2 = s_comb[(at * 2 + 1) * kCsTile + r];
+        const float m2 = comb[(at * 2 + 0) * kCsTile + r], l2 = comb[(at * 2 + 1) * kCsTile + r];
         const float mm = fmaxf(m_run, m2);
         const float ll = (m_run > -INFINITY ? l_run * exp2f(m_run - mm) : 0.f) +
                          (m2 > -INFINITY ? l2 * exp2f(m2 - mm) : 0.f);
-        a.neg_lse2[bh * lse_row(a.P) + arow] = s_fail ? NAN : -(mm + log2f(ll));
+        a.neg_lse2[it.layer * a.lse_stride + it.bh * lse_row(a.P) + arow] = s_fail ? NAN : -(mm + log2f(ll));
       }
     } else {
-      double* dcomb = reinterpret_cast<double*>(s_comb);
+      double* dcomb = reinterpret_cast<double*>(comb);
       if (bhalf == 1) dcomb[at * kCsTile + r] = col_acc;
       asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
-      if (bhalf == 0 && arow < P) 
-        a.colsum[(size_t)bh * a.P + arow] = s_fail ? NAN : (float)(col_acc + dcomb[at * kCsTile + r]);
+      if (bhalf == 0 && arow < P)
+        a.colsum[((size_t)it.layer * a.BHq + it.bh) * a.P + arow] = s_fail ? NAN : (float)(col_acc + dcomb[at * kCsTile + r]);
+    }
     }
   }
   tc::fence_before_sync();
@@ -362,45 +446,64 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ CUtensorMap map_q, const 
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem_base, 512);
   }
-  if (tid == 0 && s_fail && a.status) report_error(a.status, D2O_ERR_TIMEOUT, 0xC5C00000u | (uint32_t)(bh & 0xfffff));
+  if (tid == 0) {                                            // the last CTA leaves the counters at zero for the next launch
+    __threadfence();
+    if (atomicAdd(&a.sched[1], 1u) == gridDim.x - 1) { a.sched[0] = 0u; a.sched[1] = 0u; }
+  }
+  if (tid == 0 && s_fail && a.status) report_error(a.status, D2O_ERR_TIMEOUT, 0xC5C00000u | (uint32_t)(blockIdx.x & 0xfffff));
 }
 
-// natural-log row normalisers supplied by the caller -> negated log2 domain, padded rows; one (sequence, head) per blockIdx.x
-__global__ void lse_to_log2_kernel(const float* __restrict__ lse, float* __restrict__ neg_lse2, int P) {
+// natural-log row normalisers supplied by the caller -> negated log2 domain, padded rows; one (sequence, head) per
+// blockIdx.x, one layer per blockIdx.z
+struct LseIn { const float* p[kColsumLayers]; };
+__global__ void lse_to_log2_kernel(LseIn lse, float* __restrict__ neg_lse2, size_t lse_stride, int P) {
   const int i = blockIdx.y * blockDim.x + threadIdx.x;
-  if (i < P) neg_lse2[blockIdx.x * lse_row(P) + i] = -(lse[(size_t)blockIdx.x * P + i] * kLog2e);
+  if (i < P)
+    neg_lse2[blockIdx.z * lse_stride + blockIdx.x * lse_row(P) + i] = -(lse.p[blockIdx.z][(size_t)blockIdx.x * P + i] * kLog2e);
 }
 
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P) { return (size_t)batch * n_q_heads * lse_row(P) * 4; }
 
-// Column sums of one layer of 16-bit Q, K on the tensor cores.  `lse_in` (natural log, may be NULL) replaces sweep 1;
-// `neg_lse2` is scratch of colsum_tc_lse_bytes(); `plen` (DEVICE, may be NULL) holds every sequence's prompt length,
-// `status` (may be NULL) the error word.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that
-// are not a multiple of four used to take the FFMA kernels: 17.5 ms instead of 1.1 for two layers of 6001 tokens.)
-cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
-                             const float* lse_in, float* neg_lse2, float* colsum, const int32_t* plen, uint32_t* status,
-                             cudaStream_t st) {
-  CUtensorMap map_q, map_k;
-  if (!encode_rows_2d(&map_q, dtype, Q, (uint64_t)B * Hq * P, D, kCsTile)) return cudaErrorNotSupported;
-  if (!encode_rows_2d(&map_k, dtype, K, (uint64_t)B * Hkv * P, D, kCsTile)) return cudaErrorNotSupported;
+// Column sums of n <= kColsumLayers layers of 16-bit Q, K on the tensor cores.  `lse_in` (natural log; NULL, or a pointer
+// per layer) replaces sweep 1; `neg_lse2` is scratch of n times colsum_tc_lse_bytes(), `lse_stride` bytes apart; `colsum` of
+// the layers lies one after another; `plen` (DEVICE, may be NULL) holds every sequence's prompt length, `status` (may be
+// NULL) the error word, `sched` two words that are zero between launches.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that are not a multiple of
+// four used to take the FFMA kernels: 17.5 ms instead of 1.0 for two layers of 6001 tokens.)
+cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, int n, const void* const* Q,
+                             const void* const* K, const float* const* lse_in, float* neg_lse2, size_t lse_stride,
+                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st) {
+  ColsumTcMaps maps;
+  LseIn lse;
+  for (int l = 0; l < n; ++l) {
+    if (!encode_rows_2d(&maps.q[l], dtype, Q[l], (uint64_t)B * Hq * P, D, kCsTile)) return cudaErrorNotSupported;
+    if (!encode_rows_2d(&maps.k[l], dtype, K[l], (uint64_t)B * Hkv * P, D, kCsTile)) return cudaErrorNotSupported;
+    if (lse_in) lse.p[l] = lse_in[l];
+  }
   ColsumTcArgs a;
   a.neg_lse2 = neg_lse2;
+  a.lse_stride = lse_stride / sizeof(float);
   a.colsum = colsum;
   a.status = status;
-  a.P = P; a.Hq = Hq; a.group = Hq / Hkv;
+  a.sched = sched;
+  a.P = P; a.Hq = Hq; a.group = Hq / Hkv; a.BHq = B * Hq;
   a.plen = plen;
   const int KB = D / 64;
-  const size_t smem = (size_t)(2 + kCsStages) * KB * kCsTile * 128 + (size_t)kCsStages * kCsTile * 4 + 4 * kCsTile * 4;
-  const int n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile);
-  // heaviest CTAs first over the whole launch: the pair index is the slow grid dimension
-  dim3 grid(B * Hq, n_pairs);
+  const size_t smem = (size_t)(2 + kCsStages) * KB * kCsTile * 128 + (size_t)kCsStages * kCsTile * 4 + 8 * kCsTile * 4;
+  a.n_pairs = (P + 2 * kCsTile - 1) / (2 * kCsTile);
+  const long items = (long)n * B * Hq * a.n_pairs;
+  if (items >= (1l << 30)) return cudaErrorInvalidValue;
+  a.n_items = (int)items;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return cudaGetLastError();
+  const dim3 grid((unsigned)std::min(items, (long)sms));     // one CTA per SM (shared and tensor memory)
   const int fmt = dtype == D2O_F16 ? 0 : 1;
   cudaError_t e;
 #define D2O_LAUNCH_CS(DD, FF, SW)                                                                                  \
   do {                                                                                                             \
     e = cudaFuncSetAttribute(attn_tc_kernel<DD, FF, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
     if (e != cudaSuccess) return e;                                                                                \
-    attn_tc_kernel<DD, FF, SW><<<grid, kCsThreads, smem, st>>>(a, map_q, map_k);                                   \
+    attn_tc_kernel<DD, FF, SW><<<grid, kCsThreads, smem, st>>>(a, maps);                                              \
   } while (0)
 #define D2O_LAUNCH_CS_ALL(SW)                                                                    \
   do {                                                                                           \
@@ -408,7 +511,7 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, co
     else          { if (fmt == 0) D2O_LAUNCH_CS(64, 0, SW); else D2O_LAUNCH_CS(64, 1, SW); }     \
   } while (0)
   if (lse_in) {
-    lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256)), 256, 0, st>>>(lse_in, neg_lse2, P);
+    lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256), (unsigned)n), 256, 0, st>>>(lse, neg_lse2, a.lse_stride, P);
   } else {
     D2O_LAUNCH_CS_ALL(kSweepRows);
   }

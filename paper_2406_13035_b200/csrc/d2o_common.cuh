@@ -146,16 +146,17 @@ enum Counter { kCntDecodeSteps = 0, kCntEvictions, kCntMerges, kCntDiscards, kCn
 
 // ----------------------------------------------------------------------------- context
 struct Layout {            // byte offsets into `state`
-  size_t status, counters, density, budgets, windows, row_off, order, plen, len, tau, steps_done, sim_items, colsum, pos, score, rnorm, kpool, vpool, end;
+  size_t status, counters, colsum_sched, density, budgets, windows, row_off, order, plen, len, tau, steps_done, sim_items, colsum, pos, score, rnorm, kpool, vpool, end;
 };
 struct ScratchLayout {     // byte offsets into `scratch`
   size_t lse, evict_idx, evict_mx, evict_nn, seg_start, seg_items, seg_tmp, part_key, pl_spill, stage_q, stage_k, stage_v, stage_out, end;
-  size_t lse_stride;       // `lse` exists kStatsLanes times, this far apart (d2o_layer_stats_layers)
+  size_t lse_stride;       // `lse` exists kColsumLayers times, this far apart (d2o_layer_stats_layers)
   size_t stage_stride;     // stage_q .. stage_out exist 2 * kHostBlock times, this far apart (d2o_decode_steps_host)
   size_t lane_stride;      // evict_idx .. part_key are the working set of one layer's compression: kCompressLanes copies, this far apart
 };
 constexpr int kHostBlock = 4;       // steps per block of d2o_decode_steps_host (two blocks of staging sets)
-constexpr int kStatsLanes = 2;      // layers whose column sums d2o_layer_stats_layers computes side by side
+constexpr int kStatsLanes = 2;      // layers whose column sums d2o_layer_stats_layers computes side by side (FFMA kernels)
+constexpr int kColsumLayers = 8;    // layers whose column sums share a launch (tensor-core kernels)
 constexpr int kCompressLanes = 4;   // layers that d2o_prefill_compress_layers works on side by side
 
 }  // namespace d2o
@@ -217,6 +218,9 @@ namespace d2o {
 // launchers (one per .cu file); all return cudaError_t of the launch
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
                                cudaStream_t st, int lane = 0);
+// the layers [layer, layer + n), n <= kColsumLayers, in one launch per kernel (16-bit inputs)
+cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
+                                  const float* const* lse, cudaStream_t st);
 cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, int P, float rho, int min_budget,
                            int max_budget, float gamma, int head_reduce, int budget_rule, int n_sink, int window,
                            float nm_ratio, int32_t* budgets, int32_t* windows, int64_t* row_off, uint32_t* status_word,
@@ -234,9 +238,9 @@ size_t sim_tc_part_key_bytes(const d2o_config* cfg, int max_budget);
 size_t sim_tc_max_items(const d2o_config* cfg, int max_budget);
 size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count, int32_t* first);
 // tensor-core column sums of the prompt attention for 16-bit Q/K (d2o_colsum_tc.cu)
-cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, const void* Q, const void* K,
-                             const float* lse_in, float* neg_lse2, float* colsum, const int32_t* plen, uint32_t* status,
-                             cudaStream_t st);
+cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, int n, const void* const* Q,
+                             const void* const* K, const float* const* lse_in, float* neg_lse2, size_t lse_stride,
+                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st);
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P);      // its row normalisers
 
 // remembers the text of a failed CUDA runtime call for d2o_last_cuda_error(); returns D2O_ERR_CUDA

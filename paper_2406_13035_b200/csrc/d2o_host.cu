@@ -101,6 +101,7 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
   l->status = take(16);
   l->counters = take(kNumCounters * 8);
+  l->colsum_sched = take(8);
   l->density = take(B * L * Hq * 8);
   l->budgets = take(B * L * Hkv * 4);
   l->windows = take(B * L * Hkv * 4);
@@ -121,7 +122,7 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   o = 0;
   s->lse = take(colsum_tc_lse_bytes(c->batch, c->n_q_heads, c->prompt_len));
   s->lse_stride = o - s->lse;
-  o += (size_t)(kStatsLanes - 1) * s->lse_stride;
+  o += (size_t)(kColsumLayers - 1) * s->lse_stride;
   s->evict_idx = take(B * Hkv * P * 4);
   s->evict_mx = take(B * Hkv * P * 4);
   s->evict_nn = take(B * Hkv * P * 4);
@@ -268,6 +269,14 @@ extern "C" d2o_status d2o_layer_stats_layers(d2o_ctx* c, int32_t l0, int32_t l1,
   cudaStream_t st = (cudaStream_t)stream;
   if (l1 - l0 == 1) {
     CUDA_TRY(launch_layer_stats(c, l0, Q[0], K[0], lse ? lse[0] : nullptr, st));
+  } else if (c->stats_path == 0 && c->cfg.dtype != D2O_F32) {
+    // several layers per launch; a group is all with or all without the caller's normalisers
+    for (int l = l0, n; l < l1; l += n) {
+      auto has = [&](int i) { return lse != nullptr && lse[i - l0] != nullptr; };
+      n = 1;
+      while (n < kColsumLayers && l + n < l1 && has(l + n) == has(l)) ++n;
+      CUDA_TRY(launch_layer_stats_tc(c, l, n, Q + (l - l0), K + (l - l0), has(l) ? lse + (l - l0) : nullptr, st));
+    }
   } else {
     const d2o_status ls = ensure_lanes(c);
     if (ls != D2O_OK) return ls;

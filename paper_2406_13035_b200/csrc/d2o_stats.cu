@@ -186,39 +186,61 @@ colsum_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __r
 }
 
 // F[b, layer, hq] = (1/P) sum_j (s_j - mean)^2, mean = (1/P) sum_j s_j   (Eq. 4; population variance)
-__global__ void __launch_bounds__(256)
-density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer,
+// One CTA per (sequence, head) and layer (blockIdx.y).  Two passes in fp64; a thread keeps its values of the first pass in
+// registers (up to 8, P <= 4096) or reads them again (8192 tokens, 32 heads: 21.6 us with 256 threads that read everything
+// twice and one value at a time; the kernel is a chain of load latencies).
+constexpr int kDensityThreads = 512;
+__global__ void __launch_bounds__(kDensityThreads)
+density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
                const int32_t* __restrict__ plen) {
-  __shared__ double part[8];
-  __shared__ double mean_s;
-  const int bh = blockIdx.x;
+  constexpr int kKeep = 8, kWarps = kDensityThreads / 32;
+  __shared__ double part[kWarps];
+  const int bh = blockIdx.x, layer = layer0 + (int)blockIdx.y;
   const int b = bh / Hq, hq = bh % Hq;
   const int P = plen ? plen[b] : Pmax;
-  const float* s = colsum + (size_t)bh * Pmax;
+  const float* s = colsum + ((size_t)blockIdx.y * gridDim.x + bh) * Pmax;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto block_total = [&](double t) {                                 // every thread gets it
+    t = warp_sum(t);
+    __syncthreads();
+    if (lane == 0) part[warp] = t;
+    __syncthreads();
+    t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) t += part[w];
+    return t;
+  };
+  float v[kKeep];
   double t = 0.0;
-  for (int j = threadIdx.x; j < P; j += blockDim.x) t += (double)s[j];
-  t = warp_sum(t);
-  if (lane == 0) part[warp] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0;
-    for (int w = 0; w < 8; ++w) a += part[w];
-    mean_s = a / (double)P;
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) {
+    const int j = threadIdx.x + i * kDensityThreads;
+    v[i] = j < P ? s[j] : 0.f;
   }
-  __syncthreads();
-  const double mean = mean_s;
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i) t += (double)v[i];
+  for (int j0 = threadIdx.x + kKeep * kDensityThreads; j0 < P; j0 += 4 * kDensityThreads) {
+    float f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = j0 + i * kDensityThreads < P ? s[j0 + i * kDensityThreads] : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t += (double)f[i];
+  }
+  const double mean = block_total(t) / (double)P;
   t = 0.0;
-  for (int j = threadIdx.x; j < P; j += blockDim.x) { const double dlt = (double)s[j] - mean; t += dlt * dlt; }
-  t = warp_sum(t);
-  __syncthreads();
-  if (lane == 0) part[warp] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0;
-    for (int w = 0; w < 8; ++w) a += part[w];
-    density[((size_t)b * L + layer) * Hq + hq] = a / (double)P;
+#pragma unroll
+  for (int i = 0; i < kKeep; ++i)
+    if (threadIdx.x + i * kDensityThreads < P) { const double dlt = (double)v[i] - mean; t += dlt * dlt; }
+  for (int j0 = threadIdx.x + kKeep * kDensityThreads; j0 < P; j0 += 4 * kDensityThreads) {
+    float f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = j0 + i * kDensityThreads < P ? s[j0 + i * kDensityThreads] : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (j0 + i * kDensityThreads < P) { const double dlt = (double)f[i] - mean; t += dlt * dlt; }
   }
+  t = block_total(t);
+  if (threadIdx.x == 0) density[((size_t)b * L + layer) * Hq + hq] = t / (double)P;
 }
 
 // Cache sizes from the densities.  budget_rule 0 (Eq. 5): S_l = clip(lambda * w_l, S_min, S_max) with
@@ -447,14 +469,6 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
   float* colsum = (float*)(c->state + c->lay.colsum) + (size_t)layer * B * Hq * P;
   double* density = (double*)(c->state + c->lay.density);
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
-  if (c->stats_path == 0 && g.dtype != D2O_F32) {
-    cudaError_t e = launch_colsum_tc(g.dtype, D, B, Hq, g.n_kv_heads, P, Q, K, lse_in,
-                                     (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride), colsum, plen,
-                                     (uint32_t*)(c->state + c->lay.status), st);
-    if (e != cudaSuccess) return e;
-    density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, g.n_layers, layer, plen);
-    return cudaGetLastError();
-  }
   const float* lse = lse_in;
   dim3 grid(nT, B * Hq);
   if (!lse) {
@@ -469,12 +483,28 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
   cudaError_t e = cudaFuncSetAttribute(colsum_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
   if (e != cudaSuccess) return e;
   colsum_kernel<T, D><<<grid, kStatThreads, sm2, st>>>((const T*)Q, (const T*)K, lse, colsum, P, Hq, c->group, plen);
-  density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, g.n_layers, layer, plen);
+  density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, g.n_layers, layer, plen);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
+                                  const float* const* lse, cudaStream_t st) {
+  const d2o_config& g = c->cfg;
+  const int P = g.prompt_len, Hq = g.n_q_heads, B = g.batch;
+  float* colsum = (float*)(c->state + c->lay.colsum) + (size_t)layer * B * Hq * P;
+  const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
+  cudaError_t e = launch_colsum_tc(g.dtype, g.d_head, B, Hq, g.n_kv_heads, P, n, Q, K, lse, (float*)(c->scratch + c->slay.lse),
+                                   c->slay.lse_stride, colsum, plen, (uint32_t*)(c->state + c->lay.status),
+                                   (uint32_t*)(c->state + c->lay.colsum_sched), st);
+  if (e != cudaSuccess) return e;
+  density_kernel<<<dim3((unsigned)(B * Hq), (unsigned)n), kDensityThreads, 0, st>>>(colsum, (double*)(c->state + c->lay.density), P, Hq,
+                                                                                 g.n_layers, layer, plen);
   return cudaGetLastError();
 }
 
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
                                cudaStream_t st, int lane) {
+  if (c->stats_path == 0 && c->cfg.dtype != D2O_F32) return launch_layer_stats_tc(c, layer, 1, &Q, &K, lse ? &lse : nullptr, st);
   const int d = c->cfg.d_head;
   switch (c->cfg.dtype) {
     case D2O_F32: return d == 64 ? run_stats<float, 64>(c, layer, Q, K, lse, st, lane) : run_stats<float, 128>(c, layer, Q, K, lse, st, lane);
@@ -506,7 +536,9 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
 // Scratch for the row normalisers of d2o_layer_stats_static: part of the library image, one copy per GPU.  The
 // tensor-core kernels pad every (sequence, head) row to a multiple of four floats.
 constexpr int kStaticMaxRows = 65535;                // (sequence, head) pairs: one grid row of the generic kernels each
-static __device__ __align__(256) float g_static_lse[D2O_STATIC_LSE_FLOATS + 3 * kStaticMaxRows];
+// The two words behind them are its work counter (zero in the image, and left at zero by every launch).
+constexpr size_t kStaticFloats = (size_t)D2O_STATIC_LSE_FLOATS + 3 * kStaticMaxRows + 1;
+static __device__ __align__(256) float g_static_lse[kStaticFloats + 2];
 constexpr int kMaxDevices = 64;
 static float* g_static_lse_addr[kMaxDevices];        // device address of g_static_lse, per device (host-side cache)
 
@@ -514,9 +546,10 @@ template <typename T, int D>
 static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, float* lse_buf, float* colsum, double* density,
                                     int B, int Hq, int group, int P, cudaStream_t st) {
   if (sizeof(T) == 2) {
-    cudaError_t e = launch_colsum_tc(dtype, D, B, Hq, Hq / group, P, Q, K, nullptr, lse_buf, colsum, nullptr, nullptr, st);
+    cudaError_t e = launch_colsum_tc(dtype, D, B, Hq, Hq / group, P, 1, &Q, &K, nullptr, lse_buf, 0, colsum, nullptr, nullptr,
+                                     (uint32_t*)(lse_buf + kStaticFloats), st);
     if (e != cudaSuccess) return e;
-    density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
+    density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
     return cudaGetLastError();
   }
   const int nT = (P + kTile - 1) / kTile;
@@ -529,7 +562,7 @@ static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, flo
   e = cudaFuncSetAttribute(colsum_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
   if (e != cudaSuccess) return e;
   colsum_kernel<T, D><<<grid, kStatThreads, sm2, st>>>((const T*)Q, (const T*)K, lse_buf, colsum, P, Hq, group, nullptr);
-  density_kernel<<<B * Hq, 256, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
+  density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
   return cudaGetLastError();
 }
 
