@@ -155,8 +155,7 @@ d2o_status d2o_layer_stats(d2o_ctx* ctx, int32_t layer, const void* Q, const voi
  * layers' Q and K can hand them over together).  Q, K: HOST arrays of l1-l0 DEVICE pointers;
  * lse: NULL, or a HOST array of l1-l0 DEVICE pointers (entries may be NULL).  16-bit inputs: up to
  * eight layers share a launch, so that short prompts fill the GPU.  fp32 inputs: two layers are
- * worked on side by side on streams of the library's own (as d2o_prefill_compress_layers does,
- * same fork / join on `stream`, same first-call creation of streams and events), each with its
+ * worked on side by side on streams of the library's own, each with its
  * own row-normaliser scratch, so that one layer's last CTAs share the GPU with the next layer's
  * first.  Results are those of l1-l0 calls of d2o_layer_stats, bit for bit. */
 d2o_status d2o_layer_stats_layers(d2o_ctx* ctx, int32_t l0, int32_t l1, const void* const* Q,
@@ -188,11 +187,9 @@ d2o_status d2o_prefill_compress(d2o_ctx* ctx, int32_t layer, const void* K, cons
 /* The same for layers [l0, l1) in one call (Eq. 5 needs every layer's density before any layer
  * can be compressed, so at this point the caller holds all layers' K and V anyway).
  * K, V: HOST arrays of l1-l0 DEVICE pointers, each [B, Hkv, P, d].  The layers are independent
- * (Eq. 6-12 act per layer and head); the library works on up to four of them side by side, each
- * on a stream of its own with its own part of `scratch`, so that the per-layer kernels of a small
- * batch (B * Hkv CTAs each) fill the GPU together.  The internal streams start behind everything
- * `stream` holds at the call, and `stream` continues behind all of them; the first call creates
- * them (streams and events only, no device memory).  Results are those of l1-l0 calls of
+ * (Eq. 6-12 act per layer and head): up to 16 of them share every launch, each with its own part
+ * of `scratch` (fewer where that would take more than 256 MB, but at least four), so that the
+ * per-layer work of a small batch fills the GPU together.  Results are those of l1-l0 calls of
  * d2o_prefill_compress, bit for bit; the inspection arrays of d2o_get_view (evicted positions,
  * Max(U), Argmax) then show one of the layers, not necessarily the last. */
 d2o_status d2o_prefill_compress_layers(d2o_ctx* ctx, int32_t l0, int32_t l1, const void* const* K,

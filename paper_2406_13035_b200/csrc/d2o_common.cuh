@@ -149,15 +149,16 @@ struct Layout {            // byte offsets into `state`
   size_t status, counters, colsum_sched, density, budgets, windows, row_off, order, plen, len, tau, steps_done, sim_items, colsum, pos, score, rnorm, kpool, vpool, end;
 };
 struct ScratchLayout {     // byte offsets into `scratch`
-  size_t lse, evict_idx, evict_mx, evict_nn, seg_start, seg_items, seg_tmp, part_key, pl_spill, stage_q, stage_k, stage_v, stage_out, end;
+  size_t lse, evict_idx, evict_mx, evict_nn, seg_start, seg_items, seg_tmp, part_key, prompt_rn, pl_spill, stage_q, stage_k, stage_v, stage_out, end;
   size_t lse_stride;       // `lse` exists kColsumLayers times, this far apart (d2o_layer_stats_layers)
   size_t stage_stride;     // stage_q .. stage_out exist 2 * kHostBlock times, this far apart (d2o_decode_steps_host)
-  size_t lane_stride;      // evict_idx .. part_key are the working set of one layer's compression: kCompressLanes copies, this far apart
+  size_t lane_stride;      // evict_idx .. prompt_rn are the working set of one layer's compression: n_lanes copies, this far apart
+  int n_lanes;
 };
 constexpr int kHostBlock = 4;       // steps per block of d2o_decode_steps_host (two blocks of staging sets)
 constexpr int kStatsLanes = 2;      // layers whose column sums d2o_layer_stats_layers computes side by side (FFMA kernels)
 constexpr int kColsumLayers = 8;    // layers whose column sums share a launch (tensor-core kernels)
-constexpr int kCompressLanes = 4;   // layers that d2o_prefill_compress_layers works on side by side
+constexpr int kCompressLayers = 16; // most layers whose compression shares the launches (d2o_prefill_compress_layers)
 
 }  // namespace d2o
 
@@ -202,9 +203,9 @@ struct d2o_ctx {
   int stats_path;              // tuning: 0 = tensor cores for the column sums of 16-bit Q/K, 1 = FFMA kernels
   int wait_limit_us;           // failure-detection tests: limit of a device-side wait in microseconds (0 = one second)
   int producer_stop_stage;     // failure-detection tests: the decode producer issues no copy from this stage on (-1 = never)
-  // d2o_prefill_compress_layers: one stream per lane, created with the first call (no device memory involved)
-  cudaStream_t lane_stream[d2o::kCompressLanes];
-  cudaEvent_t lane_done[d2o::kCompressLanes];
+  // d2o_layer_stats_layers, fp32: one stream per lane, created with the first call (no device memory involved)
+  cudaStream_t lane_stream[d2o::kStatsLanes];
+  cudaEvent_t lane_done[d2o::kStatsLanes];
   cudaEvent_t lane_fork;
   bool lanes_ready;
   // d2o_decode_steps_host: a stream for the copies to the device, one for the copies back; created with the first call
@@ -225,7 +226,9 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
                            int max_budget, float gamma, int head_reduce, int budget_rule, int n_sink, int window,
                            float nm_ratio, int32_t* budgets, int32_t* windows, int64_t* row_off, uint32_t* status_word,
                            const int32_t* plen, cudaStream_t st);
-cudaError_t launch_prefill_compress(const d2o_ctx* c, int layer, const void* K, const void* V, cudaStream_t st, int lane = 0);
+// the layers [layer, layer + n), n <= kCompressLayers and <= ScratchLayout::n_lanes, in one launch per kernel
+cudaError_t launch_prefill_compress(const d2o_ctx* c, int layer, int n, const void* const* K, const void* const* V,
+                                    cudaStream_t st);
 cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const void* k, const void* v, void* out,
                           cudaStream_t st, d2o_status* why, bool chained = false, bool publish = false);
 cudaError_t launch_full_decode(int dtype, int d, int n_slices, int group, int capacity, int len, void* kc, void* vc,
@@ -233,7 +236,7 @@ cudaError_t launch_full_decode(int dtype, int d, int n_slices, int group, int ca
                                d2o_status* why);
 
 // tensor-core similarity + nearest neighbour for 16-bit keys (d2o_sim_tc.cu); fills evict_mx / evict_nn
-cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, const void* K, int max_S, cudaStream_t st, int lane = 0);
+cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, int n, const void* const* K, int max_evicted, cudaStream_t st);
 size_t sim_tc_part_key_bytes(const d2o_config* cfg, int max_budget);
 size_t sim_tc_max_items(const d2o_config* cfg, int max_budget);
 size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* count, int32_t* first);

@@ -130,8 +130,12 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   s->seg_items = take(B * Hkv * P * 4);
   s->seg_tmp = take(B * Hkv * P * 4);
   s->part_key = take(c->dtype == D2O_F32 ? 0 : sim_tc_part_key_bytes(c, max_budget));
-  s->lane_stride = o - s->evict_idx;                       // the arrays above, once more per further lane
-  o += (size_t)(kCompressLanes - 1) * s->lane_stride;
+  s->prompt_rn = take(c->dtype == D2O_F32 ? 0 : B * Hkv * P * 4);
+  // the arrays above, once per layer that shares the launches of d2o_prefill_compress_layers: four, more of small batches
+  s->lane_stride = o - s->evict_idx;
+  s->n_lanes = (int)std::min<size_t>(L, s->lane_stride * kCompressLayers <= (256u << 20) ? kCompressLayers
+                                        : std::max<size_t>(4, (256u << 20) / s->lane_stride));
+  o += (size_t)(s->n_lanes - 1) * s->lane_stride;
   s->pl_spill = take((rows + 8 * L * B * Hkv) * (Hq / Hkv) * 4);
   s->stage_q = take(L * B * Hq * d * e);
   s->stage_k = take(L * B * Hkv * d * e);
@@ -229,7 +233,7 @@ extern "C" void d2o_destroy(d2o_ctx* c) {
     }
   }
   if (c->lanes_ready) {
-    for (int i = 0; i < kCompressLanes; ++i) { cudaStreamDestroy(c->lane_stream[i]); cudaEventDestroy(c->lane_done[i]); }
+    for (int i = 0; i < kStatsLanes; ++i) { cudaStreamDestroy(c->lane_stream[i]); cudaEventDestroy(c->lane_done[i]); }
     cudaEventDestroy(c->lane_fork);
   }
   free(c->h_tables); free(c->h_sim_off); free(c->h_pair_max); free(c->h_pair_sum);
@@ -251,7 +255,7 @@ extern "C" d2o_status d2o_layer_stats(d2o_ctx* c, int32_t layer, const void* Q, 
 // the library's own streams for the multi-layer calls: streams and events only, no device memory
 static d2o_status ensure_lanes(d2o_ctx* c) {
   if (c->lanes_ready) return D2O_OK;
-  for (int i = 0; i < kCompressLanes; ++i) {
+  for (int i = 0; i < kStatsLanes; ++i) {
     CUDA_TRY(cudaStreamCreateWithFlags(&c->lane_stream[i], cudaStreamNonBlocking));
     CUDA_TRY(cudaEventCreateWithFlags(&c->lane_done[i], cudaEventDisableTiming));
   }
@@ -375,7 +379,7 @@ extern "C" d2o_status d2o_prefill_compress(d2o_ctx* c, int32_t layer, const void
   if (!c || layer < 0 || layer >= c->cfg.n_layers) return D2O_ERR_INVALID_ARG;
   if (!aligned16(K) || !aligned16(V)) return D2O_ERR_INVALID_ARG;
   if (!c->have_budgets) return D2O_ERR_STATE;
-  CUDA_TRY(launch_prefill_compress(c, layer, K, V, (cudaStream_t)stream));
+  CUDA_TRY(launch_prefill_compress(c, layer, 1, &K, &V, (cudaStream_t)stream));
   c->layer_compressed[layer] = 1;
   c->layer_steps[layer] = 0;
   c->layer_published[layer] = 1;                              // the compression sets the step counters to zero
@@ -389,23 +393,11 @@ extern "C" d2o_status d2o_prefill_compress_layers(d2o_ctx* c, int32_t l0, int32_
     if (!aligned16(K[l - l0]) || !aligned16(V[l - l0])) return D2O_ERR_INVALID_ARG;
   if (!c->have_budgets) return D2O_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
-  if (l1 - l0 == 1) {
-    CUDA_TRY(launch_prefill_compress(c, l0, K[0], V[0], st));
-  } else {
-    const d2o_status ls = ensure_lanes(c);
-    if (ls != D2O_OK) return ls;
-    // the lanes start behind everything the caller's stream holds, the caller's stream goes on behind every lane
-    const int lanes = min(kCompressLanes, l1 - l0);
-    CUDA_TRY(cudaEventRecord(c->lane_fork, st));
-    for (int i = 0; i < lanes; ++i) CUDA_TRY(cudaStreamWaitEvent(c->lane_stream[i], c->lane_fork, 0));
-    for (int l = l0; l < l1; ++l) {
-      const int lane = (l - l0) % lanes;                     // a lane's layers follow one another on its stream
-      CUDA_TRY(launch_prefill_compress(c, l, K[l - l0], V[l - l0], c->lane_stream[lane], lane));
-    }
-    for (int i = 0; i < lanes; ++i) {
-      CUDA_TRY(cudaEventRecord(c->lane_done[i], c->lane_stream[i]));
-      CUDA_TRY(cudaStreamWaitEvent(st, c->lane_done[i], 0));
-    }
+  // equal groups of at most n_lanes layers, one after another
+  const int groups = (l1 - l0 + c->slay.n_lanes - 1) / c->slay.n_lanes;
+  for (int g = 0; g < groups; ++g) {
+    const int a = l0 + (int)((long)(l1 - l0) * g / groups), b = l0 + (int)((long)(l1 - l0) * (g + 1) / groups);
+    CUDA_TRY(launch_prefill_compress(c, a, b - a, K + (a - l0), V + (a - l0), st));
   }
   for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; c->layer_published[l] = 1; }
   return D2O_OK;

@@ -17,11 +17,24 @@
 
 namespace d2o {
 
+// Every kernel works on up to kCompressLayers layers per launch (blockIdx.z, or the work list of the similarity kernel):
+// a layer of a small batch is 8 to 32 slices, a fraction of the GPU.  `stride` bytes separate the working arrays of two
+// layers of the launch.
+struct LayerRows {
+  const void* K[kCompressLayers];
+  const void* V[kCompressLayers];
+};
+template <typename T>
+__device__ __forceinline__ T* of_layer(T* p, size_t stride, int z) {
+  return reinterpret_cast<T*>(const_cast<char*>(reinterpret_cast<const char*>(p)) + stride * z);
+}
+
 // ------------------------------------------------------------------------------------ select
 constexpr int kSelThreads = 1024;
+constexpr int kSelItems = 4;            // consecutive positions per thread in the compaction
 
 struct SelectArgs {
-  const float* colsum;     // [B, Hq, P] of this layer
+  const float* colsum;     // [layers][B, Hq, P]
   const int32_t* budgets;  // [B, L, Hkv]
   const int32_t* windows;  // [B, L, Hkv]
   const int64_t* row_off;  // [B, L, Hkv]
@@ -30,10 +43,11 @@ struct SelectArgs {
   int32_t* steps_done;                        // [L, B, Hkv] decode steps completed on the slice
   int32_t* evict_idx;      // [B, Hkv, P]
   float* keys_spill;       // [B, Hkv, P] group scores when P does not fit in shared memory (may alias evict_mx)
+  size_t stride;           // bytes between two layers' evict_idx, keys_spill
   unsigned long long* counters;
   uint32_t* status;
   const int32_t* plen;     // [B] prompt length of every sequence; P below is the length the tensors are laid out for
-  int L, layer, B, Hq, Hkv, G, P, T;
+  int L, layer0, B, Hq, Hkv, G, P, T;
   int keys_in_smem;
   long long pool_rows;     // rows of the cache pool (bounds of the checked build)
   int value_feature;       // 1: the similarity of Eq. 9 is taken on the value rows (ablation), so the norms are theirs
@@ -60,10 +74,11 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
   return inc - v + warp_tot[warp];
 }
 
-template <typename T, int D>
+// One CTA per slice.  A chain of block-wide steps: what costs is the number of barriers and the serial pieces between
+// them (32 slices of 1200 tokens: 28 us when one thread walked through the 256 bins of every radix round and the
+// compaction scanned twice per 1024 positions).
 __global__ void __launch_bounds__(kSelThreads)
-select_kernel(SelectArgs a, const T* __restrict__ K, const T* __restrict__ V, T* __restrict__ kpool,
-              T* __restrict__ vpool) {
+select_kernel(SelectArgs a) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
   __shared__ int hist[256];
   __shared__ int warp_tot[32];
@@ -71,23 +86,25 @@ select_kernel(SelectArgs a, const T* __restrict__ K, const T* __restrict__ V, T*
   __shared__ uint32_t s_prefix;
   __shared__ int s_need;
   const int slice = blockIdx.x;                 // b * Hkv + h
+  const int layer = a.layer0 + (int)blockIdx.z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
   const int Pmax = a.P;                         // row stride of the per-position arrays
   const int P = a.plen[b];                      // this sequence's prompt length
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int e = slice_entry(b, layer, h, a.L, a.Hkv);
+  const int S = a.budgets[e];
   const int Tn = a.T < S ? a.T : S;
-  const int M = a.windows[slice_entry(b, a.layer, h, a.L, a.Hkv)];
-  const int64_t row0 = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)];
-  const int sidx = (a.layer * a.B + b) * a.Hkv + h;
-  float* keys = a.keys_in_smem ? reinterpret_cast<float*>(sel_smem) : a.keys_spill + (size_t)slice * Pmax;
+  const int M = a.windows[e];
+  const int64_t row0 = a.row_off[e];
+  const int sidx = (layer * a.B + b) * a.Hkv + h;
+  int32_t* const evict_idx = of_layer(a.evict_idx, a.stride, blockIdx.z) + (size_t)slice * Pmax;
+  float* keys = a.keys_in_smem ? reinterpret_cast<float*>(sel_smem) : of_layer(a.keys_spill, a.stride, blockIdx.z) + (size_t)slice * Pmax;
   // group score: sum over the G query heads of this KV head, fixed order (Eq. 6 case 1)
-  const float* cs = a.colsum + ((size_t)b * a.Hq + (size_t)h * a.G) * Pmax;
+  const float* cs = a.colsum + ((size_t)blockIdx.z * a.B * a.Hq + (size_t)b * a.Hq + (size_t)h * a.G) * Pmax;
   for (int j = threadIdx.x; j < P; j += blockDim.x) {
     float t = cs[j];
     for (int g = 1; g < a.G; ++g) t += cs[(size_t)g * Pmax + j];
     keys[j] = t;
   }
-  __syncthreads();
   const bool keep_all = S >= P;
   const int lo = Tn, hi = keep_all ? Tn : P - M;   // candidate range [lo, hi)
   const int N = S - Tn - M;
@@ -104,55 +121,78 @@ select_kernel(SelectArgs a, const T* __restrict__ K, const T* __restrict__ V, T*
         if ((o & mask) == prefix) atomicAdd(&hist[(o >> shift) & 255], 1);
       }
       __syncthreads();
-      if (threadIdx.x == 0) {
-        int acc = 0, bin = 255;
-        for (; bin > 0; --bin) { if (acc + hist[bin] >= need) break; acc += hist[bin]; }
-        s_prefix = prefix | ((uint32_t)bin << shift);
-        s_need = need - acc;
+      if (threadIdx.x < 32) {
+        // the bin, from the top, in which the running count reaches `need`: eight bins per lane
+        const int lane = threadIdx.x;
+        int c[8], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { c[i] = hist[255 - (lane * 8 + i)]; sum += c[i]; }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+        int acc = inc - sum;
+        if (acc < need && (need <= inc || lane == 31)) {
+          int i = 0;
+          while (i < 7 && acc + c[i] < need) acc += c[i++];
+          s_prefix = prefix | ((uint32_t)(255 - (lane * 8 + i)) << shift);
+          s_need = need - acc;
+        }
       }
       __syncthreads();
       prefix = s_prefix; need = s_need; mask |= 255u << shift;
-      __syncthreads();
     }
     kth = prefix; need_eq = need;                 // keep all keys > kth and the first need_eq keys == kth
   }
-  // ordered compaction over positions, 1024 at a time
-  int n_ret = 0, n_ev = 0, n_eq = 0;
-  for (int base = 0; base < P; base += blockDim.x) {
-    const int j = base + threadIdx.x;
-    int is_eq = 0, keep = 0;
-    uint32_t o = 0;
-    if (j < P) {
-      if (keep_all || j < Tn || j >= P - M) keep = 1;
-      else if (N > 0) { o = float_ord(keys[j]); if (o > kth) keep = 1; else if (o == kth) is_eq = 1; }
+  __syncthreads();
+  // Ordered compaction over positions, 4096 at a time.  One scan carries two counts: positions kept for certain (low half)
+  // and positions equal to the N-th score (high half), of which the first need_eq are kept.
+  int n_ret = 0, n_eq = 0;                        // before the current block: kept for certain, equal
+  for (int base = 0; base < P; base += kSelItems * kSelThreads) {
+    const int j0 = base + threadIdx.x * kSelItems;
+    int sure = 0, eq = 0;                         // bit i: position j0 + i
+#pragma unroll
+    for (int i = 0; i < kSelItems; ++i) {
+      const int j = j0 + i;
+      if (j < P) {
+        if (keep_all || j < Tn || j >= P - M) sure |= 1 << i;
+        else if (N > 0) {
+          const uint32_t o = float_ord(keys[j]);
+          if (o > kth) sure |= 1 << i;
+          else if (o == kth) eq |= 1 << i;
+        }
+      }
     }
-    const int eq_rank = block_exclusive_scan(is_eq, warp_tot, &s_total);
-    const int eq_tot = s_total;
-    if (is_eq && n_eq + eq_rank < need_eq) keep = 1;
-    const int kr = block_exclusive_scan(keep, warp_tot, &s_total);
-    const int keep_tot = s_total;
-    if (j < P) {
+    const int before = block_exclusive_scan(__popc(sure) | (__popc(eq) << 16), warp_tot, &s_total);
+    const int tot = s_total;
+    int n_sure = n_ret + (before & 0xffff), e_rank = n_eq + (before >> 16);
+#pragma unroll
+    for (int i = 0; i < kSelItems; ++i) {
+      const int j = j0 + i;
+      if (j >= P) break;
+      const bool is_eq = (eq >> i) & 1;
+      const bool keep = ((sure >> i) & 1) || (is_eq && e_rank < need_eq);
+      const int slot = n_sure + min(e_rank, need_eq);             // kept positions before j
       if (keep) {
-        const int slot = n_ret + kr;
         if (D2O_GUARD(slot < (keep_all ? P : S) && row0 + slot < a.pool_rows, a.status, 0xC4EC0001u)) {
           a.pos[row0 + slot] = j;
           a.score[row0 + slot] = keys[j];
         }
       } else {
-        const int at = n_ev + (threadIdx.x - kr);
-        if (D2O_GUARD(at >= 0 && at < P, a.status, 0xC4EC0002u)) a.evict_idx[(size_t)slice * Pmax + at] = j;
+        const int at = j - slot;
+        if (D2O_GUARD(at >= 0 && at < P, a.status, 0xC4EC0002u)) evict_idx[at] = j;
       }
+      n_sure += (sure >> i) & 1;
+      e_rank += is_eq ? 1 : 0;
     }
-    const int valid = min((int)blockDim.x, P - base);
-    n_ret += keep_tot; n_ev += valid - keep_tot; n_eq += eq_tot;
-    __syncthreads();
+    n_ret += tot & 0xffff; n_eq += tot >> 16;
+    __syncthreads();                              // s_total and warp_tot are used again
   }
   const int n_keep = keep_all ? P : S;
   if (threadIdx.x == 0) {
     a.len[sidx] = n_keep;
     a.steps_done[sidx] = 0;
     a.tau[sidx] = 0.f;
-    if (n_ret != n_keep) report_error(a.status, D2O_ERR_STATE, 0x5E000000u | (uint32_t)slice);
+    if (n_ret + min(n_eq, need_eq) != n_keep) report_error(a.status, D2O_ERR_STATE, 0x5E000000u | (uint32_t)slice);
     atomicAdd(&a.counters[kCntPrefillEvicted], (unsigned long long)(P - n_keep));
   }
 }
@@ -161,19 +201,18 @@ select_kernel(SelectArgs a, const T* __restrict__ K, const T* __restrict__ V, T*
 // (a kernel of its own so that a single sequence still fills the GPU).
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
-gather_kernel(SelectArgs a, const T* __restrict__ K, const T* __restrict__ V, T* __restrict__ kpool,
-              T* __restrict__ vpool) {
+gather_kernel(SelectArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__ vpool) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;                   // lanes per row
-  const int slice = blockIdx.y;
+  const int slice = blockIdx.y, layer = a.layer0 + (int)blockIdx.z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
   const int P = a.plen[b];
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int n_keep = S >= P ? P : S;
-  const int64_t row0 = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int64_t row0 = a.row_off[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int grp = threadIdx.x / LPR, lig = threadIdx.x % LPR;
-  const T* Ks = K + (size_t)slice * a.P * D;
-  const T* Vs = V + (size_t)slice * a.P * D;
+  const T* Ks = (const T*)rows.K[blockIdx.z] + (size_t)slice * a.P * D;
+  const T* Vs = (const T*)rows.V[blockIdx.z] + (size_t)slice * a.P * D;
   const int r1 = min(n_keep, ((int)blockIdx.x + 1) * 64);
   for (int r = blockIdx.x * 64 + grp; r < r1; r += blockDim.x / LPR) {
     const int j = a.pos[row0 + r];
@@ -201,26 +240,27 @@ struct SimArgs {
   const float* rnorm; const int32_t* pos;
   uint32_t* status;
   const int32_t* plen;
-  int L, layer, Hkv, P;
+  size_t stride;           // bytes between two layers' evict_idx, evict_mx, evict_nn
+  int L, layer0, Hkv, P;
 };
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kSimThreads)
-similarity_kernel(SimArgs a, const T* __restrict__ K, const T* __restrict__ kpool) {
+similarity_kernel(SimArgs a, LayerRows rows, int value_feature, const T* __restrict__ kpool) {
   extern __shared__ __align__(16) float sim_smem[];
   float* et = sim_smem;                     // [D][64] evicted tile, transposed
   float* ct = et + D * kSimTile;            // [D][64] retained tile, transposed
   float* ern = ct + D * kSimTile;           // [64] inverse norms of the evicted rows
   float* crn = ern + kSimTile;              // [64] inverse norms of the retained rows
-  const int slice = blockIdx.y;
+  const int slice = blockIdx.y, layer = a.layer0 + (int)blockIdx.z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int Le = a.plen[b] - S;
   const int i0 = blockIdx.x * kSimTile;
   if (Le <= 0 || i0 >= Le) return;
-  const int64_t row0 = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)];
-  const T* Ks = K + (size_t)slice * a.P * D;
-  const int32_t* ev = a.evict_idx + (size_t)slice * a.P;
+  const int64_t row0 = a.row_off[slice_entry(b, layer, h, a.L, a.Hkv)];
+  const T* Ks = (const T*)(value_feature ? rows.V : rows.K)[blockIdx.z] + (size_t)slice * a.P * D;
+  const int32_t* ev = of_layer(a.evict_idx, a.stride, blockIdx.z) + (size_t)slice * a.P;
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int VPR = D / EPV;
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
@@ -315,8 +355,8 @@ similarity_kernel(SimArgs a, const T* __restrict__ K, const T* __restrict__ kpoo
       // a row whose similarities are all NaN keeps the initial key: maximum -inf, neighbour 0, never merged
       const int slot = 0x7fffffff - (int)(uint32_t)(key & 0xffffffffu);
       const bool found = (unsigned)slot < (unsigned)S;
-      a.evict_mx[(size_t)slice * a.P + i] = found ? ord_float((uint32_t)(key >> 32)) : -INFINITY;
-      a.evict_nn[(size_t)slice * a.P + i] = found ? slot : 0;
+      of_layer(a.evict_mx, a.stride, blockIdx.z)[(size_t)slice * a.P + i] = found ? ord_float((uint32_t)(key >> 32)) : -INFINITY;
+      of_layer(a.evict_nn, a.stride, blockIdx.z)[(size_t)slice * a.P + i] = found ? slot : 0;
     }
   }
 }
@@ -329,7 +369,8 @@ struct SegArgs {
   unsigned long long* counters;
   uint32_t* status;
   const int32_t* plen;
-  int L, layer, B, Hkv, P, seg_stride;
+  size_t stride;           // bytes between two layers' working arrays
+  int L, layer0, B, Hkv, P, seg_stride;
   float tau_override;
 };
 
@@ -340,15 +381,15 @@ segment_kernel(SegArgs a) {
   __shared__ float s_thr;
   __shared__ int warp_tot[32];
   __shared__ int s_total;
-  const int slice = blockIdx.x;
+  const int slice = blockIdx.x, layer = a.layer0 + (int)blockIdx.z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int Le = a.plen[b] - S;
-  const int sidx = (a.layer * a.B + b) * a.Hkv + h;
-  const float* mx = a.evict_mx + (size_t)slice * a.P;
-  const int32_t* nn = a.evict_nn + (size_t)slice * a.P;
-  int32_t* start = a.seg_start + (size_t)slice * a.seg_stride;
-  int32_t* items = a.seg_items + (size_t)slice * a.P;
+  const int sidx = (layer * a.B + b) * a.Hkv + h;
+  const float* mx = of_layer(a.evict_mx, a.stride, blockIdx.z) + (size_t)slice * a.P;
+  const int32_t* nn = of_layer(a.evict_nn, a.stride, blockIdx.z) + (size_t)slice * a.P;
+  int32_t* start = of_layer(a.seg_start, a.stride, blockIdx.z) + (size_t)slice * a.seg_stride;
+  int32_t* items = of_layer(a.seg_items, a.stride, blockIdx.z) + (size_t)slice * a.P;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (Le <= 0) {
     for (int j = threadIdx.x; j <= S && j < a.seg_stride; j += blockDim.x) start[j] = 0;
@@ -401,7 +442,7 @@ segment_kernel(SegArgs a) {
   // chunk in order (lanes with the same digit are ranked with match_any).
   if (run == 0) return;
   int* hist = reinterpret_cast<int*>(seg_smem);         // [32 warps][64 digits]; the cursors are not needed any more
-  int32_t* tmp = a.seg_tmp + (size_t)slice * a.P;
+  int32_t* tmp = of_layer(a.seg_tmp, a.stride, blockIdx.z) + (size_t)slice * a.P;
   int bits = 0;
   while ((S >> bits) != 0) ++bits;                      // slots are < S
   const int passes = (bits + 5) / 6;
@@ -467,7 +508,8 @@ struct MergeArgs {
   const int32_t* seg_start; const int32_t* seg_items;
   float* rnorm;
   const int32_t* plen;
-  int L, layer, Hkv, P, seg_stride;
+  size_t stride;           // bytes between two layers' working arrays
+  int L, layer0, Hkv, P, seg_stride;
   uint32_t* status;
   int average;             // 1: average merge (every token of a merge weighs the same) instead of Eq. 12
   int value_feature;       // 1: the cached inverse norms belong to the value rows
@@ -477,28 +519,27 @@ constexpr int kMergeFlight = 4;     // merged tokens whose rows a row group has 
 
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
-merge_kernel(MergeArgs a, const T* __restrict__ K, const T* __restrict__ V, T* __restrict__ kpool,
-             T* __restrict__ vpool) {
+merge_kernel(MergeArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__ vpool) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;
-  const int slice = blockIdx.y;
+  const int slice = blockIdx.y, layer = a.layer0 + (int)blockIdx.z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int Le = a.plen[b] - S;
   if (Le <= 0) return;
   const int grp = threadIdx.x / LPR, lig = threadIdx.x % LPR;
   const int j = blockIdx.x * (blockDim.x / LPR) + grp;
   if (j >= S) return;
-  const int32_t* start = a.seg_start + (size_t)slice * a.seg_stride;
+  const int32_t* start = of_layer(a.seg_start, a.stride, blockIdx.z) + (size_t)slice * a.seg_stride;
   const int s0 = start[j], s1 = start[j + 1];
   if (s1 == s0) return;                              // nothing merged: the row stays bit-identical
   if (!D2O_GUARD(s0 >= 0 && s0 < s1 && s1 <= Le, a.status, 0xC4EC0007u)) return;
-  const int64_t row = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)] + j;
-  const int32_t* items = a.seg_items + (size_t)slice * a.P;
-  const int32_t* ev = a.evict_idx + (size_t)slice * a.P;
-  const float* mx = a.evict_mx + (size_t)slice * a.P;
-  const T* Ks = K + (size_t)slice * a.P * D;
-  const T* Vs = V + (size_t)slice * a.P * D;
+  const int64_t row = a.row_off[slice_entry(b, layer, h, a.L, a.Hkv)] + j;
+  const int32_t* items = of_layer(a.seg_items, a.stride, blockIdx.z) + (size_t)slice * a.P;
+  const int32_t* ev = of_layer(a.evict_idx, a.stride, blockIdx.z) + (size_t)slice * a.P;
+  const float* mx = of_layer(a.evict_mx, a.stride, blockIdx.z) + (size_t)slice * a.P;
+  const T* Ks = (const T*)rows.K[blockIdx.z] + (size_t)slice * a.P * D;
+  const T* Vs = (const T*)rows.V[blockIdx.z] + (size_t)slice * a.P * D;
   float ka[EPV], va[EPV], f[EPV];
   Elem<T>::unpack(ld_global_v4(kpool + row * D + lig * EPV), f);
   const float own = a.average ? 1.0f : kEuler;       // weight of the retained token itself: e^{self-similarity}, or 1
@@ -562,16 +603,24 @@ merge_kernel(MergeArgs a, const T* __restrict__ K, const T* __restrict__ V, T* _
 }
 
 // ------------------------------------------------------------------------------------ launcher
+// Layers [layer, layer + n) in one launch per kernel; their working arrays are the first n sets of `scratch`.
 template <typename T, int D>
-static cudaError_t run_prefill(const d2o_ctx* c, int layer, const void* K, const void* V, cudaStream_t st, int lane) {
+static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* const* K, const void* const* V, cudaStream_t st) {
   const d2o_config& g = c->cfg;
   const int B = g.batch, Hkv = g.n_kv_heads, P = g.prompt_len, L = g.n_layers;
   const int n_slices = B * Hkv;
-  char* S = c->state; char* X = c->scratch + (size_t)lane * c->slay.lane_stride;   // only the lane's arrays are used below
+  char* S = c->state; char* X = c->scratch;
   T* kpool = (T*)(S + c->lay.kpool);
   T* vpool = (T*)(S + c->lay.vpool);
-  int maxS = 0;
-  for (int b = 0; b < B; ++b) maxS = max(maxS, c->h_pair_max[b * L + layer]);
+  LayerRows rows;
+  int maxS = 0, maxLe = 0;                       // rows of the longest slice, most evicted rows of any slice
+  for (int l = 0; l < n; ++l) {
+    rows.K[l] = K[l]; rows.V[l] = V[l];
+    for (int b = 0; b < B; ++b) {
+      maxS = max(maxS, c->h_pair_max[b * L + layer + l]);
+      for (int h = 0; h < Hkv; ++h) maxLe = max(maxLe, c->h_plen[b] - c->h_budgets[(b * L + layer + l) * Hkv + h]);
+    }
+  }
   const int seg_stride = c->max_budget + 2;
 
   SelectArgs sa;
@@ -584,46 +633,43 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, const void* K, const
   sa.steps_done = (int32_t*)(S + c->lay.steps_done);
   sa.evict_idx = (int32_t*)(X + c->slay.evict_idx);
   sa.keys_spill = (float*)(X + c->slay.evict_mx);
+  sa.stride = c->slay.lane_stride;
   sa.counters = (unsigned long long*)(S + c->lay.counters);
   sa.status = (uint32_t*)(S + c->lay.status);
   sa.plen = (const int32_t*)(S + c->lay.plen);
-  sa.L = L; sa.layer = layer; sa.B = B; sa.Hq = g.n_q_heads; sa.Hkv = Hkv; sa.G = c->group; sa.P = P; sa.T = g.n_sink;
+  sa.L = L; sa.layer0 = layer; sa.B = B; sa.Hq = g.n_q_heads; sa.Hkv = Hkv; sa.G = c->group; sa.P = P; sa.T = g.n_sink;
   const size_t key_bytes = (size_t)P * sizeof(float);
   sa.keys_in_smem = key_bytes <= 200 * 1024;
   sa.pool_rows = c->pool_rows;
   sa.value_feature = g.sim_feature;
   const size_t sel_sm = sa.keys_in_smem ? key_bytes : 0;
-  cudaError_t e = cudaFuncSetAttribute(select_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sel_sm > 48 * 1024 ? sel_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  select_kernel<T, D><<<n_slices, kSelThreads, sel_sm, st>>>(sa, (const T*)K, (const T*)V, kpool, vpool);
+  select_kernel<<<dim3((unsigned)n_slices, 1, (unsigned)n), kSelThreads, sel_sm, st>>>(sa);
   {
     const int keep_max = min(maxS, P);
-    dim3 ggrid((unsigned)((keep_max + 63) / 64), (unsigned)n_slices);
-    gather_kernel<T, D><<<ggrid, 256, 0, st>>>(sa, (const T*)K, (const T*)V, kpool, vpool);
+    dim3 ggrid((unsigned)((keep_max + 63) / 64), (unsigned)n_slices, (unsigned)n);
+    gather_kernel<T, D><<<ggrid, 256, 0, st>>>(sa, rows, kpool, vpool);
   }
-
-  int maxLe = 0;                                 // most evicted rows of any slice of this layer
-  for (int b = 0; b < B; ++b)
-    for (int h = 0; h < Hkv; ++h) maxLe = max(maxLe, c->h_plen[b] - c->h_budgets[(b * L + layer) * Hkv + h]);
   if (maxLe <= 0) return cudaGetLastError();
 
   SimArgs ma;
   ma.budgets = sa.budgets; ma.row_off = sa.row_off;
   ma.evict_idx = sa.evict_idx; ma.evict_mx = (float*)(X + c->slay.evict_mx); ma.evict_nn = (int32_t*)(X + c->slay.evict_nn);
-  ma.rnorm = sa.rnorm; ma.pos = sa.pos; ma.status = sa.status; ma.plen = sa.plen; ma.L = L; ma.layer = layer; ma.Hkv = Hkv; ma.P = P;
-  const size_t sim_sm = ((size_t)2 * D * kSimTile + 2 * kSimTile) * sizeof(float);
-  e = cudaFuncSetAttribute(similarity_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sim_sm);
-  if (e != cudaSuccess) return e;
+  ma.rnorm = sa.rnorm; ma.pos = sa.pos; ma.status = sa.status; ma.plen = sa.plen; ma.L = L; ma.layer0 = layer; ma.Hkv = Hkv; ma.P = P;
+  ma.stride = sa.stride;
   // rows the similarity is computed on: the keys (Eq. 9), or the values (ablation "Feature choice")
-  const void* feat = g.sim_feature ? V : K;
   const T* feat_pool = g.sim_feature ? vpool : kpool;
   if (sizeof(T) == 2 && c->similarity_path == 0) {
-    e = launch_similarity_tc(c, layer, feat, maxS, st, lane);
+    e = launch_similarity_tc(c, layer, n, g.sim_feature ? V : K, maxLe, st);
     if (e != cudaSuccess) return e;
   } else {
-    dim3 sgrid((maxLe + kSimTile - 1) / kSimTile, n_slices);
-    similarity_kernel<T, D><<<sgrid, kSimThreads, sim_sm, st>>>(ma, (const T*)feat, feat_pool);
+    const size_t sim_sm = ((size_t)2 * D * kSimTile + 2 * kSimTile) * sizeof(float);
+    e = cudaFuncSetAttribute(similarity_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sim_sm);
+    if (e != cudaSuccess) return e;
+    dim3 sgrid((unsigned)((maxLe + kSimTile - 1) / kSimTile), (unsigned)n_slices, (unsigned)n);
+    similarity_kernel<T, D><<<sgrid, kSimThreads, sim_sm, st>>>(ma, rows, g.sim_feature, feat_pool);
   }
 
   SegArgs ga;
@@ -631,36 +677,37 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, const void* K, const
   ga.seg_start = (int32_t*)(X + c->slay.seg_start); ga.seg_items = (int32_t*)(X + c->slay.seg_items);
   ga.seg_tmp = (int32_t*)(X + c->slay.seg_tmp);
   ga.tau = sa.tau; ga.counters = sa.counters; ga.status = sa.status;
-  ga.plen = sa.plen;
-  ga.L = L; ga.layer = layer; ga.B = B; ga.Hkv = Hkv; ga.P = P; ga.seg_stride = seg_stride;
+  ga.plen = sa.plen; ga.stride = sa.stride;
+  ga.L = L; ga.layer0 = layer; ga.B = B; ga.Hkv = Hkv; ga.P = P; ga.seg_stride = seg_stride;
   ga.tau_override = g.tau_override;
   // counts / cursors per retained slot, later the radix histograms (32 warps x 64 digits)
   const size_t seg_sm = (size_t)max(maxS + 1, 32 * 64) * sizeof(int);
   e = cudaFuncSetAttribute(segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(seg_sm > 48 * 1024 ? seg_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  segment_kernel<<<n_slices, 1024, seg_sm, st>>>(ga);
+  segment_kernel<<<dim3((unsigned)n_slices, 1, (unsigned)n), 1024, seg_sm, st>>>(ga);
 
   MergeArgs mg;
   mg.budgets = sa.budgets; mg.row_off = sa.row_off; mg.evict_idx = sa.evict_idx; mg.evict_mx = ma.evict_mx;
   mg.seg_start = ga.seg_start; mg.seg_items = ga.seg_items; mg.rnorm = sa.rnorm;
-  mg.plen = sa.plen;
-  mg.L = L; mg.layer = layer; mg.Hkv = Hkv; mg.P = P; mg.seg_stride = seg_stride; mg.average = g.merge_policy;
+  mg.plen = sa.plen; mg.stride = sa.stride;
+  mg.L = L; mg.layer0 = layer; mg.Hkv = Hkv; mg.P = P; mg.seg_stride = seg_stride; mg.average = g.merge_policy;
   mg.value_feature = g.sim_feature; mg.status = sa.status;
   constexpr int LPR = D / Elem<T>::kPerVec;
   const int rows_per_cta = 256 / LPR;
-  dim3 mgrid((maxS + rows_per_cta - 1) / rows_per_cta, n_slices);
-  merge_kernel<T, D><<<mgrid, 256, 0, st>>>(mg, (const T*)K, (const T*)V, kpool, vpool);
+  dim3 mgrid((unsigned)((maxS + rows_per_cta - 1) / rows_per_cta), (unsigned)n_slices, (unsigned)n);
+  merge_kernel<T, D><<<mgrid, 256, 0, st>>>(mg, rows, kpool, vpool);
   return cudaGetLastError();
 }
 
-cudaError_t launch_prefill_compress(const d2o_ctx* c, int layer, const void* K, const void* V, cudaStream_t st, int lane) {
+cudaError_t launch_prefill_compress(const d2o_ctx* c, int layer, int n, const void* const* K, const void* const* V,
+                                    cudaStream_t st) {
   const int d = c->cfg.d_head;
   switch (c->cfg.dtype) {
-    case D2O_F32: return d == 64 ? run_prefill<float, 64>(c, layer, K, V, st, lane) : run_prefill<float, 128>(c, layer, K, V, st, lane);
-    case D2O_F16: return d == 64 ? run_prefill<__half, 64>(c, layer, K, V, st, lane) : run_prefill<__half, 128>(c, layer, K, V, st, lane);
-    default: return d == 64 ? run_prefill<__nv_bfloat16, 64>(c, layer, K, V, st, lane)
-                            : run_prefill<__nv_bfloat16, 128>(c, layer, K, V, st, lane);
+    case D2O_F32: return d == 64 ? run_prefill<float, 64>(c, layer, n, K, V, st) : run_prefill<float, 128>(c, layer, n, K, V, st);
+    case D2O_F16: return d == 64 ? run_prefill<__half, 64>(c, layer, n, K, V, st) : run_prefill<__half, 128>(c, layer, n, K, V, st);
+    default: return d == 64 ? run_prefill<__nv_bfloat16, 64>(c, layer, n, K, V, st)
+                            : run_prefill<__nv_bfloat16, 128>(c, layer, n, K, V, st);
   }
 }
 

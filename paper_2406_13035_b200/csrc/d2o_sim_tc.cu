@@ -48,10 +48,16 @@ struct SimTcArgs {
   const int32_t* budgets; const int64_t* row_off;
   const float* rnorm;                       // pool-wide 1/|k_c|
   unsigned long long* part_key;             // [slices][n_chunks_max][P]
+  float* prompt_rn;                         // [slices][P] 1/|k| of the prompt rows (written with chunk 0)
+  size_t stride;                            // bytes between two layers' part_key, prompt_rn
   uint32_t* status;
   const int32_t* plen;                      // [B] prompt length of every sequence; P is the row stride per slice
-  const int4* items;                        // work list of this layer: (slice, chunk, first tile, end tile) per CTA
-  int L, layer, Hkv, P, n_chunks_max;
+  const int4* items;                        // work lists of the layers of the launch: (slice, chunk, first tile, end tile) per CTA
+  int item0[kCompressLayers];               // first item of every layer
+  int n, L, layer0, Hkv, P, n_chunks_max;
+};
+struct SimTcMaps {
+  CUtensorMap k[kCompressLayers], pool;     // prompt rows per layer; the cache rows
 };
 
 // Retained rows per chunk for a slice of S rows: ceil(S / kChunkN) chunks of equal size, rounded up to the MMA's
@@ -133,9 +139,9 @@ __device__ __forceinline__ void scan_block(const uint32_t (&r)[32], const float*
   if (tb[0] > best) { best = tb[0]; best_col = c0 + cl0 + ti[0]; }   // ascending blocks: the first maximum stays
 }
 
-template <int D, int FMT>
+template <typename T, int D, int FMT>
 __global__ void __launch_bounds__(kTcThreads, 1)
-sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_pool) {
+sim_tc_kernel(SimTcArgs a, const __grid_constant__ SimTcMaps maps) {
   constexpr int KB = D / 64;                                 // 64-element (128-byte) blocks along d
   constexpr int A_BLOCK = kTileM * 128;                      // bytes of one A k-block
   constexpr int A_TILE = KB * A_BLOCK;
@@ -151,10 +157,13 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int4 item = a.items[blockIdx.x];
+  int z = 0;                                                 // layer of the launch
+  while (z + 1 < a.n && (int)blockIdx.x >= a.item0[z + 1]) ++z;
+  const int layer = a.layer0 + z;
   const int slice = item.x;
   const int nc = item.y;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int chunk_cols = chunk_columns(S);                   // the retained rows are split evenly over the chunks
   const int c0 = nc * chunk_cols;                            // first retained slot of the chunk
   const int Pb = a.plen[b];                                  // this sequence's prompt length
@@ -166,8 +175,8 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
   const int t0 = item.z;
   const int t1 = min(n_tiles_all, item.w);
   if (t0 >= t1) return;
-  const int T = t1 - t0;                                     // prompt tiles of this CTA; part p takes tiles p, p + 4, ...
-  const int64_t row0 = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int n_t = t1 - t0;                                     // prompt tiles of this CTA; part p takes tiles p, p + 4, ...
+  const int64_t row0 = a.row_off[slice_entry(b, layer, h, a.L, a.Hkv)];
   if ((tc::smem_u32(tc_smem) & 1023u) != 0u) {               // swizzled tiles need 1024-byte aligned shared memory
     if (tid == 0) report_error(a.status, D2O_ERR_STATE, 0x51C10000u);
     return;
@@ -177,7 +186,7 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
     s_fail = 0;
     tc::mbar_init(&b_full, 1);
     for (int p = 0; p < kParts; ++p) {
-      tc::mbar_init(&a_full[p], 1); tc::mbar_init(&a_empty[p], 1);
+      tc::mbar_init(&a_full[p], 1); tc::mbar_init(&a_empty[p], nc == 0 ? 1 + kTcEpiWarps / kParts : 1);
       tc::mbar_init(&tm_full[p], 1); tc::mbar_init(&tm_empty[p], kTcEpiWarps / kParts);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -199,13 +208,13 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
       tc::mbar_expect_tx(&b_full, (uint32_t)(KB * n_box * kBBoxRows * 128));
       for (int kb = 0; kb < KB; ++kb)
         for (int j = 0; j < n_box; ++j)
-          tc::tma_load_2d(sB + kb * B_BLOCK + j * kBBoxRows * 128, &map_pool, kb * 64, (int)(row0 + c0 + j * kBBoxRows), &b_full);
-      for (int i = 0; i < T; ++i) {                            // tile i goes to part i % 4, its k-th tile with k = i / 4
+          tc::tma_load_2d(sB + kb * B_BLOCK + j * kBBoxRows * 128, &maps.pool, kb * 64, (int)(row0 + c0 + j * kBBoxRows), &b_full);
+      for (int i = 0; i < n_t; ++i) {                            // tile i goes to part i % 4, its k-th tile with k = i / 4
         const int p = i % kParts, k = i / kParts;
         if (k >= 1 && !s_fail && !tc::mbar_wait(&a_empty[p], (uint32_t)((k - 1) & 1))) s_fail = 1;
         tc::mbar_expect_tx(&a_full[p], (uint32_t)A_TILE);
         for (int kb = 0; kb < KB; ++kb)
-          tc::tma_load_2d(sA + p * A_TILE + kb * A_BLOCK, &map_k, kb * 64, slice * a.P + (t0 + i) * kTileM, &a_full[p]);
+          tc::tma_load_2d(sA + p * A_TILE + kb * A_BLOCK, &maps.k[z], kb * 64, slice * a.P + (t0 + i) * kTileM, &a_full[p]);
       }
     }
   } else if (warp == 1) {
@@ -214,11 +223,11 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
     // cores work for the other three.
     if (lane == 0) {
       if (!tc::mbar_wait(&b_full, 0)) s_fail = 1;
-      const int rounds = (T + kParts - 1) / kParts;
+      const int rounds = (n_t + kParts - 1) / kParts;
       for (int k = 0; k < rounds; ++k)
         for (int j = 0; j < n_j; ++j)
           for (int p = 0; p < kParts; ++p) {
-            if (k * kParts + p >= T) continue;
+            if (k * kParts + p >= n_t) continue;
             if (j == 0 && !s_fail && !tc::mbar_wait(&a_full[p], (uint32_t)(k & 1))) s_fail = 1;
             const int cnt = k * n_j + j;                         // jobs issued to this part before this one
             // the part's epilogue must have drained its accumulator (the first use passes at once)
@@ -250,10 +259,12 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
     for (int i = tid - 64; i < kChunkN; i += kTcEpiWarps * 32)
       s_rn[i] = i < n_cols ? a.rnorm[row0 + c0 + i] : 0.f;
     asm volatile("bar.sync 1, %0;" ::"n"(kTcEpiWarps * 32) : "memory");
-    unsigned long long* out_keys = a.part_key + ((size_t)slice * a.n_chunks_max + nc) * a.P;
+    unsigned long long* out_keys = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(a.part_key) + a.stride * z) +
+                                   ((size_t)slice * a.n_chunks_max + nc) * a.P;
+    float* out_rn = reinterpret_cast<float*>(reinterpret_cast<char*>(a.prompt_rn) + a.stride * z) + (size_t)slice * a.P;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(p * kJobN);
     uint32_t ra[32], rb[32];
-    const int n_tp = p < T ? (T - p + kParts - 1) / kParts : 0;   // tiles of this part
+    const int n_tp = p < n_t ? (n_t - p + kParts - 1) / kParts : 0;   // tiles of this part
     // every load of a job has landed in registers: hand the accumulator back to the MMA warp
     auto release = [&]() {
       tc::fence_before_sync();
@@ -263,6 +274,27 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
 #pragma unroll 1
     for (int k = 0; k < n_tp; ++k) {
       float best = -INFINITY; int best_col = 0x7fffffff;
+      const int pos = (t0 + k * kParts + p) * kTileM + row;
+      if (nc == 0) {
+        // 1/|k| of this thread's prompt row, from the tile itself (16-byte segment c of a row at c ^ (row & 7)), while the
+        // tensor cores work on it: the reduction then reads 4 bytes per evicted row instead of its key
+        if (!s_fail && !tc::mbar_wait(&a_full[p], (uint32_t)(k & 1))) s_fail = 1;
+        float ss = 0.f;
+#pragma unroll
+        for (int kb = 0; kb < KB; ++kb) {
+          const unsigned char* r = sA + p * A_TILE + kb * A_BLOCK + row * 128;
+#pragma unroll
+          for (int cc = 0; cc < 8; ++cc) {
+            float f[8];
+            Elem<T>::unpack(*reinterpret_cast<const uint4*>(r + ((cc ^ (row & 7)) << 4)), f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ss = fmaf(f[i], f[i], ss);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&a_empty[p]);
+        if (pos < Pb) out_rn[pos] = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
+      }
 #pragma unroll 1
       for (int j = 0; j < n_j; ++j) {
         const int cnt = k * n_j + j;
@@ -295,7 +327,6 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ CUtensorMap map_k, const __gr
       if (best == 0.f) best = 0.f;
       const unsigned long long key = best > -INFINITY
           ? (((unsigned long long)float_ord(best) << 32) | (uint32_t)(0x7fffffff - best_col)) : 0ull;
-      const int pos = (t0 + k * kParts + p) * kTileM + row;
       if (pos < Pb) out_keys[pos] = key;
     }
   }
@@ -313,96 +344,78 @@ struct NnReduceArgs {
   const int32_t* budgets; const int64_t* row_off;
   const int32_t* evict_idx;
   const unsigned long long* part_key;
+  const float* prompt_rn;                   // 1/|k| of the prompt rows
   const float* rnorm;                       // pool-wide 1/|k_c|
   float* evict_mx; int32_t* evict_nn;
+  size_t stride;                            // bytes between two layers' working arrays
   uint32_t* status;
   const int32_t* plen;
-  int L, layer, Hkv, P, n_chunks_max;
+  int L, layer0, Hkv, P, n_chunks_max;
+  const void* K[kCompressLayers];
 };
 
-constexpr int kNnRows = 4;                  // evicted rows per row group and pass: their loads are issued together
-
+// One evicted row per thread: the positions ascend, so that neighbouring threads read neighbouring entries.  (With 16 lanes
+// per row, which read the row's key for its norm, the kernel took 138 us on 128 slices of 8192 tokens; the chain position ->
+// key and partial maxima is what it waited for.)
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
-neighbour_reduce_kernel(NnReduceArgs a, const T* __restrict__ K, const T* __restrict__ kpool) {
+neighbour_reduce_kernel(NnReduceArgs a, const T* __restrict__ kpool) {
   constexpr int EPV = Elem<T>::kPerVec;
-  constexpr int LPR = D / EPV;
-  constexpr int NGRP = 256 / LPR;
-  const int slice = blockIdx.y;
+  const int slice = blockIdx.y, z = blockIdx.z, layer = a.layer0 + z;
   const int b = slice / a.Hkv, h = slice % a.Hkv;
-  const int S = a.budgets[slice_entry(b, a.layer, h, a.L, a.Hkv)];
+  const int S = a.budgets[slice_entry(b, layer, h, a.L, a.Hkv)];
   const int Pb = a.plen[b];
   const int Le = Pb - S;
-  const int grp = threadIdx.x / LPR, lig = threadIdx.x % LPR;
-  const int i0 = blockIdx.x * (NGRP * kNnRows) + grp;       // this group's rows: i0 + r * NGRP
-  if (i0 >= Le) return;
-  const unsigned gmask = group_mask<LPR>();
+  if ((int)(blockIdx.x * blockDim.x) >= Le) return;
+  auto lane_of = [&](const void* p) { return reinterpret_cast<const char*>(p) + a.stride * z; };
+  const int32_t* evict_idx = reinterpret_cast<const int32_t*>(lane_of(a.evict_idx)) + (size_t)slice * a.P;
+  const unsigned long long* part_key = reinterpret_cast<const unsigned long long*>(lane_of(a.part_key)) + (size_t)slice * a.n_chunks_max * a.P;
+  const float* prompt_rn = reinterpret_cast<const float*>(lane_of(a.prompt_rn)) + (size_t)slice * a.P;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   const int n_chunks = (S + kChunkN - 1) / kChunkN;
-  // The three dependent loads of a row (its position, its key, its partial maxima) are issued for four rows at a
-  // time; the partial maxima of a row are spread over the lanes of its group (chunk c is lane c mod LPR's).
-  int pos[kNnRows];
-#pragma unroll
-  for (int r = 0; r < kNnRows; ++r) {
-    const int i = i0 + r * NGRP;
-    pos[r] = i < Le ? a.evict_idx[(size_t)slice * a.P + i] : -1;
-    if (pos[r] >= 0 && !D2O_GUARD(pos[r] < Pb, a.status, 0xC4EC0008u)) pos[r] = -1;    // uniform for the row's lanes
-  }
-  uint4 raw[kNnRows];
-  unsigned long long key[kNnRows];
-#pragma unroll
-  for (int r = 0; r < kNnRows; ++r) {
-    raw[r] = make_uint4(0, 0, 0, 0);
-    key[r] = 0ull;
-    if (pos[r] >= 0) {
-      raw[r] = ld_global_v4(K + ((size_t)slice * a.P + pos[r]) * D + lig * EPV);
-      for (int c = lig; c < n_chunks; c += LPR) {
-        const unsigned long long k2 = a.part_key[((size_t)slice * a.n_chunks_max + c) * a.P + pos[r]];
-        key[r] = k2 > key[r] ? k2 : key[r];
-      }
+  int pos = i < Le ? evict_idx[i] : -1;
+  if (pos >= 0 && !D2O_GUARD(pos < Pb, a.status, 0xC4EC0008u)) pos = -1;
+  unsigned long long key = 0ull;
+  float rn = 0.f;
+  if (pos >= 0) {
+    rn = prompt_rn[pos];
+    for (int c = 0; c < n_chunks; ++c) {
+      const unsigned long long k2 = part_key[(size_t)c * a.P + pos];
+      key = k2 > key ? k2 : key;
     }
   }
-#pragma unroll
-  for (int r = 0; r < kNnRows; ++r) {
-    if (pos[r] < 0) continue;                                // uniform for the row's lanes
-    float f[EPV];
-    Elem<T>::unpack(raw[r], f);
-    float ss = 0.f;
-#pragma unroll
-    for (int e = 0; e < EPV; ++e) ss = fmaf(f[e], f[e], ss);
-    ss = group_sum<LPR>(ss, gmask);
-    const float rn = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
-    unsigned long long kk = key[r];
-#pragma unroll
-    for (int o = LPR / 2; o >= 1; o >>= 1) {
-      const unsigned long long other = __shfl_xor_sync(gmask, kk, o);
-      kk = other > kk ? other : kk;
-    }
-    int slot = 0x7fffffff - (int)(uint32_t)(kk & 0xffffffffu);
-    float mx = ord_float((uint32_t)(kk >> 32)) * rn;
-    const bool found = kk != 0ull && (unsigned)slot < (unsigned)S;
-    if (!found) {
-      // No chunk reported a maximum (no finite similarity in the row: non-finite keys).  The row is redone here in
-      // fp32, all retained rows in slot order (the first maximum stays); without any finite similarity it gets maximum
-      // -inf and neighbour 0 and is never merged.
-      const int64_t row0 = a.row_off[slice_entry(b, a.layer, h, a.L, a.Hkv)];
-      float best = -INFINITY; int bj = 0;
-      for (int j = 0; j < S; ++j) {
-        float g[EPV];
-        Elem<T>::unpack(ld_global_v4(kpool + (row0 + j) * D + lig * EPV), g);
-        float dot = 0.f;
+  int slot = 0x7fffffff - (int)(uint32_t)(key & 0xffffffffu);
+  float mx = ord_float((uint32_t)(key >> 32)) * rn;
+  // No chunk reported a maximum (no finite similarity in the row: non-finite keys).  The row is redone by the whole warp in
+  // fp32, all retained rows in slot order (the first maximum stays); without any finite similarity it gets maximum -inf and
+  // neighbour 0 and is never merged.
+  unsigned redo = __ballot_sync(0xffffffffu, pos >= 0 && !(key != 0ull && (unsigned)slot < (unsigned)S));
+  while (redo) {
+    const int src = __ffs(redo) - 1;
+    redo &= redo - 1;
+    const int rp = __shfl_sync(0xffffffffu, pos, src);
+    const float rr = __shfl_sync(0xffffffffu, rn, src);
+    const T* row = (const T*)a.K[z] + ((size_t)slice * a.P + rp) * D;
+    const int64_t row0 = a.row_off[slice_entry(b, layer, h, a.L, a.Hkv)];
+    float best = -INFINITY; int bj = 0;
+    for (int j = 0; j < S; ++j) {
+      float dot = 0.f;
+      if (lane < D / EPV) {
+        float f[EPV], g[EPV];
+        Elem<T>::unpack(ld_global_v4(row + lane * EPV), f);
+        Elem<T>::unpack(ld_global_v4(kpool + (row0 + j) * D + lane * EPV), g);
 #pragma unroll
         for (int e = 0; e < EPV; ++e) dot = fmaf(f[e], g[e], dot);
-        dot = group_sum<LPR>(dot, gmask);
-        const float u = __fadd_rn(dot * rn * a.rnorm[row0 + j], 0.f);
-        if (u > best) { best = u; bj = j; }
       }
-      mx = best; slot = bj;
+      dot = warp_sum(dot);
+      const float u = __fadd_rn(dot * rr * a.rnorm[row0 + j], 0.f);
+      if (u > best) { best = u; bj = j; }
     }
-    if (lig == 0) {
-      const int i = i0 + r * NGRP;
-      a.evict_mx[(size_t)slice * a.P + i] = mx;
-      a.evict_nn[(size_t)slice * a.P + i] = slot;
-    }
+    if (lane == src) { mx = best; slot = bj; }
+  }
+  if (pos >= 0) {
+    (reinterpret_cast<float*>(reinterpret_cast<char*>(a.evict_mx) + a.stride * z) + (size_t)slice * a.P)[i] = mx;
+    (reinterpret_cast<int32_t*>(reinterpret_cast<char*>(a.evict_nn) + a.stride * z) + (size_t)slice * a.P)[i] = slot;
   }
 }
 
@@ -502,65 +515,62 @@ size_t sim_tc_part_key_bytes(const d2o_config* cfg, int max_budget) {
   return (size_t)cfg->batch * cfg->n_kv_heads * chunks * cfg->prompt_len * 8;
 }
 
-// Returns cudaErrorNotSupported if the tensor maps cannot be built.
-cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, const void* K, int max_S, cudaStream_t st, int lane) {
+// Layers [layer, layer + n) in one launch per kernel.  Returns cudaErrorNotSupported if the tensor maps cannot be built.
+cudaError_t launch_similarity_tc(const d2o_ctx* c, int layer, int n, const void* const* K, int max_evicted, cudaStream_t st) {
   const d2o_config& g = c->cfg;
   const int B = g.batch, Hkv = g.n_kv_heads, P = g.prompt_len, D = g.d_head;
   const int n_slices = B * Hkv;
-  char* S = c->state; char* X = c->scratch + (size_t)lane * c->slay.lane_stride;   // only the lane's arrays are used below
-  CUtensorMap map_k, map_pool;
-  if (!encode_rows_2d(&map_k, g.dtype, K, (uint64_t)n_slices * P, D, kTileM)) return cudaErrorNotSupported;
+  char* S = c->state; char* X = c->scratch;
+  SimTcMaps maps;
   // the retained rows of the same kind: K_c, or V_c when the similarity is taken on the values
   char* pool = S + (g.sim_feature ? c->lay.vpool : c->lay.kpool);
-  if (!encode_rows_2d(&map_pool, g.dtype, pool, (uint64_t)c->pool_rows, D, kBBoxRows)) return cudaErrorNotSupported;
-  const int n_chunks_max = (c->max_budget + kChunkN - 1) / kChunkN;
-  (void)max_S;
-  const int n_items = c->h_sim_count[layer];
-  if (n_items == 0) return cudaSuccess;                      // nothing was evicted in this layer
-
+  if (!encode_rows_2d(&maps.pool, g.dtype, pool, (uint64_t)c->pool_rows, D, kBBoxRows)) return cudaErrorNotSupported;
   SimTcArgs a;
+  NnReduceArgs r;
+  int n_items = 0;
+  for (int l = 0; l < n; ++l) {
+    if (!encode_rows_2d(&maps.k[l], g.dtype, K[l], (uint64_t)n_slices * P, D, kTileM)) return cudaErrorNotSupported;
+    a.item0[l] = n_items;
+    n_items += c->h_sim_count[layer + l];
+    r.K[l] = K[l];
+  }
+  if (n_items == 0) return cudaSuccess;                      // nothing was evicted in these layers
   a.budgets = (const int32_t*)(S + c->lay.budgets); a.row_off = (const int64_t*)(S + c->lay.row_off);
   a.rnorm = (const float*)(S + c->lay.rnorm);
   a.part_key = (unsigned long long*)(X + c->slay.part_key);
+  a.prompt_rn = (float*)(X + c->slay.prompt_rn);
+  a.stride = c->slay.lane_stride;
   a.status = (uint32_t*)(S + c->lay.status);
   a.plen = (const int32_t*)(S + c->lay.plen);
-  a.L = g.n_layers; a.layer = layer; a.Hkv = Hkv; a.P = P; a.n_chunks_max = n_chunks_max;
+  a.n = n; a.L = g.n_layers; a.layer0 = layer; a.Hkv = Hkv; a.P = P; a.n_chunks_max = (c->max_budget + kChunkN - 1) / kChunkN;
   a.items = (const int4*)(S + c->lay.sim_items) + c->h_sim_off[layer];
   const int KB = D / 64;
   const size_t smem = (size_t)KB * kChunkN * 128 + (size_t)kParts * KB * kTileM * 128 + kChunkN * 4;
   dim3 grid((unsigned)n_items);
-  const int fmt = g.dtype == D2O_F16 ? 0 : 1;
   cudaError_t e;
-#define D2O_LAUNCH_TC(DD, FF)                                                                                     \
-  do {                                                                                                            \
-    e = cudaFuncSetAttribute(sim_tc_kernel<DD, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
-    if (e != cudaSuccess) return e;                                                                               \
-    sim_tc_kernel<DD, FF><<<grid, kTcThreads, smem, st>>>(a, map_k, map_pool);                                    \
+#define D2O_LAUNCH_TC(TT, DD, FF)                                                                                     \
+  do {                                                                                                                \
+    e = cudaFuncSetAttribute(sim_tc_kernel<TT, DD, FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
+    if (e != cudaSuccess) return e;                                                                                   \
+    sim_tc_kernel<TT, DD, FF><<<grid, kTcThreads, smem, st>>>(a, maps);                                               \
   } while (0)
-  if (D == 128) { if (fmt == 0) D2O_LAUNCH_TC(128, 0); else D2O_LAUNCH_TC(128, 1); }
-  else          { if (fmt == 0) D2O_LAUNCH_TC(64, 0); else D2O_LAUNCH_TC(64, 1); }
+  if (D == 128) { if (g.dtype == D2O_F16) D2O_LAUNCH_TC(__half, 128, 0); else D2O_LAUNCH_TC(__nv_bfloat16, 128, 1); }
+  else          { if (g.dtype == D2O_F16) D2O_LAUNCH_TC(__half, 64, 0); else D2O_LAUNCH_TC(__nv_bfloat16, 64, 1); }
 #undef D2O_LAUNCH_TC
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
-  NnReduceArgs r;
   r.budgets = a.budgets; r.row_off = a.row_off; r.rnorm = a.rnorm; r.status = a.status; r.plen = a.plen;
-  r.evict_idx = (const int32_t*)(X + c->slay.evict_idx); r.part_key = a.part_key;
-  r.evict_mx = (float*)(X + c->slay.evict_mx); r.evict_nn = (int32_t*)(X + c->slay.evict_nn);
-  r.L = g.n_layers; r.layer = layer; r.Hkv = Hkv; r.P = P; r.n_chunks_max = n_chunks_max;
-  int maxLe = 0;
-  for (int bb = 0; bb < B; ++bb)
-    for (int hh = 0; hh < Hkv; ++hh) maxLe = max(maxLe, c->h_plen[bb] - c->h_budgets[(bb * g.n_layers + layer) * Hkv + hh]);
-  if (maxLe <= 0) return cudaSuccess;
-  const int lpr = D * 2 / 16;
-  const int rows_per_cta = (256 / lpr) * kNnRows;
-  dim3 rgrid((maxLe + rows_per_cta - 1) / rows_per_cta, n_slices);
+  r.evict_idx = (const int32_t*)(X + c->slay.evict_idx); r.part_key = a.part_key; r.prompt_rn = a.prompt_rn;
+  r.evict_mx = (float*)(X + c->slay.evict_mx); r.evict_nn = (int32_t*)(X + c->slay.evict_nn); r.stride = a.stride;
+  r.L = g.n_layers; r.layer0 = layer; r.Hkv = Hkv; r.P = P; r.n_chunks_max = a.n_chunks_max;
+  dim3 rgrid((unsigned)((max_evicted + 255) / 256), (unsigned)n_slices, (unsigned)n);
   if (g.dtype == D2O_F16) {
-    if (D == 128) neighbour_reduce_kernel<__half, 128><<<rgrid, 256, 0, st>>>(r, (const __half*)K, (const __half*)pool);
-    else neighbour_reduce_kernel<__half, 64><<<rgrid, 256, 0, st>>>(r, (const __half*)K, (const __half*)pool);
+    if (D == 128) neighbour_reduce_kernel<__half, 128><<<rgrid, 256, 0, st>>>(r, (const __half*)pool);
+    else neighbour_reduce_kernel<__half, 64><<<rgrid, 256, 0, st>>>(r, (const __half*)pool);
   } else {
-    if (D == 128) neighbour_reduce_kernel<__nv_bfloat16, 128><<<rgrid, 256, 0, st>>>(r, (const __nv_bfloat16*)K, (const __nv_bfloat16*)pool);
-    else neighbour_reduce_kernel<__nv_bfloat16, 64><<<rgrid, 256, 0, st>>>(r, (const __nv_bfloat16*)K, (const __nv_bfloat16*)pool);
+    if (D == 128) neighbour_reduce_kernel<__nv_bfloat16, 128><<<rgrid, 256, 0, st>>>(r, (const __nv_bfloat16*)pool);
+    else neighbour_reduce_kernel<__nv_bfloat16, 64><<<rgrid, 256, 0, st>>>(r, (const __nv_bfloat16*)pool);
   }
   return cudaGetLastError();
 }
