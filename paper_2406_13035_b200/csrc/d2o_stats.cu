@@ -3,193 +3,305 @@
 // (Eq. 5, Appendix A.2).
 //
 // Kernels in this file
-//   lse_kernel      row normalisers log sum_j exp(q_i.k_j/sqrt(d)) of the causal attention
-//   colsum_kernel   s_j = sum_{i>=j} exp(q_i.k_j/sqrt(d) - lse_i); one CTA owns a block of
-//                   columns and walks down the rows, so the column reduction needs neither
-//                   atomics nor scratch and is bit-reproducible
+//   sweep_kernel    row normalisers log sum_j exp(q_i.k_j/sqrt(d)) of the causal attention, and the
+//                   column sums s_j = sum_{i>=j} exp(q_i.k_j/sqrt(d) - lse_i)
 //   density_kernel  warp-shuffle mean / variance of s per query head (double accumulation)
 //   budget_kernel   Eq. 5 with clamping and exact-sum integerisation, one CTA per sequence
 // The two attention sweeps here are the generic FFMA implementation (any dtype, fp32 math);
 // 16-bit inputs take the tensor-core path of d2o_colsum_tc.cu.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "d2o_common.cuh"
 
 namespace d2o {
 
-constexpr int kTile = 64;        // rows and columns per CTA tile
-constexpr int kStatThreads = 256;
+namespace cg = cooperative_groups;
 
-// Loads a [64 x D] tile (rows row0.., zero beyond n_rows) transposed into smem as t[k][r], times `mul`.
-template <typename T, int D>
-__device__ __forceinline__ void load_tile_transposed(float* t, const T* base, int row0, int n_rows, float mul) {
-  constexpr int EPV = Elem<T>::kPerVec;
-  constexpr int VPR = D / EPV;                       // vectors per row
-  const int r = threadIdx.x % kTile;
-  for (int vi = threadIdx.x / kTile; vi < VPR; vi += kStatThreads / kTile) {
-    float f[EPV];
-    if (row0 + r < n_rows) {
-      uint4 v = ld_global_v4(base + (size_t)(row0 + r) * D + vi * EPV);
-      Elem<T>::unpack(v, f);
+// Both sweeps multiply 64 x 64 tiles of the causal triangle: one tile stays (a row tile of Q for the normalisers, a column
+// tile of K for the column sums), those of the other operand stream past it, and the reduction runs along the stream.
+//
+// A triangle of nT tiles has long and short strips.  Strips u and nT - 1 - u are nT + 1 tiles together for every u, so a
+// pair is the unit of work; a cluster of C CTAs divides the pair's tiles evenly and combines its 128 results through
+// distributed shared memory in rank order (no atomics, no scratch, the same bits every time).  With one CTA per strip the
+// last of 16 strips was the launch.
+//
+// 128 threads hold 8 x 4 results each as two partial sums over the even and odd elements (fma.rn.f32x2 on operands as they
+// lie in memory); tiles are copied as they are (cp.async, two buffers, one barrier per slab) into rows of d + 4 floats,
+// which keeps the 16-byte reads of both operands free of bank conflicts.  The FMA pipe is busy 55 - 60 % of the time (twelve
+// warps per SM wait for shared memory); 8 x 8 results on 64 threads were no faster for d = 64 and 25 % slower for d = 128.
+// fp32, both sweeps and the densities, one CTA per strip -> now: 8 heads of 1024 tokens 132 -> 70 us, of 100 tokens 29 -> 25;
+// 16 heads of 1500 tokens, d = 128, 675 -> 335; 8 layers of 32 heads of 1999 tokens 4.53 -> 3.94 ms.
+constexpr int kTile = 64;             // rows and columns per tile
+constexpr int kStatThreads = 128;
+constexpr int kStripA = 8, kStripB = 4;   // results per thread: rows of the resident tile x rows of the streaming tile
+constexpr int kSlab = 64;                 // elements of d per streamed copy
+
+template <int D> struct SweepSmem {
+  static constexpr int kLdX = D + 4, kLdY = kSlab + 4;
+  float x[kTile * kLdX], y[2][kTile * kLdY], yl[2][kTile];
+  double res[2][2][kTile];            // column sums, or (maximum, sum) as two floats: [strip of the pair][half of the warps]
+};
+
+// Elements [0, W) of rows [row0, row0 + 64) of a [n_rows, D] matrix into shared memory; rows past the end are zero.  fp32
+// rows travel asynchronously (the caller commits and waits), 16-bit rows are converted on the way.
+template <typename T, int D, int W>
+__device__ __forceinline__ void load_tile(float* t, const T* base, int row0, int n_rows) {
+  constexpr int EPV = Elem<T>::kPerVec, VPR = W / EPV, LD = W + 4;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kTile * VPR; i += kStatThreads) {
+    const int r = i / VPR, v = i % VPR;
+    const bool in = row0 + r < n_rows;
+    const T* src = base + (size_t)(in ? row0 + r : 0) * D + v * EPV;
+    float* dst = t + r * LD + v * EPV;
+    if (sizeof(T) == 4) {
+      const uint32_t to = (uint32_t)__cvta_generic_to_shared(dst);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src), "r"(in ? 16 : 0) : "memory");
     } else {
+      float f[EPV];
+      if (in) Elem<T>::unpack(ld_global_v4(src), f);
 #pragma unroll
-      for (int i = 0; i < EPV; ++i) f[i] = 0.f;
+      for (int e = 0; e < EPV; ++e) dst[e] = in ? f[e] : 0.f;
     }
-#pragma unroll
-    for (int i = 0; i < EPV; ++i) t[(vi * EPV + i) * kTile + r] = f[i] * mul;
   }
 }
 
-// 4x4 register tile of S = Q K^T for this thread: rows ty*4.., cols tx*4..
-template <int D>
-__device__ __forceinline__ void tile_dot(const float* qt, const float* kt, int ty, int tx, float s[4][4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) s[r][c] = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < D; ++k) {
-    const float4 a = *reinterpret_cast<const float4*>(qt + k * kTile + ty * 4);
-    const float4 b = *reinterpret_cast<const float4*>(kt + k * kTile + tx * 4);
-    const float av[4] = {a.x, a.y, a.z, a.w};
-    const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) s[r][c] = fmaf(av[r], bv[c], s[r][c]);
-  }
+// A kernel that the library launches right behind another of its own may start while that one drains: `wait` returns when
+// the kernel ahead has finished and its results are visible.
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// 2^x; terms below 2^-126 count as zero
+__device__ __forceinline__ float exp2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// lse2[b,hq,i] = log2 sum_{j<=i} 2^{(q_i.k_j) * scale * log2e}, stored as natural log.
-template <typename T, int D>
-__global__ void __launch_bounds__(kStatThreads)
-lse_kernel(const T* __restrict__ Q, const T* __restrict__ K, float* __restrict__ lse, int Pmax, int Hq, int group,
-           const int32_t* __restrict__ plen) {
-  extern __shared__ __align__(16) float smem[];
-  float* qt = smem;
-  float* kt = smem + D * kTile;
-  const int it = gridDim.x - 1 - blockIdx.x;          // heaviest row tiles first
-  const int bh = blockIdx.y;
-  const int b = bh / Hq, hq = bh % Hq;
+// (m, l) <- log2-domain maximum and sum of 2^(x - m) over two sets
+__device__ __forceinline__ void combine_lse(float& m, float& l, float mo, float lo) {
+  const float mn = fmaxf(m, mo);
+  const float a = m > -INFINITY ? l * exp2f(m - mn) : 0.f;
+  const float b = mo > -INFINITY ? lo * exp2f(mo - mn) : 0.f;
+  l = a + b;
+  m = mn;
+}
+
+// kSum: colsum_j = sum_{i >= j} exp(q_i.k_j / sqrt(d) - lse_i); else lse_i = log sum_{j <= i} exp(q_i.k_j / sqrt(d)).
+template <typename T, int D, bool kSum>
+__global__ void __launch_bounds__(kStatThreads, 3)
+sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __restrict__ lse_in, float* __restrict__ out,
+             int Pmax, int Hq, int group, const int32_t* __restrict__ plen) {
+  extern __shared__ __align__(16) unsigned char sweep_smem[];
+  SweepSmem<D>& sm = *reinterpret_cast<SweepSmem<D>*>(sweep_smem);
+  constexpr int LDX = SweepSmem<D>::kLdX, LDY = SweepSmem<D>::kLdY, kSlabs = D / kSlab;
+  start_dependents();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int u = blockIdx.x / C;
+  const int b = blockIdx.y / Hq, hq = blockIdx.y % Hq;
   const int P = plen ? plen[b] : Pmax;                 // this sequence's prompt length; tensors are laid out for Pmax
-  if (it * kTile >= P) return;
-  const int Hkv = Hq / group;
-  const T* q = Q + ((size_t)b * Hq + hq) * (size_t)Pmax * D;
-  const T* k = K + ((size_t)b * Hkv + hq / group) * (size_t)Pmax * D;
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+  const int nT = (P + kTile - 1) / kTile;
+  if (2 * u >= nT + (nT & 1)) return;                  // the whole cluster
+  const T* q = Q + (size_t)blockIdx.y * Pmax * D;
+  const T* k = K + ((size_t)b * (Hq / group) + hq / group) * (size_t)Pmax * D;
+  const float* ls = kSum ? lse_in + (size_t)blockIdx.y * Pmax : nullptr;
+  // strip `part` of the pair: its resident tile and its number of streamed tiles
+  const int n0 = nT - u, n = u != nT - 1 - u ? nT + 1 : n0;
+  auto resident = [&](int part) { return (part == 0) == kSum ? u : nT - 1 - u; };
+  const int s0 = rank * n / C, s1 = (rank + 1) * n / C;
+  // resident rows ty + 8 r, streamed rows tx + 16 c; a warp is 4 x 8 threads, the CTA 2 x 2 warps
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp >> 1;
+  const int ty = (warp & 1) * 4 + (lane >> 3), tx = half * 8 + (lane & 7);
   const float mul = (D == 64 ? 0.125f : 0.08838834764831845f) * kLog2e;
-  load_tile_transposed<T, D>(qt, q, it * kTile, P, mul);
-  float m[4], l[4];
+
+#pragma unroll 1
+  for (int part = 0; part < 2; ++part) {
+    const int at = resident(part), from = part == 0 ? 0 : n0;
+    const int i0 = max(s0, from) - from, i1 = min(s1, part == 0 ? n0 : n) - from;   // streamed tiles of this CTA
+    float m[kStripA], l[kStripA];
+    double acc[kStripA];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) { m[r] = -INFINITY; l[r] = 0.f; }
-  for (int jt = 0; jt <= it; ++jt) {
-    __syncthreads();
-    load_tile_transposed<T, D>(kt, k, jt * kTile, P, 1.0f);
-    __syncthreads();
-    float s[4][4];
-    tile_dot<D>(qt, kt, ty, tx, s);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = it * kTile + ty * 4 + r;
-      float mx = m[r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = jt * kTile + tx * 4 + c;
-        if (col > row) s[r][c] = -INFINITY;
-        mx = fmaxf(mx, s[r][c]);
+    for (int r = 0; r < kStripA; ++r) { m[r] = -INFINITY; l[r] = 0.f; acc[r] = 0.0; }
+    auto request = [&](int step) {                    // slab `step` of the stream into its buffer
+      const int i = i0 + step / kSlabs, row0 = (kSum ? at + i : i) * kTile, buf = step & 1;
+      load_tile<T, D, kSlab>(sm.y[buf], (kSum ? q : k) + (step % kSlabs) * kSlab, row0, P);
+      if (kSum && step == 0) wait_for_prior_grid();   // the normalisers
+      if (kSum && step % kSlabs == kSlabs - 1 && threadIdx.x < kTile) {
+        const bool in = row0 + (int)threadIdx.x < P;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                     ::"r"((uint32_t)__cvta_generic_to_shared(&sm.yl[buf][threadIdx.x])),
+                       "l"(ls + (in ? row0 + (int)threadIdx.x : 0)), "r"(in ? 4 : 0) : "memory");
       }
-      if (mx > -INFINITY) {
-        float add = 0.f;
+    };
+    if (i0 < i1) {
+      load_tile<T, D, D>(sm.x, kSum ? k : q, at * kTile, P);
+      request(0);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int n_steps = (i1 - i0) * kSlabs;
+    unsigned long long s[kStripA][kStripB];
+#pragma unroll 1
+    for (int step = 0; step < n_steps; ++step) {
+      const int i = i0 + step / kSlabs, slab = step % kSlabs, buf = step & 1;
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();                                // the slab is there; every warp is done with the one before it
+      if (step + 1 < n_steps) request(step + 1);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (slab == 0) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) add += exp2f(s[r][c] - mx);
-        l[r] = l[r] * exp2f(m[r] - mx) + add;
-        m[r] = mx;
+        for (int r = 0; r < kStripA; ++r)
+#pragma unroll
+          for (int c = 0; c < kStripB; ++c) s[r][c] = 0ull;
+      }
+      const float* xr = sm.x + ty * LDX + slab * kSlab;
+      const float* yr = sm.y[buf] + tx * LDY;
+#pragma unroll 4
+      for (int e = 0; e < kSlab; e += 4) {
+        ulonglong2 yv[kStripB];
+#pragma unroll
+        for (int c = 0; c < kStripB; ++c) yv[c] = *reinterpret_cast<const ulonglong2*>(yr + c * 16 * LDY + e);
+#pragma unroll
+        for (int r = 0; r < kStripA; ++r) {
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(xr + r * 8 * LDX + e);
+#pragma unroll
+          for (int c = 0; c < kStripB; ++c) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s[r][c]) : "l"(xv.x), "l"(yv[c].x));
+#pragma unroll
+          for (int c = 0; c < kStripB; ++c) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s[r][c]) : "l"(xv.y), "l"(yv[c].y));
+        }
+      }
+      if (slab < kSlabs - 1) continue;
+      // the tile on the diagonal, and the last rows of the prompt, need a mask
+      const int res0 = at * kTile + ty, str0 = (kSum ? at + i : i) * kTile + tx;
+      const bool masked = (kSum ? i == 0 : i == at) || (kSum && (at + i + 1) * kTile > P);
+      float lr[kStripB];
+#pragma unroll
+      for (int c = 0; c < kStripB; ++c) lr[c] = kSum ? sm.yl[buf][tx + 16 * c] * kLog2e : 0.f;
+#pragma unroll
+      for (int r = 0; r < kStripA; ++r) {
+        float x[kStripB];
+#pragma unroll
+        for (int c = 0; c < kStripB; ++c) {
+          float lo, hi;
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(s[r][c]));
+          x[c] = fmaf(lo + hi, mul, -lr[c]);
+        }
+        if (masked) {
+#pragma unroll
+          for (int c = 0; c < kStripB; ++c) {
+            const int row = kSum ? str0 + 16 * c : res0 + 8 * r, col = kSum ? res0 + 8 * r : str0 + 16 * c;
+            if (col > row || (kSum && row >= P)) x[c] = -INFINITY;
+          }
+        }
+        if (kSum) {
+          acc[r] += (double)((exp2_ftz(x[0]) + exp2_ftz(x[1])) + (exp2_ftz(x[2]) + exp2_ftz(x[3])));
+        } else {
+          const float mx = fmaxf(m[r], fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])));
+          if (mx > -INFINITY) {
+            l[r] = l[r] * exp2_ftz(m[r] - mx) +
+                   ((exp2_ftz(x[0] - mx) + exp2_ftz(x[1] - mx)) + (exp2_ftz(x[2] - mx) + exp2_ftz(x[3] - mx)));
+            m[r] = mx;
+          }
+        }
+      }
+    }
+    __syncthreads();                                  // the next strip uses the same buffers
+    if (i0 >= i1) {                                   // nothing of this strip here
+      if (kSum) sm.res[part][0][threadIdx.x] = 0.0;
+      else reinterpret_cast<float2*>(sm.res[part][0])[threadIdx.x] = make_float2(-INFINITY, 0.f);
+      continue;
+    }
+    // the 8 lanes that share a resident row; the other half of the warps has the rest of it
+#pragma unroll
+    for (int r = 0; r < kStripA; ++r) {
+      if (kSum) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+        if ((lane & 7) == 0) sm.res[part][half][ty + 8 * r] = acc[r];
+      } else {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+          combine_lse(m[r], l[r], __shfl_xor_sync(0xffffffffu, m[r], o), __shfl_xor_sync(0xffffffffu, l[r], o));
+        if ((lane & 7) == 0) reinterpret_cast<float2*>(sm.res[part][half])[ty + 8 * r] = make_float2(m[r], l[r]);
       }
     }
   }
-  // combine the 16 threads (tx) that share a row: contiguous lanes
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      const float mo = __shfl_xor_sync(0xffffffffu, m[r], o);
-      const float lo = __shfl_xor_sync(0xffffffffu, l[r], o);
-      const float mn = fmaxf(m[r], mo);
-      const float a = (m[r] > -INFINITY) ? l[r] * exp2f(m[r] - mn) : 0.f;
-      const float bb = (mo > -INFINITY) ? lo * exp2f(mo - mn) : 0.f;
-      l[r] = a + bb;
-      m[r] = mn;
+  cluster.sync();
+  const int share = 2 * kTile / C;                    // results this CTA writes
+  for (int i = threadIdx.x; i < share; i += kStatThreads) {
+    const int e = rank * share + i, part = e / kTile, row = resident(part) * kTile + e % kTile;
+    double t = 0.0;
+    float m = -INFINITY, l = 0.f;
+    for (int c = 0; c < 2 * C; ++c) {
+      const double* from = &cluster.map_shared_rank(&sm, c >> 1)->res[part][c & 1][e % kTile];
+      if (kSum) t += *from;
+      else { const float2 o = *reinterpret_cast<const float2*>(from); combine_lse(m, l, o.x, o.y); }
     }
-    const int row = it * kTile + ty * 4 + r;
-    if (tx == 0 && row < P) lse[((size_t)b * Hq + hq) * Pmax + row] = (m[r] + log2f(l[r])) * 0.6931471805599453f;
+    if (row < P && (part == 0 || n > n0))
+      out[(size_t)blockIdx.y * Pmax + row] = kSum ? (float)t : (m + log2f(l)) * 0.6931471805599453f;
   }
+  cluster.sync();                                     // no CTA ends while another reads its results
 }
 
+// One sweep over all heads.  CTAs per cluster: enough to give every SM its CTAs (three fit), and more while every CTA
+// keeps eight tiles, so that the last wave is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms with four
+// tiles per CTA, where the copies that start a strip weigh as much, 4.20 with eight).
+template <typename T, int D, bool kSum>
+static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, float* out, int P, int n_heads, int Hq, int group,
+                                const int32_t* plen, cudaStream_t st, bool overlap) {
+  const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
+  const long long units = (long long)pairs * n_heads;
+  int C = 1;
+  while (C < 8 && 2 * C <= nT + 1 && (units * C < 4 * 148 || (units * C < 16 * 148 && nT + 1 >= 16 * C))) C *= 2;
+  const size_t smem = sizeof(SweepSmem<D>);
+  cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, D, kSum>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(pairs * C), (unsigned)n_heads);
+  cfg.blockDim = dim3(kStatThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = overlap ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, sweep_kernel<T, D, kSum>, Q, K, lse_in, out, P, Hq, group, plen);
+}
+
+__global__ void density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
+                               const int32_t* __restrict__ plen);
+constexpr int kDensityThreads = 512;
+
+// Row normalisers (unless the caller has them), column sums and densities of one layer.  Each kernel may start beside the
+// tail of the one before it: only what this call wrote is waited for inside the kernels.
 template <typename T, int D>
-__global__ void __launch_bounds__(kStatThreads)
-colsum_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __restrict__ lse,
-              float* __restrict__ colsum, int Pmax, int Hq, int group, const int32_t* __restrict__ plen) {
-  extern __shared__ __align__(16) float smem[];
-  float* qt = smem;
-  float* kt = smem + D * kTile;
-  float* lse2 = kt + D * kTile;                        // [64]
-  double* red = reinterpret_cast<double*>(lse2 + kTile);  // [16][64]
-  const int jt = blockIdx.x;                          // column tile 0 has the most rows: first
-  const int bh = blockIdx.y;
-  const int b = bh / Hq, hq = bh % Hq;
-  const int P = plen ? plen[b] : Pmax;
-  const int nT = (P + kTile - 1) / kTile;
-  if (jt >= nT) return;
-  const int Hkv = Hq / group;
-  const T* q = Q + ((size_t)b * Hq + hq) * (size_t)Pmax * D;
-  const T* k = K + ((size_t)b * Hkv + hq / group) * (size_t)Pmax * D;
-  const float* ls = lse + ((size_t)b * Hq + hq) * Pmax;
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-  const float mul = (D == 64 ? 0.125f : 0.08838834764831845f) * kLog2e;
-  load_tile_transposed<T, D>(kt, k, jt * kTile, P, 1.0f);
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int it = jt; it < nT; ++it) {
-    __syncthreads();
-    load_tile_transposed<T, D>(qt, q, it * kTile, P, mul);
-    if (threadIdx.x < kTile) {
-      const int row = it * kTile + threadIdx.x;
-      lse2[threadIdx.x] = row < P ? ls[row] * kLog2e : INFINITY;    // +inf -> probability 0 for padding rows
-    }
-    __syncthreads();
-    float s[4][4];
-    tile_dot<D>(qt, kt, ty, tx, s);
-    float p[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = it * kTile + ty * 4 + r;
-      const float lr = lse2[ty * 4 + r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int col = jt * kTile + tx * 4 + c;
-        p[r][c] = (col <= row) ? exp2f(s[r][c] - lr) : 0.f;
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[c] += (double)((p[0][c] + p[1][c]) + (p[2][c] + p[3][c]));
+static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float* lse_buf, float* colsum, double* density, int P,
+                                 int B, int Hq, int group, int L, int layer, const int32_t* plen, cudaStream_t st) {
+  const bool own = lse == nullptr;
+  if (own) {
+    cudaError_t e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, B * Hq, Hq, group, plen, st, false);
+    if (e != cudaSuccess) return e;
+    lse = lse_buf;
   }
-  __syncthreads();
-#pragma unroll
-  for (int c = 0; c < 4; ++c) red[ty * kTile + tx * 4 + c] = acc[c];
-  __syncthreads();
-  if (threadIdx.x < kTile) {
-    double t = 0.0;
-#pragma unroll
-    for (int y = 0; y < 16; ++y) t += red[y * kTile + threadIdx.x];
-    const int col = jt * kTile + threadIdx.x;
-    if (col < P) colsum[((size_t)b * Hq + hq) * Pmax + col] = (float)t;
-  }
+  cudaError_t e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, B * Hq, Hq, group, plen, st, own);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(B * Hq));
+  cfg.blockDim = dim3(kDensityThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, density_kernel, (const float*)colsum, density, P, Hq, L, layer, plen);
 }
 
 // F[b, layer, hq] = (1/P) sum_j (s_j - mean)^2, mean = (1/P) sum_j s_j   (Eq. 4; population variance)
 // One CTA per (sequence, head) and layer (blockIdx.y).  Two passes in fp64; a thread keeps its values of the first pass in
 // registers (up to 8, P <= 4096) or reads them again (8192 tokens, 32 heads: 21.6 us with 256 threads that read everything
 // twice and one value at a time; the kernel is a chain of load latencies).
-constexpr int kDensityThreads = 512;
 __global__ void __launch_bounds__(kDensityThreads)
 density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
                const int32_t* __restrict__ plen) {
@@ -198,6 +310,7 @@ density_kernel(const float* __restrict__ colsum, double* __restrict__ density, i
   const int bh = blockIdx.x, layer = layer0 + (int)blockIdx.y;
   const int b = bh / Hq, hq = bh % Hq;
   const int P = plen ? plen[b] : Pmax;
+  wait_for_prior_grid();
   const float* s = colsum + ((size_t)blockIdx.y * gridDim.x + bh) * Pmax;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto block_total = [&](double t) {                                 // every thread gets it
@@ -465,26 +578,11 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
                              cudaStream_t st, int lane) {
   const d2o_config& g = c->cfg;
   const int P = g.prompt_len, Hq = g.n_q_heads, B = g.batch;
-  const int nT = (P + kTile - 1) / kTile;
   float* colsum = (float*)(c->state + c->lay.colsum) + (size_t)layer * B * Hq * P;
   double* density = (double*)(c->state + c->lay.density);
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
-  const float* lse = lse_in;
-  dim3 grid(nT, B * Hq);
-  if (!lse) {
-    float* lse_buf = (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride);
-    const size_t sm = (size_t)2 * D * kTile * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(lse_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    lse_kernel<T, D><<<grid, kStatThreads, sm, st>>>((const T*)Q, (const T*)K, lse_buf, P, Hq, c->group, plen);
-    lse = lse_buf;
-  }
-  const size_t sm2 = (size_t)2 * D * kTile * sizeof(float) + kTile * sizeof(float) + 16 * kTile * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(colsum_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<T, D><<<grid, kStatThreads, sm2, st>>>((const T*)Q, (const T*)K, lse, colsum, P, Hq, c->group, plen);
-  density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, g.n_layers, layer, plen);
-  return cudaGetLastError();
+  return launch_sweeps<T, D>((const T*)Q, (const T*)K, lse_in, (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride),
+                             colsum, density, P, B, Hq, c->group, g.n_layers, layer, plen, st);
 }
 
 cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
@@ -552,18 +650,7 @@ static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, flo
     density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
     return cudaGetLastError();
   }
-  const int nT = (P + kTile - 1) / kTile;
-  dim3 grid(nT, B * Hq);
-  const size_t sm = (size_t)2 * D * kTile * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(lse_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  lse_kernel<T, D><<<grid, kStatThreads, sm, st>>>((const T*)Q, (const T*)K, lse_buf, P, Hq, group, nullptr);
-  const size_t sm2 = sm + kTile * sizeof(float) + 16 * kTile * sizeof(double);
-  e = cudaFuncSetAttribute(colsum_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<T, D><<<grid, kStatThreads, sm2, st>>>((const T*)Q, (const T*)K, lse_buf, colsum, P, Hq, group, nullptr);
-  density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
-  return cudaGetLastError();
+  return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st);
 }
 
 }  // namespace d2o

@@ -49,3 +49,29 @@ def test_colsum_at_any_prompt_length(cuda_device, dtype, d, P):
     F = torch.empty(b, hq, dtype=torch.float64, device=cuda_device)
     B.d2o_layer_stats_static(Q, K, cs, F)
     assert torch.equal(cs, own)
+
+
+@pytest.mark.parametrize("hq,hkv", [(1, 1), (8, 4), (96, 96)])
+@pytest.mark.parametrize("P", [1, 63, 64, 65, 128, 129, 300, 513, 960, 1025])
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp32_colsum_at_any_prompt_length(cuda_device, d, P, hq, hkv):
+    """Lengths around one tile, odd and even numbers of strips, and head counts that take one to eight CTAs per pair of
+    strips.  An fp32 dot product of magnitudes summing to about 11 errs by a few times 11 * 2^-24: the bound above holds."""
+    b = 2
+    g = torch.Generator(device=cuda_device).manual_seed(P + hq)
+    Q = 1.5 * torch.randn(b, hq, P, d, generator=g, device=cuda_device)
+    K = torch.randn(b, hkv, P, d, generator=g, device=cuda_device)
+    lens = [P, max(1, (2 * P) // 3)]
+    ctx = _context("f32", b, hq, hkv, d, P)
+    ctx.d2o_set_prompt_lens(torch.tensor(lens, dtype=torch.int32))
+    given = torch.zeros(b, hq, P, device=cuda_device)
+    refs = []
+    for i, p in enumerate(lens):
+        logits, ref = _reference(Q[i:i + 1, :, :p], K[i:i + 1, :, :p])
+        given[i, :, :p] = torch.logsumexp(logits[0], -1).float()
+        refs.append(ref[0])
+    for lse in (None, given):
+        ctx.d2o_layer_stats(0, Q, K, lse)
+        for i, p in enumerate(lens):
+            assert float(((ctx.colsum(0)[i, :, :p].double() - refs[i]).abs() / refs[i]).max()) < 2e-5
+    assert ctx.d2o_get_stats().error_word == 0
