@@ -487,8 +487,10 @@ size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* cou
           total += (double)tiles * (cols + 64);                // + a per-tile cost that does not depend on the columns
         }
       }
-    // aim at five waves of equal items, at least eight tiles each (a CTA first loads its chunk of retained rows and keeps four tiles in flight)
-    const double target = total / ((double)n_sms * 5.0);
+    // Aim at two waves of equal items per layer (the layers of a launch follow one another), at least eight tiles each: a CTA
+    // costs about 10 us before its first and after its last tile (128 slices of 8192 tokens, four layers, compression as a
+    // whole: 1900 us with five waves, 1860 with three, 1850 with two).
+    const double target = total / ((double)n_sms * 2.0);
     for (size_t i = 0; i < pieces.size(); ++i) {
       const Piece& p = pieces[i];
       const double work = (double)p.tiles * (p.cols + 64);
