@@ -76,6 +76,24 @@ __device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
   return v;
 }
 
+// ----------------------------------------------------------------------------- kernels that follow one another
+// A kernel launched with launch_behind may start while the kernel ahead of it on the stream drains, once all CTAs of that one
+// have called start_dependents.  wait_for_prior_grid returns when it has finished and its results are visible; it comes first
+// in such a kernel, before any return, so that the order of completion on the stream stays what it was.  What the kernel ahead
+// writes is not read through const __restrict__ pointers there (it changes while the kernel behind is already running).
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ----------------------------------------------------------------------------- reductions
 template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

@@ -79,6 +79,8 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
 // compaction scanned twice per 1024 positions).
 __global__ void __launch_bounds__(kSelThreads)
 select_kernel(SelectArgs a) {
+  start_dependents();
+  wait_for_prior_grid();
   extern __shared__ __align__(16) unsigned char sel_smem[];
   __shared__ int hist[256];
   __shared__ int warp_tot[32];
@@ -202,6 +204,8 @@ select_kernel(SelectArgs a) {
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
 gather_kernel(SelectArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__ vpool) {
+  start_dependents();
+  wait_for_prior_grid();
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;                   // lanes per row
   const int slice = blockIdx.y, layer = a.layer0 + (int)blockIdx.z;
@@ -246,7 +250,8 @@ struct SimArgs {
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kSimThreads)
-similarity_kernel(SimArgs a, LayerRows rows, int value_feature, const T* __restrict__ kpool) {
+similarity_kernel(SimArgs a, LayerRows rows, int value_feature, const T* kpool) {
+  wait_for_prior_grid();                    // no start_dependents: see sim_tc_kernel
   extern __shared__ __align__(16) float sim_smem[];
   float* et = sim_smem;                     // [D][64] evicted tile, transposed
   float* ct = et + D * kSimTile;            // [D][64] retained tile, transposed
@@ -376,6 +381,8 @@ struct SegArgs {
 
 __global__ void __launch_bounds__(1024)
 segment_kernel(SegArgs a) {
+  start_dependents();
+  wait_for_prior_grid();
   extern __shared__ __align__(16) int seg_smem[];       // [max(S + 1, 32 * 64)] counts / cursors, then radix histograms
   __shared__ double part[32];
   __shared__ float s_thr;
@@ -524,6 +531,8 @@ constexpr int kMergeThreads = 64;
 template <typename T, int D>
 __global__ void __launch_bounds__(kMergeThreads, 14)
 merge_kernel(MergeArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__ vpool) {
+  start_dependents();
+  wait_for_prior_grid();
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;
   const int slice = blockIdx.y, layer = a.layer0 + (int)blockIdx.z;
@@ -650,13 +659,17 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sel_sm > 48 * 1024 ? sel_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  select_kernel<<<dim3((unsigned)n_slices, 1, (unsigned)n), kSelThreads, sel_sm, st>>>(sa);
+  // Six kernels of a few microseconds each for a small batch: each may move in while the one ahead drains (one layer of 32
+  // slices of 777 tokens 53 -> 42 us, 32 layers of 1200 tokens 1269 -> 1250 with the column sums; large batches as before).
+  e = launch_behind(select_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), kSelThreads, sel_sm, st, sa);
+  if (e != cudaSuccess) return e;
   {
     const int keep_max = min(maxS, P);
     dim3 ggrid((unsigned)((keep_max + 63) / 64), (unsigned)n_slices, (unsigned)n);
-    gather_kernel<T, D><<<ggrid, 256, 0, st>>>(sa, rows, kpool, vpool);
+    e = launch_behind(gather_kernel<T, D>, ggrid, 256, 0, st, sa, rows, kpool, vpool);
+    if (e != cudaSuccess) return e;
   }
-  if (maxLe <= 0) return cudaGetLastError();
+  if (maxLe <= 0) return cudaSuccess;
 
   SimArgs ma;
   ma.budgets = sa.budgets; ma.row_off = sa.row_off;
@@ -673,7 +686,8 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
     e = cudaFuncSetAttribute(similarity_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sim_sm);
     if (e != cudaSuccess) return e;
     dim3 sgrid((unsigned)((maxLe + kSimTile - 1) / kSimTile), (unsigned)n_slices, (unsigned)n);
-    similarity_kernel<T, D><<<sgrid, kSimThreads, sim_sm, st>>>(ma, rows, g.sim_feature, feat_pool);
+    e = launch_behind(similarity_kernel<T, D>, sgrid, kSimThreads, sim_sm, st, ma, rows, g.sim_feature, feat_pool);
+    if (e != cudaSuccess) return e;
   }
 
   SegArgs ga;
@@ -689,7 +703,8 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   e = cudaFuncSetAttribute(segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(seg_sm > 48 * 1024 ? seg_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  segment_kernel<<<dim3((unsigned)n_slices, 1, (unsigned)n), 1024, seg_sm, st>>>(ga);
+  e = launch_behind(segment_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), 1024, seg_sm, st, ga);
+  if (e != cudaSuccess) return e;
 
   MergeArgs mg;
   mg.budgets = sa.budgets; mg.row_off = sa.row_off; mg.evict_idx = sa.evict_idx; mg.evict_mx = ma.evict_mx;
@@ -700,8 +715,7 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   constexpr int LPR = D / Elem<T>::kPerVec;
   const int rows_per_cta = kMergeThreads / LPR;
   dim3 mgrid((unsigned)((maxS + rows_per_cta - 1) / rows_per_cta), (unsigned)n_slices, (unsigned)n);
-  merge_kernel<T, D><<<mgrid, kMergeThreads, 0, st>>>(mg, rows, kpool, vpool);
-  return cudaGetLastError();
+  return launch_behind(merge_kernel<T, D>, mgrid, kMergeThreads, 0, st, mg, rows, kpool, vpool);
 }
 
 cudaError_t launch_prefill_compress(const d2o_ctx* c, int layer, int n, const void* const* K, const void* const* V,

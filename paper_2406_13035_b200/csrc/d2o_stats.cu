@@ -66,11 +66,6 @@ __device__ __forceinline__ void load_tile(float* t, const T* base, int row0, int
   }
 }
 
-// A kernel that the library launches right behind another of its own may start while that one drains: `wait` returns when
-// the kernel ahead has finished and its results are visible.
-__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // 2^x; terms below 2^-126 count as zero
 __device__ __forceinline__ float exp2_ftz(float x) {
   float y;
@@ -270,7 +265,7 @@ static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, flo
   return cudaLaunchKernelEx(&cfg, sweep_kernel<T, D, kSum>, Q, K, lse_in, out, P, Hq, group, plen);
 }
 
-__global__ void density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
+__global__ void density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
                                const int32_t* __restrict__ plen);
 constexpr int kDensityThreads = 512;
 
@@ -287,15 +282,7 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
   }
   cudaError_t e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, B * Hq, Hq, group, plen, st, own);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(B * Hq));
-  cfg.blockDim = dim3(kDensityThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, density_kernel, (const float*)colsum, density, P, Hq, L, layer, plen);
+  return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, L, layer, plen);
 }
 
 // F[b, layer, hq] = (1/P) sum_j (s_j - mean)^2, mean = (1/P) sum_j s_j   (Eq. 4; population variance)
@@ -303,14 +290,14 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
 // registers (up to 8, P <= 4096) or reads them again (8192 tokens, 32 heads: 21.6 us with 256 threads that read everything
 // twice and one value at a time; the kernel is a chain of load latencies).
 __global__ void __launch_bounds__(kDensityThreads)
-density_kernel(const float* __restrict__ colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
+density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
                const int32_t* __restrict__ plen) {
   constexpr int kKeep = 8, kWarps = kDensityThreads / 32;
   __shared__ double part[kWarps];
   const int bh = blockIdx.x, layer = layer0 + (int)blockIdx.y;
   const int b = bh / Hq, hq = bh % Hq;
-  const int P = plen ? plen[b] : Pmax;
   wait_for_prior_grid();
+  const int P = plen ? plen[b] : Pmax;
   const float* s = colsum + ((size_t)blockIdx.y * gridDim.x + bh) * Pmax;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto block_total = [&](double t) {                                 // every thread gets it
