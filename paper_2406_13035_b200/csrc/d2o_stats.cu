@@ -296,6 +296,7 @@ density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int 
   __shared__ double part[kWarps];
   const int bh = blockIdx.x, layer = layer0 + (int)blockIdx.y;
   const int b = bh / Hq, hq = bh % Hq;
+  start_dependents();
   wait_for_prior_grid();
   const int P = plen ? plen[b] : Pmax;
   const float* s = colsum + ((size_t)blockIdx.y * gridDim.x + bh) * Pmax;
@@ -582,9 +583,8 @@ cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void
                                    c->slay.lse_stride, colsum, plen, (uint32_t*)(c->state + c->lay.status),
                                    (uint32_t*)(c->state + c->lay.colsum_sched), st);
   if (e != cudaSuccess) return e;
-  density_kernel<<<dim3((unsigned)(B * Hq), (unsigned)n), kDensityThreads, 0, st>>>(colsum, (double*)(c->state + c->lay.density), P, Hq,
-                                                                                 g.n_layers, layer, plen);
-  return cudaGetLastError();
+  return launch_behind(density_kernel, dim3((unsigned)(B * Hq), (unsigned)n), kDensityThreads, 0, st, (const float*)colsum,
+                       (double*)(c->state + c->lay.density), P, Hq, g.n_layers, layer, plen);
 }
 
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
@@ -634,8 +634,7 @@ static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, flo
     cudaError_t e = launch_colsum_tc(dtype, D, B, Hq, Hq / group, P, 1, &Q, &K, nullptr, lse_buf, 0, colsum, nullptr, nullptr,
                                      (uint32_t*)(lse_buf + kStaticFloats), st);
     if (e != cudaSuccess) return e;
-    density_kernel<<<B * Hq, kDensityThreads, 0, st>>>(colsum, density, P, Hq, 1, 0, nullptr);
-    return cudaGetLastError();
+    return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, 1, 0, nullptr);
   }
   return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st);
 }
