@@ -1,0 +1,77 @@
+"""Kernels that divide their work by size, at the sizes where the division changes: the decode kernel with one cluster of
+CTAs per slice (against the float64 oracle, with the tolerances of parity.py), the selection of the retained positions across
+its blocks of 4096 and with ties (exact), and the uncompressed decode around its row groups."""
+import dataclasses
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2406_13035_b200 import binding as B
+from paper_2406_13035_b200 import workloads as W
+
+from parity import assert_report, close, np64, run_parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("P,rho,hq,hkv,d,dtype", [
+    (40, 0.5, 1, 1, 64, "f32"),            # fewer rows than warps in the cluster
+    (129, 0.99, 2, 2, 128, "f16"),         # 127 - 129 rows around a copy of 64
+    (642, 0.5, 4, 1, 128, "bf16"),         # 321 rows: four CTAs instead of two
+    (640, 0.5, 40, 40, 64, "f16"),         # more slices than a quarter of the SMs: two
+    (1501, 0.7, 8, 1, 128, "bf16"),        # eight heads per slice
+    (1900, 0.9, 2, 1, 128, "f32"),         # rows that need eight CTAs
+    (2600, 0.97, 1, 1, 128, "f16")])       # more rows than four CTAs hold
+def test_decode_cluster(P, rho, hq, hkv, d, dtype):
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=1, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype,
+                             prompt_len=P, rho=rho, decode_steps=4, min_budget=8)
+    rep = run_parity(wl, slices=[(0, 0, h) for h in sorted({0, hkv - 1})])
+    assert rep.steps == 4
+    assert_report(rep, dtype)
+
+
+@pytest.mark.parametrize("P", [17, 1023, 4095, 4096, 4097, 8193])
+def test_retained_positions_with_ties(cuda_device, P):
+    """Scores of seven distinct values over 17 layers (one more than share a launch): retained are the sinks, the window and
+    the highest scores, equal ones by the earlier position; every other position is evicted."""
+    L, S, sinks, window, d = 17, max(8, P // 5), 1, 4, 64
+    ctx = B.D2OContext(B.make_config(n_layers=L, batch=1, n_q_heads=2, n_kv_heads=1, d_head=d, dtype="f16", prompt_len=P,
+                                     max_new_tokens=2, rho=S / P, n_sink=sinks, window=window, min_budget=8,
+                                     density_temp=1e30, max_budget=P))
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    x = torch.randn(L, 1, 2, P, d, generator=g, device=cuda_device).half()
+    for l in range(L):
+        ctx.d2o_layer_stats(l, x[l], x[l, :, :1])
+        ctx.colsum(l).copy_(torch.randint(0, 7, (1, 2, P), generator=g, device=cuda_device).float())
+    ctx.density().fill_(1.0)
+    ctx.d2o_layer_budgets()
+    keys = [x[l, :, :1].contiguous() for l in range(L)]
+    ctx.d2o_prefill_compress_layers(0, L, keys, keys)
+    tabs = ctx.tables()
+    for l in (0, 15, 16):
+        score = ctx.colsum(l)[0].sum(0).cpu().numpy()
+        st = ctx.slice_state(l, 0, 0, tabs)
+        middle = np.arange(sinks, P - st["M"])
+        best = middle[np.lexsort((middle, -score[middle]))][:st["S"] - sinks - st["M"]]
+        np.testing.assert_array_equal(st["pos"].numpy(), np.sort(np.r_[np.arange(sinks), best, np.arange(P - st["M"], P)]))
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("length", [1, 31, 32, 63, 64, 255, 1024])
+@pytest.mark.parametrize("dtype,d,G,n", [("f16", 128, 1, 1), ("bf16", 64, 4, 150), ("f32", 128, 2, 3)])
+def test_full_decode_lengths(cuda_device, dtype, d, G, n, length):
+    """Slices in one wave of CTAs, several CTAs per slice for few of them; fp32 softmax and sums against float64: 2^-24 of
+    the logits (below 60) and of the sums, plus the rounding of the stored output, as in parity.py."""
+    td = W.TORCH_DTYPES[dtype]
+    g = torch.Generator(device=cuda_device).manual_seed(length)
+    kc, vc = (torch.randn(n, length + 3, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    q = torch.randn(n, G, d, generator=g, device=cuda_device).to(td)
+    k, v = (torch.randn(n, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    out = torch.empty_like(q)
+    B.d2o_full_decode_step(kc, vc, length, q, k, v, out)
+    K, V = torch.cat([kc[:, :length], k[:, None]], 1).double(), torch.cat([vc[:, :length], v[:, None]], 1).double()
+    ref = torch.softmax(q.double() @ K.transpose(1, 2) / math.sqrt(d), -1) @ V
+    assert close(np64(out), ref.cpu().numpy(), dtype) <= 1.0
