@@ -32,7 +32,9 @@ struct DecodeArgs {
   long long pool_rows;              // rows of the cache pool (bounds of the checked build)
   int32_t* steps_done;              // [L, B, Hkv] decode steps completed on the slice: written as a CTA's last act
   int chained;                      // 1: the previous step's grids may still be running (see slice_ready)
-  int early;                        // decode_split_kernel: 1: the slice may be read (once slice_ready) before the grid ahead is done
+  int early;                        // decode_split_kernel: 1: the slice may be read (once slice_ready) before the grid ahead is done.
+                                    // Only behind a step that published the counter: a compression's grids may still be writing
+                                    // the slice, and until they are done the counter may be an earlier conversation's
   int publish;                      // 1: a chained step follows: the CTA publishes the slice's step counter at its end
 };
 

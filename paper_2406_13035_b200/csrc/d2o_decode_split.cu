@@ -23,8 +23,10 @@
 // 16-bit caches run both passes and the cosines on mma.sync (d2o_decode.cu describes the layout), fp32 caches on FMAs.
 //
 // Launched with programmatic stream serialisation: the grid starts beside the one before it on the stream, loads the
-// slice's state as soon as the slice's step counter shows that the previous step on the slice is complete (the state
-// depends on nothing else), and only then waits for the grid before it, whose outputs the queries may be.
+// slice's state as soon as the slice's step counter shows that the previous step on the slice is complete (from the second
+// step after a compression on the state depends on nothing else), and only then waits for the grid before it, whose outputs
+// the queries may be.  The first step after a compression waits for the grids ahead before it reads anything: the counter
+// says nothing about the prompt stage, whose last kernels may still be at work.
 //
 // A CTA writes into another's shared memory only before a barrier that both wait for, and reads from another's only
 // before the last barrier.  Nothing of the slice is written before barrier 2 has shown that no CTA's wait ran out.
@@ -105,7 +107,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lig = lane % LPR, wg = lane / LPR, gid = lane >> 2, tig = lane & 3;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (a.early) start_dependents();
 
   // ---- which slice
   const int item = (int)blockIdx.x / C;
@@ -143,7 +145,12 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   }
   // barrier 0: every CTA of the cluster has started before anything is written into its shared memory
   cluster_arrive();
-  if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!a.early) {
+    // the grids ahead may still write the slice (the end of the prompt stage): its next step, which looks at the step
+    // counter alone, must not start before they are done either
+    wait_for_prior_grid();
+    start_dependents();
+  }
   if (tid == 0) {
     int stop = *reinterpret_cast<volatile uint32_t*>(a.status) != 0u;
     if (!stop && a.early) {
@@ -840,7 +847,7 @@ static cudaError_t launch_g(int G, const DecodeArgs& a, const CUtensorMap* maps,
 }
 
 // One step of `n_slices` slices (in index order) with `C` CTAs each.  `a.chained`, `a.publish`: see launch_decode;
-// `a.early`: the step counters of the slices are kept up to date, so the kernel may look at them.
+// `a.early`: see DecodeArgs.
 cudaError_t launch_decode_split(const d2o_ctx* c, DecodeArgs a, int C, int n_slices, int max_rows, const void* q,
                                 const void* k, const void* v, void* out, void* kpool, void* vpool, cudaStream_t st) {
   const d2o_config& g = c->cfg;

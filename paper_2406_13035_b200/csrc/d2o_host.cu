@@ -382,7 +382,7 @@ extern "C" d2o_status d2o_prefill_compress(d2o_ctx* c, int32_t layer, const void
   CUDA_TRY(launch_prefill_compress(c, layer, 1, &K, &V, (cudaStream_t)stream));
   c->layer_compressed[layer] = 1;
   c->layer_steps[layer] = 0;
-  c->layer_published[layer] = 1;                              // the compression sets the step counters to zero
+  c->layer_published[layer] = 0;                              // the first step waits for the compression's grids (DecodeArgs::early)
   return D2O_OK;
 }
 
@@ -399,7 +399,7 @@ extern "C" d2o_status d2o_prefill_compress_layers(d2o_ctx* c, int32_t l0, int32_
     const int a = l0 + (int)((long)(l1 - l0) * g / groups), b = l0 + (int)((long)(l1 - l0) * (g + 1) / groups);
     CUDA_TRY(launch_prefill_compress(c, a, b - a, K + (a - l0), V + (a - l0), st));
   }
-  for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; c->layer_published[l] = 1; }
+  for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; c->layer_published[l] = 0; }
   return D2O_OK;
 }
 
