@@ -28,8 +28,9 @@
 // the queries may be.  The first step after a compression waits for the grids ahead before it reads anything: the counter
 // says nothing about the prompt stage, whose last kernels may still be at work.
 //
-// A CTA writes into another's shared memory only before a barrier that both wait for, and reads from another's only
-// before the last barrier.  Nothing of the slice is written before barrier 2 has shown that no CTA's wait ran out.
+// A CTA writes into another's shared memory only before it arrives at a barrier that the other waits for before it ends (on the
+// way out after a wait that ran out there is a barrier for that), and reads from another's only before the last barrier.
+// Nothing of the slice is written before barrier 2 has shown that no CTA's wait ran out.
 #include <cooperative_groups.h>
 #include <math.h>
 #include <string.h>
@@ -571,8 +572,12 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   // A chained grid must not be complete before its predecessor (whatever the stream runs next is ordered behind this
   // grid only): one CTA that stays until then is enough.
   auto hold = [&]() { if (a.chained && blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory"); };
-  // A CTA must not end while copies are on their way into its shared memory; a cluster that gives up sees its own land.
+  // A CTA must not end while copies are on their way into its shared memory (a cluster that gives up sees its own land), nor
+  // while a peer that has arrived at the barrier before may still store into it: one more barrier.  The flags are the same in
+  // every CTA, so all of them come here or none.
   auto leave = [&](uint32_t detail) {
+    cluster_arrive();
+    cluster_wait();
     if (tid == 0) {
       if (s_timeout == 2) report_error(a.status, D2O_ERR_TIMEOUT, detail | (uint32_t)(sl & 0xffff));
       for (int i = 0; i < issued; ++i)

@@ -78,3 +78,35 @@ def test_decode_wait_that_runs_out_is_reported(cuda_device, name):
     small = dataclasses.replace(W.CONFIGS["cfg0"], prompt_len=128, decode_steps=2)
     rep = run_parity(small)
     assert_report(rep, small.dtype)
+
+
+@pytest.mark.parametrize("P,rho,hq,hkv,d,dtype,stage", [
+    (400, 0.5, 8, 8, 64, "f32", 4),             # 200 rows on two CTAs: the first copy of values
+    (640, 0.505, 8, 2, 128, "bf16", 3),         # 323 rows on four
+    (640, 0.505, 8, 2, 128, "bf16", 5),         # the last copy of values
+    (1900, 0.9, 2, 1, 128, "f32", 7)])          # 1710 rows on eight
+def test_decode_cluster_whose_values_do_not_arrive(cuda_device, P, rho, hq, hkv, d, dtype, stage):
+    """The CTAs of a cluster leave together, after the stores that they send one another (outputs and the new token's entry)
+    have landed; nothing of the slice is written, and later steps, which leave at the first barrier, do nothing either."""
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=1, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype,
+                             prompt_len=P, rho=rho, decode_steps=8, min_budget=8, max_budget=0)
+    ctx = make_ctx(wl)
+    s = W.LayerStream(wl, 0, "cuda:0")
+    Q, K, V = s.prompt()
+    ctx.d2o_layer_stats(0, Q, K)
+    ctx.d2o_layer_budgets()
+    ctx.d2o_prefill_compress(0, K, V)
+    q, k, v = s.decode()
+    out = torch.zeros_like(q)
+    ctx.d2o_decode_step(0, 1, q, k, v, out)
+    before, first = _state(ctx, wl), out.clone()
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.d2o_set_fault_injection(wait_limit_us=2000, producer_stop_stage=stage)
+    for _ in range(4):                                           # the step that runs out of time, then steps that find the error
+        t0 = time.perf_counter()
+        ctx.d2o_decode_step(0, 1, q, k, v, out)
+        torch.cuda.synchronize()
+        assert time.perf_counter() - t0 < 0.5
+        assert ctx.d2o_get_stats().error_word == D2O_ERR_TIMEOUT
+        assert _same(before, _state(ctx, wl)) and torch.equal(out, first)
+    ctx.close()
