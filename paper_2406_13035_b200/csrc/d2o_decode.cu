@@ -41,7 +41,6 @@ namespace d2o {
 // vectors per stage.
 __host__ __device__ constexpr int stage_bytes_of(int cw) { return 4 * cw * 32 * 16; }
 constexpr int kMaxStages = 12;
-constexpr int kTensorMinG = 2;                          // query heads per KV head from which the tensor-core path is used
 
 template <int CW>
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(CW * 32) : "memory"); }
@@ -68,8 +67,6 @@ __device__ __forceinline__ void block_arg_extreme(unsigned long long key, int li
   }
 }
 
-// 16-bit caches take the tensor-core path (more registers per thread, fewer instructions per row)
-__host__ __device__ constexpr bool tensor_path(int elem_size, int G) { return elem_size == 2 && G >= kTensorMinG; }
 // CTAs per SM the kernel is compiled for
 __host__ __device__ constexpr int ctas_per_sm(int cw, int G, int elem_size) {
   const bool t = tensor_path(elem_size, G);

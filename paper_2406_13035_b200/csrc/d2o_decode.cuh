@@ -12,6 +12,12 @@ namespace d2o {
 constexpr unsigned long long kWaitNs = 1000000000ull;   // an mbarrier wait gives up after 1 s
 constexpr uint32_t kSuspendNs = 4000u;                  // a waiting thread may stay suspended this long before it looks again
 
+// 16-bit caches with several query heads per KV head take the tensor-core path (more registers per thread, fewer
+// instructions per row); the weights enter its value pass as two 16-bit terms.  With one head the FMA loops are as fast, use
+// every warp, and keep the weights in fp32.
+constexpr int kTensorMinG = 2;
+__host__ __device__ constexpr bool tensor_path(int elem_size, int G) { return elem_size == 2 && G >= kTensorMinG; }
+
 struct DecodeArgs {
   const int32_t* budgets; const int32_t* windows; const int64_t* row_off;   // [B, L, Hkv]
   int32_t* pos; float* score; float* rnorm;                                  // pool-wide

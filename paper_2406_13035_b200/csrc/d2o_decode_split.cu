@@ -20,7 +20,8 @@
 // The kernel is bound by this chain of latencies, not by bandwidth or arithmetic, so a warp works alone wherever it can:
 // it owns every eighth tile of 16 rows from the logits to the cosines and writes its own entries (maximum and sum, best
 // victim, best neighbour) into every CTA of the cluster; the only block-wide step is the sum of the warps' outputs.
-// 16-bit caches run both passes and the cosines on mma.sync (d2o_decode.cu describes the layout), fp32 caches on FMAs.
+// 16-bit caches with several heads per slice run both passes and the cosines on mma.sync (d2o_decode.cu describes the
+// layout), fp32 caches and single heads on FMAs (tensor_path).
 //
 // Launched with programmatic stream serialisation: the grid starts beside the one before it on the stream, loads the
 // slice's state as soon as the slice's step counter shows that the previous step on the slice is complete (from the second
@@ -94,10 +95,10 @@ __global__ void __launch_bounds__(kSplitThreads, G <= 4 ? 2 : 1)
 decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const T* __restrict__ q_in, const T* __restrict__ k_in, const T* __restrict__ v_in, T* __restrict__ out,
                     T* __restrict__ kpool, T* __restrict__ vpool) {
-  constexpr bool kTensor = sizeof(T) == 2;                // both passes and the cosines on mma.sync
+  constexpr bool kTensor = tensor_path((int)sizeof(T), G);      // both passes and the cosines on mma.sync
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;                            // 16-byte segments of a row; lanes that share a row
-  constexpr int WG = 32 / LPR;                            // rows a warp's lanes cover at a time (FMA path: 1 or 2)
+  constexpr int WG = 32 / LPR;                            // rows a warp's lanes cover at a time
   constexpr int QL = LPR / 4;                             // lanes that end up with the same row total after reduce4
   constexpr int ROWB = D * (int)sizeof(T);
   constexpr int NH = kTensor ? ROWB / 128 : 1;            // 128-byte halves of a row
@@ -119,8 +120,8 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   const T* k_new = k_in + (size_t)sl * D;
   const T* v_new = v_in + (size_t)sl * D;
 
-  // ---- shared memory.  Keys and values lie as the copies bring them: 16-bit rows in pieces of [half][32 rows][128 B] with
-  // the 128-byte swizzle (16-byte segment c of row r at c ^ (r & 7)), fp32 rows one after another.
+  // ---- shared memory.  Keys and values lie as the copies bring them: on the tensor path in pieces of [half][32 rows][128 B]
+  // with the 128-byte swizzle (16-byte segment c of row r at c ^ (r & 7)), else rows one after another.
   extern __shared__ __align__(1024) unsigned char dsm[];
   const int cap = a.row_cap;
   uint4* sK = reinterpret_cast<uint4*>(dsm);                              // [cap][LPR]
@@ -859,7 +860,7 @@ cudaError_t launch_decode_split(const d2o_ctx* c, DecodeArgs a, int C, int n_sli
   a.row_cap = split_rows(max_rows, C);
   CUtensorMap maps[2];
   memset(maps, 0, sizeof(maps));
-  if (c->elem_size == 2 && (!encode_rows_2d(&maps[0], g.dtype, kpool, (uint64_t)c->pool_rows, g.d_head, kSplitPiece) ||
+  if (tensor_path(c->elem_size, c->group) && (!encode_rows_2d(&maps[0], g.dtype, kpool, (uint64_t)c->pool_rows, g.d_head, kSplitPiece) ||
                             !encode_rows_2d(&maps[1], g.dtype, vpool, (uint64_t)c->pool_rows, g.d_head, kSplitPiece)))
     return cudaErrorNotSupported;
   if (g.dtype == D2O_F32)

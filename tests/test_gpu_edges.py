@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("P,rho,hq,hkv,d,dtype", [
     (40, 0.5, 1, 1, 64, "f32"),            # fewer rows than warps in the cluster
-    (129, 0.99, 2, 2, 128, "f16"),         # 127 - 129 rows around a copy of 64
+    (129, 0.99, 2, 2, 128, "f16"),         # 127 - 129 rows on two CTAs, in copies of 32
     (642, 0.5, 4, 1, 128, "bf16"),         # 321 rows: four CTAs instead of two
     (640, 0.5, 40, 40, 64, "f16"),         # more slices than a quarter of the SMs: two
     (1501, 0.7, 8, 1, 128, "bf16"),        # eight heads per slice
@@ -30,6 +30,47 @@ def test_decode_cluster(P, rho, hq, hkv, d, dtype):
     rep = run_parity(wl, slices=[(0, 0, h) for h in sorted({0, hkv - 1})])
     assert rep.steps == 4
     assert_report(rep, dtype)
+
+
+@pytest.mark.parametrize("P,rho,hq,hkv,d,dtype", [
+    (40, 0.5, 1, 1, 64, "f32"), (129, 0.99, 2, 2, 128, "f16"), (642, 0.5, 4, 1, 128, "bf16"), (640, 0.5, 40, 40, 64, "f16"),
+    (1501, 0.7, 8, 1, 128, "bf16"), (1900, 0.9, 2, 1, 128, "f32"), (2600, 0.97, 1, 1, 128, "f16"),
+    (800, 0.99, 32, 32, 128, "bf16"), (333, 0.6, 64, 64, 64, "bf16"), (700, 0.8, 16, 8, 64, "f16"), (517, 0.9, 16, 4, 64, "f32"),
+    (450, 0.7, 16, 2, 128, "f16")])
+def test_decode_cluster_values(cuda_device, P, rho, hq, hkv, d, dtype):
+    """Attention spread over all rows (logits of variance 1), so that every value row counts: outputs of one step against
+    float64 on the rows the cache holds.  An output is the rounding of something within e of the reference.  A logit errs by a
+    few 2^-24 of the magnitudes it sums (about 7), a weight by as much; over the rows the errors are of random sign, so that
+    the output errs by about 2e-7 of its root mean square: e = 1.5e-6 of it.  With several heads on bf16 caches the weights
+    enter as two bf16 terms, up to 2^-17 off: 4e-6, e = 3e-5.  A missing row would be 1e-3 or more."""
+    ctx = B.D2OContext(B.make_config(n_layers=1, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=P,
+                                     max_new_tokens=4, rho=rho, n_sink=1, min_budget=8, density_temp=1e30))
+    td, G = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]], hq // hkv
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    draw = lambda *s: torch.randn(*s, generator=g, device=cuda_device).to(td)
+    K, V = draw(1, hkv, P, d), draw(1, hkv, P, d)
+    ctx.d2o_layer_stats(0, draw(1, hq, P, d), K)
+    ctx.d2o_layer_budgets()
+    ctx.d2o_prefill_compress(0, K, V)
+    for _ in range(2):
+        q, k, v = draw(1, 1, hq, d), draw(1, 1, hkv, d), draw(1, 1, hkv, d)
+        tabs = ctx.tables()
+        refs = []
+        for h in range(hkv):
+            st = ctx.slice_state(0, 0, h, tabs)
+            Kh, Vh = np.r_[np64(st["K"]), np64(k[0, :, h])], np.r_[np64(st["V"]), np64(v[0, :, h])]
+            x = np64(q[0, 0, h * G:(h + 1) * G]) @ Kh.T / math.sqrt(d)
+            w = np.exp(x - x.max(1, keepdims=True))
+            refs.append(w @ Vh / w.sum(1, keepdims=True))
+        ref = np.concatenate(refs)
+        out = torch.empty_like(q)
+        ctx.d2o_decode_step(0, 1, q, k, v, out)
+        got, rms = np64(out[0, 0]), math.sqrt(np.mean(ref * ref))
+        e = (3e-5 if dtype == "bf16" and G > 1 else 1.5e-6) * rms
+        lo, hi = np64(torch.tensor(ref - e).to(td)), np64(torch.tensor(ref + e).to(td))
+        assert np.all((lo <= got) & (got <= hi)), (float(np.max(np.abs(got - ref) / rms)), int(np.sum((got < lo) | (got > hi))))
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.close()
 
 
 @pytest.mark.parametrize("P", [17, 1023, 4095, 4096, 4097, 8193])
