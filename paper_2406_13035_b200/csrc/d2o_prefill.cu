@@ -51,6 +51,7 @@ struct SelectArgs {
   int keys_in_smem;
   long long pool_rows;     // rows of the cache pool (bounds of the checked build)
   int value_feature;       // 1: the similarity of Eq. 9 is taken on the value rows (ablation), so the norms are theirs
+  int generic_next;        // 1: similarity_kernel comes behind the gather
 };
 
 __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total) {
@@ -204,7 +205,9 @@ select_kernel(SelectArgs a) {
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
 gather_kernel(SelectArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__ vpool) {
-  start_dependents();
+  // Not when similarity_kernel follows: its long CTAs, moving in beside these, end up several on one SM (8 slices of 1024
+  // fp32 tokens, all of the compression: 77 us that way, 46 so).
+  if (!a.generic_next) start_dependents();
   wait_for_prior_grid();
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;                   // lanes per row
@@ -655,6 +658,8 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   sa.keys_in_smem = key_bytes <= 200 * 1024;
   sa.pool_rows = c->pool_rows;
   sa.value_feature = g.sim_feature;
+  const bool sim_tc = sizeof(T) == 2 && c->similarity_path == 0;
+  sa.generic_next = maxLe > 0 && !sim_tc;
   const size_t sel_sm = sa.keys_in_smem ? key_bytes : 0;
   cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sel_sm > 48 * 1024 ? sel_sm : 48 * 1024));
@@ -678,7 +683,7 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   ma.stride = sa.stride;
   // rows the similarity is computed on: the keys (Eq. 9), or the values (ablation "Feature choice")
   const T* feat_pool = g.sim_feature ? vpool : kpool;
-  if (sizeof(T) == 2 && c->similarity_path == 0) {
+  if (sim_tc) {
     e = launch_similarity_tc(c, layer, n, g.sim_feature ? V : K, maxLe, st);
     if (e != cudaSuccess) return e;
   } else {
