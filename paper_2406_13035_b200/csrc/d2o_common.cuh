@@ -173,6 +173,7 @@ struct ScratchLayout {     // byte offsets into `scratch`
   size_t lane_stride;      // evict_idx .. prompt_rn are the working set of one layer's compression: n_lanes copies, this far apart
   int n_lanes;
 };
+constexpr int kSplitSizes = 4;      // cluster sizes of decode_split_kernel: 2, 4, 8, 16
 constexpr int kHostBlock = 4;       // steps per block of d2o_decode_steps_host (two blocks of staging sets)
 constexpr int kStatsLanes = 2;      // layers whose column sums d2o_layer_stats_layers computes side by side (FFMA kernels)
 constexpr int kColsumLayers = 8;    // layers whose column sums share a launch (tensor-core kernels)
@@ -186,7 +187,7 @@ struct d2o_ctx {
   int elem_size;
   int max_budget;
   int n_sms;                   // multiprocessors of the device the context was created on
-  int max_cluster;             // largest thread-block cluster of decode_split_kernel there
+  int split_clusters[d2o::kSplitSizes];  // clusters of 2, 4, 8, 16 CTAs of decode_split_kernel resident there, at one CTA per SM
   int64_t total_budget;        // S_tot per sequence = round(rho * L * P)
   int64_t pool_rows;           // B * Hkv * S_tot
   d2o::Layout lay;

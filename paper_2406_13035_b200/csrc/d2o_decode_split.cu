@@ -785,41 +785,60 @@ static size_t split_smem(int rows, int G, int D, int esz) {
 
 // CTAs per slice, or 0 when one CTA per slice (decode_kernel) is the better choice or the rows do not fit.
 //
-// What counts here is how quickly one slice is done, so the kernel wins while all CTAs of the call are resident at once:
-// two CTAs for every SM and 20 MB of keys and values (us per call, this kernel / decode_kernel: 8 slices of 1640 rows
-// 11.0 / 39, 32 of 800 rows 12.9 / 30, 96 of 320 rows (16 MB) 16.8 / 20; but 128 of 400 rows (26 MB) 24 / 22 and 96 of
-// 800 rows (39 MB) 36 / 31).  Larger clusters shorten the passes, but every barrier and every exchange takes longer: two
-// CTAs, four for longer slices while there is an SM for each (32 slices of 800 rows 12.9 us with four, 14.2 with two,
-// 17 with eight; 96 of 320 rows 16.8 with two, 22 with four), more only where the rows do not fit otherwise.
+// What counts here is how quickly one slice is done, and how many rounds of resident clusters the call takes: about 11 us
+// each, plus the time for the longest slice's rows, which the one-CTA kernel pays in full (us per call, this kernel /
+// decode_kernel: 8 fp16 slices of 1640 rows, one head, 13.8 / 37, 32 of 820 rows 13.8 / 25, 72 of 160 bf16 rows, four heads,
+// 12.7 / 14.5).  Rows are long where one layer holds most of the budget, and then shared memory admits one CTA per SM: 144
+// slices of which the longest has 1460 rows are four rounds of four CTAs or eight of eight, 99 / 27; 100 slices of 320 rows
+// are two rounds, 21.8 / 16.5; but 64 slices of up to 1345 rows in two rounds 21.5 / 26.  Single heads of few rows are faster
+// in one CTA (24 slices of 40 rows 11.9 / 10.4).  Larger clusters shorten the passes, but every barrier and every exchange
+// takes longer: two CTAs, four for longer slices while there is an SM for each (32 slices of 800 rows 12.9 us with four, 14.2
+// with two, 17 with eight), more only where the rows do not fit otherwise, two where four would take a second round (36
+// slices of 640 rows 15.6 instead of 19.9).  From 20 MB of keys and values on, the passes count more than the chain of steps
+// (96 of 800 rows (39 MB) 36 / 31).
 int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows) {
   const d2o_config& g = c->cfg;
+  const int G = c->group;
   if (total_rows * 2 * g.d_head * c->elem_size > 20e6 || n_slices > c->n_sms) return 0;
-  int C = max_rows > 320 && 4 * n_slices <= c->n_sms ? 4 : 2;
-  const size_t room = 227 * 1024 - 1024 - 14 * 1024;                      // 14 KB: the static shared arrays at G = 8
-  for (; C <= c->max_cluster; C *= 2) {
-    const int rows = split_rows(max_rows, C);
-    if (rows <= kSplitMaxRows && split_smem(rows, c->group, g.d_head, c->elem_size) <= room) return C;
-  }
-  return 0;
+  const size_t fixed = (size_t)G * 1024 + 5 * 1024;                       // static shared arrays
+  // rounds of resident clusters; 0: the rows do not fit
+  auto rounds = [&](int i) {
+    const int rows = split_rows(max_rows, 2 << i);
+    const size_t smem = split_smem(rows, G, g.d_head, c->elem_size) + fixed + 1024;
+    if (c->split_clusters[i] == 0 || rows > kSplitMaxRows || smem > 227 * 1024) return 0;
+    const int resident = c->split_clusters[i] * (G <= 4 && 2 * smem <= 228 * 1024 ? 2 : 1);
+    return (n_slices + resident - 1) / resident;
+  };
+  int i = max_rows > 320 && 4 * n_slices <= c->n_sms ? 1 : 0, n = 0;
+  while (i < kSplitSizes && (n = rounds(i)) == 0) ++i;
+  if (n == 0) return 0;
+  if (n > 1 && i == 1 && rounds(0) == 1) { i = 0; n = 1; }
+  const double row_us = 3.1e-5 * 2 * g.d_head * c->elem_size * max_rows;  // the longest slice in one CTA
+  const double one_us = (G == 1 ? 10.0 : G <= 4 ? 12.3 : 16.0) + row_us;
+  const double split_us = (c->elem_size == 4 ? 11.0 : 11.5) * n + row_us / (2 << i);
+  return split_us < one_us ? 2 << i : 0;
 }
 
-// Largest cluster the kernels can be launched with on the current device (8 is always possible).
-int decode_split_max_cluster() {
+// Clusters of 2, 4, 8 and 16 CTAs that the current device holds at one CTA per SM.
+void decode_split_places(int* clusters) {
   auto kern = decode_split_kernel<float, 128, 8>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kSplitMaxCluster); cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = 212 * 1024;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kSplitMaxCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 8;
+  const size_t smem = 150 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  for (int i = 0; i < kSplitSizes; ++i) {
+    const int C = 2 << i;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C); cfg.blockDim = dim3(kSplitThreads); cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    clusters[i] = 0;
+    if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess || cudaOccupancyMaxActiveClusters(&clusters[i], kern, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      clusters[i] = 0;
+    }
   }
-  return n > 0 ? kSplitMaxCluster : 8;
 }
 
 template <typename T, int D, int G>

@@ -190,7 +190,7 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
       return D2O_ERR_CUDA;
     }
     c->n_sms = sms;
-    c->max_cluster = decode_split_max_cluster();
+    decode_split_places(c->split_clusters);
   }
   c->state = (char*)state; c->scratch = (char*)scratch;
   c->state_bytes = state_bytes; c->scratch_bytes = scratch_bytes;

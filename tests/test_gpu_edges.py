@@ -36,7 +36,8 @@ def test_decode_cluster(P, rho, hq, hkv, d, dtype):
     (40, 0.5, 1, 1, 64, "f32"), (129, 0.99, 2, 2, 128, "f16"), (642, 0.5, 4, 1, 128, "bf16"), (640, 0.5, 40, 40, 64, "f16"),
     (1501, 0.7, 8, 1, 128, "bf16"), (1900, 0.9, 2, 1, 128, "f32"), (2600, 0.97, 1, 1, 128, "f16"),
     (800, 0.99, 32, 32, 128, "bf16"), (333, 0.6, 64, 64, 64, "bf16"), (700, 0.8, 16, 8, 64, "f16"), (517, 0.9, 16, 4, 64, "f32"),
-    (450, 0.7, 16, 2, 128, "f16")])
+    (450, 0.7, 16, 2, 128, "f16"), (40, 0.5, 4, 1, 128, "bf16"), (129, 0.99, 4, 2, 128, "f16"), (640, 0.5, 80, 40, 64, "f16"),
+    (640, 0.99, 72, 36, 128, "bf16")])
 def test_decode_cluster_values(cuda_device, P, rho, hq, hkv, d, dtype):
     """Attention spread over all rows (logits of variance 1), so that every value row counts: outputs of one step against
     float64 on the rows the cache holds.  An output is the rounding of something within e of the reference.  A logit errs by a
