@@ -391,13 +391,15 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
       m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
       m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
     }
+    // a warp whose logits are all -inf: weights 0, as against the slice's maximum
+    const float b0 = m0 > -INFINITY ? m0 : 0.f, b1 = m1 > -INFINITY ? m1 : 0.f;
 #pragma unroll
     for (int i = 0; i < TW; ++i) {
       const int t = warp + i * kSplitWarps;
       if (t >= n_tiles) break;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float p = t * 16 + gid + (j >> 1) * 8 < cnt ? exp2f(acc[i][j] - ((j & 1) ? m1 : m0)) : 0.f;
+        const float p = t * 16 + gid + (j >> 1) * 8 < cnt ? exp2f(acc[i][j] - ((j & 1) ? b1 : b0)) : 0.f;
         if (j & 1) l1 += p; else l0 += p;
         if (2 * tig + (j & 1) < G) pl[(size_t)(2 * tig + (j & 1)) * cap + t * 16 + gid + (j >> 1) * 8] = p;
       }
@@ -437,9 +439,10 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       lw[g] = 0.f;
+      const float base = mw[g] > -INFINITY ? mw[g] : 0.f;                 // all -inf: weights 0, as against the slice's maximum
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        const float p = run && row_of(r) < cnt ? exp2f(x[r][g] - mw[g]) : 0.f;
+        const float p = run && row_of(r) < cnt ? exp2f(x[r][g] - base) : 0.f;
         if (run && (row_of(r) >> 4) < n_tiles) pl[(size_t)g * cap + row_of(r)] = p;       // 0 past the last row
         lw[g] += p;
       }

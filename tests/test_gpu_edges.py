@@ -74,6 +74,39 @@ def test_decode_cluster_values(cuda_device, P, rho, hq, hkv, d, dtype):
     ctx.close()
 
 
+@pytest.mark.parametrize("P,hq,d,dtype", [(65, 4, 128, "bf16"), (65, 2, 64, "f32"), (225, 1, 128, "bf16"), (225, 8, 64, "bf16")])
+def test_decode_cluster_warp_without_a_finite_logit(cuda_device, P, hq, d, dtype):
+    """The new token's tile of 16 rows holds no other row, and its logits overflow to -inf for every head: the token has
+    weight 0 in its own step and in the next, and the outputs are those of the other rows (bounds as above)."""
+    ctx = B.D2OContext(B.make_config(n_layers=1, batch=1, n_q_heads=hq, n_kv_heads=1, d_head=d, dtype=dtype, prompt_len=P,
+                                     max_new_tokens=8, rho=(P + 8) / P, n_sink=1, min_budget=8, max_budget=P + 8))
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    draw = lambda *s: torch.randn(*s, generator=g, device=cuda_device).to(td)
+    K, V = draw(1, 1, P, d), draw(1, 1, P, d)
+    K[..., 0] = 0.0
+    ctx.d2o_layer_stats(0, draw(1, hq, P, d), K)
+    ctx.d2o_layer_budgets()
+    ctx.d2o_prefill_compress(0, K, V)
+    Kh, Vh = np64(K[0, 0]), np64(V[0, 0])
+    for step in range(2):
+        q, k, v = draw(1, 1, hq, d), draw(1, 1, 1, d), draw(1, 1, 1, d)
+        q[..., 0] = 64.0
+        k[..., 0] = -3e38 if step == 0 else 0.0
+        if step > 0:
+            Kh, Vh = np.r_[Kh, np64(k[0, 0])], np.r_[Vh, np64(v[0, 0])]
+        x = np64(q[0, 0]) @ Kh.T / math.sqrt(d)
+        w = np.exp(x - x.max(1, keepdims=True))
+        ref = w @ Vh / w.sum(1, keepdims=True)
+        out = torch.empty_like(q)
+        ctx.d2o_decode_step(0, 1, q, k, v, out)
+        e = (3e-5 if dtype == "bf16" and hq > 1 else 1.5e-6) * math.sqrt(np.mean(ref * ref))
+        got, lo, hi = np64(out[0, 0]), np64(torch.tensor(ref - e).to(td)), np64(torch.tensor(ref + e).to(td))
+        assert np.all((lo <= got) & (got <= hi))
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.close()
+
+
 @pytest.mark.parametrize("P", [17, 1023, 4095, 4096, 4097, 8193])
 def test_retained_positions_with_ties(cuda_device, P):
     """Scores of seven distinct values over 17 layers (one more than share a launch): retained are the sinks, the window and
