@@ -369,7 +369,7 @@ extern "C" d2o_status d2o_layer_budgets(d2o_ctx* c, int32_t* budgets_host, void*
     if (n_items > 0)
       CUDA_TRY(cudaMemcpyAsync(c->state + c->lay.sim_items, c->h_sim_items, n_items * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
-  // (the two host arrays change again only in a later call, behind its own synchronisation above)
+  CUDA_TRY(cudaStreamSynchronize(st));      // the tables are complete for calls on any stream, and the host arrays may change again
   c->have_budgets = true;
   if (budgets_host) memcpy(budgets_host, c->h_budgets, BLH * 4);
   return D2O_OK;

@@ -73,3 +73,22 @@ def test_first_steps_behind_a_compression(cuda_device, mode, L, hq, hkv, P, d, d
                 assert a["len"] == b["len"] and np.float32(a["tau"]).tobytes() == np.float32(b["tau"]).tobytes()
                 for key in ("pos", "score", "rnorm", "K", "V"):
                     assert torch.equal(a[key].view(torch.uint8), b[key].view(torch.uint8)), key
+
+
+@pytest.mark.parametrize("L,B_,hkv,P", [(4, 1, 8, 512), (32, 16, 32, 1024)])
+def test_budgets_are_complete_on_return(cuda_device, L, B_, hkv, P):
+    """d2o_layer_budgets synchronises its stream: what it uploads for the calls behind it is there for calls on any stream.
+    The larger case uploads half a megabyte of work lists."""
+    d, td = 64, torch.float16
+    ctx = B.D2OContext(B.make_config(n_layers=L, batch=B_, n_q_heads=hkv, n_kv_heads=hkv, d_head=d, dtype="f16", prompt_len=P,
+                                     max_new_tokens=2, rho=0.3, n_sink=1, min_budget=16))
+    Q = torch.randn(B_, hkv, P, d, device=cuda_device).to(td)
+    ctx.d2o_layer_stats_layers(0, L, [Q] * L, [Q] * L)
+    call, handle, stream = ctx.lib.d2o_layer_budgets, ctx.handle, torch.cuda.current_stream()
+    at, done = stream.cuda_stream, []
+    for _ in range(50):
+        status = call(handle, None, at)
+        done.append(status == 0 and stream.query())
+    assert all(done)
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.close()
