@@ -168,7 +168,8 @@ struct Layout {            // byte offsets into `state`
 };
 struct ScratchLayout {     // byte offsets into `scratch`
   size_t lse, evict_idx, evict_mx, evict_nn, seg_start, seg_items, seg_tmp, part_key, prompt_rn, pl_spill, stage_q, stage_k, stage_v, stage_out, end;
-  size_t lse_stride;       // `lse` exists kColsumLayers times, this far apart (d2o_layer_stats_layers)
+  size_t lse_stride;       // `lse` exists once per layer that is worked on at a time, this far apart (d2o_layer_stats_layers): at
+                           // most kColsumLayers, kStatsLanes for fp32 caches, and never more than there are layers
   size_t stage_stride;     // stage_q .. stage_out exist 2 * kHostBlock times, this far apart (d2o_decode_steps_host)
   size_t lane_stride;      // evict_idx .. prompt_rn are the working set of one layer's compression: n_lanes copies, this far apart
   int n_lanes;

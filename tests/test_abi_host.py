@@ -60,6 +60,15 @@ def test_workspace_size_and_validation(lib):
     assert lib.d2o_workspace_size(C.byref(good()), None, None) == 1
 
 
+@pytest.mark.parametrize("dtype,n_layers,copies", [("f32", 1, 1), ("f32", 16, 2), ("bf16", 1, 1), ("bf16", 3, 3), ("f16", 16, 8)])
+def test_scratch_holds_the_normalisers_of_the_layers_at_work(lib, dtype, n_layers, copies):
+    """32 more query heads of 2^17 tokens: 16 MiB for every layer whose column sums are computed at a time (what else
+    grows with the heads is below a third of that)."""
+    size = [B.d2o_workspace_size(good(dtype=dtype, n_layers=n_layers, batch=1, n_kv_heads=8, n_q_heads=h, prompt_len=1 << 17,
+                                      rho=0.01, max_budget=4096))[1] for h in (32, 64)]
+    assert (size[1] - size[0]) // (32 * (1 << 17) * 4) == copies
+
+
 def test_null_and_misaligned_arguments(lib):
     cfg = good()
     h = C.c_void_p()
