@@ -376,9 +376,11 @@ budget_kernel(const double* __restrict__ density, int L, int H, int Hkv, int Pma
   extern __shared__ __align__(16) double dsm[];
   const int n = budget_rule == 1 ? L * Hkv : L;                       // allocation units
   const int G = H / Hkv;
+  int n_pad = 2;                                                      // kinks, padded for the sort
+  while (n_pad < 2 * n) n_pad *= 2;
   double* w = dsm;              // [n] weights
   double* x = w + n;            // [n] scaled sizes, then remainders
-  double* kinks = x + n;        // [2n]
+  double* kinks = x + n;        // [n_pad]
   __shared__ double part[kBudgetThreads / 32], s_lam;
   __shared__ int s_lo, s_hi, s_open;
   __shared__ long long s_left;
@@ -440,20 +442,19 @@ budget_kernel(const double* __restrict__ density, int L, int H, int Hkv, int Pma
       kinks[2 * u] = __ddiv_rn(lo, w[u]);
       kinks[2 * u + 1] = __ddiv_rn(hi, w[u]);
     }
-    const int nk = 2 * n;
-    // Bitonic sort whose exchanges all put the smaller value first: entries past the end count as +inf and never move, so
-    // they take no room (6400 units fit as they always did).
-    for (int k = 2; k < 2 * nk; k *= 2)
+    for (int i = 2 * n + tid; i < n_pad; i += kBudgetThreads) kinks[i] = INFINITY;
+    for (int k = 2; k <= n_pad; k *= 2)                               // bitonic sort
       for (int j = k / 2; j > 0; j /= 2) {
         __syncthreads();
-        for (int i = tid; i < nk; i += kBudgetThreads) {
-          const int o = j == k / 2 ? i ^ (k - 1) : i ^ j;
-          if (o > i && o < nk) {
+        for (int i = tid; i < n_pad; i += kBudgetThreads) {
+          const int o = i ^ j;
+          if (o > i) {
             const double p = kinks[i], q = kinks[o];
-            if (p > q) { kinks[i] = q; kinks[o] = p; }
+            if ((p > q) == ((i & k) == 0)) { kinks[i] = q; kinks[o] = p; }
           }
         }
       }
+    const int nk = 2 * n;
     auto total = [&](double lam) {
       double t = 0.0;
       for (int u = 0; u < n; ++u) t = __dadd_rn(t, clipd(__dmul_rn(lam, w[u]), lo, hi));
@@ -603,7 +604,9 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
                            float nm_ratio, int32_t* budgets, int32_t* windows, int64_t* row_off, uint32_t* status_word,
                            const int32_t* plen, cudaStream_t st) {
   const size_t n = budget_rule == 1 ? (size_t)L * Hkv : (size_t)L;
-  const size_t sm = 4 * n * sizeof(double);
+  size_t n_pad = 2;
+  while (n_pad < 2 * n) n_pad *= 2;
+  const size_t sm = (2 * n + n_pad) * sizeof(double);
   if (sm > 200 * 1024) return cudaErrorInvalidValue;          // more allocation units than the work arrays hold
   cudaError_t e = cudaFuncSetAttribute(budget_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;

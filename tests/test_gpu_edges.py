@@ -150,16 +150,3 @@ def test_full_decode_lengths(cuda_device, dtype, d, G, n, length):
     K, V = torch.cat([kc[:, :length], k[:, None]], 1).double(), torch.cat([vc[:, :length], v[:, None]], 1).double()
     ref = torch.softmax(q.double() @ K.transpose(1, 2) / math.sqrt(d), -1) @ V
     assert close(np64(out), ref.cpu().numpy(), dtype) <= 1.0
-
-
-@pytest.mark.parametrize("L,hkv", [(1, 1), (1, 3), (73, 64), (100, 64)])
-def test_budgets_of_many_units(cuda_device, L, hkv):
-    """Per-head budgets for 1, 3, 4672 and 6400 allocation units, the most that are accepted."""
-    from oracle import d2o_oracle as O
-    P, rho = 300, B.f32(0.3)
-    F = np.random.default_rng(L).gamma(1.0, size=(2, L, hkv)) * 30.0
-    bud, _, _, status = B.d2o_budgets_from_density(torch.tensor(F, device=cuda_device), n_kv_heads=hkv, prompt_len=P, rho=rho,
-                                                   min_budget=4, density_temp=10.0, budget_rule=1)
-    assert int(status[0]) == 0
-    for b in range(2):
-        np.testing.assert_array_equal(bud[b].cpu().numpy(), O.head_budgets(F[b], P, rho, 1, 4, 10.0, 0))
