@@ -275,9 +275,10 @@ d2o_status d2o_full_decode_step(int32_t dtype, int32_t d_head, int32_t n_slices,
  * made with that device current) and keeps it for the life of the process; make that first call
  * outside of any stream capture.  After cudaDeviceReset() the kept address is stale: a process
  * that resets a device must not call this entry point on it again.
- * All calls share the one array: it is fully rewritten by each call before it is read, so
- * nothing needs clearing, but two calls whose work overlaps on the GPU (different streams)
- * race on it.  Asynchronous on `stream` like the other calls. */
+ * All calls share the one array and the work counter behind it: the array is fully rewritten by
+ * each call before it is read and the counter is left at zero, so nothing needs clearing, but two
+ * calls whose work overlaps on the GPU (different streams) race on them: the results of both are
+ * then undefined, those of later calls are not affected.  Asynchronous on `stream` like the other calls. */
 #define D2O_STATIC_LSE_FLOATS (1u << 20)
 d2o_status d2o_layer_stats_static(int32_t dtype, int32_t d_head, int32_t batch, int32_t n_q_heads,
                                   int32_t n_kv_heads, int32_t prompt_len, const void* Q, const void* K,

@@ -266,7 +266,7 @@ static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, flo
 }
 
 __global__ void density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
-                               const int32_t* __restrict__ plen);
+                               const int32_t* __restrict__ plen, uint32_t* sched);
 constexpr int kDensityThreads = 512;
 
 // Row normalisers (unless the caller has them), column sums and densities of one layer.  Each kernel may start beside the
@@ -282,7 +282,8 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
   }
   cudaError_t e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, B * Hq, Hq, group, plen, st, own);
   if (e != cudaSuccess) return e;
-  return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, L, layer, plen);
+  return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, L, layer, plen,
+                       (uint32_t*)nullptr);
 }
 
 // F[b, layer, hq] = (1/P) sum_j (s_j - mean)^2, mean = (1/P) sum_j s_j   (Eq. 4; population variance)
@@ -291,13 +292,16 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
 // twice and one value at a time; the kernel is a chain of load latencies).
 __global__ void __launch_bounds__(kDensityThreads)
 density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
-               const int32_t* __restrict__ plen) {
+               const int32_t* __restrict__ plen, uint32_t* sched) {
   constexpr int kKeep = 8, kWarps = kDensityThreads / 32;
   __shared__ double part[kWarps];
   const int bh = blockIdx.x, layer = layer0 + (int)blockIdx.y;
   const int b = bh / Hq, hq = bh % Hq;
   start_dependents();
   wait_for_prior_grid();
+  // The column sums' work counter (NULL: there is none) is zero for the next call whatever became of it in this one, so that
+  // calls that overlap on the GPU against the rules spoil their own results only.
+  if (sched && bh == 0 && blockIdx.y == 0 && threadIdx.x < 2) sched[threadIdx.x] = 0u;
   const int P = plen ? plen[b] : Pmax;
   const float* s = colsum + ((size_t)blockIdx.y * gridDim.x + bh) * Pmax;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -584,7 +588,8 @@ cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void
                                    (uint32_t*)(c->state + c->lay.colsum_sched), st);
   if (e != cudaSuccess) return e;
   return launch_behind(density_kernel, dim3((unsigned)(B * Hq), (unsigned)n), kDensityThreads, 0, st, (const float*)colsum,
-                       (double*)(c->state + c->lay.density), P, Hq, g.n_layers, layer, plen);
+                       (double*)(c->state + c->lay.density), P, Hq, g.n_layers, layer, plen,
+                       (uint32_t*)(c->state + c->lay.colsum_sched));
 }
 
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
@@ -621,7 +626,7 @@ cudaError_t launch_budgets(const double* density, int B, int L, int H, int Hkv, 
 // Scratch for the row normalisers of d2o_layer_stats_static: part of the library image, one copy per GPU.  The
 // tensor-core kernels pad every (sequence, head) row to a multiple of four floats.
 constexpr int kStaticMaxRows = 65535;                // (sequence, head) pairs: one grid row of the generic kernels each
-// The two words behind them are its work counter (zero in the image, and left at zero by every launch).
+// The two words behind them are its work counter (zero in the image, and left at zero by every call).
 constexpr size_t kStaticFloats = (size_t)D2O_STATIC_LSE_FLOATS + 3 * kStaticMaxRows + 1;
 static __device__ __align__(256) float g_static_lse[kStaticFloats + 2];
 constexpr int kMaxDevices = 64;
@@ -631,10 +636,12 @@ template <typename T, int D>
 static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, float* lse_buf, float* colsum, double* density,
                                     int B, int Hq, int group, int P, cudaStream_t st) {
   if (sizeof(T) == 2) {
+    uint32_t* sched = (uint32_t*)(lse_buf + kStaticFloats);
     cudaError_t e = launch_colsum_tc(dtype, D, B, Hq, Hq / group, P, 1, &Q, &K, nullptr, lse_buf, 0, colsum, nullptr, nullptr,
-                                     (uint32_t*)(lse_buf + kStaticFloats), st);
+                                     sched, st);
     if (e != cudaSuccess) return e;
-    return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, 1, 0, nullptr);
+    return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, 1, 0,
+                         nullptr, sched);
   }
   return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st);
 }

@@ -75,3 +75,25 @@ def test_fp32_colsum_at_any_prompt_length(cuda_device, d, P, hq, hkv):
         for i, p in enumerate(lens):
             assert float(((ctx.colsum(0)[i, :, :p].double() - refs[i]).abs() / refs[i]).max()) < 2e-5
     assert ctx.d2o_get_stats().error_word == 0
+
+
+def test_work_counter_is_zero_after_every_call(cuda_device):
+    """The tensor-core kernels take their work from a counter.  Whatever it holds before a call (as after two calls that
+    overlapped), the call after that one computes everything."""
+    b, hq, hkv, d, P = 1, 32, 8, 64, 1281                          # 192 items: more than the GPU has SMs
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    Q = torch.randn(b, hq, P, d, generator=g, device=cuda_device).bfloat16()
+    K = torch.randn(b, hkv, P, d, generator=g, device=cuda_device).bfloat16()
+    ctx = _context("bf16", b, hq, hkv, d, P)
+    ctx.d2o_layer_stats(0, Q, K)
+    want = ctx.colsum(0).clone()
+    at = ctx._view(0).density - ctx.state.data_ptr() - 256         # the counter's 256 bytes lie ahead of the densities
+    counter = ctx.state[at:at + 8].view(torch.int32)
+    assert counter.tolist() == [0, 0]
+    for dirty in ([3, 1000], [1 << 20, 1], [7, 0]):
+        counter.copy_(torch.tensor(dirty, dtype=torch.int32))
+        ctx.d2o_layer_stats(0, Q, K)
+        ctx.colsum(0).zero_()
+        ctx.d2o_layer_stats(0, Q, K)
+        assert torch.equal(ctx.colsum(0), want) and counter.tolist() == [0, 0]
+    ctx.close()
