@@ -52,6 +52,8 @@ struct ColsumTcArgs {
   uint32_t* status;                          // NULL: no error word (the allocation-free entry point)
   const int32_t* plen;                       // [B] prompt length of every sequence (<= P); NULL: all P
   int P, Hq, group, BHq;                     // P: the length the tensors are laid out for; BHq: (sequence, head) pairs of a layer
+  unsigned long long wait_ns;                // limit of every wait
+  int stop_job;                              // failure-detection tests: no copy from this streamed tile of a CTA on (-1: never)
 };
 
 // Layers of one launch: a short prompt's layer alone (32 heads, 1200 tokens: 160 items) is little more than one item per
@@ -218,6 +220,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   float* s_comb = s_lse + kCsStages * kCsTile;               // [2][2][2][128] partner values for the final combination
   __shared__ unsigned long long a_full, a_empty, b_full[kCsStages], b_empty[kCsStages], tm_full[2], tm_empty[2], it_full[2], it_empty[2];
   __shared__ int s_item[2];                                  // the CTA's current and next item, -1: no more
+  __shared__ int s_now[2], s_lost;                           // the epilogue's current item; taken after a wait had run out
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
 
@@ -228,11 +231,11 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   }
 
   if (tid == 0) {
-    s_fail = 0;
+    s_fail = 0; s_lost = s_item[0] = s_item[1] = -1;
     tc::mbar_init(&a_full, 1); tc::mbar_init(&a_empty, 1);
     for (int s = 0; s < kCsStages; ++s) { tc::mbar_init(&b_full[s], 1); tc::mbar_init(&b_empty[s], 1 + kCsEpiWarps); }
     for (int i = 0; i < 2; ++i) { tc::mbar_init(&tm_full[i], 1); tc::mbar_init(&tm_empty[i], kCsEpiWarps);
-                                  tc::mbar_init(&it_full[i], 1); tc::mbar_init(&it_empty[i], 1 + kCsEpiWarps); }
+                                  tc::mbar_init(&it_full[i], 1); tc::mbar_init(&it_empty[i], 2); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -244,18 +247,19 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem_base = s_tmem;
+  auto wait = [&](unsigned long long* bar, uint32_t parity) { return tc::mbar_wait(bar, parity, a.wait_ns); };
   // The set-up above ran beside the tail of the kernel ahead (both sweeps and the densities of 32 heads of 300 tokens 26.7 ->
   // 20.5 us, three layers of 32 heads of 1100 tokens, d = 64, 71.9 -> 66.8; large calls as before).
   wait_for_prior_grid();
 
-  // The k-th item of this CTA as the consumers see it; false: no more.  All lanes of an epilogue warp, or the MMA thread.
-  auto next_item = [&](int k, CsItem<SWEEP>& it) {
-    if (!tc::mbar_wait(&it_full[k & 1], (uint32_t)((k >> 1) & 1))) { s_fail = 1; return false; }
+  // The k-th item of this CTA as its two consumers see it (the MMA thread, one thread of the epilogue); -1: no more.
+  auto next_item = [&](int k) {
+    if (!wait(&it_full[k & 1], (uint32_t)((k >> 1) & 1))) { s_fail = 1; return -1; }
     const int i = s_item[k & 1];
-    if (i < 0) return false;
-    it.decode(a, i);
-    return true;
+    tc::mbar_arrive(&it_empty[k & 1]);
+    return i;
   };
+  int jb_copies = 0, ia_copies = 0;                          // the producer's streamed tiles and items with copies
 
   if (warp == 0) {
     // ======================================================================= TMA producer
@@ -265,12 +269,12 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
       int jb = 0, ia = 0;                                    // jobs and items so far
       int item = (int)blockIdx.x;
       for (int k = 0;; ++k) {
-        if (k >= 2 && !tc::mbar_wait(&it_empty[k & 1], (uint32_t)(((k >> 1) - 1) & 1))) s_fail = 1;
+        if (k >= 2 && !wait(&it_empty[k & 1], (uint32_t)(((k >> 1) - 1) & 1))) s_fail = 1;
+        if (s_fail) { s_lost = item; break; }                // the consumers find no further item and leave
         s_item[k & 1] = item < a.n_items ? item : -1;
         tc::mbar_arrive(&it_full[k & 1]);
         if (item >= a.n_items) { start_dependents(); break; }  // the next kernel may set itself up during the last items
         it.decode(a, item);
-        if (s_fail) it.n_jobs = 0;                           // after a wait that ran out: the epilogue writes NaN
         const CUtensorMap* map_a = SWEEP == kSweepRows ? &maps.q[it.layer] : &maps.k[it.layer];
         const CUtensorMap* map_b = SWEEP == kSweepRows ? &maps.k[it.layer] : &maps.q[it.layer];
         const int a_row = (SWEEP == kSweepRows ? it.q_base(a) : it.k_base(a)) + it.a0;
@@ -279,8 +283,8 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
         for (int job = 0; job < it.n_jobs; ++job, ++jb) {
           // the first streamed tile goes ahead of the resident ones: its stage is free earlier than they are
           const int s = jb % kCsStages;
-          if (jb >= kCsStages && !s_fail && !tc::mbar_wait(&b_empty[s], (uint32_t)(((jb / kCsStages) - 1) & 1))) s_fail = 1;
-          if (s_fail) break;
+          if (jb >= kCsStages && !s_fail && !wait(&b_empty[s], (uint32_t)(((jb / kCsStages) - 1) & 1))) s_fail = 1;
+          if (s_fail || jb == a.stop_job) break;
           const int r0 = (it.bt0 + job) * kCsTile;           // first B row of the tile
           // 16-byte granules: up to three entries past the prompt come from the row's padding and are masked
           const int n_lse = SWEEP == kSweepCols ? min(kCsTile, ((it.P + 3) & ~3) - r0) : 0;
@@ -289,7 +293,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
             tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
           if (n_lse > 0) tc::bulk_g2s(s_lse + s * kCsTile, neg_lse2 + r0, (uint32_t)(n_lse * 4), &b_full[s]);
           if (job == 0) {
-            if (ia >= 1 && !tc::mbar_wait(&a_empty, (uint32_t)((ia - 1) & 1))) { s_fail = 1; ++jb; break; }
+            if (ia >= 1 && !wait(&a_empty, (uint32_t)((ia - 1) & 1))) { s_fail = 1; ++jb; break; }
             tc::mbar_expect_tx(&a_full, (uint32_t)(2 * TILE));
             for (int t = 0; t < 2; ++t)
               for (int kb = 0; kb < KB; ++kb)
@@ -297,32 +301,31 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
             ++ia;
           }
         }
+        if (jb == a.stop_job) break;
         // Not earlier: this thread is up to four tiles ahead of the epilogue, which covers the counter's latency, and an
         // item taken at the beginning of a long one would wait while other CTAs run out of work (2048 tokens, 32 heads:
         // 80 us instead of 62).
         item = (int)(gridDim.x + atomicAdd(&a.sched[0], 1u));
       }
-      if (s_fail) {                                          // see the copies on their way land before the CTA may end
-        for (int i = max(0, jb - kCsStages); i < jb; ++i)
-          if (!tc::mbar_wait(&b_full[i % kCsStages], (uint32_t)((i / kCsStages) & 1))) break;
-        if (ia > 0) (void)tc::mbar_wait(&a_full, (uint32_t)((ia - 1) & 1));
-      }
+      jb_copies = jb; ia_copies = ia;
     }
   } else if (warp == 1) {
     // ======================================================================= MMA issuer
     if (lane == 0) {
       CsItem<SWEEP> it;
       int jb = 0, ia = 0;
-      for (int k = 0; next_item(k, it); ++k) {
-      tc::mbar_arrive(&it_empty[k & 1]);
+      for (int k = 0;; ++k) {
+      const int item = next_item(k);
+      if (item < 0) break;
+      it.decode(a, item);
       if (it.n_jobs == 0) continue;
-      if (!s_fail && !tc::mbar_wait(&a_full, (uint32_t)(ia & 1))) s_fail = 1;
+      if (!s_fail && !wait(&a_full, (uint32_t)(ia & 1))) s_fail = 1;
       ++ia;
       for (int job = 0; job < it.n_jobs && !s_fail; ++job, ++jb) {
         const int s = jb % kCsStages, buf = jb & 1;
-        if (!s_fail && !tc::mbar_wait(&b_full[s], (uint32_t)((jb / kCsStages) & 1))) s_fail = 1;
+        if (!s_fail && !wait(&b_full[s], (uint32_t)((jb / kCsStages) & 1))) s_fail = 1;
         // the epilogue must have drained this buffer (the first use of each buffer passes at once)
-        if (!s_fail && !tc::mbar_wait(&tm_empty[buf], (uint32_t)(((jb >> 1) & 1) ^ 1))) s_fail = 1;
+        if (!s_fail && !wait(&tm_empty[buf], (uint32_t)(((jb >> 1) & 1) ^ 1))) s_fail = 1;
         if (s_fail) break;
         tc::fence_after_sync();
 #pragma unroll
@@ -342,6 +345,8 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
         if (job == it.n_jobs - 1) tc::mma_commit(&a_empty);  // the resident tiles have been read
       }
       }
+      if (s_fail)                                            // tensor memory is freed behind the last products
+        for (int j = max(0, jb - 2); j < jb; ++j) (void)wait(&tm_full[j & 1], (uint32_t)((j >> 1) & 1));
     }
   } else {
     // ======================================================================= epilogue warps
@@ -350,24 +355,34 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
     const int part = e >> 2;                                 // 0,1: first A tile, B rows 0-63 / 64-127; 2,3: second A tile
     const int at = part >> 1, bhalf = part & 1;
     CsItem<SWEEP> it;
-    int jb = 0, ia = 0;
+    int jb = 0;
     uint32_t ra[32], rb[32];
+    // One thread looks at the next item, for all, ahead of the barrier that ends the one before: warps that waited for it each
+    // by itself could run out of time apart, and those that stayed would wait at the barrier for good.
+    auto end_item = [&](int k) {
+      if (e == 0 && lane == 0) s_now[(k + 1) & 1] = next_item(k + 1);
+      __syncwarp();
+      asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
+    };
+    end_item(-1);
 #pragma unroll 1
-    for (int k = 0; next_item(k, it); ++k) {
-    __syncwarp();
-    if (lane == 0) tc::mbar_arrive(&it_empty[k & 1]);
-    if (it.n_jobs == 0) continue;
+    for (int k = 0;; ++k) {
+    const int item = s_now[k & 1];
+    if (item < 0) break;
+    it.decode(a, item);
+    if (it.n_jobs == 0) { end_item(k); continue; }
     const int P = it.P, w0 = it.a0 + at * kCsTile + quarter * 32;        // first A row of this warp
     const int arow = w0 + lane;                              // position of this thread's A row (query or key)
     // sweep 1: running maximum m of the log2-domain logits and sum of 2^{c s - m}; sweep 2: column sum
     float m_run = -INFINITY, l_run = 0.f;
     double col_acc = 0.0;
 #pragma unroll 1
-    for (int job = 0; job < it.n_jobs && !s_fail; ++job, ++jb) {
+    for (int job = 0; job < it.n_jobs; ++job, ++jb) {
       const int s = jb % kCsStages, buf = jb & 1;
       const int brow0 = (it.bt0 + job) * kCsTile + bhalf * 64;   // position of the first B row this warp looks at
-      if (!tc::mbar_wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1))) s_fail = 1;
+      if (!wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1))) s_fail = 1;
       __syncwarp();
+      if (s_fail) break;                                       // one read by lanes in step: the same for all
       tc::fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + at * kCsTile + bhalf * 64);
       tc::tmem_ld32_issue(taddr, ra);
@@ -423,11 +438,10 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
     // combine the two warps that share an A row (B-row halves), fixed order; after a wait that ran out: NaN.  The exchange
     // area alternates between items: whoever writes it again has passed the barrier of the item in between.
     const int r = quarter * 32 + lane;
-    float* comb = s_comb + (ia & 1) * 4 * kCsTile;
-    ++ia;
+    float* comb = s_comb + (k & 1) * 4 * kCsTile;
     if (SWEEP == kSweepRows) {
       if (bhalf == 1) { comb[(at * 2 + 0) * kCsTile + r] = m_run; comb[(at * 2 + 1) * kCsTile + r] = l_run; }
-      asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
+      end_item(k);
       if (bhalf == 0 && arow < P) {
         const float m2 = comb[(at * 2 + 0) * kCsTile + r], l2 = comb[(at * 2 + 1) * kCsTile + r];
         const float mm = fmaxf(m_run, m2);
@@ -438,7 +452,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
     } else {
       double* dcomb = reinterpret_cast<double*>(comb);
       if (bhalf == 1) dcomb[at * kCsTile + r] = col_acc;
-      asm volatile("bar.sync 1, %0;" ::"n"(kCsEpiWarps * 32) : "memory");
+      end_item(k);
       if (bhalf == 0 && arow < P)
         a.colsum[((size_t)it.layer * a.BHq + it.bh) * a.P + arow] = s_fail ? NAN : (float)(col_acc + dcomb[at * kCsTile + r]);
     }
@@ -449,6 +463,29 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   if (warp == 1) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem_base, 512);
+  }
+  if (s_fail) {
+    if (tid == 0) {                                          // see the copies on their way land before the CTA may end
+      for (int i = max(0, jb_copies - kCsStages); i < jb_copies; ++i)
+        if (!wait(&b_full[i % kCsStages], (uint32_t)((i / kCsStages) & 1))) break;
+      if (ia_copies > 0) (void)wait(&a_full, (uint32_t)((ia_copies - 1) & 1));
+    }
+    // NaN for the items this CTA had in hand, and for those that nobody has taken
+    for (int n = 0;; ++n) {
+      if (tid == 0) s_now[0] = n < 2 ? s_item[n] : n == 2 ? s_lost : (int)(gridDim.x + atomicAdd(&a.sched[0], 1u));
+      __syncthreads();
+      const int i = s_now[0];
+      __syncthreads();
+      if (i >= a.n_items && n > 2) break;
+      if (i < 0 || i >= a.n_items) continue;
+      CsItem<SWEEP> it;
+      it.decode(a, i);
+      if (it.n_jobs == 0) continue;
+      for (int r = it.a0 + tid; r < min(it.P, it.a0 + 2 * kCsTile); r += kCsThreads) {
+        if (SWEEP == kSweepRows) a.neg_lse2[it.layer * a.lse_stride + it.bh * lse_row(a.P) + r] = NAN;
+        else a.colsum[((size_t)it.layer * a.BHq + it.bh) * a.P + r] = NAN;
+      }
+    }
   }
   if (tid == 0) {                                            // the last CTA leaves the counters at zero for the next launch
     __threadfence();
@@ -471,11 +508,13 @@ size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P) { return (size_t)bat
 // Column sums of n <= kColsumLayers layers of 16-bit Q, K on the tensor cores.  `lse_in` (natural log; NULL, or a pointer
 // per layer) replaces sweep 1; `neg_lse2` is scratch of n times colsum_tc_lse_bytes(), `lse_stride` bytes apart; `colsum` of
 // the layers lies one after another; `plen` (DEVICE, may be NULL) holds every sequence's prompt length, `status` (may be
-// NULL) the error word, `sched` two words that are zero between launches.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that are not a multiple of
+// NULL) the error word, `sched` two words that are zero between launches; `wait_ns` (0: one second) and `stop_job` are for the
+// failure-detection tests.  Any prompt length: the rows of a TMA box need no alignment.  (Lengths that are not a multiple of
 // four used to take the FFMA kernels: 17.5 ms instead of 1.0 for two layers of 6001 tokens.)
 cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, int n, const void* const* Q,
                              const void* const* K, const float* const* lse_in, float* neg_lse2, size_t lse_stride,
-                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st) {
+                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st,
+                             unsigned long long wait_ns, int stop_job) {
   ColsumTcMaps maps;
   LseIn lse;
   for (int l = 0; l < n; ++l) {
@@ -489,6 +528,7 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, in
   a.colsum = colsum;
   a.status = status;
   a.sched = sched;
+  a.wait_ns = wait_ns > 0 ? wait_ns : kTcWaitNs; a.stop_job = stop_job;
   a.P = P; a.Hq = Hq; a.group = Hq / Hkv; a.BHq = B * Hq;
   a.plen = plen;
   const int KB = D / 64;

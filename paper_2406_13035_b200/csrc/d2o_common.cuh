@@ -222,7 +222,7 @@ struct d2o_ctx {
   int similarity_path;         // tuning: 0 = tensor cores for 16-bit keys, 1 = FFMA kernel for every dtype
   int stats_path;              // tuning: 0 = tensor cores for the column sums of 16-bit Q/K, 1 = FFMA kernels
   int wait_limit_us;           // failure-detection tests: limit of a device-side wait in microseconds (0 = one second)
-  int producer_stop_stage;     // failure-detection tests: the decode producer issues no copy from this stage on (-1 = never)
+  int producer_stop_stage;     // failure-detection tests: the producers of decode and column sums issue no copy from this stage on (-1 = never)
   // d2o_layer_stats_layers, fp32: one stream per lane, created with the first call (no device memory involved)
   cudaStream_t lane_stream[d2o::kStatsLanes];
   cudaEvent_t lane_done[d2o::kStatsLanes];
@@ -263,7 +263,8 @@ size_t sim_tc_build_items(const d2o_ctx* c, int n_sms, int4* items, int32_t* cou
 // tensor-core column sums of the prompt attention for 16-bit Q/K (d2o_colsum_tc.cu)
 cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, int n, const void* const* Q,
                              const void* const* K, const float* const* lse_in, float* neg_lse2, size_t lse_stride,
-                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st);
+                             float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st,
+                             unsigned long long wait_ns = 0, int stop_job = -1);
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P);      // its row normalisers
 
 // remembers the text of a failed CUDA runtime call for d2o_last_cuda_error(); returns D2O_ERR_CUDA

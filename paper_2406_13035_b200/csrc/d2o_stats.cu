@@ -585,7 +585,8 @@ cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
   cudaError_t e = launch_colsum_tc(g.dtype, g.d_head, B, Hq, g.n_kv_heads, P, n, Q, K, lse, (float*)(c->scratch + c->slay.lse),
                                    c->slay.lse_stride, colsum, plen, (uint32_t*)(c->state + c->lay.status),
-                                   (uint32_t*)(c->state + c->lay.colsum_sched), st);
+                                   (uint32_t*)(c->state + c->lay.colsum_sched), st,
+                                   (unsigned long long)c->wait_limit_us * 1000ull, c->producer_stop_stage);
   if (e != cudaSuccess) return e;
   return launch_behind(density_kernel, dim3((unsigned)(B * Hq), (unsigned)n), kDensityThreads, 0, st, (const float*)colsum,
                        (double*)(c->state + c->lay.density), P, Hq, g.n_layers, layer, plen,

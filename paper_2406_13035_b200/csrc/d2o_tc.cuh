@@ -32,12 +32,12 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t 
       : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait; false = the phase did not complete within kTcWaitNs.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity) {
+// Bounded wait; false = the phase did not complete within the limit.
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, unsigned long long limit_ns = kTcWaitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
   while (!mbar_try_wait(bar, parity)) {
-    if (global_ns() - t0 > kTcWaitNs) return false;
+    if (global_ns() - t0 > limit_ns) return false;
   }
   return true;
 }

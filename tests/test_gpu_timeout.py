@@ -110,3 +110,33 @@ def test_decode_cluster_whose_values_do_not_arrive(cuda_device, P, rho, hq, hkv,
         assert ctx.d2o_get_stats().error_word == D2O_ERR_TIMEOUT
         assert _same(before, _state(ctx, wl)) and torch.equal(out, first)
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f16", 64)])
+@pytest.mark.parametrize("P,hq,stage", [(1025, 2, 0), (1025, 2, 1), (1025, 2, 3), (700, 64, 5), (2000, 40, 9)])
+def test_column_sums_whose_tiles_do_not_arrive(cuda_device, dtype, d, P, hq, stage):
+    """Fewer items than SMs and more (those that a CTA takes behind its first one, and those that nobody takes any more), a
+    wait that runs out in the first item or later.  Every column sum that the missing tiles could have entered is NaN; a call
+    without the knob afterwards computes everything."""
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    Q = torch.randn(1, hq, P, d, generator=g, device=cuda_device).to(td)
+    K = torch.randn(1, hq, P, d, generator=g, device=cuda_device).to(td)
+    make = lambda: B.D2OContext(B.make_config(n_layers=1, batch=1, n_q_heads=hq, n_kv_heads=hq, d_head=d, dtype=dtype,
+                                              prompt_len=P, max_new_tokens=2, rho=0.5, n_sink=1, min_budget=8))
+    ctx, other = make(), make()
+    other.d2o_layer_stats(0, Q, K)
+    ctx.d2o_set_fault_injection(wait_limit_us=2000, producer_stop_stage=stage)
+    t0 = time.perf_counter()
+    ctx.d2o_layer_stats(0, Q, K)
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t0 < 1.0
+    assert ctx.d2o_get_stats().error_word == D2O_ERR_TIMEOUT
+    cs = ctx.colsum(0)
+    # the last rows' normalisers take every tile of the keys; they enter every column of their head
+    assert torch.isnan(cs).all()
+    ctx.d2o_set_fault_injection(0, -1)
+    ctx.d2o_layer_stats(0, Q, K)
+    assert torch.equal(ctx.colsum(0), other.colsum(0))
+    ctx.close()
+    other.close()
