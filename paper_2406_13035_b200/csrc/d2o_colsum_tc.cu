@@ -41,7 +41,7 @@ constexpr int kCsEpiWarps = 16;
 constexpr int kCsThreads = (2 + kCsEpiWarps) * 32;
 constexpr int kCsTile = 128;                 // rows per MMA operand tile (M and N)
 constexpr int kCsStages = 4;                 // B ring
-enum { kSweepRows = 0, kSweepCols = 1 };
+enum { kSweepRows = 0, kSweepCols = 1, kSweepColsGiven = 2 };    // Given: with the caller's normalisers
 
 struct ColsumTcArgs {
   float* neg_lse2;                           // [layers][B * Hq][lse_row(P)] negated log2-domain row normalisers (sweep 1 -> sweep 2)
@@ -86,10 +86,15 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// maximum that keeps a NaN
+// maximum and minimum that keep a NaN
 __device__ __forceinline__ float max_nan(float a, float b) {
   float d;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
 // global -> this CTA's shared memory, 16-byte aligned on both sides, size a multiple of 16
@@ -115,12 +120,17 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // the nearest integer and leaves n in the low mantissa bits), 2^f by the polynomial of degree 5 with constant term 1
 // whose largest relative error on [-1/2, 1/2] is smallest (9.1e-8; found as a linear program over 4001 Chebyshev points;
 // 1.7e-7 with the fp32 roundings of Horner's rule, the same size as the special-function unit's), 2^n as exponent bits.
-// Exponents below -127 count as -127, whose exponent bits are those of zero: such a term is 0.  A NaN stays one.
+// Exponents below -127 count as -127, whose exponent bits are those of zero: such a term is 0.  A NaN stays one.  HIGH:
+// exponents that round to 128 and more count as 128, whose exponent bits are those of infinity (normalisers that the caller
+// made too low, or -inf); the sweeps' own normalisers leave none above 0, but for rounding, and skip it.
+template <bool HIGH>
 __device__ __forceinline__ tc::f32x2 exp2_poly_pair(tc::f32x2 xy, tc::f32x2 acc) {
   const float kRound = 12582912.0f;
   float x, y;
   tc::unpack2(xy, x, y);
-  xy = tc::pack2(tc::max_nan(x, -127.f), tc::max_nan(y, -127.f));
+  x = tc::max_nan(x, -127.f); y = tc::max_nan(y, -127.f);
+  if (HIGH) { x = tc::min_nan(x, 128.f); y = tc::min_nan(y, 128.f); }
+  xy = tc::pack2(x, y);
   const tc::f32x2 t = tc::add2(xy, tc::pack2(kRound, kRound));
   const tc::f32x2 n = tc::add2(t, tc::pack2(-kRound, -kRound));
   const tc::f32x2 f = tc::fma2(n, tc::pack2(-1.f, -1.f), xy);                 // exact
@@ -142,7 +152,7 @@ __host__ __device__ constexpr bool poly_pair(int k) { return (kPolyPairs >> (k &
 
 // Sum of 2^{c s_i + b_i} over the 64 logits s_i of one accumulator row (in two register blocks).  Rows: every b_i is
 // `b`; columns: b_i comes from shared memory (the negated normalisers of the 64 streamed rows).
-template <bool PER_ROW>
+template <bool PER_ROW, bool HIGH>
 __device__ __forceinline__ float exp_sum_64(const uint32_t (&ra)[32], const uint32_t (&rb)[32], float c, float b,
                                             const float* s_b) {
   const tc::f32x2 c2 = tc::pack2(c, c), b2 = tc::pack2(b, b);
@@ -163,7 +173,7 @@ __device__ __forceinline__ float exp_sum_64(const uint32_t (&ra)[32], const uint
                                       : tc::pack2(__uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
         const tc::f32x2 x = tc::fma2(s, c2, bb[w]);
         if (poly_pair(i4 * 4 + half * 2 + w)) {
-          pac[w] = exp2_poly_pair(x, pac[w]);
+          pac[w] = exp2_poly_pair<HIGH>(x, pac[w]);
         } else {
           float x0, x1;
           tc::unpack2(x, x0, x1);
@@ -264,7 +274,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
   if (warp == 0) {
     // ======================================================================= TMA producer
     if (lane == 0) {
-      if (SWEEP == kSweepCols) asm volatile("fence.proxy.async.global;" ::: "memory");    // normalisers: stored by the kernel ahead, copied in bulk here
+      if (SWEEP != kSweepRows) asm volatile("fence.proxy.async.global;" ::: "memory");    // normalisers: stored by the kernel ahead, copied in bulk here
       CsItem<SWEEP> it{};
       int jb = 0, ia = 0;                                    // jobs and items so far
       int item = (int)blockIdx.x;
@@ -287,7 +297,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
           if (s_fail || jb == a.stop_job) break;
           const int r0 = (it.bt0 + job) * kCsTile;           // first B row of the tile
           // 16-byte granules: up to three entries past the prompt come from the row's padding and are masked
-          const int n_lse = SWEEP == kSweepCols ? min(kCsTile, ((it.P + 3) & ~3) - r0) : 0;
+          const int n_lse = SWEEP != kSweepRows ? min(kCsTile, ((it.P + 3) & ~3) - r0) : 0;
           tc::mbar_expect_tx(&b_full[s], (uint32_t)(TILE + n_lse * 4));
           for (int kb = 0; kb < KB; ++kb)
             tc::tma_load_2d(sB + s * TILE + kb * BLOCK, map_b, kb * 64, b_base + r0, &b_full[s]);
@@ -411,13 +421,13 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
         for (int i = 0; i < 32; ++i) bmx[i & 3] = tc::max3(bmx[i & 3], __uint_as_float(ra[i]), __uint_as_float(rb[i]));
         const float bm = fmaxf(fmaxf(bmx[0], bmx[1]), fmaxf(bmx[2], bmx[3])) * c;     // in the log2 domain, rounded once
         if (bm > m_run) { l_run *= exp2f(m_run - bm); m_run = bm; }            // exp2f(-inf) = 0 on the first block
-        if (m_run > -INFINITY) l_run += exp_sum_64<false>(ra, rb, c, -m_run, nullptr);
+        if (m_run > -INFINITY) l_run += exp_sum_64<false, false>(ra, rb, c, -m_run, nullptr);
       } else {
         // B rows are queries: valid iff query >= key and query < P
         const float* ls = s_lse + s * kCsTile + bhalf * 64;
         float part;
         if (brow0 >= w0 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
-          part = exp_sum_64<true>(ra, rb, c, 0.f, ls);
+          part = exp_sum_64<true, SWEEP == kSweepColsGiven>(ra, rb, c, 0.f, ls);
         } else {
           const int first = arow - brow0, end = P - brow0;     // the row's valid columns of the 64
           float p0 = 0.f, p1 = 0.f;
@@ -559,10 +569,11 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, in
     lse_to_log2_kernel<<<dim3((unsigned)(B * Hq), (unsigned)((P + 255) / 256), (unsigned)n), 256, 0, st>>>(lse, neg_lse2, a.lse_stride, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    D2O_LAUNCH_CS_ALL(kSweepColsGiven);
   } else {
     D2O_LAUNCH_CS_ALL(kSweepRows);
+    D2O_LAUNCH_CS_ALL(kSweepCols);
   }
-  D2O_LAUNCH_CS_ALL(kSweepCols);
 #undef D2O_LAUNCH_CS_ALL
 #undef D2O_LAUNCH_CS
   return cudaSuccess;

@@ -97,3 +97,29 @@ def test_work_counter_is_zero_after_every_call(cuda_device):
         ctx.d2o_layer_stats(0, Q, K)
         assert torch.equal(ctx.colsum(0), want) and counter.tolist() == [0, 0]
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,d,P", [("bf16", 128, 700), ("f16", 64, 513)])
+def test_normalisers_far_too_low(cuda_device, dtype, d, P):
+    """A row whose normaliser is -inf, or 200 below the true one, contributes +inf to every column it attends to (its
+    probabilities are 2^288 and more times too large) and nothing else: no NaN, no finite value, in no place of the tiles."""
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    Q = torch.randn(1, 4, P, d, generator=g, device=cuda_device).to(td)
+    K = torch.randn(1, 2, P, d, generator=g, device=cuda_device).to(td)
+    logits, _ = _reference(Q, K)
+    lse = torch.logsumexp(logits, -1)
+    at = (P * 3) // 4                                              # from here on the columns see no such row
+    low = lse.clone()
+    low[0, 0, at - 1] = -float("inf")
+    low[0, 1, at - 1] -= 200.0
+    low[0, 2, 17] = -float("inf")
+    ref = torch.exp(logits - lse[..., None]).sum(-2)
+    ctx = _context(dtype, 1, 4, 2, d, P)
+    ctx.d2o_layer_stats(0, Q, K, low.float().contiguous())
+    cs = ctx.colsum(0)[0]
+    for h, n in ((0, at), (1, at), (2, 18), (3, 0)):
+        assert torch.isposinf(cs[h, :n]).all()
+        assert float(((cs[h, n:].double() - ref[0, h, n:]).abs() / ref[0, h, n:]).max()) < 2e-5
+    assert ctx.d2o_get_stats().error_word == 0
+    ctx.close()
