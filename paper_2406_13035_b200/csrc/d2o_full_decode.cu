@@ -136,9 +136,10 @@ full_decode_kernel(FullArgs a, const T* __restrict__ q_in, const T* __restrict__
       const float mn = fmaxf(m[g], mx);
       const float old = mn > -INFINITY ? exp2f(m[g] - mn) : 0.f;
       m[g] = mn;
+      const float base = mn > -INFINITY ? mn : 0.f;                  // rows past the end, and logits of -inf: 0; a NaN stays one
       float p[U / 4], s = 0.f;
 #pragma unroll
-      for (int b = 0; b < U / 4; ++b) { p[b] = x[g][b] > -INFINITY ? exp2f(x[g][b] - mn) : 0.f; s += p[b]; }
+      for (int b = 0; b < U / 4; ++b) { p[b] = exp2f(x[g][b] - base); s += p[b]; }
       l[g] = fmaf(l[g], old, s);                                     // this lane's rows only: summed over the group at the end
 #pragma unroll
       for (int e = 0; e < EPV; ++e) acc[g][e] *= old;

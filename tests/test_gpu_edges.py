@@ -150,3 +150,25 @@ def test_full_decode_lengths(cuda_device, dtype, d, G, n, length):
     K, V = torch.cat([kc[:, :length], k[:, None]], 1).double(), torch.cat([vc[:, :length], v[:, None]], 1).double()
     ref = torch.softmax(q.double() @ K.transpose(1, 2) / math.sqrt(d), -1) @ V
     assert close(np64(out), ref.cpu().numpy(), dtype) <= 1.0
+
+
+@pytest.mark.parametrize("dtype,d,G,length", [("f16", 128, 1, 200), ("bf16", 64, 4, 65), ("f32", 128, 2, 1000), ("bf16", 128, 8, 1)])
+def test_full_decode_non_finite_keys(cuda_device, dtype, d, G, length):
+    """A NaN in a cached key reaches every output of its slice, as it does in the softmax; a logit of -inf is weight 0."""
+    td, n, row = W.TORCH_DTYPES[dtype], 4, length // 2
+    g = torch.Generator(device=cuda_device).manual_seed(length)
+    kc, vc = (torch.randn(n, length + 2, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    q = torch.randn(n, G, d, generator=g, device=cuda_device).to(td)
+    k, v = (torch.randn(n, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    kc[..., 0], k[:, 0] = 0.0, 0.0
+    q[..., 0] = 4.0
+    kc[1, row, 1] = float("nan")
+    kc[2, row, 0] = -float("inf")
+    k[3, 5] = float("nan")
+    out = torch.empty_like(q)
+    K, V = torch.cat([kc[:, :length], k[:, None]], 1).double(), torch.cat([vc[:, :length], v[:, None]], 1).double()
+    B.d2o_full_decode_step(kc, vc, length, q, k, v, out)
+    ref = torch.softmax(q.double() @ K.transpose(1, 2) / math.sqrt(d), -1) @ V
+    assert torch.isnan(out[1]).all() and torch.isnan(out[3]).all()
+    for s in (0, 2):
+        assert close(np64(out[s]), ref[s].cpu().numpy(), dtype) <= 1.0
