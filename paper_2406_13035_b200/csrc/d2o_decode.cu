@@ -1148,7 +1148,7 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
 
   // Few slices: a cluster of CTAs for each (the knobs of d2o_set_tuning belong to the kernel below)
   if (c->decode_warps == 0 && c->decode_stages == 0 && c->decode_smem_rows == 0 && c->decode_long_pairs == 0) {
-    const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows, sum_rows * Hkv, ordered);
+    const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows, sum_rows * Hkv);
     if (C > 0) {
       bool published = true;                                          // the last step of every layer of the call
       for (int l = l0; l < l1; ++l) published = published && c->layer_published[l];

@@ -46,7 +46,7 @@ struct DecodeArgs {
 
 // d2o_decode_split.cu
 void decode_split_places(int* clusters);
-int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows, bool all_layers);
+int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows);
 cudaError_t launch_decode_split(const d2o_ctx* c, DecodeArgs a, int C, int n_slices, int max_rows, const void* q,
                                 const void* k, const void* v, void* out, void* kpool, void* vpool, cudaStream_t st);
 

@@ -790,18 +790,17 @@ static size_t split_smem(int rows, int G, int D, int esz) {
 //
 // What counts here is how quickly one slice is done, and how many rounds of resident clusters the call takes: about 11 us
 // for one and less for those behind it, plus the time for the longest slice's rows, which the one-CTA kernel pays in full (us
-// per call, this kernel /
-// decode_kernel: 8 fp16 slices of 1640 rows, one head, 13.8 / 37, 32 of 820 rows 13.8 / 25, 72 of 160 bf16 rows, four heads,
-// 12.7 / 14.5).  Rows are long where one layer holds most of the budget, and then shared memory admits one CTA per SM: 144
-// slices of which the longest has 1460 rows are four rounds of four CTAs or eight of eight, 99 / 27; 100 slices of 320 rows
-// are two rounds, 21.8 / 16.5; but 64 slices of up to 1345 rows in two rounds 21.5 / 26.  Single heads of few rows are faster
-// in one CTA when the same slices' next step comes behind (24 slices of 40 rows 11.9 / 10.4), but not when another layer does,
-// whose clusters start beside these (56 fp32 slices of 172 rows 8.7 / 9.9).  Larger clusters shorten the passes, but every barrier and every exchange
-// takes longer: two CTAs, four for longer slices while there is an SM for each (32 slices of 800 rows 12.9 us with four, 14.2
-// with two, 17 with eight), more only where the rows do not fit otherwise, two where four would take a second round (36
-// slices of 640 rows 15.6 instead of 19.9).  From 20 MB of keys and values on, the passes count more than the chain of steps
-// (96 of 800 rows (39 MB) 36 / 31).
-int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows, bool all_layers) {
+// per call, this kernel / decode_kernel: 8 fp16 slices of 1640 rows, one head, 13.8 / 37, 32 of 820 rows 13.8 / 25, 72 of 160
+// bf16 rows, four heads, 12.7 / 14.5).  One round of clusters is the better choice, also for short slices: repeated steps on
+// 24 slices of 40 rows and one head take 11.9 / 10.4, but in a model that calls layer by layer the clusters of one call start
+// beside those of the call before (56 fp32 slices of 172 rows 8.7 / 9.9).  Rows are long where one layer holds most of the
+// budget, and then shared memory admits one CTA per SM: 144 slices of which the longest has 1460 rows are four rounds of four
+// CTAs or eight of eight, 99 / 27; 100 slices of 320 rows are two rounds, 21.8 / 16.5; but 64 slices of up to 1345 rows in two
+// rounds 21.5 / 26.  Larger clusters shorten the passes, but every barrier and every exchange takes longer: two CTAs, four for
+// longer slices while there is an SM for each (32 slices of 800 rows 12.9 us with four, 14.2 with two, 17 with eight), more
+// only where the rows do not fit otherwise, two where four would take a second round (36 slices of 640 rows 15.6 instead of
+// 19.9).  From 20 MB of keys and values on, the passes count more than the chain of steps (96 of 800 rows (39 MB) 36 / 31).
+int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double total_rows) {
   const d2o_config& g = c->cfg;
   const int G = c->group;
   if (total_rows * 2 * g.d_head * c->elem_size > 20e6 || n_slices > c->n_sms) return 0;
@@ -818,10 +817,10 @@ int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double to
   while (i < kSplitSizes && (n = rounds(i)) == 0) ++i;
   if (n == 0) return 0;
   if (n > 1 && i == 1 && rounds(0) == 1) { i = 0; n = 1; }
-  if (n == 1 && !all_layers) return 2 << i;
+  if (n == 1) return 2 << i;
   const double row_us = 3.1e-5 * 2 * g.d_head * c->elem_size * max_rows;  // the longest slice in one CTA
   const double one_us = (G == 1 ? 10.0 : G <= 4 ? 12.3 : 16.0) + row_us;
-  const double split_us = (c->elem_size == 4 ? 11.0 : 11.5) + 9.5 * (n - 1) + row_us / (2 << i);
+  const double split_us = 11.5 + 9.5 * (n - 1) + row_us / (2 << i);
   return split_us < one_us ? 2 << i : 0;
 }
 
