@@ -1,4 +1,4 @@
-"""d2o_prefill_compress_layers (several layers per call, up to four side by side on the library's own streams)
+"""d2o_prefill_compress_layers (several layers per call, up to sixteen of which share every launch)
 against d2o_prefill_compress called layer by layer: the compressed caches, thresholds and the decode steps that
 follow must be identical bit for bit."""
 import dataclasses

@@ -3,10 +3,9 @@
 Some users of the library cannot call cudaMalloc while it runs: an inference server whose memory
 pool has taken the whole device, or a host application that passes tensors in but keeps its
 allocator to itself.  d2o_layer_stats_static serves them with a scratch array that lives inside
-the library image.  It runs the library's generic kernels: where d2o_layer_stats runs them too
-(fp32 inputs, or a prompt length that is not a multiple of 4) the two must agree bit for bit, and
-where d2o_layer_stats takes its tensor-core kernels they must agree within the parity tolerance;
-in both cases also on a second call that finds the first call's leftovers in the scratch array.
+the library image.  It runs the kernels of d2o_layer_stats, so the two agree bit for bit (checked
+for fp32 inputs and for a prompt length that is no multiple of 4) and within the parity tolerance,
+also on a second call that finds the first call's leftovers in the scratch array.
 The results are checked against the CPU oracle as well, and the free device memory must not move
 across the call.
 This file sorts last on purpose, so that a run which stops at the first failure has already
