@@ -381,18 +381,17 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
     if (item < 0) break;
     it.decode(a, item);
     if (it.n_jobs == 0) { end_item(k); continue; }
+    const int n_jobs = __any_sync(0xffffffffu, s_fail != 0) ? 0 : it.n_jobs;     // after a wait that ran out: NaN, at once
     const int P = it.P, w0 = it.a0 + at * kCsTile + quarter * 32;        // first A row of this warp
     const int arow = w0 + lane;                              // position of this thread's A row (query or key)
     // sweep 1: running maximum m of the log2-domain logits and sum of 2^{c s - m}; sweep 2: column sum
     float m_run = -INFINITY, l_run = 0.f;
     double col_acc = 0.0;
 #pragma unroll 1
-    for (int job = 0; job < it.n_jobs; ++job, ++jb) {
+    for (int job = 0; job < n_jobs; ++job, ++jb) {
       const int s = jb % kCsStages, buf = jb & 1;
       const int brow0 = (it.bt0 + job) * kCsTile + bhalf * 64;   // position of the first B row this warp looks at
-      if (!wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1))) s_fail = 1;
-      __syncwarp();
-      if (s_fail) break;                                       // one read by lanes in step: the same for all
+      if (!__all_sync(0xffffffffu, wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1)))) { s_fail = 1; break; }
       tc::fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + at * kCsTile + bhalf * 64);
       tc::tmem_ld32_issue(taddr, ra);
