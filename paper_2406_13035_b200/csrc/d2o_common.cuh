@@ -168,6 +168,7 @@ struct Layout {            // byte offsets into `state`
 };
 struct ScratchLayout {     // byte offsets into `scratch`
   size_t lse, evict_idx, evict_mx, evict_nn, seg_start, seg_items, seg_tmp, part_key, prompt_rn, pl_spill, stage_q, stage_k, stage_v, stage_out, end;
+  size_t logits, logits_stride;   // fp32: logits between the two sweeps of the column sums, one set per lane (stride 0: none)
   size_t lse_stride;       // `lse` exists once per layer that is worked on at a time, this far apart (d2o_layer_stats_layers): at
                            // most kColsumLayers, kStatsLanes for fp32 caches, and never more than there are layers
   size_t stage_stride;     // stage_q .. stage_out exist 2 * kHostBlock times, this far apart (d2o_decode_steps_host)
@@ -266,6 +267,7 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, in
                              float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st,
                              unsigned long long wait_ns = 0, int stop_job = -1);
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P);      // its row normalisers
+size_t stored_logits_bytes(int heads, int P, int lanes);                     // logits that one lane of the fp32 kernels keeps (d2o_stats.cu)
 
 // remembers the text of a failed CUDA runtime call for d2o_last_cuda_error(); returns D2O_ERR_CUDA
 d2o_status record_cuda_error(cudaError_t e, const char* where);

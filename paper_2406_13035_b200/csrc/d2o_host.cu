@@ -123,6 +123,9 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   s->lse = take(colsum_tc_lse_bytes(c->batch, c->n_q_heads, c->prompt_len));
   s->lse_stride = o - s->lse;
   o += (std::min<size_t>(L, c->dtype == D2O_F32 ? kStatsLanes : kColsumLayers) - 1) * s->lse_stride;
+  const size_t lanes = std::min<size_t>(L, kStatsLanes);
+  s->logits_stride = c->dtype == D2O_F32 ? stored_logits_bytes((int)(B * Hq), (int)P, (int)lanes) : 0;
+  s->logits = take(lanes * s->logits_stride);
   s->evict_idx = take(B * Hkv * P * 4);
   s->evict_mx = take(B * Hkv * P * 4);
   s->evict_nn = take(B * Hkv * P * 4);

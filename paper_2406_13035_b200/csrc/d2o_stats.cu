@@ -5,12 +5,15 @@
 // Kernels in this file
 //   sweep_kernel    row normalisers log sum_j exp(q_i.k_j/sqrt(d)) of the causal attention, and the
 //                   column sums s_j = sum_{i>=j} exp(q_i.k_j/sqrt(d) - lse_i)
+//   colsum_stored_kernel  the same column sums from dot products that the row sweep stored (fp32 caches)
 //   density_kernel  warp-shuffle mean / variance of s per query head (double accumulation)
 //   budget_kernel   Eq. 5 with clamping and exact-sum integerisation, one CTA per sequence
 // The two attention sweeps here are the generic FFMA implementation (any dtype, fp32 math);
 // 16-bit inputs take the tensor-core path of d2o_colsum_tc.cu.
 #include <cooperative_groups.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "d2o_common.cuh"
 
@@ -82,11 +85,17 @@ __device__ __forceinline__ void combine_lse(float& m, float& l, float mo, float 
   m = mn;
 }
 
+// log2(e) / sqrt(d)
+__host__ __device__ constexpr float logit_scale(int d) { return (d == 64 ? 0.125f : 0.08838834764831845f) * kLog2e; }
+
+// tiles of the causal triangle of P rows
+__host__ __device__ __forceinline__ size_t triangle_tiles(int P) { const size_t n = (size_t)(P + kTile - 1) / kTile; return n * (n + 1) / 2; }
+
 // kSum: colsum_j = sum_{i >= j} exp(q_i.k_j / sqrt(d) - lse_i); else lse_i = log sum_{j <= i} exp(q_i.k_j / sqrt(d)).
 template <typename T, int D, bool kSum>
 __global__ void __launch_bounds__(kStatThreads, 3)
 sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __restrict__ lse_in, float* __restrict__ out,
-             int Pmax, int Hq, int group, const int32_t* __restrict__ plen) {
+             int Pmax, int Hq, int group, const int32_t* __restrict__ plen, int head0, float4* __restrict__ logits) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];
   SweepSmem<D>& sm = *reinterpret_cast<SweepSmem<D>*>(sweep_smem);
   constexpr int LDX = SweepSmem<D>::kLdX, LDY = SweepSmem<D>::kLdY, kSlabs = D / kSlab;
@@ -94,13 +103,13 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int u = blockIdx.x / C;
-  const int b = blockIdx.y / Hq, hq = blockIdx.y % Hq;
+  const int bh = head0 + (int)blockIdx.y, b = bh / Hq, hq = bh % Hq;
   const int P = plen ? plen[b] : Pmax;                 // this sequence's prompt length; tensors are laid out for Pmax
   const int nT = (P + kTile - 1) / kTile;
   if (2 * u >= nT + (nT & 1)) return;                  // the whole cluster
-  const T* q = Q + (size_t)blockIdx.y * Pmax * D;
+  const T* q = Q + (size_t)bh * Pmax * D;
   const T* k = K + ((size_t)b * (Hq / group) + hq / group) * (size_t)Pmax * D;
-  const float* ls = kSum ? lse_in + (size_t)blockIdx.y * Pmax : nullptr;
+  const float* ls = kSum ? lse_in + (size_t)bh * Pmax : nullptr;
   // strip `part` of the pair: its resident tile and its number of streamed tiles
   const int n0 = nT - u, n = u != nT - 1 - u ? nT + 1 : n0;
   auto resident = [&](int part) { return (part == 0) == kSum ? u : nT - 1 - u; };
@@ -108,7 +117,7 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
   // resident rows ty + 8 r, streamed rows tx + 16 c; a warp is 4 x 8 threads, the CTA 2 x 2 warps
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = warp >> 1;
   const int ty = (warp & 1) * 4 + (lane >> 3), tx = half * 8 + (lane & 7);
-  const float mul = (D == 64 ? 0.125f : 0.08838834764831845f) * kLog2e;
+  const float mul = logit_scale(D);
 
 #pragma unroll 1
   for (int part = 0; part < 2; ++part) {
@@ -179,8 +188,13 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
         for (int c = 0; c < kStripB; ++c) {
           float lo, hi;
           asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(s[r][c]));
-          x[c] = fmaf(lo + hi, mul, -lr[c]);
+          x[c] = lo + hi;
         }
+        if (!kSum && logits)                          // for colsum_stored_kernel, in the order of the threads
+          logits[(blockIdx.y * triangle_tiles(Pmax) + (size_t)at * (at + 1) / 2 + i) * (kTile * kTile / 4) + r * kStatThreads + threadIdx.x] =
+              make_float4(x[0], x[1], x[2], x[3]);
+#pragma unroll
+        for (int c = 0; c < kStripB; ++c) x[c] = fmaf(x[c], mul, -lr[c]);
         if (masked) {
 #pragma unroll
           for (int c = 0; c < kStripB; ++c) {
@@ -233,9 +247,108 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
       else { const float2 o = *reinterpret_cast<const float2*>(from); combine_lse(m, l, o.x, o.y); }
     }
     if (row < P && (part == 0 || n > n0))
-      out[(size_t)blockIdx.y * Pmax + row] = kSum ? (float)t : (m + log2f(l)) * 0.6931471805599453f;
+      out[(size_t)bh * Pmax + row] = kSum ? (float)t : (m + log2f(l)) * 0.6931471805599453f;
   }
   cluster.sync();                                     // no CTA ends while another reads its results
+}
+
+// Column sums from the dot products that the row sweep left in `logits` (whole tiles; rows >= P: 0), one pair of
+// column tiles per cluster as above.  A thread holds the entries that it would have computed: rows ty + 8 r, columns tx + 16 c.
+//
+// The row sweep is bound by its FMAs (one per element of d and logit); repeating them for the column sums took half of the call.
+// A logit costs 8 bytes of traffic instead (kStoredLogits: how many are kept at a time).  Row sweep, column sums and densities,
+// us, repeated / stored: 8 heads of 1024 tokens, d = 64, 70 / 48, of 100 tokens 24.6 / 20.5, of 450 tokens 33.5 / 24.5; 32
+// heads of 1999 tokens 540 / 367; six layers of 16 heads of 1500 tokens 893 / 569.
+__global__ void __launch_bounds__(kStatThreads)
+colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__ out, int Pmax, int Hq, const int32_t* __restrict__ plen,
+                     int head0, float mul) {
+  __shared__ double res[2][2][kTile];                  // [strip of the pair][warps that share columns][column]
+  start_dependents();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int u = blockIdx.x / C, bh = head0 + (int)blockIdx.y;
+  const int P = plen ? plen[bh / Hq] : Pmax;
+  const int nT = (P + kTile - 1) / kTile;
+  wait_for_prior_grid();
+  if (2 * u >= nT + (nT & 1)) return;                  // the whole cluster
+  const int n0 = nT - u, n = u != nT - 1 - u ? nT + 1 : n0;
+  const int s0 = rank * n / C, s1 = (rank + 1) * n / C;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ty = (warp & 1) * 4 + (lane >> 3), tx = (warp >> 1) * 8 + (lane & 7);
+  logits += blockIdx.y * triangle_tiles(Pmax) * (kTile * kTile / 4) + threadIdx.x;
+  lse += (size_t)bh * Pmax;
+#pragma unroll 1
+  for (int part = 0; part < 2; ++part) {
+    const int col = part == 0 ? u : nT - 1 - u, from = part == 0 ? 0 : n0;            // column tile
+    const int i0 = max(s0, from) - from, i1 = min(s1, part == 0 ? n0 : n) - from;     // its row tiles of this CTA, from the diagonal on
+    double acc[kStripB] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int i = i0; i < i1; ++i) {
+      const int at = col + i;
+      const float4* t = logits + ((size_t)at * (at + 1) / 2 + col) * (kTile * kTile / 4);
+      float4 x[kStripA];
+      float l[kStripA];
+#pragma unroll
+      for (int r = 0; r < kStripA; ++r) x[r] = t[r * kStatThreads];
+#pragma unroll
+      for (int r = 0; r < kStripA; ++r) { const int row = at * kTile + ty + 8 * r; l[r] = row < P ? -(lse[row] * kLog2e) : -INFINITY; }
+#pragma unroll
+      for (int q = 0; q < kStripA; q += 4) {
+        float p[4][kStripB];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float d[kStripB] = {x[q + r].x, x[q + r].y, x[q + r].z, x[q + r].w};
+#pragma unroll
+          for (int c = 0; c < kStripB; ++c) {
+            const float e = exp2_ftz(fmaf(d[c], mul, l[q + r]));
+            p[r][c] = i == 0 && tx + 16 * c > ty + 8 * (q + r) ? 0.f : e;             // the tile on the diagonal
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < kStripB; ++c) acc[c] += (double)((p[0][c] + p[1][c]) + (p[2][c] + p[3][c]));
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < kStripB; ++c) {                // the four row groups of a warp, then the two warps
+      acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 8);
+      acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 16);
+      if (lane < 8) res[part][warp & 1][tx + 16 * c] = acc[c];
+    }
+  }
+  cluster.sync();
+  const int share = 2 * kTile / C;                     // results this CTA writes
+  for (int i = threadIdx.x; i < share; i += kStatThreads) {
+    const int e = rank * share + i, part = e / kTile, col = (part == 0 ? u : nT - 1 - u) * kTile + e % kTile;
+    double t = 0.0;
+    for (int c = 0; c < 2 * C; ++c) t += cluster.map_shared_rank(&res[0][0][0], c >> 1)[(part * 2 + (c & 1)) * kTile + e % kTile];
+    if (col < P && (part == 0 || n > n0)) out[(size_t)bh * Pmax + col] = (float)t;
+  }
+  cluster.sync();                                      // no CTA ends while another reads its results
+}
+
+// Bytes of logits that one of `lanes` lanes keeps: whole heads, for all lanes at most kStoredLogits; 0 where one head's
+// triangle is larger.  Fewer heads at a time mean more launches with a start and an end each, which weighs more than keeping
+// the logits in L2: 32 heads of 1999 tokens, one lane, 517 us with 32 MB, 437 with 64, 367 with 256.
+constexpr size_t kStoredLogits = (size_t)256 << 20;
+static size_t stored_head_bytes(int P) { return triangle_tiles(P) * kTile * kTile * sizeof(float); }
+size_t stored_logits_bytes(int heads, int P, int lanes) {
+  return std::min<size_t>(heads, kStoredLogits / lanes / stored_head_bytes(P)) * stored_head_bytes(P);
+}
+
+static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, float* colsum, int P, int D, int head0, int n_heads, int Hq,
+                                        const int32_t* plen, cudaStream_t st) {
+  const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
+  int C = 1;
+  while (C < 8 && 2 * C <= nT + 1 && (long long)pairs * n_heads * C < 4 * 148) C *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(pairs * C), (unsigned)n_heads); cfg.blockDim = dim3(kStatThreads); cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, colsum_stored_kernel, logits, lse, colsum, P, Hq, plen, head0, logit_scale(D));
 }
 
 // One sweep over all heads.  CTAs per cluster: enough to give every SM its CTAs (three fit), and more while every CTA
@@ -243,7 +356,7 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
 // tiles per CTA, where the copies that start a strip weigh as much, 4.20 with eight).
 template <typename T, int D, bool kSum>
 static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, float* out, int P, int n_heads, int Hq, int group,
-                                const int32_t* plen, cudaStream_t st, bool overlap) {
+                                const int32_t* plen, cudaStream_t st, bool overlap, int head0 = 0, float4* logits = nullptr) {
   const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
   const long long units = (long long)pairs * n_heads;
   int C = 1;
@@ -262,7 +375,7 @@ static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, flo
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = overlap ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, sweep_kernel<T, D, kSum>, Q, K, lse_in, out, P, Hq, group, plen);
+  return cudaLaunchKernelEx(&cfg, sweep_kernel<T, D, kSum>, Q, K, lse_in, out, P, Hq, group, plen, head0, logits);
 }
 
 __global__ void density_kernel(const float* colsum, double* __restrict__ density, int Pmax, int Hq, int L, int layer0,
@@ -273,15 +386,30 @@ constexpr int kDensityThreads = 512;
 // tail of the one before it: only what this call wrote is waited for inside the kernels.
 template <typename T, int D>
 static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float* lse_buf, float* colsum, double* density, int P,
-                                 int B, int Hq, int group, int L, int layer, const int32_t* plen, cudaStream_t st) {
+                                 int B, int Hq, int group, int L, int layer, const int32_t* plen, cudaStream_t st, float4* logits,
+                                 size_t logits_bytes) {
   const bool own = lse == nullptr;
-  if (own) {
-    cudaError_t e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, B * Hq, Hq, group, plen, st, false);
+  const int heads = B * Hq;
+  cudaError_t e;
+  if (own && logits) {
+    // as many heads at a time as leave their logits behind, in groups of about the same size
+    const int fit = (int)(logits_bytes / stored_head_bytes(P)), groups = (heads + fit - 1) / fit;
+    for (int i = 0; i < groups; ++i) {
+      const int h0 = (int)((long long)heads * i / groups), n = (int)((long long)heads * (i + 1) / groups) - h0;
+      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, n, Hq, group, plen, st, false, h0, logits);
+      if (e != cudaSuccess) return e;
+      e = launch_colsum_stored(logits, lse_buf, colsum, P, D, h0, n, Hq, plen, st);
+      if (e != cudaSuccess) return e;
+    }
+  } else {
+    if (own) {
+      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, heads, Hq, group, plen, st, false);
+      if (e != cudaSuccess) return e;
+      lse = lse_buf;
+    }
+    e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, heads, Hq, group, plen, st, own);
     if (e != cudaSuccess) return e;
-    lse = lse_buf;
   }
-  cudaError_t e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, B * Hq, Hq, group, plen, st, own);
-  if (e != cudaSuccess) return e;
   return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, L, layer, plen,
                        (uint32_t*)nullptr);
 }
@@ -574,7 +702,9 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
   double* density = (double*)(c->state + c->lay.density);
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
   return launch_sweeps<T, D>((const T*)Q, (const T*)K, lse_in, (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride),
-                             colsum, density, P, B, Hq, c->group, g.n_layers, layer, plen, st);
+                             colsum, density, P, B, Hq, c->group, g.n_layers, layer, plen, st,
+                             c->slay.logits_stride ? (float4*)(c->scratch + c->slay.logits + (size_t)lane * c->slay.logits_stride) : nullptr,
+                             c->slay.logits_stride);
 }
 
 cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
@@ -644,7 +774,7 @@ static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, flo
     return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, 1, 0,
                          nullptr, sched);
   }
-  return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st);
+  return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st, nullptr, 0);
 }
 
 }  // namespace d2o
