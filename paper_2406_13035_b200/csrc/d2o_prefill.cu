@@ -30,7 +30,6 @@ __device__ __forceinline__ T* of_layer(T* p, size_t stride, int z) {
 }
 
 // ------------------------------------------------------------------------------------ select
-constexpr int kSelThreads = 1024;
 constexpr int kSelItems = 4;            // consecutive positions per thread in the compaction
 
 struct SelectArgs {
@@ -78,7 +77,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
 // One CTA per slice.  A chain of block-wide steps: what costs is the number of barriers and the serial pieces between
 // them (32 slices of 1200 tokens: 28 us when one thread walked through the 256 bins of every radix round and the
 // compaction scanned twice per 1024 positions).
-__global__ void __launch_bounds__(kSelThreads)
+__global__ void __launch_bounds__(1024)
 select_kernel(SelectArgs a) {
   start_dependents();
   wait_for_prior_grid();
@@ -147,10 +146,10 @@ select_kernel(SelectArgs a) {
     kth = prefix; need_eq = need;                 // keep all keys > kth and the first need_eq keys == kth
   }
   __syncthreads();
-  // Ordered compaction over positions, 4096 at a time.  One scan carries two counts: positions kept for certain (low half)
+  // Ordered compaction over positions, four per thread at a time.  One scan carries two counts: positions kept for certain (low half)
   // and positions equal to the N-th score (high half), of which the first need_eq are kept.
   int n_ret = 0, n_eq = 0;                        // before the current block: kept for certain, equal
-  for (int base = 0; base < P; base += kSelItems * kSelThreads) {
+  for (int base = 0; base < P; base += kSelItems * (int)blockDim.x) {
     const int j0 = base + threadIdx.x * kSelItems;
     int sure = 0, eq = 0;                         // bit i: position j0 + i
 #pragma unroll
@@ -386,7 +385,7 @@ __global__ void __launch_bounds__(1024)
 segment_kernel(SegArgs a) {
   start_dependents();
   wait_for_prior_grid();
-  extern __shared__ __align__(16) int seg_smem[];       // [max(S + 1, 32 * 64)] counts / cursors, then radix histograms
+  extern __shared__ __align__(16) int seg_smem[];       // [max(S + 1, 64 per warp)] counts / cursors, then radix histograms
   __shared__ double part[32];
   __shared__ float s_thr;
   __shared__ int warp_tot[32];
@@ -406,15 +405,18 @@ segment_kernel(SegArgs a) {
     if (threadIdx.x == 0) a.tau[sidx] = 0.f;
     return;
   }
-  // tau_0 = (1/Le) sum_i mx_i   (Eq. 10, t = 0); fixed reduction tree, double accumulation
-  double t = 0.0;
-  for (int i = threadIdx.x; i < Le; i += blockDim.x) t += (double)mx[i];
-  t = warp_sum(t);
-  if (lane == 0) part[warp] = t;
+  // tau_0 = (1/Le) sum_i mx_i   (Eq. 10, t = 0); double accumulation, one reduction tree (that of 1024 threads) whatever the
+  // number of threads
+  for (int v = threadIdx.x; v < 1024; v += blockDim.x) {
+    double t = 0.0;
+    for (int i = v; i < Le; i += 1024) t += (double)mx[i];
+    t = warp_sum(t);
+    if (lane == 0) part[v >> 5] = t;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
+    for (int w = 0; w < 32; ++w) s += part[w];
     const float tau0 = (float)(s / (double)Le);
     a.tau[sidx] = tau0;
     s_thr = isnan(a.tau_override) ? tau0 : a.tau_override;
@@ -619,6 +621,16 @@ merge_kernel(MergeArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__
 }
 
 // ------------------------------------------------------------------------------------ launcher
+// Threads of a CTA of select_kernel and segment_kernel, which take one slice each.  A CTA is a chain of block-wide steps: with
+// no more slices than SMs as many threads as there are shorten it; with more slices, smaller CTAs of which several fit an SM
+// do not wait for a place (select_kernel: one CTA of 1024 threads per SM, four of 256).  us, with 1024 threads / so: 32 layers of
+// 32 slices of 1200 tokens, the prompt stage as a whole 1230 / 1185; four layers of 128 slices of 8192 tokens, compression 1783 /
+// 1766 and, on another GPU, 1785 / 1717 (256 threads: 1877); but 64 slices of 3000 tokens 146 / 155 with 512 threads, so few
+// slices keep 1024.
+static int slice_threads(const d2o_ctx* c, int n_ctas, int rows) {
+  return n_ctas <= c->n_sms ? 1024 : rows <= 2048 ? 256 : rows <= 16384 ? 512 : 1024;
+}
+
 // Layers [layer, layer + n) in one launch per kernel; their working arrays are the first n sets of `scratch`.
 template <typename T, int D>
 static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* const* K, const void* const* V, cudaStream_t st) {
@@ -666,7 +678,7 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   if (e != cudaSuccess) return e;
   // Six kernels of a few microseconds each for a small batch: each may move in while the one ahead drains (one layer of 32
   // slices of 777 tokens 53 -> 42 us, 32 layers of 1200 tokens 1269 -> 1250 with the column sums; large batches as before).
-  e = launch_behind(select_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), kSelThreads, sel_sm, st, sa);
+  e = launch_behind(select_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), slice_threads(c, n_slices * n, P), sel_sm, st, sa);
   if (e != cudaSuccess) return e;
   {
     const int keep_max = min(maxS, P);
@@ -703,12 +715,13 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   ga.plen = sa.plen; ga.stride = sa.stride;
   ga.L = L; ga.layer0 = layer; ga.B = B; ga.Hkv = Hkv; ga.P = P; ga.seg_stride = seg_stride;
   ga.tau_override = g.tau_override;
-  // counts / cursors per retained slot, later the radix histograms (32 warps x 64 digits)
-  const size_t seg_sm = (size_t)max(maxS + 1, 32 * 64) * sizeof(int);
+  // counts / cursors per retained slot, later the radix histograms (64 digits per warp)
+  const int seg_threads = slice_threads(c, n_slices * n, maxLe);
+  const size_t seg_sm = (size_t)max(maxS + 1, seg_threads / 32 * 64) * sizeof(int);
   e = cudaFuncSetAttribute(segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(seg_sm > 48 * 1024 ? seg_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  e = launch_behind(segment_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), 1024, seg_sm, st, ga);
+  e = launch_behind(segment_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), seg_threads, seg_sm, st, ga);
   if (e != cudaSuccess) return e;
 
   MergeArgs mg;

@@ -86,6 +86,14 @@ def test_fp32_config_0_shape():
     _run(wl, [(0, 6)])
 
 
+@pytest.mark.parametrize("dtype,P,rho", [("f32", 41, 0.7), ("f16", 300, 0.2), ("bf16", 1029, 0.3), ("f16", 2048, 0.1), ("bf16", 2300, 0.05)])
+def test_more_slices_than_sms(dtype, P, rho):
+    """160 slices per launch, selected and sorted by smaller CTAs than a layer's sixteen."""
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=20, batch=2, dtype=dtype, prompt_len=P, rho=rho, decode_steps=2,
+                             density_temp=50.0, min_budget=8, max_budget=0)
+    _run(wl, [(0, 20)], steps=2)
+
+
 @pytest.mark.parametrize("name", ["cfg0", "cfg1", "cfg2"])
 def test_layer_stats_of_several_layers_in_one_call(name):
     """d2o_layer_stats_layers against layer-by-layer calls: column sums, densities and budgets bit for bit."""
