@@ -93,7 +93,7 @@ __device__ __forceinline__ unsigned long long keys_extreme(const unsigned long l
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(kSplitThreads, G <= 4 ? 2 : 1)
 decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                    const T* __restrict__ q_in, const T* __restrict__ k_in, const T* __restrict__ v_in, T* __restrict__ out,
+                    const T* q_in, const T* k_in, const T* v_in, T* __restrict__ out,
                     T* __restrict__ kpool, T* __restrict__ vpool) {
   constexpr bool kTensor = tensor_path((int)sizeof(T), G);      // both passes and the cosines on mma.sync
   constexpr int EPV = Elem<T>::kPerVec;
@@ -341,6 +341,8 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   push_key(best, best_li, false, false);
   // ---- from here on the inputs: the grid ahead on the stream must be done (unless the call promised them complete)
   if (a.early && !a.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // an anomaly of the grids ahead that was recorded while this one waited: looked at again below, beside the key pass
+  const uint32_t word = tid == 0 ? *reinterpret_cast<volatile uint32_t*>(a.status) : 0u;
   const float qscale = (D == 64 ? 0.125f : 0.08838834764831845f) * kLog2e;   // log2(e)/sqrt(d)
   float qf[kTensor ? 1 : G][EPV];
   uint4 qb[D / 32];                                                       // tensor path: this lane's pieces of query gid
@@ -457,6 +459,8 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
       for (int g = 0; g < G; ++g) { to->m[my_entry][g] = mw[g]; to->l[my_entry][g] = lw[g]; }
     }
   }
+  if (word != 0u && s_timeout == 0) s_timeout = 1;
+  __syncwarp();
   if (lane < C) cluster.map_shared_rank(&xch, lane)->bad1[my_entry] = s_timeout;
   cluster_arrive();                                                       // barrier 1
   if (warp == 0 || own_new) {

@@ -40,7 +40,7 @@ __host__ __device__ constexpr int full_ctas(int G) { return G <= 4 ? 2 : 1; }
 
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(kFullThreads, full_ctas(G))
-full_decode_kernel(FullArgs a, const T* __restrict__ q_in, const T* __restrict__ k_in, const T* __restrict__ v_in,
+full_decode_kernel(FullArgs a, const T* q_in, const T* k_in, const T* v_in,      // the grid ahead may still be writing them: see wait_for_prior_grid
                    T* __restrict__ out, T* __restrict__ kcache, T* __restrict__ vcache) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;                  // lanes that share one row (16-byte segment each)

@@ -75,6 +75,62 @@ def test_first_steps_behind_a_compression(cuda_device, mode, L, hq, hkv, P, d, d
                     assert torch.equal(a[key].view(torch.uint8), b[key].view(torch.uint8)), key
 
 
+@pytest.mark.parametrize("hq,hkv,P,d,dtype,rho", [
+    (32, 8, 700, 128, "bf16", 0.3), (32, 8, 2000, 128, "bf16", 0.4), (16, 16, 300, 128, "f16", 0.5), (8, 8, 400, 64, "f32", 0.4)])
+def test_outputs_of_a_layer_are_the_queries_of_the_next(cuda_device, hq, hkv, P, d, dtype, rho):
+    """The inputs of a step are still being written when its kernel starts: they are read behind the wait."""
+    L, td = 12, B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    Q, K, V, q, k, v = _prompt(5, L, hq, hkv, P, d, td, cuda_device)
+
+    def run(synced):
+        ctx = B.D2OContext(B.make_config(n_layers=L, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=P,
+                                         max_new_tokens=8, rho=rho, n_sink=1, window=8, min_budget=16, density_temp=1e30))
+        ctx.d2o_layer_stats_layers(0, L, list(Q), list(K))
+        ctx.d2o_layer_budgets()
+        ctx.d2o_prefill_compress_layers(0, L, list(K), list(V))
+        out = torch.zeros(STEPS, L, 1, hq, d, dtype=td, device=cuda_device)
+        for s in range(STEPS):
+            for l in range(L):
+                ctx.d2o_decode_step(l, l + 1, q[s, 0] if l == 0 else out[s, l - 1], k[s, l], v[s, l], out[s, l])
+                if synced:
+                    torch.cuda.synchronize()
+        assert ctx.d2o_get_stats().error_word == 0
+        ctx.close()
+        return out
+
+    want = run(True)
+    for _ in range(5):
+        assert torch.equal(want.view(torch.uint8), run(False).view(torch.uint8))
+
+
+@pytest.mark.parametrize("n,G,P,d,dtype", [(8, 4, 900, 128, "bf16"), (64, 1, 500, 128, "f16"), (5, 2, 70, 64, "f32")])
+def test_uncompressed_outputs_are_the_next_queries(cuda_device, n, G, P, d, dtype):
+    L, td = 12, B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    kc, vc = (torch.randn(L, n, P + 2, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    q = torch.randn(n, G, d, generator=g, device=cuda_device).to(td)
+    k, v = (torch.randn(L, n, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+
+    def run(synced):
+        kk, vv = kc.clone(), vc.clone()
+        out = torch.zeros(L, n, G, d, dtype=td, device=cuda_device)
+        torch.cuda.synchronize()
+        for l in range(L):
+            B.d2o_full_decode_step(kk[l], vv[l], P, q if l == 0 else out[l - 1], k[l], v[l], out[l])
+            if synced:
+                torch.cuda.synchronize()
+        # the second token reads the row that the first one has just appended
+        for l in range(L):
+            B.d2o_full_decode_step(kk[l], vv[l], P + 1, out[l - 1], k[l], v[l], out[l])
+            if synced:
+                torch.cuda.synchronize()
+        return out, kk, vv
+
+    want = run(True)
+    for _ in range(5):
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(want, run(False)))
+
+
 @pytest.mark.parametrize("L,B_,hkv,P", [(4, 1, 8, 512), (32, 16, 32, 1024)])
 def test_budgets_are_complete_on_return(cuda_device, L, B_, hkv, P):
     """d2o_layer_budgets synchronises its stream: what it uploads for the calls behind it is there for calls on any stream.

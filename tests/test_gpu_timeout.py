@@ -112,6 +112,45 @@ def test_decode_cluster_whose_values_do_not_arrive(cuda_device, P, rho, hq, hkv,
     ctx.close()
 
 
+@pytest.mark.parametrize("P,rho,hq,hkv,d,dtype", [(400, 0.5, 8, 8, 64, "f32"), (640, 0.505, 8, 2, 128, "bf16")])
+def test_layers_behind_one_that_ran_out_of_time(cuda_device, P, rho, hq, hkv, d, dtype):
+    """The next layers' clusters are already resident when a layer's wait runs out; they too do nothing."""
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=3, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype,
+                             prompt_len=P, rho=rho, decode_steps=8, min_budget=8, max_budget=0)
+    ctx = make_ctx(wl)
+    streams = [W.LayerStream(wl, l, "cuda:0") for l in range(3)]
+    kv = []
+    for l, s in enumerate(streams):
+        Q, K, V = s.prompt()
+        ctx.d2o_layer_stats(l, Q, K)
+        kv.append((K, V))
+    ctx.d2o_layer_budgets()
+    for l in range(3):
+        ctx.d2o_prefill_compress(l, *kv[l])
+    first = [s.decode() for s in streams]
+    second = [s.decode() for s in streams]
+    out = [torch.zeros_like(q) for q, _, _ in first]
+    for l in range(3):
+        ctx.d2o_decode_step(l, l + 1, *first[l], out[l])
+    torch.cuda.synchronize()
+    assert ctx.d2o_get_stats().error_word == 0
+
+    def state():
+        tabs = ctx.tables()
+        return [ctx.slice_state(l, 0, h, tabs) for l in range(3) for h in range(hkv)]
+
+    before, first_out = state(), [o.clone() for o in out]
+    ctx.d2o_set_fault_injection(wait_limit_us=2000, producer_stop_stage=1)
+    ctx.d2o_decode_step(0, 1, *second[0], out[0])
+    ctx.d2o_set_fault_injection(0, -1)
+    for l in (1, 2):
+        ctx.d2o_decode_step(l, l + 1, *second[l], out[l])
+    torch.cuda.synchronize()
+    assert ctx.d2o_get_stats().error_word == D2O_ERR_TIMEOUT
+    assert _same(before, state()) and all(torch.equal(a, b) for a, b in zip(first_out, out))
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f16", 64)])
 @pytest.mark.parametrize("P,hq,stage", [(1025, 2, 0), (1025, 2, 1), (1025, 2, 3), (700, 64, 5), (2000, 40, 9)])
 def test_column_sums_whose_tiles_do_not_arrive(cuda_device, dtype, d, P, hq, stage):
