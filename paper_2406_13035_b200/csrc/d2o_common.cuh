@@ -209,6 +209,9 @@ struct d2o_ctx {
   uint8_t* layer_compressed;   // [L]
   int32_t* layer_steps;        // [L] decode steps taken
   uint8_t* layer_published;    // [L] the slices' step counters of the last decode step were (or will be) written
+  // the last decode call, and whether it left its slices' step counters to the next one (launch_decode)
+  mutable struct { int l0, l1, step; cudaStream_t stream; bool deferred; } last_decode;
+  cudaStream_t* layer_stream;  // [L] the stream of the call that writes the layer's step counters
   int32_t* h_plen;             // [B] prompt length of every sequence (prompt_len unless d2o_set_prompt_lens was called)
   int32_t* h_sim_count;        // [L] work items of the tensor-core similarity kernel per layer
   int32_t* h_sim_off;          // [L] first item of the layer in the work list

@@ -1151,16 +1151,26 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows, sum_rows * Hkv);
     if (C > 0) {
       bool published = true;                                          // the last step of every layer of the call
-      for (int l = l0; l < l1; ++l) published = published && c->layer_published[l];
+      for (int l = l0; l < l1; ++l) published = published && c->layer_published[l] && c->layer_stream[l] == st;
       a.early = published ? 1 : 0;
-      a.publish = 1;
+      // behind a call on other layers of the same stream: that call's counters, if it left them, and not this one's own
+      auto& last = c->last_decode;
+      const bool other = last.l1 > last.l0 && last.stream == st && (l1 <= last.l0 || l0 >= last.l1);
+      const bool theirs = other && last.deferred && !chained;
+      if (theirs) { a.pub_first = last.l0 * B * Hkv; a.pub_count = (last.l1 - last.l0) * B * Hkv; a.pub_step = last.step + 1; }
+      a.publish = publish || !other ? 1 : 0;
       c->decode_launches += 1;
       const cudaError_t e = launch_decode_split(c, a, C, n_pairs * Hkv, max_rows, q, k, v, out, kpool, vpool, st);
-      if (e == cudaSuccess) memset(c->layer_published + l0, 1, l1 - l0);
+      memset(c->layer_published + l0, e == cudaSuccess && a.publish, l1 - l0);
+      if (e == cudaSuccess && theirs) memset(c->layer_published + last.l0, 1, last.l1 - last.l0);
+      last = {l0, l1, a.step, st, e == cudaSuccess && !a.publish};
+      for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
       return e;
     }
   }
   memset(c->layer_published + l0, 0, l1 - l0);                          // set again below once the launch has succeeded
+  c->last_decode = {l0, l1, a.step, st, false};
+  for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
   auto launched = [&](cudaError_t e) {
     if (publish && e == cudaSuccess && *why == D2O_OK) memset(c->layer_published + l0, 1, l1 - l0);
     return e;

@@ -41,7 +41,9 @@ struct DecodeArgs {
   int early;                        // decode_split_kernel: 1: the slice may be read (once slice_ready) before the grid ahead is done.
                                     // Only behind a step that published the counter: a compression's grids may still be writing
                                     // the slice, and until they are done the counter may be an earlier conversation's
-  int publish;                      // 1: a chained step follows: the CTA publishes the slice's step counter at its end
+  int publish;                      // 1: the CTA (cluster) publishes the slice's step counter at its end: a chained step follows, or
+                                    // (decode_split_kernel) the next call is likely to work on the same layers
+  int pub_first, pub_count, pub_step;   // decode_split_kernel: slices of the call before whose counters this grid writes, and their value
 };
 
 // d2o_decode_split.cu

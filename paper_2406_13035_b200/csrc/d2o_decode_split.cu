@@ -12,10 +12,9 @@
 //   ----- up to here only the slice's state is read, nothing of the step's inputs -----
 //   keys     logits of the G heads; maximum and sum per head                    -> barrier 1 (softmax normaliser)
 //   values   un-normalised outputs, between arriving at barrier 1 and waiting for it
-//   scores   AttnScore += probabilities (Eq. 6); victim (Eq. 7-8)               -> barrier 2 (victim, failures)
+//   scores   AttnScore += probabilities (Eq. 6); victim (Eq. 7-8); partial outputs -> barrier 2 (victim, outputs, failures)
 //            a wrong guess: cosines of the true victim, one more barrier
-//   merge    tau_t, merge or discard, the new token's row (Eq. 10-12), by the CTA that holds the neighbour; outputs
-//                                                                               -> barrier 3, outputs, step counter
+//   outputs, merge: tau_t, merge or discard, the new token's row (Eq. 10-12), by the CTA that holds the neighbour
 //
 // The kernel is bound by this chain of latencies, not by bandwidth or arithmetic, so a warp works alone wherever it can:
 // it owns every eighth tile of 16 rows from the logits to the cosines and writes its own entries (maximum and sum, best
@@ -29,8 +28,16 @@
 // the queries may be.  The first step after a compression waits for the grids ahead before it reads anything: the counter
 // says nothing about the prompt stage, whose last kernels may still be at work.
 //
+// Who writes the step counter.  A step that tells by itself that a slice is complete has to collect the stores of the whole
+// cluster first: one more cluster barrier and a release, 1.5 us of every call.  Where calls alternate between layers the next
+// call does it instead: behind its wait for the grid ahead that grid's stores are all visible, and a warp of its last CTA writes
+// the counters (DecodeArgs::pub_first).  A chained step, and one that follows a step on the same layers, writes its own.
+// Calls layer by layer, us a call, with the barrier / so: 32 layers of 8 slices of 1640 bf16 rows, four heads, 11.5 / 10.7; 24 layers of
+// 32 fp16 slices of 450 rows, one head, 10.2 / 9.5; 5 layers of 24 fp32 slices of 180 rows 7.8 / 7.0.  (A release by every rank in
+// the place of the barrier: 11.4 and 9.9.)
+//
 // A CTA writes into another's shared memory only before it arrives at a barrier that the other waits for before it ends (on the
-// way out after a wait that ran out there is a barrier for that), and reads from another's only before the last barrier.
+// way out after a wait that ran out there is a barrier for that), and reads from another's only before such a barrier.
 // Nothing of the slice is written before barrier 2 has shown that no CTA's wait ran out.
 #include <cooperative_groups.h>
 #include <math.h>
@@ -119,6 +126,15 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   const int sidx = (layer * a.B + b) * a.Hkv + h;
   const T* k_new = k_in + (size_t)sl * D;
   const T* v_new = v_in + (size_t)sl * D;
+  // The inputs may still be on their way from the grid ahead and are not read before it is done, but their lines can be in L2 by
+  // then.
+  if (a.early) {
+    constexpr int kQ = G * D * (int)sizeof(T) / 128, kR = D * (int)sizeof(T) / 128;            // lines of the queries, of a row
+    const char* line = tid < kQ ? reinterpret_cast<const char*>(q_in + (size_t)sl * G * D) + tid * 128
+                     : tid < kQ + kR ? reinterpret_cast<const char*>(k_new) + (tid - kQ) * 128
+                                     : reinterpret_cast<const char*>(v_new) + (tid - kQ - kR) * 128;
+    if (tid < kQ + 2 * kR) asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+  }
 
   // ---- shared memory.  Keys and values lie as the copies bring them: on the tensor path in pieces of [half][32 rows][128 B]
   // with the 128-byte swizzle (16-byte segment c of row r at c ^ (r & 7)), else rows one after another.
@@ -343,6 +359,11 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   if (a.early && !a.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
   // an anomaly of the grids ahead that was recorded while this one waited: looked at again below, beside the key pass
   const uint32_t word = tid == 0 ? *reinterpret_cast<volatile uint32_t*>(a.status) : 0u;
+  if (a.pub_count > 0 && warp == kSplitWarps - 1 && blockIdx.x == gridDim.x - 1) {
+    // the slices of the call before: its grid is done
+    for (int i = lane; i < a.pub_count; i += 32)
+      asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + a.pub_first + i), "r"(a.pub_step) : "memory");
+  }
   const float qscale = (D == 64 ? 0.125f : 0.08838834764831845f) * kLog2e;   // log2(e)/sqrt(d)
   float qf[kTensor ? 1 : G][EPV];
   uint4 qb[D / 32];                                                       // tensor path: this lane's pieces of query gid
@@ -645,20 +666,24 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
     const float ns = __shfl_sync(0xffffffffu, (tl >> 1) == 0 ? sc[0] : sc[R - 1], (tl & 1) * 16 + (new_li & 15));
     if (lane < C) cluster.map_shared_rank(&xch, lane)->new_score = ns;
   }
-  cluster_arrive();                                                       // barrier 2
-  // scaled outputs, each to the rank that finishes it (read after barrier 3)
+  // scaled outputs, each to the rank that finishes it: read behind the cluster's last barrier
   const int share = G * D / C;                                            // outputs a rank finishes
+  auto send_outputs = [&]() {
 #pragma unroll
-  for (int i = 0; i < OUT; ++i) {
-    const int at = tid + i * kSplitThreads;
-    if (at < G * D) {
-      float o = 0.f;
+    for (int i = 0; i < OUT; ++i) {
+      const int at = tid + i * kSplitThreads;
+      if (at < G * D) {
+        float o = 0.f;
 #pragma unroll
-      for (int w = 0; w < kSplitWarps; ++w) o = fmaf(red[w * G * D + at], s_fac[w][at / D], o);
-      cluster.map_shared_rank(part, at / share)[rank * share + at % share] = o;
+        for (int w = 0; w < kSplitWarps; ++w) o = fmaf(red[w * G * D + at], s_fac[w][at / D], o);
+        cluster.map_shared_rank(part, at / share)[rank * share + at % share] = o;
+      }
     }
-  }
-  cluster_wait();                                                         // barrier 2
+  };
+  if (!a.publish) send_outputs();
+  cluster_arrive();                                                       // barrier 2
+  if (a.publish) send_outputs();                                          // beside the barrier: there is another one
+  cluster_wait();
   if (any_bad(xch.bad2)) { leave(0xDEC10000u); return; }                  // the values did not arrive: nothing written yet
 
   // ---- the victim and its neighbour
@@ -666,6 +691,16 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   unsigned long long nbest = 0ull;
   const unsigned long long vbest = keys_extreme<true>(xch.vkey, xch.vli, entries, &vic_li);
   const bool none = evict && vbest == ~0ull;                              // S_l < T + M: nothing may be evicted
+  // ---- this rank's share of the outputs (Eq. 3)
+  auto write_outputs = [&](int first) {
+    if (none) return;
+    for (int i = first; i < share; i += kSplitThreads) {
+      float t = 0.f;
+      for (int r = 0; r < C; ++r) t += part[r * share + i];
+      out[(size_t)sl * G * D + rank * share + i] = Elem<T>::from_float(t);
+    }
+  };
+  if (!a.publish) write_outputs(kSplitThreads - 1 - tid);                 // the first warp goes on to the merge
   if (!evict) vic_li = -1;
   if (evict && !none) {
     if (!D2O_GUARD(vic_li >= 0 && vic_li <= n_old, a.status, 0xC4EC0011u)) vic_li = n_old;
@@ -697,7 +732,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
     const int li = row_of(r);
     if ((li < old_cnt && r0 + li != vic_li) || (li == new_li && !evict)) a.score[row0 + r0 + li] = sc[r];
   }
-  cluster_arrive();                                                       // barrier 3
+  if (a.publish) cluster_arrive();                                        // barrier 3
   // ---- threshold, merge or discard (Eq. 10-12), the new token's row: by the CTA that holds the neighbour (or, while
   // the cache still fills, the new token)
   const bool writer = warp == 0 && !none && (evict ? max(nn_li, 0) : n_old) / chunk == rank;
@@ -764,21 +799,15 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   if (none && rank == 0 && tid == 0)                                      // drop the new token, keep the cache as it is
     report_error(a.status, D2O_ERR_STATE, 0xDEC00000u | (uint32_t)(sl & 0xfffff));
   hold();
-  cluster_wait();                                                         // barrier 3
-  // every other CTA's stores to the state were ordered before barrier 3, this warp's before the release
+  if (a.publish) cluster_wait();                                          // barrier 3
   if (writer) {
     asm volatile("fence.proxy.async.global;" ::: "memory");
     __syncwarp();
-    if (lane == 0) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + sidx), "r"(a.step + 1) : "memory");
+    // every other CTA's stores to the state were ordered before barrier 3, this warp's before the release
+    if (lane == 0 && a.publish)
+      asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + sidx), "r"(a.step + 1) : "memory");
   }
-  // ---- this rank's share of the outputs (Eq. 3)
-  if (!none) {
-    for (int i = tid; i < share; i += kSplitThreads) {
-      float t = 0.f;
-      for (int r = 0; r < C; ++r) t += part[r * share + i];
-      out[(size_t)sl * G * D + rank * share + i] = Elem<T>::from_float(t);
-    }
-  }
+  if (a.publish) write_outputs(tid);
 }
 
 // ------------------------------------------------------------------------------------ launch

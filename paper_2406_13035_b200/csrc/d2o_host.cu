@@ -211,6 +211,7 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
   c->layer_compressed = (uint8_t*)calloc(cfg->n_layers, 1);
   c->layer_steps = (int32_t*)calloc(cfg->n_layers, 4);
   c->layer_published = (uint8_t*)calloc(cfg->n_layers, 1);
+  c->layer_stream = (cudaStream_t*)calloc(cfg->n_layers, sizeof(cudaStream_t));
   c->h_order = (int32_t*)calloc(BL, 4);
   c->h_plen = (int32_t*)calloc(cfg->batch, 4);
   c->h_sim_count = (int32_t*)calloc(cfg->n_layers, 4);
@@ -240,7 +241,7 @@ extern "C" void d2o_destroy(d2o_ctx* c) {
     cudaEventDestroy(c->lane_fork);
   }
   free(c->h_tables); free(c->h_sim_off); free(c->h_pair_max); free(c->h_pair_sum);
-  free(c->layer_fed); free(c->layer_compressed); free(c->layer_steps); free(c->layer_published); free(c->h_order); free(c->h_plen); free(c->h_sim_count); free(c->h_sim_items);
+  free(c->layer_fed); free(c->layer_compressed); free(c->layer_steps); free(c->layer_published); free(c->layer_stream); free(c->h_order); free(c->h_plen); free(c->h_sim_count); free(c->h_sim_items);
   free(c);
 }
 
@@ -386,6 +387,7 @@ extern "C" d2o_status d2o_prefill_compress(d2o_ctx* c, int32_t layer, const void
   c->layer_compressed[layer] = 1;
   c->layer_steps[layer] = 0;
   c->layer_published[layer] = 0;                              // the first step waits for the compression's grids (DecodeArgs::early)
+  c->last_decode.l1 = c->last_decode.l0 = 0;                  // and nobody writes the counters of steps before it
   return D2O_OK;
 }
 
@@ -403,6 +405,7 @@ extern "C" d2o_status d2o_prefill_compress_layers(d2o_ctx* c, int32_t l0, int32_
     CUDA_TRY(launch_prefill_compress(c, a, b - a, K + (a - l0), V + (a - l0), st));
   }
   for (int l = l0; l < l1; ++l) { c->layer_compressed[l] = 1; c->layer_steps[l] = 0; c->layer_published[l] = 0; }
+  c->last_decode.l1 = c->last_decode.l0 = 0;
   return D2O_OK;
 }
 

@@ -103,6 +103,82 @@ def test_outputs_of_a_layer_are_the_queries_of_the_next(cuda_device, hq, hkv, P,
         assert torch.equal(want.view(torch.uint8), run(False).view(torch.uint8))
 
 
+@pytest.mark.parametrize("hq,hkv,P,d,dtype", [(32, 8, 500, 128, "bf16"), (8, 8, 300, 64, "f32")])
+def test_step_counters_in_any_order_of_calls(cuda_device, hq, hkv, P, d, dtype):
+    """Who writes a slice's step counter depends on the call behind it: other layers, the same ones, a chain of steps, another
+    stream, a new prompt."""
+    L, td = 4, B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    one = lambda *layers: [(l, l + 1) for l in layers]
+    tokens = [one(0, 1, 2, 3), one(0, 1, 2, 3), one(3, 1, 0, 2), [(0, 4)], [(0, 4)], one(1, 0, 3, 2), [(0, 2), (2, 4)], [(0, 2), (2, 4)],
+              "chain", one(2, 3, 0, 1), "side stream", one(0, 1, 2, 3), "chain", "new prompt", one(0, 1, 2, 3), one(1, 2, 3, 0)]
+    prompts = [_prompt(seed, L, hq, hkv, P, d, td, cuda_device) for seed in (7, 8)]
+    g = torch.Generator(device=cuda_device).manual_seed(9)
+    q = torch.randn(40, L, 1, hq, d, generator=g, device=cuda_device).to(td)
+    k, v = (torch.randn(40, L, 1, hkv, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+
+    def run(synced):
+        ctx = B.D2OContext(B.make_config(n_layers=L, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=P,
+                                         max_new_tokens=40, rho=0.3, n_sink=1, window=8, min_budget=16, density_temp=1e30))
+        out = torch.zeros_like(q)
+        side = torch.cuda.Stream()
+        torch.cuda.synchronize()
+
+        def wait():
+            if synced:
+                torch.cuda.synchronize()
+
+        def prompt(Q, K, V, *_):
+            ctx.d2o_layer_stats_layers(0, L, list(Q), list(K))
+            ctx.d2o_layer_budgets()
+            ctx.d2o_prefill_compress_layers(0, L, list(K), list(V))
+            wait()
+
+        def calls(t, ranges):
+            for l0, l1 in ranges:
+                ctx.d2o_decode_step(l0, l1, q[t, l0:l1], k[t, l0:l1], v[t, l0:l1], out[t, l0:l1])
+                wait()
+
+        prompt(*prompts[0])
+        t = 0
+        for token in tokens:
+            if token == "new prompt":
+                prompt(*prompts[1])
+                continue
+            if token == "chain":
+                ctx.d2o_decode_steps(0, L, 3, q[t:t + 3], k[t:t + 3], v[t:t + 3], out[t:t + 3])
+                wait()
+                t += 3
+                continue
+            if token == "side stream":
+                # layers in turn on two streams, each behind the call before
+                for i, r in enumerate(one(0, 1, 2, 3, 0, 1, 2, 3)):
+                    here, there = torch.cuda.current_stream(), side
+                    if i % 3 == 1:
+                        there.wait_stream(here)
+                        with torch.cuda.stream(there):
+                            calls(t + i // L, [r])
+                        here.wait_stream(there)
+                    else:
+                        calls(t + i // L, [r])
+                t += 2
+                continue
+            calls(t, token)
+            t += 1
+        torch.cuda.synchronize()
+        assert ctx.d2o_get_stats().error_word == 0
+        tabs = ctx.tables()
+        state = [ctx.slice_state(l, 0, h, tabs) for l in range(L) for h in range(hkv)]
+        ctx.close()
+        return out, state
+
+    want, ws = run(True)
+    for _ in range(3):
+        got, gs = run(False)
+        assert torch.equal(want.view(torch.uint8), got.view(torch.uint8))
+        for a, b in zip(ws, gs):
+            assert all(torch.equal(a[key].view(torch.uint8), b[key].view(torch.uint8)) for key in ("pos", "score", "rnorm", "K", "V"))
+
+
 @pytest.mark.parametrize("n,G,P,d,dtype", [(8, 4, 900, 128, "bf16"), (64, 1, 500, 128, "f16"), (5, 2, 70, 64, "f32")])
 def test_uncompressed_outputs_are_the_next_queries(cuda_device, n, G, P, d, dtype):
     L, td = 12, B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
