@@ -253,16 +253,19 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
 }
 
 // Column sums from the dot products that the row sweep left in `logits` (whole tiles; rows >= P: 0), one pair of
-// column tiles per cluster as above.  A thread holds the entries that it would have computed: rows ty + 8 r, columns tx + 16 c.
+// column tiles per cluster as above.  A thread holds the entries that it computed there: rows ty + 8 r, columns tx + 16 c.  The
+// sums run in the order of sweep_kernel, so that the bits are the same whoever computes them: groups of rows 16 apart in fp32
+// (r even: group ty, r odd: group ty + 8), the tiles of a CTA, and the groups as its butterfly takes them (4 apart, 2, 1).
 //
 // The row sweep is bound by its FMAs (one per element of d and logit); repeating them for the column sums took half of the call.
 // A logit costs 8 bytes of traffic instead (kStoredLogits: how many are kept at a time).  Row sweep, column sums and densities,
-// us, repeated / stored: 8 heads of 1024 tokens, d = 64, 70 / 48, of 100 tokens 24.6 / 20.5, of 450 tokens 33.5 / 24.5; 32
-// heads of 1999 tokens 540 / 367; six layers of 16 heads of 1500 tokens 893 / 569.
+// us, repeated / stored: 8 heads of 1024 tokens, d = 64, 70.5 / 50.2, of 100 tokens 24.7 / 22.6, of 450 tokens 33.3 / 26.7; 32
+// heads of 1999 tokens 539 / 371; six layers of 16 heads of 1500 tokens 893 / 576.
 __global__ void __launch_bounds__(kStatThreads)
 colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__ out, int Pmax, int Hq, const int32_t* __restrict__ plen,
                      int head0, float mul) {
-  __shared__ double res[2][2][kTile];                  // [strip of the pair][warps that share columns][column]
+  __shared__ double res[2][2][kTile];                  // [strip of the pair][groups below 8, from 8 on][column]
+  __shared__ double upper[2 * kStripB][kStatThreads / 2];           // of the warps with groups 4 to 7 and 12 to 15
   start_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
@@ -281,7 +284,7 @@ colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__
   for (int part = 0; part < 2; ++part) {
     const int col = part == 0 ? u : nT - 1 - u, from = part == 0 ? 0 : n0;            // column tile
     const int i0 = max(s0, from) - from, i1 = min(s1, part == 0 ? n0 : n) - from;     // its row tiles of this CTA, from the diagonal on
-    double acc[kStripB] = {0.0, 0.0, 0.0, 0.0};
+    double acc[2][kStripB] = {};
 #pragma unroll 1
     for (int i = i0; i < i1; ++i) {
       const int at = col + i;
@@ -293,27 +296,38 @@ colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__
 #pragma unroll
       for (int r = 0; r < kStripA; ++r) { const int row = at * kTile + ty + 8 * r; l[r] = row < P ? -(lse[row] * kLog2e) : -INFINITY; }
 #pragma unroll
-      for (int q = 0; q < kStripA; q += 4) {
+      for (int g = 0; g < 2; ++g) {
         float p[4][kStripB];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float d[kStripB] = {x[q + r].x, x[q + r].y, x[q + r].z, x[q + r].w};
+        for (int q = 0; q < 4; ++q) {
+          const int r = 2 * q + g;
+          const float d[kStripB] = {x[r].x, x[r].y, x[r].z, x[r].w};
 #pragma unroll
           for (int c = 0; c < kStripB; ++c) {
-            const float e = exp2_ftz(fmaf(d[c], mul, l[q + r]));
-            p[r][c] = i == 0 && tx + 16 * c > ty + 8 * (q + r) ? 0.f : e;             // the tile on the diagonal
+            const float e = exp2_ftz(fmaf(d[c], mul, l[r]));
+            p[q][c] = i == 0 && tx + 16 * c > ty + 8 * r ? 0.f : e;                   // the tile on the diagonal
           }
         }
 #pragma unroll
-        for (int c = 0; c < kStripB; ++c) acc[c] += (double)((p[0][c] + p[1][c]) + (p[2][c] + p[3][c]));
+        for (int c = 0; c < kStripB; ++c) acc[g][c] += (double)((p[0][c] + p[1][c]) + (p[2][c] + p[3][c]));
       }
     }
+    const int peer = (warp >> 1) * 32 + lane;
+    if (warp & 1) {
 #pragma unroll
-    for (int c = 0; c < kStripB; ++c) {                // the four row groups of a warp, then the two warps
-      acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 8);
-      acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 16);
-      if (lane < 8) res[part][warp & 1][tx + 16 * c] = acc[c];
+      for (int k = 0; k < 2 * kStripB; ++k) upper[k][peer] = acc[k / kStripB][k % kStripB];
     }
+    __syncthreads();
+    if (!(warp & 1)) {
+#pragma unroll
+      for (int k = 0; k < 2 * kStripB; ++k) {
+        double t = acc[k / kStripB][k % kStripB] + upper[k][peer];
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+        if (lane < 8) res[part][k / kStripB][tx + 16 * (k % kStripB)] = t;
+      }
+    }
+    __syncthreads();                                   // `upper` is used again
   }
   cluster.sync();
   const int share = 2 * kTile / C;                     // results this CTA writes
@@ -328,7 +342,7 @@ colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__
 
 // Bytes of logits that one of `lanes` lanes keeps: whole heads, for all lanes at most kStoredLogits; 0 where one head's
 // triangle is larger.  Fewer heads at a time mean more launches with a start and an end each, which weighs more than keeping
-// the logits in L2: 32 heads of 1999 tokens, one lane, 517 us with 32 MB, 437 with 64, 367 with 256.
+// the logits in L2: 32 heads of 1999 tokens, one lane, 517 us with 32 MB, 437 with 64, 367 with 256 (in another order of the sums).
 constexpr size_t kStoredLogits = (size_t)256 << 20;
 static size_t stored_head_bytes(int P) { return triangle_tiles(P) * kTile * kTile * sizeof(float); }
 size_t stored_logits_bytes(int heads, int P, int lanes) {
@@ -336,10 +350,8 @@ size_t stored_logits_bytes(int heads, int P, int lanes) {
 }
 
 static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, float* colsum, int P, int D, int head0, int n_heads, int Hq,
-                                        const int32_t* plen, cudaStream_t st) {
-  const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
-  int C = 1;
-  while (C < 8 && 2 * C <= nT + 1 && (long long)pairs * n_heads * C < 4 * 148) C *= 2;
+                                        const int32_t* plen, cudaStream_t st, int C) {
+  const int pairs = ((P + kTile - 1) / kTile + 1) / 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(pairs * C), (unsigned)n_heads); cfg.blockDim = dim3(kStatThreads); cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -351,16 +363,23 @@ static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, 
   return cudaLaunchKernelEx(&cfg, colsum_stored_kernel, logits, lse, colsum, P, Hq, plen, head0, logit_scale(D));
 }
 
-// One sweep over all heads.  CTAs per cluster: enough to give every SM its CTAs (three fit), and more while every CTA
+// CTAs per cluster of a sweep over `heads` heads: enough to give every SM its CTAs (three fit), and more while every CTA
 // keeps eight tiles, so that the last wave is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms with four
-// tiles per CTA, where the copies that start a strip weigh as much, 4.20 with eight).
-template <typename T, int D, bool kSum>
-static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, float* out, int P, int n_heads, int Hq, int group,
-                                const int32_t* plen, cudaStream_t st, bool overlap, int head0 = 0, float4* logits = nullptr) {
+// tiles per CTA, where the copies that start a strip weigh as much, 4.20 with eight).  Sums depend on it, so it is that of all
+// heads of a call also where they go in groups.
+static int sweep_ctas(int P, int heads) {
   const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
-  const long long units = (long long)pairs * n_heads;
+  const long long units = (long long)pairs * heads;
   int C = 1;
   while (C < 8 && 2 * C <= nT + 1 && (units * C < 4 * 148 || (units * C < 16 * 148 && nT + 1 >= 16 * C))) C *= 2;
+  return C;
+}
+
+// One sweep over `n_heads` heads from `head0` on.
+template <typename T, int D, bool kSum>
+static cudaError_t launch_sweep(const T* Q, const T* K, const float* lse_in, float* out, int P, int n_heads, int Hq, int group,
+                                const int32_t* plen, cudaStream_t st, bool overlap, int C, int head0 = 0, float4* logits = nullptr) {
+  const int pairs = ((P + kTile - 1) / kTile + 1) / 2;
   const size_t smem = sizeof(SweepSmem<D>);
   cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, D, kSum>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -389,25 +408,25 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
                                  int B, int Hq, int group, int L, int layer, const int32_t* plen, cudaStream_t st, float4* logits,
                                  size_t logits_bytes) {
   const bool own = lse == nullptr;
-  const int heads = B * Hq;
+  const int heads = B * Hq, C = sweep_ctas(P, heads);
   cudaError_t e;
   if (own && logits) {
     // as many heads at a time as leave their logits behind, in groups of about the same size
     const int fit = (int)(logits_bytes / stored_head_bytes(P)), groups = (heads + fit - 1) / fit;
     for (int i = 0; i < groups; ++i) {
       const int h0 = (int)((long long)heads * i / groups), n = (int)((long long)heads * (i + 1) / groups) - h0;
-      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, n, Hq, group, plen, st, false, h0, logits);
+      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, n, Hq, group, plen, st, false, C, h0, logits);
       if (e != cudaSuccess) return e;
-      e = launch_colsum_stored(logits, lse_buf, colsum, P, D, h0, n, Hq, plen, st);
+      e = launch_colsum_stored(logits, lse_buf, colsum, P, D, h0, n, Hq, plen, st, C);
       if (e != cudaSuccess) return e;
     }
   } else {
     if (own) {
-      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, heads, Hq, group, plen, st, false);
+      e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, heads, Hq, group, plen, st, false, C);
       if (e != cudaSuccess) return e;
       lse = lse_buf;
     }
-    e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, heads, Hq, group, plen, st, own);
+    e = launch_sweep<T, D, true>(Q, K, lse, colsum, P, heads, Hq, group, plen, st, own, C);
     if (e != cudaSuccess) return e;
   }
   return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, L, layer, plen,
