@@ -32,6 +32,8 @@
 
 #include <algorithm>
 
+#include <cuda/std/type_traits>
+
 #include "d2o_common.cuh"
 #include "d2o_tc.cuh"
 
@@ -208,6 +210,11 @@ struct CsItem {
     bt0 = SWEEP == kSweepRows ? 0 : a0 / kCsTile;
     n_jobs = (SWEEP == kSweepRows ? min(n_tiles, (a0 + 2 * kCsTile) / kCsTile) : n_tiles) - bt0;
   }
+  // Has A tile t any valid logit with the streamed tile of a job?  Not beyond the diagonal, nor past the prompt.
+  __device__ __forceinline__ bool valid(int t, int job) const {
+    const int at = a0 / kCsTile + t;
+    return at * kCsTile < P && (SWEEP == kSweepRows ? bt0 + job <= at : bt0 + job >= at);
+  }
   __device__ __forceinline__ int q_base(const ColsumTcArgs& a) const { return bh * a.P; }     // first row of the head in the views
   __device__ __forceinline__ int k_base(const ColsumTcArgs& a) const {
     return (bh / a.Hq * (a.Hq / a.group) + bh % a.Hq / a.group) * a.P;
@@ -340,6 +347,7 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
         tc::fence_after_sync();
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
+          if (!it.valid(t, job)) continue;
           const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256 + t * kCsTile);
 #pragma unroll
           for (int kb = 0; kb < KB; ++kb) {
@@ -366,7 +374,6 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
     const int at = part >> 1, bhalf = part & 1;
     CsItem<SWEEP> it;
     int jb = 0;
-    uint32_t ra[32], rb[32];
     // One thread looks at the next item, for all, ahead of the barrier that ends the one before: warps that waited for it each
     // by itself could run out of time apart, and those that stayed would wait at the barrier for good.
     auto end_item = [&](int k) {
@@ -393,41 +400,61 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
       const int brow0 = (it.bt0 + job) * kCsTile + bhalf * 64;   // position of the first B row this warp looks at
       if (!__all_sync(0xffffffffu, wait(&tm_full[buf], (uint32_t)((jb >> 1) & 1)))) { s_fail = 1; break; }
       tc::fence_after_sync();
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + at * kCsTile + bhalf * 64);
-      tc::tmem_ld32_issue(taddr, ra);
-      tc::tmem_ld32_issue(taddr + 32u, rb);
-      tc::tmem_ld_wait(ra);
-      tc::tmem_ld_wait(rb);
-      // both blocks are in registers: hand the accumulator back to the MMA warp
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&tm_empty[buf]);
-      if (SWEEP == kSweepRows ? brow0 > w0 + 31 : brow0 + 63 < w0 || brow0 >= P) {
-        // nothing of this warp's block is valid (warp-uniform)
-      } else if (SWEEP == kSweepRows) {
+      // Each of the paths below loads the accumulator's block into registers of its own, and products that no path needs are
+      // not made (CsItem::valid).  us, one set for masked and unmasked paths and all products / so: 32 heads of 300 tokens
+      // 20.3 / 18.5; four layers of 2 x 16 heads of 1700 tokens, d = 64, 142.4 / 136.9; four layers of 2 x 32 heads of 600 tokens with
+      // the caller's normalisers 39.1 / 38.3; long prompts run at the power cap and take the same time (two layers of 6001
+      // tokens 714 - 726 / 716 - 719).
+      auto drained = [&]() {                                   // hand the accumulator back to the MMA warp
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&tm_empty[buf]);
+      };
+      auto load = [&](uint32_t (&ra)[32], uint32_t (&rb)[32]) {
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 256 + at * kCsTile + bhalf * 64);
+        tc::tmem_ld32_issue(taddr, ra);
+        tc::tmem_ld32_issue(taddr + 32u, rb);
+        tc::tmem_ld_wait(ra);
+        tc::tmem_ld_wait(rb);
+        drained();
+      };
+      if (SWEEP == kSweepRows) {
         // B rows are keys: valid iff key <= query (keys >= P are > every stored query)
-        if (brow0 + 63 > w0) {                                 // warp-uniform: the diagonal
-          const int last = arow - brow0;                       // the row's last valid column of the 64
+        auto rows = [&](auto diagonal) {
+          uint32_t ra[32], rb[32];
+          load(ra, rb);
+          if (decltype(diagonal)::value) {
+            const int last = arow - brow0;                     // the row's last valid column of the 64
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            if (i > last) ra[i] = 0xff800000u;
-            if (i + 32 > last) rb[i] = 0xff800000u;
+            for (int i = 0; i < 32; ++i) {
+              if (i > last) ra[i] = 0xff800000u;
+              if (i + 32 > last) rb[i] = 0xff800000u;
+            }
           }
-        }
-        // four independent chains of three-input maxima: the block maximum is on every thread's critical path
-        float bmx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+          // four independent chains of three-input maxima: the block maximum is on every thread's critical path
+          float bmx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int i = 0; i < 32; ++i) bmx[i & 3] = tc::max3(bmx[i & 3], __uint_as_float(ra[i]), __uint_as_float(rb[i]));
-        const float bm = fmaxf(fmaxf(bmx[0], bmx[1]), fmaxf(bmx[2], bmx[3])) * c;     // in the log2 domain, rounded once
-        if (bm > m_run) { l_run *= exp2f(m_run - bm); m_run = bm; }            // exp2f(-inf) = 0 on the first block
-        if (m_run > -INFINITY) l_run += exp_sum_64<false, false>(ra, rb, c, -m_run, nullptr);
+          for (int i = 0; i < 32; ++i) bmx[i & 3] = tc::max3(bmx[i & 3], __uint_as_float(ra[i]), __uint_as_float(rb[i]));
+          const float bm = fmaxf(fmaxf(bmx[0], bmx[1]), fmaxf(bmx[2], bmx[3])) * c;     // in the log2 domain, rounded once
+          if (bm > m_run) { l_run *= exp2f(m_run - bm); m_run = bm; }            // exp2f(-inf) = 0 on the first block
+          const float sum = exp_sum_64<false, false>(ra, rb, c, m_run > -INFINITY ? -m_run : 0.f, nullptr);
+          if (m_run > -INFINITY) l_run += sum;
+        };
+        if (brow0 > w0 + 31 || w0 >= P) drained();             // warp-uniform: nothing of this warp's block is valid
+        else if (brow0 + 63 > w0) rows(cuda::std::true_type{});
+        else rows(cuda::std::false_type{});
       } else {
         // B rows are queries: valid iff query >= key and query < P
         const float* ls = s_lse + s * kCsTile + bhalf * 64;
-        float part;
-        if (brow0 >= w0 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
-          part = exp_sum_64<true, SWEEP == kSweepColsGiven>(ra, rb, c, 0.f, ls);
+        if (brow0 + 63 < w0 || brow0 >= P) {                   // warp-uniform: nothing is valid
+          drained();
+        } else if (brow0 >= w0 + 31 && brow0 + 64 <= P) {      // warp-uniform: nothing is masked
+          uint32_t ra[32], rb[32];
+          load(ra, rb);
+          col_acc += (double)exp_sum_64<true, SWEEP == kSweepColsGiven>(ra, rb, c, 0.f, ls);
         } else {
+          uint32_t ra[32], rb[32];
+          load(ra, rb);
           const int first = arow - brow0, end = P - brow0;     // the row's valid columns of the 64
           float p0 = 0.f, p1 = 0.f;
 #pragma unroll
@@ -437,9 +464,8 @@ attn_tc_kernel(ColsumTcArgs a, const __grid_constant__ ColsumTcMaps maps) {
             p0 += i >= first && i < end ? x : 0.f;
             p1 += i + 32 >= first && i + 32 < end ? y : 0.f;
           }
-          part = p0 + p1;
+          col_acc += (double)(p0 + p1);
         }
-        col_acc += (double)part;
       }
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&b_empty[s]);           // this warp is done with the stage (sweep 2: its normalisers)
