@@ -28,6 +28,7 @@
 #include <stdlib.h>
 
 #include <algorithm>
+#include <cuda/std/type_traits>
 #include <utility>
 #include <vector>
 
@@ -83,61 +84,46 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-// One block of 32 accumulator columns of one row: times 1/|k_c| per column, maximum and its column (the lowest
-// on ties), merged into the row's running (best, best_col).  cl0 = chunk-local column of the block.
-__device__ __forceinline__ void scan_block(const uint32_t (&r)[32], const float* s_rn, int cl0, int n_cols, int c0,
-                                           float& best, int& best_col) {
-  const float4* rn4 = reinterpret_cast<const float4*>(s_rn + cl0);
-  if (cl0 + 32 <= n_cols) {
-    // Columns go in pairs (2i, 2i + 1): one packed multiply, one three-input maximum against the running value,
-    // one compare and two selects per pair.  The chain remembers the winning pair and that pair's first value,
-    // from which the column inside the pair follows at the end.  Two chains (pairs i mod 2) keep them short.
-    // max.f32 drops a NaN operand, as the compare of the scalar form does.
-    float pb[2] = {-INFINITY, -INFINITY}, plo[2] = {-INFINITY, -INFINITY};
-    int pi[2] = {0, 1};
+// Running maximum over the columns of a job, for one row.  Columns go in pairs (2i, 2i + 1): one packed multiply, one three-input
+// maximum against the running value, one compare and two selects per pair.  A chain remembers the winning pair and that pair's
+// first value, from which the column inside the pair follows at the end.  Two chains (pairs i mod 2) keep them short.  max.f32
+// drops a NaN operand, as a compare would.
+struct JobMax {
+  float pb[2], plo[2]; int pi[2];
+  __device__ __forceinline__ void start() {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) { pb[w] = plo[w] = -INFINITY; pi[w] = w; }
+  }
+  // Block `b` of 32 columns of the job: accumulators r times 1/|k_c| (s_rn: those of the block).  MASK: columns from `n` on hold other
+  // slices' rows.
+  template <bool MASK>
+  __device__ __forceinline__ void block(const uint32_t (&r)[32], const float* s_rn, int b, int n) {
+    const float4* rn4 = reinterpret_cast<const float4*>(s_rn);
 #pragma unroll
     for (int i4 = 0; i4 < 8; ++i4) {
       const float4 q = rn4[i4];
       const float rv[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
       for (int w = 0; w < 2; ++w) {
+        const int at = i4 * 4 + 2 * w;
         float x0, x1;
-        mul_pair(__uint_as_float(r[i4 * 4 + 2 * w]), __uint_as_float(r[i4 * 4 + 2 * w + 1]), rv[2 * w], rv[2 * w + 1], x0, x1);
+        mul_pair(__uint_as_float(r[at]), __uint_as_float(r[at + 1]), rv[2 * w], rv[2 * w + 1], x0, x1);
+        if (MASK) { x0 = at < n ? x0 : -INFINITY; x1 = at + 1 < n ? x1 : -INFINITY; }
         const float m = max3(pb[w], x0, x1);
         const bool up = m > pb[w];
-        pi[w] = up ? i4 * 2 + w : pi[w];
+        pi[w] = up ? b * 16 + i4 * 2 + w : pi[w];
         plo[w] = up ? x0 : plo[w];
         pb[w] = m;
       }
     }
-    // the later chain wins only with a larger value or an equal one from an earlier pair
+  }
+  // Merged into the row's (best, best_col); col0: the job's first column.  The later chain wins only with a larger value or an
+  // equal one from an earlier pair; equal values inside a pair go to the lower column; the first of equal jobs stays.
+  __device__ __forceinline__ void finish(int col0, float& best, int& best_col) {
     if (pb[1] > pb[0] || (pb[1] == pb[0] && pi[1] < pi[0])) { pb[0] = pb[1]; pi[0] = pi[1]; plo[0] = plo[1]; }
-    const int col = 2 * pi[0] + (plo[0] == pb[0] ? 0 : 1);        // equal values inside the pair: the lower column
-    if (pb[0] > best) { best = pb[0]; best_col = c0 + cl0 + col; }
-    return;
+    if (pb[0] > best) { best = pb[0]; best_col = col0 + 2 * pi[0] + (plo[0] == pb[0] ? 0 : 1); }
   }
-  // four interleaved running maxima (columns i mod 4) keep the compare chains short
-  float tb[4]; int ti[4];
-#pragma unroll
-  for (int w = 0; w < 4; ++w) { tb[w] = -INFINITY; ti[w] = w; }
-  {                                                               // columns past the chunk hold other slices' rows
-#pragma unroll
-    for (int i4 = 0; i4 < 8; ++i4) {
-      const float4 q = rn4[i4];
-      const float rv[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const float x = __uint_as_float(r[i4 * 4 + w]) * rv[w];
-        if (cl0 + i4 * 4 + w < n_cols && x > tb[w]) { tb[w] = x; ti[w] = i4 * 4 + w; }
-      }
-    }
-  }
-  // larger value wins, equal values go to the lower column
-#pragma unroll
-  for (int w = 1; w < 4; ++w)
-    if (tb[w] > tb[0] || (tb[w] == tb[0] && ti[w] < ti[0])) { tb[0] = tb[w]; ti[0] = ti[w]; }
-  if (tb[0] > best) { best = tb[0]; best_col = c0 + cl0 + ti[0]; }   // ascending blocks: the first maximum stays
-}
+};
 
 template <typename T, int D, int FMT>
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -173,7 +159,8 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ SimTcMaps maps) {
   if (c0 >= S || Pb - S <= 0) return;                        // uniform for the CTA: nothing to do
   const int n_cols = min(chunk_cols, S - c0);
   const int n_j = (n_cols + kJobN - 1) / kJobN;              // MMA column tiles (jobs) per prompt tile: 1 .. 3
-  const int n_last = (n_cols - (n_j - 1) * kJobN + 15) & ~15;    // columns of the last job's MMA (multiple of 16)
+  const int job_w = ((n_cols + n_j - 1) / n_j + 31) & ~31;   // columns of a job: about the same for all
+  const int n_last = (n_cols - (n_j - 1) * job_w + 15) & ~15;    // of the last one's MMA (multiple of 16)
   const int n_tiles_all = (Pb + kTileM - 1) / kTileM;
   const int t0 = item.z;
   const int t1 = min(n_tiles_all, item.w);
@@ -237,11 +224,11 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ SimTcMaps maps) {
             if (!s_fail && !tc::mbar_wait(&tm_empty[p], (uint32_t)((cnt & 1) ^ 1))) s_fail = 1;
             tc::fence_after_sync();
             const uint32_t d_tmem = tmem_base + (uint32_t)(p * kJobN);
-            const uint32_t idesc = make_idesc(FMT, kTileM, j == n_j - 1 ? (uint32_t)n_last : (uint32_t)kJobN);
+            const uint32_t idesc = make_idesc(FMT, kTileM, j == n_j - 1 ? (uint32_t)n_last : (uint32_t)job_w);
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb) {
               const uint64_t adesc = tc::smem_desc_sw128(tc::smem_u32(sA + p * A_TILE + kb * A_BLOCK));
-              const uint64_t bdesc = tc::smem_desc_sw128(tc::smem_u32(sB + kb * B_BLOCK + j * kJobN * 128));
+              const uint64_t bdesc = tc::smem_desc_sw128(tc::smem_u32(sB + kb * B_BLOCK + j * job_w * 128));
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)                     // 16 elements = 32 bytes along K per instruction
                 tc::mma_f16(d_tmem, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), idesc, (kb | kk) != 0 ? 1u : 0u);
@@ -266,7 +253,6 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ SimTcMaps maps) {
                                    ((size_t)slice * a.n_chunks_max + nc) * a.P;
     float* out_rn = reinterpret_cast<float*>(reinterpret_cast<char*>(a.prompt_rn) + a.stride * z) + (size_t)slice * a.P;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(p * kJobN);
-    uint32_t ra[32], rb[32];
     const int n_tp = p < n_t ? (n_t - p + kParts - 1) / kParts : 0;   // tiles of this part
     // every load of a job has landed in registers: hand the accumulator back to the MMA warp
     auto release = [&]() {
@@ -307,27 +293,33 @@ sim_tc_kernel(SimTcArgs a, const __grid_constant__ SimTcMaps maps) {
         const int cnt = k * n_j + j;
         if (!s_fail && !tc::mbar_wait(&tm_full[p], (uint32_t)(cnt & 1))) s_fail = 1;
         tc::fence_after_sync();
-        const int cl = j * kJobN;                              // chunk-local column of the job's first block
-        const int nb = (min(kJobN, n_cols - cl) + 31) / 32;    // 32-column blocks with retained rows: 1 .. 4
-        // loads run one block ahead of the scan
-        tc::tmem_ld32_issue(lane_base, ra);
-        tc::tmem_ld_wait(ra);
-        if (nb > 1) tc::tmem_ld32_issue(lane_base + 32u, rb); else release();
-        scan_block(ra, s_rn, cl, n_cols, c0, best, best_col);
-        if (nb > 1) {
-          tc::tmem_ld_wait(rb);
-          if (nb > 2) tc::tmem_ld32_issue(lane_base + 64u, ra); else release();
-          scan_block(rb, s_rn, cl + 32, n_cols, c0, best, best_col);
-        }
-        if (nb > 2) {
-          tc::tmem_ld_wait(ra);
-          if (nb > 3) tc::tmem_ld32_issue(lane_base + 96u, rb); else release();
-          scan_block(ra, s_rn, cl + 64, n_cols, c0, best, best_col);
-        }
-        if (nb > 3) {
-          tc::tmem_ld_wait(rb);
-          release();
-          scan_block(rb, s_rn, cl + 96, n_cols, c0, best, best_col);
+        const int cl = j * job_w;                              // chunk-local column of the job's first block
+        const int cols = min(job_w, n_cols - cl);              // its columns with retained rows: up to four blocks of 32
+        // One straight path per number of blocks, with registers of its own; loads run one block ahead of the scan.  us of
+        // compression, conditional loads into shared registers, a merge per block and jobs of 128 columns and a rest / so: three
+        // layers of 48 slices of 5000 tokens, d = 64, 293 / 278; two of 32 slices of 3000 tokens 145.7 / 142.4; 32 layers of 32 slices of
+        // 1200 tokens, the whole prompt stage, 1149 / 1135; four of 128 slices of 8192 tokens 1703 / 1704 and 1691 / 1682.
+        auto job = [&](auto blocks) {
+          constexpr int NB = decltype(blocks)::value;
+          uint32_t r[2][32];
+          JobMax mx;
+          mx.start();
+          tc::tmem_ld32_issue(lane_base, r[0]);
+          tc::tmem_ld_wait(r[0]);
+#pragma unroll
+          for (int b = 0; b < NB; ++b) {
+            if (b + 1 < NB) tc::tmem_ld32_issue(lane_base + (uint32_t)(b + 1) * 32u, r[(b + 1) & 1]); else release();
+            if (b + 1 < NB || cols == NB * 32) mx.block<false>(r[b & 1], s_rn + cl + b * 32, b, 32);
+            else mx.block<true>(r[b & 1], s_rn + cl + b * 32, b, cols - b * 32);
+            if (b + 1 < NB) tc::tmem_ld_wait(r[(b + 1) & 1]);
+          }
+          mx.finish(c0 + cl, best, best_col);
+        };
+        switch ((cols + 31) / 32) {
+          case 4: job(cuda::std::integral_constant<int, 4>()); break;
+          case 3: job(cuda::std::integral_constant<int, 3>()); break;
+          case 2: job(cuda::std::integral_constant<int, 2>()); break;
+          default: job(cuda::std::integral_constant<int, 1>()); break;
         }
       }
       // (ordered value, inverted slot): larger is better, ties go to the lower slot; -0 counts as +0
