@@ -366,15 +366,22 @@ static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, 
   return cudaLaunchKernelEx(&cfg, colsum_stored_kernel, logits, lse, colsum, P, Hq, plen, head0, logit_scale(D));
 }
 
-// CTAs per cluster of a sweep over `heads` heads: enough to give every SM its CTAs (three fit), and more while every CTA
-// keeps eight tiles, so that the last wave is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms with four
-// tiles per CTA, where the copies that start a strip weigh as much, 4.20 with eight).  Sums depend on it, so it is that of all
-// heads of a call also where they go in groups.
+// CTAs per cluster of a sweep over `heads` heads: as many as give every SM its CTAs (three fit, four leave a short second round);
+// past that only while every CTA keeps four tiles, because the copies that start a strip weigh as much as a tile or two, or
+// eight in sweeps of several rounds, so that the last one is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms
+// with four tiles per CTA, 4.20 with eight).  us, two rounds of CTAs with one or two tiles / one round: 16 heads of 700 tokens 48.3 /
+// 39.7, four layers of 32 heads of 500 tokens 183 / 139, of 16 heads of 900 tokens 199 / 174; 16 heads of 1024 tokens 72.4 / 73.4
+// (by itself 78.9 / 74.8); but 24 heads of 1000 tokens, two rounds of four tiles / one round 87.3 / 89.2.
+// Sums depend on it, so it is that of all heads of a call also where they go in groups.
 static int sweep_ctas(int P, int heads) {
+  int dev = 0, sms = 148;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) (void)cudaGetLastError();
   const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
   const long long units = (long long)pairs * heads;
   int C = 1;
-  while (C < 8 && 2 * C <= nT + 1 && (units * C < 4 * 148 || (units * C < 16 * 148 && nT + 1 >= 16 * C))) C *= 2;
+  while (C < 8 && 2 * C <= nT + 1 &&
+         (units * 2 * C <= 4 * sms || (units * C < 4 * sms && nT + 1 >= 8 * C) || (units * C < 16 * sms && nT + 1 >= 16 * C)))
+    C *= 2;
   return C;
 }
 
