@@ -100,10 +100,11 @@ sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __re
   extern __shared__ __align__(16) unsigned char sweep_smem[];
   SweepSmem<D>& sm = *reinterpret_cast<SweepSmem<D>*>(sweep_smem);
   constexpr int LDX = SweepSmem<D>::kLdX, LDY = SweepSmem<D>::kLdY, kSlabs = D / kSlab;
-  start_dependents();
   // The first kernel of a call: what is ahead of it may be writing Q and K, or reading the scratch of the call before.  Only its
-  // launch overlaps with that (8 heads of 100 tokens 22.6 -> 20.6 us a call, of 1024 tokens 49.9 -> 49.6).
+  // launch overlaps with that (8 heads of 100 tokens 22.6 -> 20.6 us a call, of 1024 tokens 49.9 -> 49.6).  The kernel behind it
+  // starts after this wait: the column sweep requests tiles of Q and K ahead of its own.
   if (!kSum) wait_for_prior_grid();
+  start_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int u = blockIdx.x / C;

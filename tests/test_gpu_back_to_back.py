@@ -224,3 +224,58 @@ def test_budgets_are_complete_on_return(cuda_device, L, B_, hkv, P):
     assert all(done)
     assert ctx.d2o_get_stats().error_word == 0
     ctx.close()
+
+
+def _appended_then_summed(cuda_device, dtype, d, n, P, sums):
+    """An uncompressed step that appends a row to a cache, and at once the column sums with that cache's keys and values as keys
+    and queries, on the same stream: the step's kernel lets the next ones start as its first act.  Bit for bit the result of the
+    calls with a synchronisation in between."""
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    g = torch.Generator(device=cuda_device).manual_seed(P + d)
+    kc, vc = (torch.randn(n, P, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    q = torch.randn(n, 1, d, generator=g, device=cuda_device).to(td)
+    k, v = (3 * torch.randn(n, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    out = torch.empty_like(q)
+
+    def run(synced):
+        kc[:, P - 1].zero_()                              # as it was before the step
+        vc[:, P - 1].zero_()
+        torch.cuda.synchronize()
+        B.d2o_full_decode_step(kc, vc, P - 1, q, k, v, out)
+        if synced:
+            torch.cuda.synchronize()
+        got = sums(vc.view(1, n, P, d), kc.view(1, n, P, d))
+        torch.cuda.synchronize()
+        return got
+
+    want = run(True)
+    for _ in range(10):
+        assert torch.equal(want, run(False))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n,P", [(2, 200), (8, 2000), (32, 2000)])
+def test_fp32_column_sums_of_a_cache_that_is_being_appended_to(cuda_device, n, P, d):
+    cs = torch.empty(1, n, P, device=cuda_device)
+    density = torch.empty(1, n, dtype=torch.float64, device=cuda_device)
+
+    def static(Q, K):
+        B.d2o_layer_stats_static(Q, K, cs, density)
+        return cs.clone()
+
+    _appended_then_summed(cuda_device, "f32", d, n, P, static)
+
+
+@pytest.mark.parametrize("dtype,d,n,P", [("f32", 64, 8, 2000), ("f32", 64, 2, 12001), ("f32", 128, 2, 12001), ("f16", 128, 8, 1000)])
+def test_column_sums_of_a_context_behind_an_appending_step(cuda_device, dtype, d, n, P):
+    """Heads with and without room for their dot products, and the CUDA-core sweeps on 16-bit inputs."""
+    ctx = B.D2OContext(B.make_config(n_layers=1, batch=1, n_q_heads=n, n_kv_heads=n, d_head=d, dtype=dtype, prompt_len=P,
+                                     max_new_tokens=1, rho=0.5, n_sink=1, min_budget=8))
+    ctx.d2o_set_tuning(stats_path=1)
+
+    def stats(Q, K):
+        ctx.d2o_layer_stats(0, Q, K)
+        return ctx.colsum(0).clone()
+
+    _appended_then_summed(cuda_device, dtype, d, n, P, stats)
+    ctx.close()
