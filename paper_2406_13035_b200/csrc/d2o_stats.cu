@@ -95,7 +95,7 @@ __host__ __device__ __forceinline__ size_t triangle_tiles(int P) { const size_t 
 // kSum: colsum_j = sum_{i >= j} exp(q_i.k_j / sqrt(d) - lse_i); else lse_i = log sum_{j <= i} exp(q_i.k_j / sqrt(d)).
 template <typename T, int D, bool kSum>
 __global__ void __launch_bounds__(kStatThreads, 3)
-sweep_kernel(const T* __restrict__ Q, const T* __restrict__ K, const float* __restrict__ lse_in, float* __restrict__ out,
+sweep_kernel(const T* Q, const T* K, const float* lse_in, float* __restrict__ out,    // inputs: see wait_for_prior_grid
              int Pmax, int Hq, int group, const int32_t* __restrict__ plen, int head0, float4* __restrict__ logits) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];
   SweepSmem<D>& sm = *reinterpret_cast<SweepSmem<D>*>(sweep_smem);

@@ -266,7 +266,8 @@ def test_fp32_column_sums_of_a_cache_that_is_being_appended_to(cuda_device, n, P
     _appended_then_summed(cuda_device, "f32", d, n, P, static)
 
 
-@pytest.mark.parametrize("dtype,d,n,P", [("f32", 64, 8, 2000), ("f32", 64, 2, 12001), ("f32", 128, 2, 12001), ("f16", 128, 8, 1000)])
+@pytest.mark.parametrize("dtype,d,n,P", [("f32", 64, 8, 2000), ("f32", 64, 2, 12001), ("f32", 128, 2, 12001), ("f16", 128, 8, 1000),
+                                          ("bf16", 64, 2, 777), ("f16", 64, 64, 300)])
 def test_column_sums_of_a_context_behind_an_appending_step(cuda_device, dtype, d, n, P):
     """Heads with and without room for their dot products, and the CUDA-core sweeps on 16-bit inputs."""
     ctx = B.D2OContext(B.make_config(n_layers=1, batch=1, n_q_heads=n, n_kv_heads=n, d_head=d, dtype=dtype, prompt_len=P,
