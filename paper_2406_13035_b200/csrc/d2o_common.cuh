@@ -242,7 +242,7 @@ namespace d2o {
 
 // launchers (one per .cu file); all return cudaError_t of the launch
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
-                               cudaStream_t st, int lane = 0);
+                               cudaStream_t st, int lane = 0, int lanes = 1);
 // the layers [layer, layer + n), n <= kColsumLayers, in one launch per kernel (16-bit inputs)
 cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
                                   const float* const* lse, cudaStream_t st);
@@ -270,7 +270,7 @@ cudaError_t launch_colsum_tc(int dtype, int D, int B, int Hq, int Hkv, int P, in
                              float* colsum, const int32_t* plen, uint32_t* status, uint32_t* sched, cudaStream_t st,
                              unsigned long long wait_ns = 0, int stop_job = -1);
 size_t colsum_tc_lse_bytes(int batch, int n_q_heads, int P);      // its row normalisers
-size_t stored_logits_bytes(int heads, int P, int lanes);                     // logits that one lane of the fp32 kernels keeps (d2o_stats.cu)
+size_t stored_logits_bytes(int heads, int P, int D, int lanes);   // logits that one lane of the fp32 kernels keeps (d2o_stats.cu)
 
 // remembers the text of a failed CUDA runtime call for d2o_last_cuda_error(); returns D2O_ERR_CUDA
 d2o_status record_cuda_error(cudaError_t e, const char* where);

@@ -124,7 +124,7 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   s->lse_stride = o - s->lse;
   o += (std::min<size_t>(L, c->dtype == D2O_F32 ? kStatsLanes : kColsumLayers) - 1) * s->lse_stride;
   const size_t lanes = std::min<size_t>(L, kStatsLanes);
-  s->logits_stride = c->dtype == D2O_F32 ? stored_logits_bytes((int)(B * Hq), (int)P, (int)lanes) : 0;
+  s->logits_stride = c->dtype == D2O_F32 ? stored_logits_bytes((int)(B * Hq), (int)P, (int)d, (int)lanes) : 0;
   s->logits = take(lanes * s->logits_stride);
   s->evict_idx = take(B * Hkv * P * 4);
   s->evict_mx = take(B * Hkv * P * 4);
@@ -293,7 +293,7 @@ extern "C" d2o_status d2o_layer_stats_layers(d2o_ctx* c, int32_t l0, int32_t l1,
     for (int i = 0; i < lanes; ++i) CUDA_TRY(cudaStreamWaitEvent(c->lane_stream[i], c->lane_fork, 0));
     for (int l = l0; l < l1; ++l) {
       const int lane = (l - l0) % lanes;                     // a lane's layers follow one another on its stream
-      CUDA_TRY(launch_layer_stats(c, l, Q[l - l0], K[l - l0], lse ? lse[l - l0] : nullptr, c->lane_stream[lane], lane));
+      CUDA_TRY(launch_layer_stats(c, l, Q[l - l0], K[l - l0], lse ? lse[l - l0] : nullptr, c->lane_stream[lane], lane, lanes));
     }
     for (int i = 0; i < lanes; ++i) {
       CUDA_TRY(cudaEventRecord(c->lane_done[i], c->lane_stream[i]));

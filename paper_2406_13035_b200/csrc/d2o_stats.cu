@@ -358,13 +358,51 @@ colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__
   cluster.sync();                                      // no CTA ends while another reads its results
 }
 
+// CTAs per cluster of a sweep over `heads` heads: as many as give every SM its CTAs (three fit, four leave a short second round);
+// past that only while every CTA keeps four tiles, because the copies that start a strip weigh as much as a tile or two, or
+// eight in sweeps of several rounds, so that the last one is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms
+// with four tiles per CTA, 4.20 with eight).  us, two rounds of CTAs with one or two tiles / one round: 16 heads of 700 tokens 48.3 /
+// 39.7, four layers of 32 heads of 500 tokens 183 / 139, of 16 heads of 900 tokens 199 / 174; 16 heads of 1024 tokens 72.4 / 73.4
+// (by itself 78.9 / 74.8); but 24 heads of 1000 tokens, two rounds of four tiles / one round 87.3 / 89.2.
+// Sums depend on it, so it is that of all heads of a call also where they go in groups.
+static int sweep_ctas(int P, int heads, int sms) {
+  const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
+  const long long units = (long long)pairs * heads;
+  int C = 1;
+  while (C < kMaxSweepCtas && 2 * C <= nT + 1 &&
+         (units * 2 * C <= 4 * sms || (units * C < 4 * sms && nT + 1 >= 8 * C) || (units * C < 16 * sms && nT + 1 >= 16 * C)))
+    C *= 2;
+  return C;
+}
+
 // Bytes of logits that one of `lanes` lanes keeps: whole heads, for all lanes at most kStoredLogits; 0 where one head's
 // triangle is larger.  Fewer heads at a time mean more launches with a start and an end each, which weighs more than keeping
 // the logits in L2: 32 heads of 1999 tokens, one lane, 517 us with 32 MB, 437 with 64, 367 with 256 (in another order of the sums).
 constexpr size_t kStoredLogits = (size_t)256 << 20;
+constexpr int kB200Sms = 148;             // the size of the scratch does not depend on the current device
 static size_t stored_head_bytes(int P) { return triangle_tiles(P) * kTile * kTile * sizeof(float); }
-size_t stored_logits_bytes(int heads, int P, int lanes) {
-  return std::min<size_t>(heads, kStoredLogits / lanes / stored_head_bytes(P)) * stored_head_bytes(P);
+
+// Are the dot products of `heads` heads better stored than computed twice, with room for `fit` heads and `lanes` layers at a time?
+// Heads that all fit: always.  In groups, one launch after another, only where the CTAs in flight come near to filling the GPU as
+// those of all heads do: its places are three per SM, and a group on half of them takes as long as both sweeps over all heads at
+// once.  ms, twice / stored, d = 64: 448 CTAs and more 0.53 / 0.37 (32 heads of 2000 tokens) to 3.46 / 2.92 (16 of 8000); 376 1.99 /
+// 1.73; 366 2.65 / 2.46; 344 3.29 / 3.06; 336 2.90 / 2.95; 320 5.09 / 5.66 and 1.43 / 1.45; 288 1.91 / 2.12; 252 6.39 / 8.21; 160 5.26 /
+// 8.31 (64 heads of 5000 tokens); clusters of four, two CTAs to an SM, are as good again: 288 2.26 / 2.25, 284 4.41 / 3.95, but 300
+// 3.70 / 3.97, 252 3.47 / 4.26.  A logit of d = 128 is twice the products: 344 6.12 / 5.45; 320 4.03 / 3.64; 288 3.72 / 3.62 and
+// 4.40 / 4.07; 252 6.80 / 7.36; 188 14.1 / 18.5.
+static bool stored_pays(int P, int D, int heads, int fit, int lanes, int sms) {
+  if (fit >= heads) return true;
+  if (fit < 1) return false;
+  const int groups = (heads + fit - 1) / fit, pairs = ((P + kTile - 1) / kTile + 1) / 2, C = sweep_ctas(P, heads, sms);
+  const long long ctas = (long long)lanes * heads * pairs * C / groups;
+  return 10 * ctas >= 19 * sms && (D == 128 || 10 * ctas >= 23 * sms || (C >= 4 && ctas <= 2 * sms));
+}
+
+size_t stored_logits_bytes(int heads, int P, int D, int lanes) {
+  const size_t head = stored_head_bytes(P);
+  const int fit = (int)std::min<size_t>(heads, kStoredLogits / lanes / head), all = (int)std::min<size_t>(heads, lanes * (size_t)fit);
+  // layers side by side, or one at a time in the room of all lanes
+  return stored_pays(P, D, heads, fit, lanes, kB200Sms) || stored_pays(P, D, heads, all, 1, kB200Sms) ? fit * head : 0;
 }
 
 static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, float* colsum, int P, int D, int head0, int n_heads, int Hq,
@@ -379,25 +417,6 @@ static cudaError_t launch_colsum_stored(const float4* logits, const float* lse, 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, colsum_stored_kernel, logits, lse, colsum, P, Hq, plen, head0, logit_scale(D));
-}
-
-// CTAs per cluster of a sweep over `heads` heads: as many as give every SM its CTAs (three fit, four leave a short second round);
-// past that only while every CTA keeps four tiles, because the copies that start a strip weigh as much as a tile or two, or
-// eight in sweeps of several rounds, so that the last one is a small part of the launch (32 heads of 1999 tokens, d = 64: 4.67 ms
-// with four tiles per CTA, 4.20 with eight).  us, two rounds of CTAs with one or two tiles / one round: 16 heads of 700 tokens 48.3 /
-// 39.7, four layers of 32 heads of 500 tokens 183 / 139, of 16 heads of 900 tokens 199 / 174; 16 heads of 1024 tokens 72.4 / 73.4
-// (by itself 78.9 / 74.8); but 24 heads of 1000 tokens, two rounds of four tiles / one round 87.3 / 89.2.
-// Sums depend on it, so it is that of all heads of a call also where they go in groups.
-static int sweep_ctas(int P, int heads) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) (void)cudaGetLastError();
-  const int nT = (P + kTile - 1) / kTile, pairs = (nT + 1) / 2;
-  const long long units = (long long)pairs * heads;
-  int C = 1;
-  while (C < kMaxSweepCtas && 2 * C <= nT + 1 &&
-         (units * 2 * C <= 4 * sms || (units * C < 4 * sms && nT + 1 >= 8 * C) || (units * C < 16 * sms && nT + 1 >= 16 * C)))
-    C *= 2;
-  return C;
 }
 
 // One sweep over `n_heads` heads from `head0` on.
@@ -426,18 +445,21 @@ __global__ void density_kernel(const float* colsum, double* __restrict__ density
                                const int32_t* __restrict__ plen, uint32_t* sched);
 constexpr int kDensityThreads = 512;
 
-// Row normalisers (unless the caller has them), column sums and densities of one layer.  Each kernel may start beside the
+// Row normalisers (unless the caller has them), column sums and densities of one layer, one of `lanes` side by side.  Each kernel may start beside the
 // tail of the one before it: only what this call wrote is waited for inside the kernels.
 template <typename T, int D>
 static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float* lse_buf, float* colsum, double* density, int P,
                                  int B, int Hq, int group, int L, int layer, const int32_t* plen, cudaStream_t st, float4* logits,
-                                 size_t logits_bytes) {
+                                 size_t logits_bytes, int lanes) {
   const bool own = lse == nullptr;
-  const int heads = B * Hq, C = sweep_ctas(P, heads);
+  int dev = 0, sms = kB200Sms;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) (void)cudaGetLastError();
+  const int heads = B * Hq, C = sweep_ctas(P, heads, sms);
+  const int fit = (int)std::min<size_t>(heads, logits_bytes / stored_head_bytes(P));
   cudaError_t e;
-  if (own && logits) {
+  if (own && stored_pays(P, D, heads, fit, lanes, sms)) {
     // as many heads at a time as leave their logits behind, in groups of about the same size
-    const int fit = (int)(logits_bytes / stored_head_bytes(P)), groups = (heads + fit - 1) / fit;
+    const int groups = (heads + fit - 1) / fit;
     for (int i = 0; i < groups; ++i) {
       const int h0 = (int)((long long)heads * i / groups), n = (int)((long long)heads * (i + 1) / groups) - h0;
       e = launch_sweep<T, D, false>(Q, K, nullptr, lse_buf, P, n, Hq, group, plen, st, true, C, h0, logits);
@@ -739,7 +761,7 @@ row_offset_kernel(const int32_t* __restrict__ budgets, int B, int L, int Hkv, in
 
 template <typename T, int D>
 static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse_in,
-                             cudaStream_t st, int lane) {
+                             cudaStream_t st, int lane, int lanes) {
   const d2o_config& g = c->cfg;
   const int P = g.prompt_len, Hq = g.n_q_heads, B = g.batch;
   float* colsum = (float*)(c->state + c->lay.colsum) + (size_t)layer * B * Hq * P;
@@ -747,8 +769,9 @@ static cudaError_t run_stats(const d2o_ctx* c, int layer, const void* Q, const v
   const int32_t* plen = (const int32_t*)(c->state + c->lay.plen);
   return launch_sweeps<T, D>((const T*)Q, (const T*)K, lse_in, (float*)(c->scratch + c->slay.lse + (size_t)lane * c->slay.lse_stride),
                              colsum, density, P, B, Hq, c->group, g.n_layers, layer, plen, st,
-                             c->slay.logits_stride ? (float4*)(c->scratch + c->slay.logits + (size_t)lane * c->slay.logits_stride) : nullptr,
-                             c->slay.logits_stride);
+                             (float4*)(c->scratch + c->slay.logits + (size_t)lane * c->slay.logits_stride),
+                             // a layer by itself has the room of all lanes
+                             (lanes == 1 ? std::min(g.n_layers, kStatsLanes) : 1) * c->slay.logits_stride, lanes);
 }
 
 cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void* const* Q, const void* const* K,
@@ -768,14 +791,14 @@ cudaError_t launch_layer_stats_tc(const d2o_ctx* c, int layer, int n, const void
 }
 
 cudaError_t launch_layer_stats(const d2o_ctx* c, int layer, const void* Q, const void* K, const float* lse,
-                               cudaStream_t st, int lane) {
+                               cudaStream_t st, int lane, int lanes) {
   if (c->stats_path == 0 && c->cfg.dtype != D2O_F32) return launch_layer_stats_tc(c, layer, 1, &Q, &K, lse ? &lse : nullptr, st);
   const int d = c->cfg.d_head;
   switch (c->cfg.dtype) {
-    case D2O_F32: return d == 64 ? run_stats<float, 64>(c, layer, Q, K, lse, st, lane) : run_stats<float, 128>(c, layer, Q, K, lse, st, lane);
-    case D2O_F16: return d == 64 ? run_stats<__half, 64>(c, layer, Q, K, lse, st, lane) : run_stats<__half, 128>(c, layer, Q, K, lse, st, lane);
-    default: return d == 64 ? run_stats<__nv_bfloat16, 64>(c, layer, Q, K, lse, st, lane)
-                            : run_stats<__nv_bfloat16, 128>(c, layer, Q, K, lse, st, lane);
+    case D2O_F32: return d == 64 ? run_stats<float, 64>(c, layer, Q, K, lse, st, lane, lanes) : run_stats<float, 128>(c, layer, Q, K, lse, st, lane, lanes);
+    case D2O_F16: return d == 64 ? run_stats<__half, 64>(c, layer, Q, K, lse, st, lane, lanes) : run_stats<__half, 128>(c, layer, Q, K, lse, st, lane, lanes);
+    default: return d == 64 ? run_stats<__nv_bfloat16, 64>(c, layer, Q, K, lse, st, lane, lanes)
+                            : run_stats<__nv_bfloat16, 128>(c, layer, Q, K, lse, st, lane, lanes);
   }
 }
 
@@ -818,7 +841,7 @@ static cudaError_t run_stats_static(int dtype, const void* Q, const void* K, flo
     return launch_behind(density_kernel, dim3((unsigned)(B * Hq)), kDensityThreads, 0, st, (const float*)colsum, density, P, Hq, 1, 0,
                          nullptr, sched);
   }
-  return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st, nullptr, 0);
+  return launch_sweeps<T, D>((const T*)Q, (const T*)K, nullptr, lse_buf, colsum, density, P, B, Hq, group, 1, 0, nullptr, st, nullptr, 0, 1);
 }
 
 }  // namespace d2o

@@ -69,6 +69,16 @@ def test_scratch_holds_the_normalisers_of_the_layers_at_work(lib, dtype, n_layer
     assert (size[1] - size[0]) // (32 * (1 << 17) * 4) == copies
 
 
+@pytest.mark.parametrize("h,d,P,n_layers,stored", [
+    (32, 64, 2000, 1, True), (32, 64, 4096, 2, True), (8, 64, 8000, 2, True), (64, 64, 4800, 1, False), (32, 128, 8000, 1, False),
+    (48, 64, 6000, 2, False), (2, 64, 12001, 1, False)])
+def test_dot_products_are_kept_where_that_pays(lib, h, d, P, n_layers, stored):
+    """fp32 scratch has room for the dot products of some heads only where the launches over those heads fill the GPU."""
+    size = B.d2o_workspace_size(good(dtype="f32", n_layers=n_layers, batch=1, n_kv_heads=h, n_q_heads=h, d_head=d, prompt_len=P, rho=0.05,
+                                     max_new_tokens=0))[1]
+    assert (size > 128 << 20) == stored              # everything else takes less than 64 MB here
+
+
 def test_null_and_misaligned_arguments(lib):
     cfg = good()
     h = C.c_void_p()

@@ -77,6 +77,34 @@ def test_fp32_colsum_at_any_prompt_length(cuda_device, d, P, hq, hkv):
     assert ctx.d2o_get_stats().error_word == 0
 
 
+@pytest.mark.parametrize("b,hq,hkv,d,P,L", [
+    (2, 1, 1, 64, 1, 1), (2, 8, 4, 128, 65, 1), (1, 8, 8, 64, 450, 3), (2, 96, 96, 64, 1025, 2), (1, 32, 8, 128, 1999, 2),
+    (1, 8, 2, 64, 6001, 2), (1, 16, 16, 64, 5000, 3), (1, 32, 32, 64, 5000, 1), (1, 32, 4, 64, 5300, 2), (1, 12, 12, 64, 9000, 1), (1, 4, 4, 64, 11000, 1),
+    (1, 2, 1, 64, 12001, 1)])
+def test_fp32_colsum_bits_whoever_computes_them(cuda_device, b, hq, hkv, d, P, L):
+    """Products stored (all heads, or in groups, with the room of one layer or of all) or computed twice: the bits are those of the
+    allocation-free entry point, which computes them twice."""
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    Q = [1.5 * torch.randn(b, hq, P, d, generator=g, device=cuda_device) for _ in range(L)]
+    K = [torch.randn(b, hkv, P, d, generator=g, device=cuda_device) for _ in range(L)]
+    want, F = torch.empty(L, b, hq, P, device=cuda_device), torch.empty(L, b, hq, dtype=torch.float64, device=cuda_device)
+    for l in range(L):
+        B.d2o_layer_stats_static(Q[l], K[l], want[l], F[l])
+    ctx = B.D2OContext(B.make_config(n_layers=L, batch=b, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype="f32", prompt_len=P,
+                                     max_new_tokens=8, rho=1.0 if P < 64 else 0.1, n_sink=0, min_budget=1))
+    for one_call in (True, False):
+        for l in range(L):
+            ctx.colsum(l).zero_()
+        if one_call:
+            ctx.d2o_layer_stats_layers(0, L, Q, K)
+        else:
+            for l in range(L):
+                ctx.d2o_layer_stats(l, Q[l], K[l])
+        assert all(torch.equal(ctx.colsum(l), want[l]) for l in range(L))
+        assert torch.equal(ctx.density(), F.permute(1, 0, 2))
+    ctx.close()
+
+
 def test_work_counter_is_zero_after_every_call(cuda_device):
     """The tensor-core kernels take their work from a counter.  Whatever it holds before a call (as after two calls that
     overlapped), the call after that one computes everything."""
