@@ -127,7 +127,10 @@ const char* d2o_status_string(d2o_status s);
 /* Text of the last CUDA runtime error seen by this thread's calls (HOST string). */
 const char* d2o_last_cuda_error(void);
 
-/* Sizes in bytes of the caller-owned DEVICE buffers for this config. */
+/* Sizes in bytes of the caller-owned DEVICE buffers for this config.  With fp32 caches scratch_bytes includes up to
+ * 256 MB for dot products that d2o_layer_stats keeps between its two sweeps over the prompt attention (two sets, for two layers
+ * at a time, where there are two); they come last, and d2o_create also takes a scratch that has no room for them: the products
+ * are then computed twice, with the same results. */
 d2o_status d2o_workspace_size(const d2o_config* cfg, size_t* state_bytes, size_t* scratch_bytes);
 
 /* Creates a context over caller-owned DEVICE buffers (256-byte aligned).  Zeroes the
@@ -156,7 +159,7 @@ d2o_status d2o_layer_stats(d2o_ctx* ctx, int32_t layer, const void* Q, const voi
  * lse: NULL, or a HOST array of l1-l0 DEVICE pointers (entries may be NULL).  16-bit inputs: up to
  * eight layers share a launch, so that short prompts fill the GPU.  fp32 inputs: two layers are
  * worked on side by side on streams of the library's own, each with its
- * own row-normaliser scratch, so that one layer's last CTAs share the GPU with the next layer's
+ * own scratch for row normalisers and dot products, so that one layer's last CTAs share the GPU with the next layer's
  * first.  Results are those of l1-l0 calls of d2o_layer_stats, bit for bit. */
 d2o_status d2o_layer_stats_layers(d2o_ctx* ctx, int32_t l0, int32_t l1, const void* const* Q,
                                   const void* const* K, const float* const* lse, void* stream);

@@ -123,9 +123,6 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   s->lse = take(colsum_tc_lse_bytes(c->batch, c->n_q_heads, c->prompt_len));
   s->lse_stride = o - s->lse;
   o += (std::min<size_t>(L, c->dtype == D2O_F32 ? kStatsLanes : kColsumLayers) - 1) * s->lse_stride;
-  const size_t lanes = std::min<size_t>(L, kStatsLanes);
-  s->logits_stride = c->dtype == D2O_F32 ? stored_logits_bytes((int)(B * Hq), (int)P, (int)d, (int)lanes) : 0;
-  s->logits = take(lanes * s->logits_stride);
   s->evict_idx = take(B * Hkv * P * 4);
   s->evict_mx = take(B * Hkv * P * 4);
   s->evict_nn = take(B * Hkv * P * 4);
@@ -146,6 +143,9 @@ static void layouts(const d2o_config* c, int64_t total_budget, int max_budget, L
   s->stage_out = take(L * B * Hq * d * e);
   s->stage_stride = o - s->stage_q;                        // further sets of the four for the pipelined host path
   o += (size_t)(2 * kHostBlock - 1) * s->stage_stride;
+  const size_t lanes = std::min<size_t>(L, kStatsLanes);
+  s->logits_stride = c->dtype == D2O_F32 ? stored_logits_bytes((int)(B * Hq), (int)P, (int)d, (int)lanes) : 0;
+  s->logits = take(lanes * s->logits_stride);              // last: d2o_create takes a scratch without them
   s->end = o;
 }
 
@@ -170,7 +170,8 @@ extern "C" d2o_status d2o_create(const d2o_config* cfg, void* state, size_t stat
   if (((uintptr_t)state & 255) || ((uintptr_t)scratch & 255)) return D2O_ERR_WORKSPACE;
   Layout l; ScratchLayout s;
   layouts(cfg, tot, maxb, &l, &s);
-  if (state_bytes < l.end || scratch_bytes < s.end) return D2O_ERR_WORKSPACE;
+  if (state_bytes < l.end || scratch_bytes < s.logits) return D2O_ERR_WORKSPACE;
+  if (scratch_bytes < s.end) s.logits_stride = 0;          // no room for dot products: they are computed twice
   d2o_ctx* c = (d2o_ctx*)calloc(1, sizeof(d2o_ctx));
   if (!c) return D2O_ERR_INVALID_ARG;
   c->cfg = *cfg;

@@ -68,6 +68,45 @@ def test_static_scratch_entry_matches_regular_entry(cuda_device, name, P, same_k
             assert abs(float(F[1, hq]) - O.attention_density(s_ref)) <= 2e-4 * O.attention_density(s_ref)
 
 
+def test_scratch_without_room_for_dot_products(cuda_device):
+    """fp32: a scratch that lacks only the room for the dot products (every head's whole tiles, for two layers) is accepted, one that
+    lacks a byte more is not; column sums and caches are those of the full scratch, bit for bit."""
+    import ctypes as C
+    from paper_2406_13035_b200 import build
+    build.build_library()
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=3, batch=1, prompt_len=300, decode_steps=2, window=8, max_budget=0)
+    products = 2 * wl.n_q_heads * 15 * 64 * 64 * 4        # 5 tiles of 64 rows: 15 on and below the diagonal
+    streams = [W.LayerStream(wl, l, "cuda:0") for l in range(3)]
+    Q, K, V = zip(*[s.prompt() for s in streams])
+
+    def results(ctx):
+        ctx.d2o_layer_stats_layers(0, 3, Q, K)
+        ctx.d2o_layer_budgets()
+        ctx.d2o_prefill_compress_layers(0, 3, K, V)
+        tabs = ctx.tables()
+        return [ctx.colsum(l).clone() for l in range(3)] + [ctx.slice_state(l, 0, h, tabs)["K"] for l in range(3) for h in range(wl.n_kv_heads)]
+
+    full = make_ctx(wl)
+    want = results(full)
+    lib, cfg = B.load_library(), full.cfg
+    sb, xb = B.d2o_workspace_size(cfg)
+    small = make_ctx(wl)
+    lib.d2o_destroy(small.handle)
+    small.scratch[small._scratch_off + xb - products:].fill_(0x5a)
+    sp, xp = (t.data_ptr() + off for t, off in ((small.state, small._state_off), (small.scratch, small._scratch_off)))
+    h = C.c_void_p()
+    st = torch.cuda.current_stream().cuda_stream
+    assert lib.d2o_create(C.byref(cfg), sp, sb, xp, xb - products - 256, st, C.byref(h)) == 3
+    assert lib.d2o_create(C.byref(cfg), sp, sb, xp, xb - products, st, C.byref(h)) == 0
+    small.handle = h
+    for a, b in zip(want, results(small)):
+        assert torch.equal(a, b)
+    torch.cuda.synchronize()
+    assert bool((small.scratch[small._scratch_off + xb - products:] == 0x5a).all())      # and left alone
+    full.close()
+    small.close()
+
+
 def test_static_scratch_entry_rejects_oversize(cuda_device):
     B.load_library()
     P = B.STATIC_LSE_FLOATS // 8 + 1                    # 1 x 8 heads x P floats: one row too many
