@@ -132,6 +132,11 @@ decode_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, const __g
       return;
     }
   }
+  if (a.pub_count > 0 && blockIdx.x == gridDim.x - 1) {
+    // the counters of the call before, a step on clusters: its grid was done before this one started
+    for (int i = tid; i < a.pub_count; i += (CW + 1) * 32)
+      asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + a.pub_first + i), "r"(a.pub_step) : "memory");
+  }
   const int n_old = a.len[sidx];
   const float tau_old = a.tau[sidx];
   if (!D2O_GUARD(S >= 1 && n_old >= 0 && n_old <= S && row0 >= 0 && row0 + slice_stride(S) <= a.pool_rows, a.status,
@@ -1146,6 +1151,17 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     return min(c->h_pair_max[(pr % B) * L + pr / B], t_now) + 1;
   };
 
+  // Behind a call on other layers of the same stream: this one writes that call's step counters, if it left them (only steps on
+  // clusters do; d2o_decode_split.cu).  Where a stack's layers take different kernels and this kernel's calls did not write
+  // them, the cluster steps waited for the grid ahead before they read anything: by-layer calls of 32 layers, 16 of them above the 20 MB of
+  // decode_split_cluster, us a token without / with: 64 fp16 slices a layer, one head, 656 / 560, 32 bf16 slices, four heads, 788 / 782;
+  // eight fp32 layers 205 / 182; layers of one sort as before.
+  auto& last = c->last_decode;
+  const auto before = last;
+  const bool other = before.l1 > before.l0 && before.stream == st && (l1 <= before.l0 || l0 >= before.l1);
+  const bool theirs = other && before.deferred && !chained;
+  if (theirs) { a.pub_first = before.l0 * B * Hkv; a.pub_count = (before.l1 - before.l0) * B * Hkv; a.pub_step = before.step + 1; }
+
   // Few slices: a cluster of CTAs for each (the knobs of d2o_set_tuning belong to the kernel below)
   if (c->decode_warps == 0 && c->decode_stages == 0 && c->decode_smem_rows == 0 && c->decode_long_pairs == 0) {
     const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows, sum_rows * Hkv);
@@ -1153,26 +1169,23 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
       bool published = true;                                          // the last step of every layer of the call
       for (int l = l0; l < l1; ++l) published = published && c->layer_published[l] && c->layer_stream[l] == st;
       a.early = published ? 1 : 0;
-      // behind a call on other layers of the same stream: that call's counters, if it left them, and not this one's own
-      auto& last = c->last_decode;
-      const bool other = last.l1 > last.l0 && last.stream == st && (l1 <= last.l0 || l0 >= last.l1);
-      const bool theirs = other && last.deferred && !chained;
-      if (theirs) { a.pub_first = last.l0 * B * Hkv; a.pub_count = (last.l1 - last.l0) * B * Hkv; a.pub_step = last.step + 1; }
-      a.publish = publish || !other ? 1 : 0;
+      a.publish = publish || !other ? 1 : 0;                          // calls alternate between layers: the next one's
       c->decode_launches += 1;
       const cudaError_t e = launch_decode_split(c, a, C, n_pairs * Hkv, max_rows, q, k, v, out, kpool, vpool, st);
       memset(c->layer_published + l0, e == cudaSuccess && a.publish, l1 - l0);
-      if (e == cudaSuccess && theirs) memset(c->layer_published + last.l0, 1, last.l1 - last.l0);
+      if (e == cudaSuccess && theirs) memset(c->layer_published + before.l0, 1, before.l1 - before.l0);
       last = {l0, l1, a.step, st, e == cudaSuccess && !a.publish};
       for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
       return e;
     }
   }
   memset(c->layer_published + l0, 0, l1 - l0);                          // set again below once the launch has succeeded
-  c->last_decode = {l0, l1, a.step, st, false};
+  last = {l0, l1, a.step, st, false};
   for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
   auto launched = [&](cudaError_t e) {
-    if (publish && e == cudaSuccess && *why == D2O_OK) memset(c->layer_published + l0, 1, l1 - l0);
+    if (e != cudaSuccess || *why != D2O_OK) return e;
+    if (publish) memset(c->layer_published + l0, 1, l1 - l0);
+    if (theirs) memset(c->layer_published + before.l0, 1, before.l1 - before.l0);
     return e;
   };
 
@@ -1226,6 +1239,7 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     c->decode_launches += 1;
     DecodeArgs ac = a;
     ac.row_cap = row_cap; ac.stages = stages; ac.pair_base = p0;
+    if (p0 > 0) ac.pub_count = 0;                                     // beside a launch of the same step, which writes them
     // 16-bit caches with grouped queries read their rows through tensor maps (swizzled stages)
     CUtensorMap map_k, map_v;
     memset(&map_k, 0, sizeof(map_k));

@@ -179,6 +179,59 @@ def test_step_counters_in_any_order_of_calls(cuda_device, hq, hkv, P, d, dtype):
             assert all(torch.equal(a[key].view(torch.uint8), b[key].view(torch.uint8)) for key in ("pos", "score", "rnorm", "K", "V"))
 
 
+@pytest.mark.parametrize("hq,hkv,d,dtype,pair", [(32, 8, 128, "bf16", False), (16, 16, 128, "f16", False), (16, 16, 64, "f32", False),
+                                                  (32, 8, 128, "bf16", True)])
+def test_step_counters_of_stacks_on_both_decode_kernels(cuda_device, hq, hkv, d, dtype, pair):
+    """Layers with small caches step on clusters and leave their step counters to the next call; layers with large ones step on one
+    CTA per slice.  The counters are written whichever kernel comes next, and the results are those of synchronised calls."""
+    L, B_, P, tokens = 6, 4, 2400, 5
+    td = B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    Q, K, V = (torch.randn(L, B_, h, P, d, generator=g, device=cuda_device).to(td) for h in (hq, hkv, hkv))
+    q = torch.randn(tokens, L, B_, hq, d, generator=g, device=cuda_device).to(td)
+    k, v = (torch.randn(tokens, L, B_, hkv, d, generator=g, device=cuda_device).to(td) for _ in range(2))
+    row = 2 * d * (4 if dtype == "f32" else 2) * B_ * hkv                  # bytes of one row of every slice of a layer
+    small, large = 12e6 / row, 26e6 / row                                  # on either side of the 20 MB where the kernels change
+    big = (1, 2, 4)
+    calls = [(0, 1), (1, 3), (3, 4), (4, 5), (5, 6)] if pair else [(l, l + 1) for l in range(L)]
+
+    def run(synced):
+        ctx = B.D2OContext(B.make_config(n_layers=L, batch=B_, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=P,
+                                         max_new_tokens=tokens + 3, rho=(small + large) / 2 / P, n_sink=1, window=8, min_budget=16))
+        for l in range(L):
+            ctx.d2o_layer_stats(l, Q[l], K[l])
+        for l in range(L):                                                 # Eq. 5 weights exp(-F)
+            ctx.density()[:, l] = 1.0 - torch.log(torch.tensor(large if l in big else small)).item()
+        budgets = ctx.d2o_layer_budgets()
+        assert all(bool((budgets[:, l] * row > 20e6).all()) == (l in big) for l in range(L))
+        ctx.d2o_prefill_compress_layers(0, L, list(K), list(V))
+        at = ctx._view(0).tau - ctx.state.data_ptr() + (L * B_ * hkv * 4 + 255) // 256 * 256      # the counters lie behind tau
+        counters = ctx.state[at:at + L * B_ * hkv * 4].view(torch.int32).view(L, -1)
+        out = torch.zeros_like(q)
+        written = []
+        for t in range(tokens):
+            for l0, l1 in calls:
+                ctx.d2o_decode_step(l0, l1, q[t, l0:l1], k[t, l0:l1], v[t, l0:l1], out[t, l0:l1])
+                if synced:
+                    torch.cuda.synchronize()
+            written.append(counters.clone())
+        torch.cuda.synchronize()
+        assert ctx.d2o_get_stats().error_word == 0
+        for t, c in enumerate(written):                                    # those of layer 5 may be written by the next token's first call
+            assert bool((c[0] == t + 1).all()) and bool((c[3] == t + 1).all()) and bool((c[5] >= t).all())
+        tabs = ctx.tables()
+        state = [ctx.slice_state(l, b, h, tabs) for l in range(L) for b in range(B_) for h in range(hkv)]
+        ctx.close()
+        return out, state
+
+    want, ws = run(True)
+    for _ in range(2):
+        got, gs = run(False)
+        assert torch.equal(want.view(torch.uint8), got.view(torch.uint8))
+        for a, b in zip(ws, gs):
+            assert all(torch.equal(a[key].view(torch.uint8), b[key].view(torch.uint8)) for key in ("pos", "score", "rnorm", "K", "V"))
+
+
 @pytest.mark.parametrize("n,G,P,d,dtype", [(8, 4, 900, 128, "bf16"), (64, 1, 500, 128, "f16"), (5, 2, 70, 64, "f32")])
 def test_uncompressed_outputs_are_the_next_queries(cuda_device, n, G, P, d, dtype):
     L, td = 12, B.TORCH_DTYPE[B.DTYPE_CODE[dtype]]
