@@ -621,14 +621,18 @@ merge_kernel(MergeArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__
 }
 
 // ------------------------------------------------------------------------------------ launcher
-// Threads of a CTA of select_kernel and segment_kernel, which take one slice each.  A CTA is a chain of block-wide steps: with
-// no more slices than SMs as many threads as there are shorten it; with more slices, smaller CTAs of which several fit an SM
-// do not wait for a place (select_kernel: one CTA of 1024 threads per SM, four of 256).  us, with 1024 threads / so: 32 layers of
-// 32 slices of 1200 tokens, the prompt stage as a whole 1230 / 1185; four layers of 128 slices of 8192 tokens, compression 1783 /
-// 1766 and, on another GPU, 1785 / 1717 (256 threads: 1877); but 64 slices of 3000 tokens 146 / 155 with 512 threads, so few
-// slices keep 1024.
+// Threads of a CTA of select_kernel and segment_kernel, which take one slice each.  A CTA is a chain of block-wide steps: more
+// threads shorten it, for as long as every thread has rows and every CTA a place at once (of select_kernel's, one of 1024 threads
+// fits an SM, two of 512, four of 256).  us of compression with 1024 / 512 / 256 threads; 160 slices of 450 rows 55 / 44.4 / 43.8, 800
+// 63.5 / 55.1 / 58.5, 3000 172 / 170 / 194, 6000 338 / 341 / 392; 256 of 450 rows 58 / 49.0 / 48.4, 2040 154 / 149 / 169, 4096 262 / 261 /
+// 301, 8192 689 / 696 / 771; 320 of 600 rows 79 / 62.5 / 59.6, 1000 108 / 93 / 95, 8192 854 / 850 / 898; 512 of 800 rows 131 / 107.7 /
+// 106.6, 1200 227 / 202 / 206, 12000 1469 / 1450 / 1497, 16384 2443 / 2460 / 2590; 1024 of 1200 rows 318 / 274 / 262, 4096 935 / 886 / 880; but
+// 64 of 3000 rows 146 / 155 with 512.
 static int slice_threads(const d2o_ctx* c, int n_ctas, int rows) {
-  return n_ctas <= c->n_sms ? 1024 : rows <= 2048 ? 256 : rows <= 16384 ? 512 : 1024;
+  const int sms = c->n_sms;
+  if (n_ctas <= sms) return 1024;
+  if (rows <= (n_ctas > 4 * sms ? 4096 : n_ctas > 2 * sms ? 800 : 450)) return 256;
+  return rows <= (n_ctas > 2 * sms ? 12288 : 5120) ? 512 : 1024;
 }
 
 // Layers [layer, layer + n) in one launch per kernel; their working arrays are the first n sets of `scratch`.

@@ -94,6 +94,16 @@ def test_more_slices_than_sms(dtype, P, rho):
     _run(wl, [(0, 20)], steps=2)
 
 
+@pytest.mark.parametrize("L,batch,P,rho", [(20, 2, 450, 0.2), (20, 2, 451, 0.2), (20, 2, 5120, 0.02), (20, 2, 5121, 0.02), (16, 3, 801, 0.1),
+                                           (16, 3, 12289, 0.01), (16, 5, 801, 0.1), (16, 5, 4097, 0.03)])
+def test_threads_per_slice(L, batch, P, rho):
+    """Launches of more slices than the GPU has SMs, at the numbers of slices and rows where the threads per slice change, against a
+    layer at a time (1024 threads)."""
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=L, batch=batch, dtype="f16", prompt_len=P, rho=rho, decode_steps=1,
+                             density_temp=50.0, min_budget=8, max_budget=0)
+    _run(wl, [(0, L)], steps=1)
+
+
 @pytest.mark.parametrize("name", ["cfg0", "cfg1", "cfg2"])
 def test_layer_stats_of_several_layers_in_one_call(name):
     """d2o_layer_stats_layers against layer-by-layer calls: column sums, densities and budgets bit for bit."""
