@@ -313,8 +313,8 @@ d2o_status d2o_set_tuning(d2o_ctx* ctx, int32_t decode_stages, int32_t decode_l2
  * engine issues no copy from this stage of a slice on (-1 = never), so that the wait for it runs out; the
  * tensor-core column sums take both for their streamed tiles (from this one of every CTA on) and give NaN.  A wait
  * that runs out sets the error word to D2O_ERR_TIMEOUT (see d2o_get_stats); the kernel returns, the slices
- * whose wait ran out during the key pass are left untouched, and every later decode step on this context does
- * nothing.  Nothing traps and the CUDA context stays usable. */
+ * whose wait ran out during the key pass are left untouched, the call's other slices may or may not have taken the step, and
+ * every later decode step on this context does nothing.  Nothing traps and the CUDA context stays usable. */
 d2o_status d2o_set_fault_injection(d2o_ctx* ctx, int32_t wait_limit_us, int32_t producer_stop_stage);
 
 #ifdef __cplusplus

@@ -357,7 +357,8 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   push_key(best, best_li, false, false);
   // ---- from here on the inputs: the grid ahead on the stream must be done (unless the call promised them complete)
   if (a.early && !a.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
-  // an anomaly of the grids ahead that was recorded while this one waited: looked at again below, beside the key pass
+  // A wait of the grids ahead that ran out while this one waited for them: looked at again below, beside the key pass.  (Other
+  // anomalies concern one slice and may be those of another cluster of this launch: its own token is dropped, no other.)
   const uint32_t word = tid == 0 ? *reinterpret_cast<volatile uint32_t*>(a.status) : 0u;
   if (a.pub_count > 0 && warp == kSplitWarps - 1 && blockIdx.x == gridDim.x - 1) {
     // the slices of the call before: its grid is done
@@ -480,7 +481,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
       for (int g = 0; g < G; ++g) { to->m[my_entry][g] = mw[g]; to->l[my_entry][g] = lw[g]; }
     }
   }
-  if (word != 0u && s_timeout == 0) s_timeout = 1;
+  if (word == D2O_ERR_TIMEOUT && s_timeout == 0) s_timeout = 1;
   __syncwarp();
   if (lane < C) cluster.map_shared_rank(&xch, lane)->bad1[my_entry] = s_timeout;
   cluster_arrive();                                                       // barrier 1

@@ -19,6 +19,7 @@ from parity import assert_report, make_ctx, run_parity
 
 pytestmark = pytest.mark.gpu
 
+D2O_ERR_STATE = 4
 D2O_ERR_TIMEOUT = 6
 
 
@@ -148,6 +149,47 @@ def test_layers_behind_one_that_ran_out_of_time(cuda_device, P, rho, hq, hkv, d,
     torch.cuda.synchronize()
     assert ctx.d2o_get_stats().error_word == D2O_ERR_TIMEOUT
     assert _same(before, state()) and all(torch.equal(a, b) for a, b in zip(first_out, out))
+    ctx.close()
+
+
+@pytest.mark.parametrize("word,taken", [(D2O_ERR_STATE, True), (D2O_ERR_TIMEOUT, False)])
+@pytest.mark.parametrize("hq,hkv,d,dtype", [(8, 8, 64, "f32"), (32, 8, 128, "bf16")])
+def test_error_recorded_while_a_step_waits(cuda_device, hq, hkv, d, dtype, word, taken):
+    """A step on clusters that is resident and waits for the kernel ahead of it when an error is recorded: one that concerns a single
+    slice (its token was dropped) does not stop it, a wait that ran out does."""
+    wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=2, batch=1, n_q_heads=hq, n_kv_heads=hkv, d_head=d, dtype=dtype, prompt_len=300,
+                             rho=0.4, decode_steps=8, min_budget=8, max_budget=0)
+    ctx = make_ctx(wl)
+    streams = [W.LayerStream(wl, l, "cuda:0") for l in range(2)]
+    Q, K, V = zip(*[s.prompt() for s in streams])
+    ctx.d2o_layer_stats_layers(0, 2, Q, K)
+    ctx.d2o_layer_budgets()
+    ctx.d2o_prefill_compress_layers(0, 2, K, V)
+    for _ in range(2):
+        for l in range(2):
+            q, k, v = streams[l].decode()
+            out = torch.empty_like(q)
+            ctx.d2o_decode_step(l, l + 1, q, k, v, out)
+    q, k, v = streams[0].decode()
+    # eight CTAs that take milliseconds over a long cache, and let the step move in at once
+    kc, vc = (torch.zeros(1, 1 << 20, 128, device=cuda_device) for _ in range(2))
+    x = torch.zeros(1, 1, 128, device=cuda_device)
+    error = torch.tensor([word], dtype=torch.int32).pin_memory()
+    at = ctx.state[ctx._state_off:ctx._state_off + 4].view(torch.int32)
+    side, done = torch.cuda.Stream(), torch.cuda.Event()
+    assert ctx.d2o_get_stats().error_word == 0
+    before = ctx.d2o_get_stats().decode_steps
+    torch.cuda.synchronize()
+    B.d2o_full_decode_step(kc, vc, (1 << 20) - 1, x, x[0], x[0], torch.empty_like(x))
+    ctx.d2o_decode_step(0, 1, q, k, v, out)
+    done.record()
+    time.sleep(2e-4)
+    with torch.cuda.stream(side):
+        at.copy_(error, non_blocking=True)
+    side.synchronize()
+    assert not done.query()                                      # the kernel ahead was still running
+    torch.cuda.synchronize()
+    assert ctx.d2o_get_stats().decode_steps - before == (hkv if taken else 0)
     ctx.close()
 
 
