@@ -270,10 +270,11 @@ sweep_kernel(const T* Q, const T* K, const float* lse_in, float* __restrict__ ou
   cluster.sync();                                     // no CTA ends while another reads its results
 }
 
-// Column sums from the dot products that the row sweep left in `logits` (whole tiles; rows >= P: 0), one pair of
-// column tiles per cluster as above.  A thread holds the entries that it computed there: rows ty + 8 r, columns tx + 16 c.  The
-// sums run in the order of sweep_kernel, so that the bits are the same whoever computes them: groups of rows 16 apart in fp32
-// (r even: group ty, r odd: group ty + 8), the tiles of a CTA, and the groups as its butterfly takes them (4 apart, 2, 1).
+// Column sums from the dot products that the row sweep left in `logits` (whole tiles; those of rows >= P are not looked at: zeros
+// times a key that is not finite are NaN), one pair of column tiles per cluster as above.  A thread holds the entries that it
+// computed there: rows ty + 8 r, columns tx + 16 c.  The sums run in the order of sweep_kernel, so that the bits are the same
+// whoever computes them: groups of rows 16 apart in fp32 (r even: group ty, r odd: group ty + 8), the tiles of a CTA, and the
+// groups as its butterfly takes them (4 apart, 2, 1).
 //
 // The row sweep is bound by its FMAs (one per element of d and logit); repeating them for the column sums took half of the call.
 // A logit costs 8 bytes of traffic instead (kStoredLogits: how many are kept at a time).  Row sweep, column sums and densities,
@@ -310,7 +311,10 @@ colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__
       float4 x[kStripA];
       float l[kStripA];
 #pragma unroll
-      for (int r = 0; r < kStripA; ++r) x[r] = t[r * kStatThreads];
+      for (int r = 0; r < kStripA; ++r) {
+        x[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (at * kTile + ty + 8 * r < P) x[r] = t[r * kStatThreads];
+      }
 #pragma unroll
       for (int r = 0; r < kStripA; ++r) { const int row = at * kTile + ty + 8 * r; l[r] = row < P ? -(lse[row] * kLog2e) : -INFINITY; }
 #pragma unroll

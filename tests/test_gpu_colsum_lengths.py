@@ -105,6 +105,31 @@ def test_fp32_colsum_bits_whoever_computes_them(cuda_device, b, hq, hkv, d, P, L
     ctx.close()
 
 
+@pytest.mark.parametrize("d,P,key", [(64, 100, 97), (64, 65, 3), (128, 449, 448), (64, 128, 70)])
+def test_fp32_keys_with_infinite_elements(cuda_device, d, P, key):
+    """A key whose logits are all -inf: its column is 0, every other one is as without it, and nothing comes from the rows past the
+    end of the last tile, whose products with it are not numbers."""
+    h = 4
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    Q = torch.randn(1, h, P, d, generator=g, device=cuda_device)
+    K = torch.randn(1, h, P, d, generator=g, device=cuda_device)
+    Q[..., 5] = Q[..., 5].abs() + 0.1
+    K[:, :, key, 5] = -float("inf")
+    logits, ref = _reference(Q, K)
+    ref[:, :, key] = 0.0
+    ctx = _context("f32", 1, h, h, d, P)
+    for _ in range(2):
+        ctx.d2o_layer_stats(0, Q, K)
+        cs = ctx.colsum(0)
+        assert bool((cs[:, :, key] == 0).all())
+        others = torch.arange(P, device=cuda_device) != key
+        assert float(((cs.double() - ref).abs() / ref)[:, :, others].max()) < 2e-5
+    static, F = torch.empty(1, h, P, device=cuda_device), torch.empty(1, h, dtype=torch.float64, device=cuda_device)
+    B.d2o_layer_stats_static(Q, K, static, F)
+    assert torch.equal(static, cs)
+    ctx.close()
+
+
 def test_work_counter_is_zero_after_every_call(cuda_device):
     """The tensor-core kernels take their work from a counter.  Whatever it holds before a call (as after two calls that
     overlapped), the call after that one computes everything."""
