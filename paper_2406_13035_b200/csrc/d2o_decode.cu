@@ -132,11 +132,6 @@ decode_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, const __g
       return;
     }
   }
-  if (a.pub_count > 0 && blockIdx.x == gridDim.x - 1) {
-    // the counters of the call before, a step on clusters: its grid was done before this one started
-    for (int i = tid; i < a.pub_count; i += (CW + 1) * 32)
-      asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + a.pub_first + i), "r"(a.pub_step) : "memory");
-  }
   const int n_old = a.len[sidx];
   const float tau_old = a.tau[sidx];
   if (!D2O_GUARD(S >= 1 && n_old >= 0 && n_old <= S && row0 >= 0 && row0 + slice_stride(S) <= a.pool_rows, a.status,
@@ -1100,6 +1095,26 @@ static int smem_rows_for(int max_rows, double mean_rows, int G) {
   return min(max_rows, max(free_rows, (int)(2.0 * mean_rows)));
 }
 
+// Rows of the longest slice of the layers [l0, l1), and the sum over their pairs of the pair's mean (a cache cannot hold more than
+// was generated).
+struct CallRows { int max_rows; double sum_rows; };
+static CallRows call_rows(const d2o_ctx* c, int l0, int l1) {
+  const int B = c->cfg.batch, L = c->cfg.n_layers, Hkv = c->cfg.n_kv_heads, t_now = c->cfg.prompt_len + c->layer_steps[l0];
+  CallRows r = {0, 0.0};
+  for (int l = l0; l < l1; ++l)
+    for (int b = 0; b < B; ++b) {
+      r.max_rows = max(r.max_rows, min(c->h_pair_max[b * L + l], t_now) + 1);
+      r.sum_rows += (double)min((long long)c->h_pair_sum[b * L + l], (long long)t_now * Hkv) / Hkv + 1.0;
+    }
+  return r;
+}
+
+// CTAs per slice of a step on the layers [l0, l1), 0: decode_kernel, to which the knobs of d2o_set_tuning belong
+static int call_cluster(const d2o_ctx* c, int l0, int l1, const CallRows& r) {
+  if (c->decode_warps != 0 || c->decode_stages != 0 || c->decode_smem_rows != 0 || c->decode_long_pairs != 0) return 0;
+  return decode_split_cluster(c, (l1 - l0) * c->cfg.batch * c->cfg.n_kv_heads, r.max_rows, r.sum_rows * c->cfg.n_kv_heads);
+}
+
 // `chained`: this step follows another decode step of the same layers on the same stream, and its inputs were
 // complete before that one was launched.  Its grids are then launched with programmatic stream serialisation and
 // may start while the previous step's last CTAs are still running; every CTA waits for its own slice's step counter
@@ -1131,15 +1146,10 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
   const int G = c->group, Hkv = g.n_kv_heads;
   const int row_bytes = g.d_head * c->elem_size;
   void* kpool = S + c->lay.kpool; void* vpool = S + c->lay.vpool;
-  // rows of the longest slice of a pair, and the mean over all slices (a cache cannot hold more than was generated)
   const int t_now = g.prompt_len + c->layer_steps[l0];
-  int max_rows = 0;
-  double sum_rows = 0.0;
-  for (int l = l0; l < l1; ++l)
-    for (int b = 0; b < B; ++b) {
-      max_rows = max(max_rows, min(c->h_pair_max[b * L + l], t_now) + 1);
-      sum_rows += (double)min((long long)c->h_pair_sum[b * L + l], (long long)t_now * g.n_kv_heads) / g.n_kv_heads + 1.0;
-    }
+  const CallRows rows = call_rows(c, l0, l1);
+  const int max_rows = rows.max_rows;
+  const double sum_rows = rows.sum_rows;
   // all layers in one call: CTAs take the slices largest cache first, so the long ones do not end up in the tail
   const bool ordered = (l0 == 0 && l1 == L);
   a.order = ordered ? (const int32_t*)(S + c->lay.order) : nullptr;
@@ -1151,41 +1161,36 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     return min(c->h_pair_max[(pr % B) * L + pr / B], t_now) + 1;
   };
 
-  // Behind a call on other layers of the same stream: this one writes that call's step counters, if it left them (only steps on
-  // clusters do; d2o_decode_split.cu).  Where a stack's layers take different kernels and this kernel's calls did not write
-  // them, the cluster steps waited for the grid ahead before they read anything: by-layer calls of 32 layers, 16 of them above the 20 MB of
-  // decode_split_cluster, us a token without / with: 64 fp16 slices a layer, one head, 656 / 560, 32 bf16 slices, four heads, 788 / 782;
-  // eight fp32 layers 205 / 182; layers of one sort as before.
-  auto& last = c->last_decode;
-  const auto before = last;
-  const bool other = before.l1 > before.l0 && before.stream == st && (l1 <= before.l0 || l0 >= before.l1);
-  const bool theirs = other && before.deferred && !chained;
-  if (theirs) { a.pub_first = before.l0 * B * Hkv; a.pub_count = (before.l1 - before.l0) * B * Hkv; a.pub_step = before.step + 1; }
-
-  // Few slices: a cluster of CTAs for each (the knobs of d2o_set_tuning belong to the kernel below)
-  if (c->decode_warps == 0 && c->decode_stages == 0 && c->decode_smem_rows == 0 && c->decode_long_pairs == 0) {
-    const int C = decode_split_cluster(c, n_pairs * Hkv, max_rows, sum_rows * Hkv);
-    if (C > 0) {
-      bool published = true;                                          // the last step of every layer of the call
-      for (int l = l0; l < l1; ++l) published = published && c->layer_published[l] && c->layer_stream[l] == st;
-      a.early = published ? 1 : 0;
-      a.publish = publish || !other ? 1 : 0;                          // calls alternate between layers: the next one's
-      c->decode_launches += 1;
-      const cudaError_t e = launch_decode_split(c, a, C, n_pairs * Hkv, max_rows, q, k, v, out, kpool, vpool, st);
-      memset(c->layer_published + l0, e == cudaSuccess && a.publish, l1 - l0);
-      if (e == cudaSuccess && theirs) memset(c->layer_published + before.l0, 1, before.l1 - before.l0);
-      last = {l0, l1, a.step, st, e == cudaSuccess && !a.publish};
-      for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
-      return e;
-    }
+  // Few slices: a cluster of CTAs for each
+  if (const int C = call_cluster(c, l0, l1, rows)) {
+    bool published = true;                                            // the last step of every layer of the call
+    for (int l = l0; l < l1; ++l) published = published && c->layer_published[l] && c->layer_stream[l] == st;
+    a.early = published ? 1 : 0;
+    // Behind a call on other layers of the same stream: that call's counters, if it left them, and not this one's own, unless the
+    // call that is likely to follow (as many layers, the next ones) takes decode_kernel.  That kernel writes none, and where nobody
+    // wrote them the cluster steps waited for the grid ahead before they read anything.  By-layer calls of 32 layers, every second
+    // one above the 20 MB of decode_split_cluster, us a token, left to the next call / so: 64 fp16 slices a layer, one head, 656 /
+    // 581, 32 bf16 slices, four heads, 788 / 787 (every eighth one 492 / 495); eight fp32 layers 205 / 188.  (decode_kernel writing
+    // them as its first act: 559, 773, 182, but 0.3 - 1 % of every other call of that kernel, with 480 us of nine layers 3.5.)
+    auto& last = c->last_decode;
+    const bool other = last.l1 > last.l0 && last.stream == st && (l1 <= last.l0 || l0 >= last.l1);
+    const bool theirs = other && last.deferred && !chained;
+    if (theirs) { a.pub_first = last.l0 * B * Hkv; a.pub_count = (last.l1 - last.l0) * B * Hkv; a.pub_step = last.step + 1; }
+    const int n0 = l1 < L ? l1 : 0, n1 = min(L, n0 + l1 - l0);
+    a.publish = publish || !other || call_cluster(c, n0, n1, call_rows(c, n0, n1)) == 0 ? 1 : 0;
+    c->decode_launches += 1;
+    const cudaError_t e = launch_decode_split(c, a, C, n_pairs * Hkv, max_rows, q, k, v, out, kpool, vpool, st);
+    memset(c->layer_published + l0, e == cudaSuccess && a.publish, l1 - l0);
+    if (e == cudaSuccess && theirs) memset(c->layer_published + last.l0, 1, last.l1 - last.l0);
+    last = {l0, l1, a.step, st, e == cudaSuccess && !a.publish};
+    for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
+    return e;
   }
   memset(c->layer_published + l0, 0, l1 - l0);                          // set again below once the launch has succeeded
-  last = {l0, l1, a.step, st, false};
+  c->last_decode = {l0, l1, a.step, st, false};
   for (int l = l0; l < l1; ++l) c->layer_stream[l] = st;
   auto launched = [&](cudaError_t e) {
-    if (e != cudaSuccess || *why != D2O_OK) return e;
-    if (publish) memset(c->layer_published + l0, 1, l1 - l0);
-    if (theirs) memset(c->layer_published + before.l0, 1, before.l1 - before.l0);
+    if (publish && e == cudaSuccess && *why == D2O_OK) memset(c->layer_published + l0, 1, l1 - l0);
     return e;
   };
 
@@ -1239,7 +1244,6 @@ cudaError_t launch_decode(const d2o_ctx* c, int l0, int l1, const void* q, const
     c->decode_launches += 1;
     DecodeArgs ac = a;
     ac.row_cap = row_cap; ac.stages = stages; ac.pair_base = p0;
-    if (p0 > 0) ac.pub_count = 0;                                     // beside a launch of the same step, which writes them
     // 16-bit caches with grouped queries read their rows through tensor maps (swizzled stages)
     CUtensorMap map_k, map_v;
     memset(&map_k, 0, sizeof(map_k));

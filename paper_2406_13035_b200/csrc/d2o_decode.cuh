@@ -43,7 +43,7 @@ struct DecodeArgs {
                                     // the slice, and until they are done the counter may be an earlier conversation's
   int publish;                      // 1: the CTA (cluster) publishes the slice's step counter at its end: a chained step follows, or
                                     // (decode_split_kernel) the next call is likely to work on the same layers
-  int pub_first, pub_count, pub_step;   // slices of the call before whose counters this grid writes, and their value
+  int pub_first, pub_count, pub_step;   // decode_split_kernel: slices of the call before whose counters this grid writes, and their value
 };
 
 // d2o_decode_split.cu

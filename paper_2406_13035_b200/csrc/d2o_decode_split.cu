@@ -31,7 +31,8 @@
 // Who writes the step counter.  A step that tells by itself that a slice is complete has to collect the stores of the whole
 // cluster first: one more cluster barrier and a release, 1.5 us of every call.  Where calls alternate between layers the next
 // call does it instead: behind its wait for the grid ahead that grid's stores are all visible, and a warp of its last CTA writes
-// the counters (DecodeArgs::pub_first); so does decode_kernel where it takes the next call's layers.  A chained step, and one that follows a step on the same layers, writes its own.
+// the counters (DecodeArgs::pub_first).  A chained step, one that follows a step on the same layers, and one whose next call is
+// likely to take decode_kernel (launch_decode) writes its own.
 // Calls layer by layer, us a call, with the barrier / so: 32 layers of 8 slices of 1640 bf16 rows, four heads, 11.5 / 10.7; 24 layers of
 // 32 fp16 slices of 450 rows, one head, 10.2 / 9.5; 5 layers of 24 fp32 slices of 180 rows 7.8 / 7.0.  (A release by every rank in
 // the place of the barrier: 11.4 and 9.9.)
