@@ -77,7 +77,12 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
 // One CTA per slice.  A chain of block-wide steps: what costs is the number of barriers and the serial pieces between
 // them (32 slices of 1200 tokens: 28 us when one thread walked through the 256 bins of every radix round and the
 // compaction scanned twice per 1024 positions).
-__global__ void __launch_bounds__(1024)
+//
+// Compiled for each number of threads (slice_threads), as is segment_kernel: with blockDim.x as the step of the compaction the
+// compiler gave this one 32 registers and spilled (52 before); with it in the tree of tau_0 that one became slower too.  us of
+// compression: 8 slices of 3908 bf16 rows 71.6, 40 of 1023 rows 49.2; so 63.3 and 45.4.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 2048 / kThreads)
 select_kernel(SelectArgs a) {
   start_dependents();
   wait_for_prior_grid();
@@ -149,7 +154,7 @@ select_kernel(SelectArgs a) {
   // Ordered compaction over positions, four per thread at a time.  One scan carries two counts: positions kept for certain (low half)
   // and positions equal to the N-th score (high half), of which the first need_eq are kept.
   int n_ret = 0, n_eq = 0;                        // before the current block: kept for certain, equal
-  for (int base = 0; base < P; base += kSelItems * (int)blockDim.x) {
+  for (int base = 0; base < P; base += kSelItems * kThreads) {
     const int j0 = base + threadIdx.x * kSelItems;
     int sure = 0, eq = 0;                         // bit i: position j0 + i
 #pragma unroll
@@ -381,7 +386,8 @@ struct SegArgs {
   float tau_override;
 };
 
-__global__ void __launch_bounds__(1024)
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 1)
 segment_kernel(SegArgs a) {
   start_dependents();
   wait_for_prior_grid();
@@ -407,16 +413,18 @@ segment_kernel(SegArgs a) {
   }
   // tau_0 = (1/Le) sum_i mx_i   (Eq. 10, t = 0); double accumulation, one reduction tree (that of 1024 threads) whatever the
   // number of threads
-  for (int v = threadIdx.x; v < 1024; v += blockDim.x) {
+  constexpr int kTurns = 1024 / kThreads;
+#pragma unroll 1
+  for (int u = 0; u < kTurns; ++u) {
     double t = 0.0;
-    for (int i = v; i < Le; i += 1024) t += (double)mx[i];
+    for (int i = u * kThreads + (int)threadIdx.x; i < Le; i += kTurns * (int)blockDim.x) t += (double)mx[i];
     t = warp_sum(t);
-    if (lane == 0) part[v >> 5] = t;
+    if (lane == 0) part[u * (kThreads / 32) + warp] = t;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < 32; ++w) s += part[w];
+    for (int w = 0; w < kTurns * (int)(blockDim.x >> 5); ++w) s += part[w];
     const float tau0 = (float)(s / (double)Le);
     a.tau[sidx] = tau0;
     s_thr = isnan(a.tau_override) ? tau0 : a.tau_override;
@@ -622,17 +630,16 @@ merge_kernel(MergeArgs a, LayerRows rows, T* __restrict__ kpool, T* __restrict__
 
 // ------------------------------------------------------------------------------------ launcher
 // Threads of a CTA of select_kernel and segment_kernel, which take one slice each.  A CTA is a chain of block-wide steps: more
-// threads shorten it, for as long as every thread has rows and every CTA a place at once (of select_kernel's, one of 1024 threads
-// fits an SM, two of 512, four of 256).  us of compression with 1024 / 512 / 256 threads; 160 slices of 450 rows 55 / 44.4 / 43.8, 800
-// 63.5 / 55.1 / 58.5, 3000 172 / 170 / 194, 6000 338 / 341 / 392; 256 of 450 rows 58 / 49.0 / 48.4, 2040 154 / 149 / 169, 4096 262 / 261 /
-// 301, 8192 689 / 696 / 771; 320 of 600 rows 79 / 62.5 / 59.6, 1000 108 / 93 / 95, 8192 854 / 850 / 898; 512 of 800 rows 131 / 107.7 /
-// 106.6, 1200 227 / 202 / 206, 12000 1469 / 1450 / 1497, 16384 2443 / 2460 / 2590; 1024 of 1200 rows 318 / 274 / 262, 4096 935 / 886 / 880; but
-// 64 of 3000 rows 146 / 155 with 512.
+// threads shorten it, for as long as every thread has rows and every CTA a place at once.  us of compression with 1024 / 512 / 256
+// threads: 160 slices of 450 rows 56 / 43.1 / 43.0, 500 56.8 / 44.6 / 46.6, 3000 172 / 166 / 188, 8192 480 / 480 / 528, 12000 610 / 618 / 679; 256
+// of 450 rows 61 / 48.6 / 47.7, 2040 156 / 146 / 163, 8192 686 / 684 / 749; 320 of 600 rows 81 / 61.4 / 59.1, 1000 111 / 92.0 / 92.0, 20000
+// 1902 / 1902 / 2048; 512 of 800 rows 137 / 106 / 103, 1200 234 / 199.1 / 199.6, 20000 2954 / 2942 / 3024; 1024 of 1200 rows 332 / 271 / 259,
+// 4096 941 / 882 / 869.
 static int slice_threads(const d2o_ctx* c, int n_ctas, int rows) {
   const int sms = c->n_sms;
   if (n_ctas <= sms) return 1024;
-  if (rows <= (n_ctas > 4 * sms ? 4096 : n_ctas > 2 * sms ? 800 : 450)) return 256;
-  return rows <= (n_ctas > 2 * sms ? 12288 : 5120) ? 512 : 1024;
+  if (rows <= (n_ctas > 4 * sms ? 4096 : n_ctas > 2 * sms ? 1024 : 450)) return 256;
+  return rows <= 8192 || n_ctas > 2 * sms ? 512 : 1024;
 }
 
 // Layers [layer, layer + n) in one launch per kernel; their working arrays are the first n sets of `scratch`.
@@ -677,12 +684,14 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   const bool sim_tc = sizeof(T) == 2 && c->similarity_path == 0;
   sa.generic_next = maxLe > 0 && !sim_tc;
   const size_t sel_sm = sa.keys_in_smem ? key_bytes : 0;
-  cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const int sel_threads = slice_threads(c, n_slices * n, P);
+  auto select = sel_threads == 1024 ? select_kernel<1024> : sel_threads == 512 ? select_kernel<512> : select_kernel<256>;
+  cudaError_t e = cudaFuncSetAttribute(select, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sel_sm > 48 * 1024 ? sel_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
   // Six kernels of a few microseconds each for a small batch: each may move in while the one ahead drains (one layer of 32
   // slices of 777 tokens 53 -> 42 us, 32 layers of 1200 tokens 1269 -> 1250 with the column sums; large batches as before).
-  e = launch_behind(select_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), slice_threads(c, n_slices * n, P), sel_sm, st, sa);
+  e = launch_behind(select, dim3((unsigned)n_slices, 1, (unsigned)n), sel_threads, sel_sm, st, sa);
   if (e != cudaSuccess) return e;
   {
     const int keep_max = min(maxS, P);
@@ -722,10 +731,11 @@ static cudaError_t run_prefill(const d2o_ctx* c, int layer, int n, const void* c
   // counts / cursors per retained slot, later the radix histograms (64 digits per warp)
   const int seg_threads = slice_threads(c, n_slices * n, maxLe);
   const size_t seg_sm = (size_t)max(maxS + 1, seg_threads / 32 * 64) * sizeof(int);
-  e = cudaFuncSetAttribute(segment_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  auto segment = seg_threads == 1024 ? segment_kernel<1024> : seg_threads == 512 ? segment_kernel<512> : segment_kernel<256>;
+  e = cudaFuncSetAttribute(segment, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(seg_sm > 48 * 1024 ? seg_sm : 48 * 1024));
   if (e != cudaSuccess) return e;
-  e = launch_behind(segment_kernel, dim3((unsigned)n_slices, 1, (unsigned)n), seg_threads, seg_sm, st, ga);
+  e = launch_behind(segment, dim3((unsigned)n_slices, 1, (unsigned)n), seg_threads, seg_sm, st, ga);
   if (e != cudaSuccess) return e;
 
   MergeArgs mg;

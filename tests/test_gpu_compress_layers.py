@@ -94,11 +94,11 @@ def test_more_slices_than_sms(dtype, P, rho):
     _run(wl, [(0, 20)], steps=2)
 
 
-@pytest.mark.parametrize("L,batch,P,rho", [(20, 2, 450, 0.2), (20, 2, 451, 0.2), (20, 2, 5120, 0.02), (20, 2, 5121, 0.02), (16, 3, 801, 0.1),
-                                           (16, 3, 12289, 0.01), (16, 5, 801, 0.1), (16, 5, 4097, 0.03)])
+@pytest.mark.parametrize("L,batch,P,rho", [(1, 5, 1023, 0.2), (1, 1, 3908, 0.1), (20, 2, 450, 0.2), (20, 2, 451, 0.2), (20, 2, 8192, 0.02),
+                                           (20, 2, 8193, 0.02), (16, 3, 1025, 0.1), (16, 3, 8193, 0.02), (16, 5, 1025, 0.1), (16, 5, 4097, 0.03)])
 def test_threads_per_slice(L, batch, P, rho):
     """Launches of more slices than the GPU has SMs, at the numbers of slices and rows where the threads per slice change, against a
-    layer at a time (1024 threads)."""
+    layer at a time (1024 threads); and few slices, for which both take 1024."""
     wl = dataclasses.replace(W.CONFIGS["cfg0"], n_layers=L, batch=batch, dtype="f16", prompt_len=P, rho=rho, decode_steps=1,
                              density_temp=50.0, min_budget=8, max_budget=0)
     _run(wl, [(0, L)], steps=1)
