@@ -98,7 +98,10 @@ __device__ __forceinline__ unsigned long long keys_extreme(const unsigned long l
 }
 
 // `a.row_cap`: rows per CTA the shared arrays are sized for (a multiple of kSplitPiece).
-template <typename T, int D, int G>
+// kPublish (DecodeArgs::publish): the step writes its own counters.  Compiled for either: with both paths in one kernel, and the
+// inputs asked into L2 for both, repeated and chained steps were slower (8 steps of 4 layers of 8 bf16 slices of 410 rows 100.7 -> 103.7
+// us, chained 99.4 -> 101.4; so 101.8 and 100.2; layer by layer, four tokens of 32 layers, 1370 -> 1345).
+template <typename T, int D, int G, bool kPublish>
 __global__ void __launch_bounds__(kSplitThreads, G <= 4 ? 2 : 1)
 decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const T* q_in, const T* k_in, const T* v_in, T* __restrict__ out,
@@ -129,7 +132,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   const T* v_new = v_in + (size_t)sl * D;
   // The inputs may still be on their way from the grid ahead and are not read before it is done, but their lines can be in L2 by
   // then.
-  if (a.early) {
+  if (!kPublish && a.early) {
     constexpr int kQ = G * D * (int)sizeof(T) / 128, kR = D * (int)sizeof(T) / 128;            // lines of the queries, of a row
     const char* line = tid < kQ ? reinterpret_cast<const char*>(q_in + (size_t)sl * G * D) + tid * 128
                      : tid < kQ + kR ? reinterpret_cast<const char*>(k_new) + (tid - kQ) * 128
@@ -360,7 +363,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   if (a.early && !a.chained) asm volatile("griddepcontrol.wait;" ::: "memory");
   // A wait of the grids ahead that ran out while this one waited for them: looked at again below, beside the key pass.  (Other
   // anomalies concern one slice and may be those of another cluster of this launch: its own token is dropped, no other.)
-  const uint32_t word = tid == 0 ? *reinterpret_cast<volatile uint32_t*>(a.status) : 0u;
+  const uint32_t word = a.early && !a.chained && tid == 0 ? *reinterpret_cast<volatile uint32_t*>(a.status) : 0u;
   if (a.pub_count > 0 && warp == kSplitWarps - 1 && blockIdx.x == gridDim.x - 1) {
     // the slices of the call before: its grid is done
     for (int i = lane; i < a.pub_count; i += 32)
@@ -682,9 +685,9 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
       }
     }
   };
-  if (!a.publish) send_outputs();
+  if (!kPublish) send_outputs();
   cluster_arrive();                                                       // barrier 2
-  if (a.publish) send_outputs();                                          // beside the barrier: there is another one
+  if (kPublish) send_outputs();                                           // beside the barrier: there is another one
   cluster_wait();
   if (any_bad(xch.bad2)) { leave(0xDEC10000u); return; }                  // the values did not arrive: nothing written yet
 
@@ -702,7 +705,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
       out[(size_t)sl * G * D + rank * share + i] = Elem<T>::from_float(t);
     }
   };
-  if (!a.publish) write_outputs(kSplitThreads - 1 - tid);                 // the first warp goes on to the merge
+  if (!kPublish) write_outputs(kSplitThreads - 1 - tid);                  // the first warp goes on to the merge
   if (!evict) vic_li = -1;
   if (evict && !none) {
     if (!D2O_GUARD(vic_li >= 0 && vic_li <= n_old, a.status, 0xC4EC0011u)) vic_li = n_old;
@@ -734,7 +737,7 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
     const int li = row_of(r);
     if ((li < old_cnt && r0 + li != vic_li) || (li == new_li && !evict)) a.score[row0 + r0 + li] = sc[r];
   }
-  if (a.publish) cluster_arrive();                                        // barrier 3
+  if (kPublish) cluster_arrive();                                         // barrier 3
   // ---- threshold, merge or discard (Eq. 10-12), the new token's row: by the CTA that holds the neighbour (or, while
   // the cache still fills, the new token)
   const bool writer = warp == 0 && !none && (evict ? max(nn_li, 0) : n_old) / chunk == rank;
@@ -801,15 +804,15 @@ decode_split_kernel(DecodeArgs a, const __grid_constant__ CUtensorMap map_k, con
   if (none && rank == 0 && tid == 0)                                      // drop the new token, keep the cache as it is
     report_error(a.status, D2O_ERR_STATE, 0xDEC00000u | (uint32_t)(sl & 0xfffff));
   hold();
-  if (a.publish) cluster_wait();                                          // barrier 3
+  if (kPublish) cluster_wait();                                           // barrier 3
   if (writer) {
     asm volatile("fence.proxy.async.global;" ::: "memory");
     __syncwarp();
     // every other CTA's stores to the state were ordered before barrier 3, this warp's before the release
-    if (lane == 0 && a.publish)
+    if (kPublish && lane == 0)
       asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.steps_done + sidx), "r"(a.step + 1) : "memory");
   }
-  if (a.publish) write_outputs(tid);
+  if (kPublish) write_outputs(tid);
 }
 
 // ------------------------------------------------------------------------------------ launch
@@ -861,7 +864,7 @@ int decode_split_cluster(const d2o_ctx* c, int n_slices, int max_rows, double to
 
 // Clusters of 2, 4, 8 and 16 CTAs that the current device holds at one CTA per SM.
 void decode_split_places(int* clusters) {
-  auto kern = decode_split_kernel<float, 128, 8>;
+  auto kern = decode_split_kernel<float, 128, 8, true>;
   const size_t smem = 150 * 1024;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   for (int i = 0; i < kSplitSizes; ++i) {
@@ -885,7 +888,7 @@ template <typename T, int D, int G>
 static cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, int C, int n_slices, const void* q, const void* k,
                               const void* v, void* out, void* kpool, void* vpool, cudaStream_t st) {
   const size_t smem = split_smem(a.row_cap, G, D, (int)sizeof(T));
-  auto kern = decode_split_kernel<T, D, G>;
+  auto kern = a.publish ? decode_split_kernel<T, D, G, true> : decode_split_kernel<T, D, G, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
