@@ -266,9 +266,9 @@ d2o_status d2o_full_decode_step(int32_t dtype, int32_t d_head, int32_t n_slices,
  *   colsum DEVICE float [B, Hq, P] (out: column sums of the causal prompt attention, Eq. 4);
  *   density DEVICE double [B, Hq] (out: F_v = Var(colsum) per query head).
  *
- * It runs the kernels that d2o_layer_stats runs with its default tuning (tensor cores for 16-bit
- * inputs, fp32 arithmetic on CUDA cores for fp32 inputs; any prompt length) and returns
- * bit-identical results.  It has no error word: should a device-side wait run out, the column sums
+ * Any prompt length.  It returns the results of d2o_layer_stats with its default tuning, bit for bit (full-length
+ * prompts): with 16-bit inputs it runs the same kernels (tensor cores); with fp32 inputs (CUDA cores) it computes the dot
+ * products a second time for the column sums, where d2o_layer_stats keeps them in its scratch and adds in the same order.  It has no error word: should a device-side wait run out, the column sums
  * concerned are NaN.
  *
  * Limit: batch * n_q_heads * prompt_len <= D2O_STATIC_LSE_FLOATS and batch * n_q_heads <= 65535,

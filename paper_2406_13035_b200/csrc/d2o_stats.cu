@@ -33,8 +33,8 @@ namespace cg = cooperative_groups;
 // lie in memory); tiles are copied as they are (cp.async, two buffers, one barrier per slab) into rows of d + 4 floats,
 // which keeps the 16-byte reads of both operands free of bank conflicts.  The FMA pipe is busy 55 - 60 % of the time (twelve
 // warps per SM wait for shared memory); 8 x 8 results on 64 threads were no faster for d = 64 and 25 % slower for d = 128.
-// fp32, both sweeps and the densities, one CTA per strip -> now: 8 heads of 1024 tokens 132 -> 70 us, of 100 tokens 29 -> 25;
-// 16 heads of 1500 tokens, d = 128, 675 -> 335; 8 layers of 32 heads of 1999 tokens 4.53 -> 3.94 ms.
+// fp32, both sweeps (no products stored) and the densities, one CTA per strip -> so: 8 heads of 1024 tokens 132 -> 66 us, of 100
+// tokens 29 -> 22; 16 heads of 1500 tokens, d = 128, 675 -> 334.
 constexpr int kTile = 64;             // rows and columns per tile
 constexpr int kStatThreads = 128;
 constexpr int kStripA = 8, kStripB = 4;   // results per thread: rows of the resident tile x rows of the streaming tile
@@ -244,9 +244,9 @@ sweep_kernel(const T* Q, const T* K, const float* lse_in, float* __restrict__ ou
   const int share = 2 * kTile / C;                    // results this CTA writes
   for (int i = threadIdx.x; i < share; i += kStatThreads) {
     const int e = rank * share + i, part = e / kTile, row = resident(part) * kTile + e % kTile;
-    // Summed in fp64 under the final maximum, so that the number of CTAs in the cluster adds no rounding.  One fp32 combination after
-    // another had errors of the column sums against fp64 of 8.9e-8 (32 heads, 500 tokens; relative, rms) and 9.5e-8 (16, 900); so: 8.5e-8
-    // and 8.9e-8.  The halves are read once, all at a time: the same 39.7 us at 16 x 700 and 139 us at 128 x 500 as one after another.
+    // Added in fp64 under the final maximum; the exponentials and products that bring the halves to it are fp32.  One fp32 combination
+    // after another had errors of the column sums against fp64 of 8.8e-8 (32 heads, 500 tokens; relative, rms) and 9.4e-8 (16, 900); so:
+    // 8.4e-8 and 8.9e-8.  The halves are read once, all at a time: the same 39.7 us at 16 x 700 and 139 us at 128 x 500 as one after another.
     double t = 0.0;
     float m = -INFINITY;
     if (kSum) {
@@ -278,8 +278,8 @@ sweep_kernel(const T* Q, const T* K, const float* lse_in, float* __restrict__ ou
 //
 // The row sweep is bound by its FMAs (one per element of d and logit); repeating them for the column sums took half of the call.
 // A logit costs 8 bytes of traffic instead (kStoredLogits: how many are kept at a time).  Row sweep, column sums and densities,
-// us, repeated / stored: 8 heads of 1024 tokens, d = 64, 70.5 / 50.2, of 100 tokens 24.7 / 22.6, of 450 tokens 33.3 / 26.7; 32
-// heads of 1999 tokens 539 / 371; six layers of 16 heads of 1500 tokens 893 / 576.
+// us, repeated / stored: 8 heads of 1024 tokens, d = 64, 65.8 / 48.7, of 100 tokens 21.7 / 19.3; 32 heads of 1999 tokens 525 / 365, 16 of
+// 1500, d = 128, 334 / 202; six layers of these 1686 / 1022.
 __global__ void __launch_bounds__(kStatThreads)
 colsum_stored_kernel(const float4* logits, const float* lse, float* __restrict__ out, int Pmax, int Hq, const int32_t* __restrict__ plen,
                      int head0, float mul) {

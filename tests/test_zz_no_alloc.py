@@ -3,8 +3,9 @@
 Some users of the library cannot call cudaMalloc while it runs: an inference server whose memory
 pool has taken the whole device, or a host application that passes tensors in but keeps its
 allocator to itself.  d2o_layer_stats_static serves them with a scratch array that lives inside
-the library image.  It runs the kernels of d2o_layer_stats, so the two agree bit for bit (checked
-for fp32 inputs and for a prompt length that is no multiple of 4) and within the parity tolerance,
+the library image.  It runs the kernels of d2o_layer_stats, or for fp32 inputs, whose dot products it cannot
+keep, other ones that add in the same order, so the two agree bit for bit (checked
+for fp32 inputs, at more lengths in test_gpu_colsum_lengths.py, and for a prompt length that is no multiple of 4) and within the parity tolerance,
 also on a second call that finds the first call's leftovers in the scratch array.
 The results are checked against the CPU oracle as well, and the free device memory must not move
 across the call.
@@ -57,7 +58,7 @@ def test_static_scratch_entry_matches_regular_entry(cuda_device, name, P, same_k
         assert free_after == free_before                 # nothing was allocated or freed on the device
         torch.testing.assert_close(cs, ref_cs, rtol=2e-4, atol=0)
         torch.testing.assert_close(F, ref_F, rtol=2e-4, atol=0)
-        if same_kernels:                                 # same kernels in the same order: bit-identical
+        if same_kernels:                                 # same kernels, or (fp32) the same order of the sums: bit-identical
             assert torch.equal(cs, ref_cs) and torch.equal(F, ref_F)
         # against the oracle, on two heads of the second sequence
         Qc, Kc = Q.cpu().double().numpy(), K.cpu().double().numpy()
