@@ -379,6 +379,25 @@ static int sweep_ctas(int P, int heads, int sms) {
   return C;
 }
 
+// The same for the column sweep by itself (the caller's normalisers): of the sizes 1, 2, 4 and 8 the one whose rounds are shortest.  A
+// round takes as long as the tiles of a CTA do (1.5 and 1.7 times as long with two and three CTAs per SM as with one) and 1.5
+// tiles to start and end.  us with the rule above / so: 32 heads of 896 tokens, where that leaves four CTAs for a second round,
+// 71.8 / 65.7, 22 of 896, d = 128, 102 / 87.7, 48 of 640, d = 128, 102 / 90.6, 12 of 1500 74.2 / 65.2, 32 of 1999 263 / 239, 28 of 832 51.3 / 51.3;
+// two layers side by side 12 of 1500 127 / 114, but 22 of 896 88 / 92 and 16 of 900 71 / 77.
+static int given_ctas(int P, int heads, int sms) {
+  const int nT = (P + kTile - 1) / kTile;
+  const long long units = (long long)((nT + 1) / 2) * heads;
+  static const int tile10[4] = {0, 10, 15, 17};
+  int best = 1;
+  long long shortest = -1;
+  for (int C = 1; C <= kMaxSweepCtas && (C == 1 || C <= nT + 1); C *= 2) {
+    const long long rounds = units * C / (3 * sms), rest = units * C % (3 * sms), tiles = (nT + C) / C;
+    const long long t = rounds * (17 * tiles + 15) + (rest > 0 ? tile10[(rest + sms - 1) / sms] * tiles + 15 : 0);
+    if (shortest < 0 || t < shortest) { shortest = t; best = C; }
+  }
+  return best;
+}
+
 // Bytes of logits that one of `lanes` lanes keeps: whole heads, for all lanes at most kStoredLogits; 0 where one head's
 // triangle is larger.  Fewer heads at a time mean more launches with a start and an end each, which weighs more than keeping
 // the logits in L2: 32 heads of 1999 tokens, one lane, 517 us with 32 MB, 437 with 64, 367 with 256 (in another order of the sums).
@@ -458,7 +477,7 @@ static cudaError_t launch_sweeps(const T* Q, const T* K, const float* lse, float
   const bool own = lse == nullptr;
   int dev = 0, sms = kB200Sms;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) (void)cudaGetLastError();
-  const int heads = B * Hq, C = sweep_ctas(P, heads, sms);
+  const int heads = B * Hq, C = own ? sweep_ctas(P, heads, sms) : given_ctas(P, heads, sms);
   const int fit = (int)std::min<size_t>(heads, logits_bytes / stored_head_bytes(P));
   cudaError_t e;
   if (own && stored_pays(P, D, heads, fit, lanes, sms)) {

@@ -105,6 +105,19 @@ def test_fp32_colsum_bits_whoever_computes_them(cuda_device, b, hq, hkv, d, P, L
     ctx.close()
 
 
+@pytest.mark.parametrize("h,d,P", [(32, 64, 896), (22, 128, 896), (12, 64, 1500), (64, 64, 500), (2, 64, 1999), (5, 128, 7)])
+def test_fp32_given_normalisers_with_every_cluster_size(cuda_device, h, d, P):
+    """The column sweep by itself, with one, two, four and eight CTAs to a pair of strips."""
+    g = torch.Generator(device=cuda_device).manual_seed(P)
+    Q = 1.5 * torch.randn(1, h, P, d, generator=g, device=cuda_device)
+    K = torch.randn(1, h, P, d, generator=g, device=cuda_device)
+    logits, ref = _reference(Q, K)
+    ctx = _context("f32", 1, h, h, d, P)
+    ctx.d2o_layer_stats(0, Q, K, torch.logsumexp(logits, -1).float().contiguous())
+    assert float(((ctx.colsum(0).double() - ref).abs() / ref).max()) < 2e-5
+    ctx.close()
+
+
 @pytest.mark.parametrize("d,P,key", [(64, 100, 97), (64, 65, 3), (128, 449, 448), (64, 128, 70)])
 def test_fp32_keys_with_infinite_elements(cuda_device, d, P, key):
     """A key whose logits are all -inf: its column is 0, every other one is as without it, and nothing comes from the rows past the
